@@ -310,7 +310,10 @@ typedef struct {
                                         items to balance a tree with few refined
                                         nodes, the halo staged twice); 0 = 2 when the
                                         tree has fewer refined nodes than twice the
-                                        kernel's resident CTAs, else 1.  Same results. */
+                                        kernel's resident CTAs, else 1.  FMM_FP64 and
+                                        FMM_DFLOAT take half of that: 1 a half, 2 a
+                                        quarter, 0 = 2 below eight refined nodes per SM.
+                                        Same results. */
     int32_t reserved;
 } fmm_tuning;
 

@@ -125,22 +125,33 @@ __device__ __forceinline__ dfloat add_u(dfloat a, dfloat b)
     df_two_sum(a.hi, b.hi, s, e);
     return dfloat(s, e + (a.lo + b.lo));
 }
+// a product likewise: the high part is the rounded product of the high
+// parts, the low part its error and the cross terms (within a few half ulps
+// of the high part), which is all that a further product needs
+__device__ __forceinline__ dfloat mul_u(dfloat a, dfloat b)
+{
+    const float p = a.hi * b.hi;
+    float e = fmaf(a.hi, b.hi, -p);
+    e = fmaf(a.hi, b.lo, e);
+    return dfloat(p, fmaf(a.lo, b.hi, e));
+}
 __device__ __forceinline__ dfloat renorm(dfloat a) { return df_fast(a.hi, a.lo); }
 
 __device__ __forceinline__ dfloat &operator+=(dfloat &a, dfloat b) { return a = a + b; }
 __device__ __forceinline__ dfloat &operator-=(dfloat &a, dfloat b) { return a = a - b; }
 __device__ __forceinline__ dfloat &operator*=(dfloat &a, dfloat b) { return a = a * b; }
 
-// 1/sqrt(v): the float estimate y refined by one Newton step for
-// f(y) = 1/y^2 - v, y' = y + y (1 - v y^2) / 2; the residual 1 - v y^2 is
-// formed in double-float (y^2 exactly), which doubles the estimate's bits
+// 1/sqrt(v): the float estimate y corrected by the binomial series of
+// (1 - e)^(-1/2) = 1 + e/2 + 3 e^2/8 + ..., e = 1 - v y^2, formed in
+// double-float (y^2 exactly; 1 - t.hi is exact, t being 1 to a few float
+// ulps).  With the first-order term alone the truncation, always of one sign,
+// was the largest error of an interaction (3/8 e^2, about 2^-45).
 __device__ __forceinline__ dfloat df_rsqrt(dfloat v)
 {
     const float y = rsqrtf(v.hi);
     const dfloat t = v * df_two_prod(y, y);
-    const dfloat res = dfloat(1.f) - t;
-    const float c = 0.5f * y * (res.hi + res.lo);
-    return df_fast(y, c);
+    const float e = (1.f - t.hi) - t.lo;
+    return df_fast(y, y * fmaf(0.375f * e, e, 0.5f * e));
 }
 
 }  // namespace fmm

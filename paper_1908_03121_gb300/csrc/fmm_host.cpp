@@ -355,6 +355,12 @@ static void slot_tables(const fmm_tree_s *t, std::vector<int64_t> &tab)
 // 3 + 51 + 18 + 30 -> 102.
 static const double kFlops[4] = {240.0, 176.0, 8.0, 199.0};
 static const double kFlops2[4] = {125.0, 107.0, 8.0, 102.0};
+// The FP64 and double-float kernels sum moments of the separations instead
+// (fmm_wide.cuh): multipole<-monopole 29 + 33 fused (95), multipole<-multipole
+// three more for the offset and 85 for the moments (183), monopole<-multipole
+// 113; order 2: 62, 103 and 65.
+static const double kFlopsWide[4] = {183.0, 95.0, 8.0, 113.0};
+static const double kFlopsWide2[4] = {103.0, 62.0, 8.0, 65.0};
 
 // Monopole<-multipole work as pair lists: for every cell of a leaf node next
 // to a refined node, the stencil entries whose source cell is refined, each
@@ -821,9 +827,12 @@ int fmm_get_stats(fmm_tree_t t, fmm_stats *o)
     if (!t || !o) return fail(FMM_ERR_INVALID_ARG, "NULL argument");
     std::memset(o, 0, sizeof *o);
     const Plan &P = t->plan;
+    const bool o2 = t->cfg.order == 2;
+    const double *flops = t->cfg.precision == FMM_MIXED ? (o2 ? kFlops2 : kFlops)
+                                                        : (o2 ? kFlopsWide2 : kFlopsWide);
     for (int k = 0; k < 4; ++k) {
         o->interactions[k] = P.interactions[k];
-        o->flops_per_interaction[k] = t->cfg.order == 2 ? kFlops2[k] : kFlops[k];
+        o->flops_per_interaction[k] = flops[k];
     }
     o->stencil_far = P.n_far[0];
     o->stencil_near = P.n_near[0];

@@ -36,12 +36,14 @@
 // floats, fmm_dfloat.cuh) evaluate offsets, derivative tensors, contraction
 // and sums in double-float, so each pair's contributions to A and to B cancel
 // in momentum and angular momentum to about 1e-13, as in FP64.
+#include <algorithm>
 #include <cstdio>
 #include <type_traits>
 
 #include "fmm_convert.cuh"
 #include "fmm_internal.h"
 #include "fmm_tensor.cuh"
+#include "fmm_wide.cuh"
 
 namespace fmm {
 
@@ -149,7 +151,10 @@ __device__ __forceinline__ void pack_float(const NodeInfo &ni, const double *__r
 //   g0 = (delta, M0), delta = (X - centre) / h (first, so that its x and y
 //        land in an aligned register pair for the paired FP32 subtraction),
 //   g1 = B2[0..3], g2 = (B2[4], B3[0..2]), g3 = B3[3..6],
-// the traceless projections of A2 = mult M2 / (2 h^2), A3 = mult M3 / (6 h^3).
+// float: the traceless projections of A2 = mult M2 / (2 h^2),
+// A3 = mult M3 / (6 h^3); double-float and double: the traceless parts
+// themselves, t2 = (3/2) T2 / h^2 (xx yy xy xz yz) and t3 = (5/2) T3 / h^3 (xxx
+// xxy xxz xyy xyz yyy yyz), see fmm_wide.cuh.
 template <typename T>
 __global__ void __launch_bounds__(512) pack_kernel(const NodeInfo *__restrict__ info,
                                                    const int32_t *__restrict__ nodes,
@@ -179,17 +184,34 @@ __global__ void __launch_bounds__(512) pack_kernel(const NodeInfo *__restrict__ 
     double d[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) d[a] = (com[(size_t(node) * 3 + a) * NCELL + c] - ctr[a]) * ih;
-    const double w2 = 0.5 * ih * ih, w3 = (1.0 / 6.0) * ih * ih * ih;
-    double A2[6], A3[10];
+    // traceless parts: T2 = M2 - delta tr/3, T3 = M3 - (delta v, three terms)/5
+    // with v_k = M3_iik; symmetric order M2 xx xy xz yy yz zz, M3 xxx xxy xxz
+    // xyy xyz xzz yyy yyz yzz zzz
+    const double w2 = 1.5 * ih * ih, w3 = 2.5 * ih * ih * ih;
+    double m2[6], m3[10];
 #pragma unroll
-    for (int q = 0; q < 6; ++q) A2[q] = mult2(q) * w2 * Mn[(4 + q) * NCELL];
+    for (int q = 0; q < 6; ++q) m2[q] = Mn[(4 + q) * NCELL];
 #pragma unroll
-    for (int q = 0; q < 10; ++q) A3[q] = mult3(q) * w3 * Mn[(10 + q) * NCELL];
-    // symmetric order: A2 xx xy xz yy yz zz; A3 xxx xxy xxz xyy xyz xzz yyy yyz yzz zzz
-    const double v[16] = {d[0],          d[1],          d[2],          Mn[0],
-                          A2[0] - A2[5], A2[3] - A2[5], A2[1],         A2[2],
-                          A2[4],         A3[0] - A3[5], A3[1] - A3[8], A3[2] - A3[9],
-                          A3[3] - A3[5], A3[4],         A3[6] - A3[8], A3[7] - A3[9]};
+    for (int q = 0; q < 10; ++q) m3[q] = Mn[(10 + q) * NCELL];
+    const double tr = (m2[0] + m2[3] + m2[5]) * (1.0 / 3.0);
+    const double vx = 0.2 * (m3[0] + m3[3] + m3[5]), vy = 0.2 * (m3[1] + m3[6] + m3[8]),
+                 vz = 0.2 * (m3[2] + m3[7] + m3[9]);
+    const double v[16] = {d[0],
+                          d[1],
+                          d[2],
+                          Mn[0],
+                          w2 * (m2[0] - tr),
+                          w2 * (m2[3] - tr),
+                          w2 * m2[1],
+                          w2 * m2[2],
+                          w2 * m2[4],
+                          w3 * (m3[0] - 3.0 * vx),
+                          w3 * (m3[1] - vy),
+                          w3 * (m3[2] - vz),
+                          w3 * (m3[3] - vx),
+                          w3 * m3[4],
+                          w3 * (m3[6] - 3.0 * vy),
+                          w3 * (m3[7] - vz)};
     T *out = mp + (size_t(ni.mp_row) * 4 * NCELL + pi) * 4;
 #pragma unroll
     for (int g = 0; g < 4; ++g)
@@ -475,16 +497,7 @@ __device__ __forceinline__ float acc_lo(const SmemAcc<N, NC> &a, int k)
     return k < NC ? a.col[(k * 2 + 1) * kThreads] : 0.f;
 }
 
-// the multipole kernel's accumulators: for float, shared-memory pairs for
-// orders 0-1 and the correction
-template <typename T, int N>
-struct MpAcc {
-    using type = Acc<T, N>;
-};
-template <int N>
-struct MpAcc<float, N> {
-    using type = SmemAcc<N, N == 16 ? 4 : N>;
-};
+// (the multipole kernel keeps shared-memory pairs for orders 0-1 and the correction)
 constexpr int kMpPairs = 4 + 3;      // compensated float components of mp_kernel
 
 // store component k of a target cell: level units; (hi, lo) float pairs for
@@ -540,16 +553,16 @@ __device__ __forceinline__ void store_target_values(const KParams &P, int node, 
     store_neg_sum<T>(P, node, 19, cell, hi, lo, 11, 15);   // zzz = -(xxz + yyz)
 }
 
-template <typename T, class LA>
+template <class LA>
 __device__ __forceinline__ void store_target(const KParams &P, int node, int cell, const LA &L)
 {
-    T hi[16], lo[16];
+    float hi[16], lo[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
         hi[k] = acc_hi(L, k);
         lo[k] = acc_lo(L, k);
     }
-    store_target_values<T>(P, node, cell, hi, lo);
+    store_target_values<float>(P, node, cell, hi, lo);
 }
 
 // packed data of one source cell (level units)
@@ -576,12 +589,11 @@ __device__ __forceinline__ void load4(const T *p, T v[4])
     }
 }
 
-template <typename T>
-__device__ __forceinline__ void load_source_at(const T *base, Src<T> &s)
+__device__ __forceinline__ void load_source_at(const float *base, Src<float> &s)
 {
-    T v[16];
+    float v[16];
 #pragma unroll
-    for (int g = 0; g < 4; ++g) load4<T>(base + size_t(g) * NCELL * 4, v + 4 * g);
+    for (int g = 0; g < 4; ++g) load4<float>(base + size_t(g) * NCELL * 4, v + 4 * g);
     s.d[0] = v[0]; s.d[1] = v[1]; s.d[2] = v[2];
     s.m0 = v[3];
 #pragma unroll
@@ -590,20 +602,33 @@ __device__ __forceinline__ void load_source_at(const T *base, Src<T> &s)
     for (int q = 0; q < 7; ++q) s.B3[q] = v[9 + q];
 }
 
+// the same for the wide types; base also names the zero row of leaf sources
 template <typename T>
-__device__ __forceinline__ void load_source(const KParams &P, int row, int pi, Src<T> &s)
+__device__ __forceinline__ void load_wide(const T *base, WideSrc<T> &s)
 {
-    load_source_at<T>(static_cast<const T *>(P.mp) + (size_t(row) * 4 * NCELL + pi) * 4, s);
+    T v[16];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) load4<T>(base + size_t(g) * NCELL * 4, v + 4 * g);
+    s.d[0] = v[0]; s.d[1] = v[1]; s.d[2] = v[2];
+    s.m0 = v[3];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) s.t2[k] = v[4 + k];
+#pragma unroll
+    for (int q = 0; q < 7; ++q) s.t3[q] = v[9 + q];
 }
 
-template <typename T>
-__device__ __forceinline__ void zero_moments(Src<T> &s)
+__device__ __forceinline__ void load_source(const KParams &P, int row, int pi, Src<float> &s)
 {
-    s.d[0] = s.d[1] = s.d[2] = T(0);
+    load_source_at(static_cast<const float *>(P.mp) + (size_t(row) * 4 * NCELL + pi) * 4, s);
+}
+
+__device__ __forceinline__ void zero_moments(Src<float> &s)
+{
+    s.d[0] = s.d[1] = s.d[2] = 0.f;
 #pragma unroll
-    for (int k = 0; k < 5; ++k) s.B2[k] = T(0);
+    for (int k = 0; k < 5; ++k) s.B2[k] = 0.f;
 #pragma unroll
-    for (int q = 0; q < 7; ++q) s.B3[q] = T(0);
+    for (int q = 0; q < 7; ++q) s.B3[q] = 0.f;
 }
 
 // One source (multipole if SRC_MP, else a point mass m0 = s.m0) into a
@@ -612,63 +637,55 @@ __device__ __forceinline__ void zero_moments(Src<T> &s)
 // with the sign of L folded in:
 //   L0 -= M0 D0 + B2.D2 - B3.D3,  L1_i -= M0 D1_i + B2.D3[i,.],
 //   L2 -= M0 D2,  L3 -= M0 D3.
-// Orders 0 and 1 (potential and field) sum each source's terms first and
-// add that sum to the chunk sum once, so every source costs one rounding at
-// the chunk sum's magnitude; orders 2-3 and the correction take each product
-// straight into their sums as one fused multiply-add.
+// Every product goes straight into its chunk sum as one fused multiply-add.
 //
 // Expansion order 2 (ORDER = 2; truncation n + m <= 2): L0 -= M0 D0 + B2.D2,
 // L1 -= M0 D1, L2 -= M0 D2, no L3, and the correction is the dropped
 // n = 1, m = 2 term with the target's share added (D3 is odd):
 //   S_i -= sum_k (B2_B + M0_B a2_A)_k D3[i, k],  a2_A = B2_A / M0_A
 // (aA holds a2_A in its first five entries then).
-template <typename T, bool SRC_MP, int ORDER = 3, class LA, class SA>
-__device__ __forceinline__ void acc_mp(T Rx, T Ry, T Rz, const Src<T> &s, const T aA[7], LA &L,
-                                       SA &S)
+template <bool SRC_MP, int ORDER = 3, class LA, class SA>
+__device__ __forceinline__ void acc_mp(float Rx, float Ry, float Rz, const Src<float> &s,
+                                       const float aA[7], LA &L, SA &S)
 {
-    DTraceless<T> D;
-    D.template eval<ORDER == 3>(Rx, Ry, Rz);
-    const T nm0 = -s.m0;
-    // float: each term straight into the chunk sum (one fused multiply-add
-    // per term); double-float and double: each source's terms summed first
-    T a = kF32<T> ? fmadd(nm0, D.D0, L.part[0]) : nm0 * D.D0;
+    DTraceless D;
+    D.eval<ORDER == 3>(Rx, Ry, Rz);
+    const float nm0 = -s.m0;
+    float a = fmaf(nm0, D.D0, L.part[0]);
     if (SRC_MP) {
 #pragma unroll
-        for (int k = 0; k < 5; ++k) a = fmadd_u(-s.B2[k], D.D2[k], a);
+        for (int k = 0; k < 5; ++k) a = fmaf(-s.B2[k], D.D2[k], a);
         if (ORDER == 3) {
 #pragma unroll
-            for (int q = 0; q < 7; ++q) a = fmadd_u(s.B3[q], D.D3[q], a);
+            for (int q = 0; q < 7; ++q) a = fmaf(s.B3[q], D.D3[q], a);
         }
     }
-    L.part[0] = kF32<T> ? a : add_u(L.part[0], renorm(a));
+    L.part[0] = a;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        T b = kF32<T> ? fmadd(nm0, D.D1[i], L.part[1 + i]) : nm0 * D.D1[i];
+        float b = fmaf(nm0, D.D1[i], L.part[1 + i]);
         if (SRC_MP && ORDER == 3) {
 #pragma unroll
-            for (int k = 0; k < 5; ++k) b = fmadd_u(-s.B2[k], D.d3slice(i, k), b);
+            for (int k = 0; k < 5; ++k) b = fmaf(-s.B2[k], D.d3slice(i, k), b);
         }
-        L.part[1 + i] = kF32<T> ? b : add_u(L.part[1 + i], renorm(b));
+        L.part[1 + i] = b;
     }
     if constexpr (ORDER == 2) {
 #pragma unroll
-        for (int k = 0; k < 5; ++k) L.part[4 + k] = fmadd_u(nm0, D.D2[k], L.part[4 + k]);
-        T wn[5];
+        for (int k = 0; k < 5; ++k) L.part[4 + k] = fmaf(nm0, D.D2[k], L.part[4 + k]);
+        float wn[5];
 #pragma unroll
-        for (int k = 0; k < 5; ++k) wn[k] = SRC_MP ? fmadd(nm0, aA[k], -s.B2[k]) : nm0 * aA[k];
+        for (int k = 0; k < 5; ++k) wn[k] = SRC_MP ? fmaf(nm0, aA[k], -s.B2[k]) : nm0 * aA[k];
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            T c = S.part[i];
+            float c = S.part[i];
 #pragma unroll
-            for (int k = 0; k < 5; ++k) c = fmadd_u(wn[k], D.d3slice(i, k), c);
-            S.part[i] = renorm(c);
+            for (int k = 0; k < 5; ++k) c = fmaf(wn[k], D.d3slice(i, k), c);
+            S.part[i] = c;
         }
-        return;
-    }
-    const T *a3A = aA;
-    if constexpr (kF32<T>) {
+    } else {
         // orders 2-3 (12 components): the pairs in which the derivative
-        // tensors come out of DTraceless<float> (xx yy | xz yz of D2, xxx yyy
+        // tensors come out of DTraceless (xx yy | xz yz of D2, xxx yyy
         // | xxz yyz of D3) on the paired FP32 pipe (fma.rn.f32x2: each half
         // rounds as fmaf does), the other four scalar
         constexpr int pair_a[4] = {4, 7, 9, 11}, pair_b[4] = {5, 8, 14, 15};
@@ -688,86 +705,75 @@ __device__ __forceinline__ void acc_mp(T Rx, T Ry, T Rz, const Src<T> &s, const 
         L.part[10] = fmaf(nm0, dv[10], L.part[10]);
         L.part[12] = fmaf(nm0, dv[12], L.part[12]);
         L.part[13] = fmaf(nm0, dv[13], L.part[13]);
-    } else {
+        float w[7];
 #pragma unroll
-        for (int k = 0; k < 5; ++k) L.part[4 + k] = fmadd_u(nm0, D.D2[k], L.part[4 + k]);
+        for (int q = 0; q < 7; ++q) w[q] = SRC_MP ? fmaf(nm0, aA[q], s.B3[q]) : nm0 * aA[q];
 #pragma unroll
-        for (int q = 0; q < 7; ++q) L.part[9 + q] = fmadd_u(nm0, D.D3[q], L.part[9 + q]);
-    }
-    T w[7];
+        for (int i = 0; i < 3; ++i) {
+            float c = S.part[i];
 #pragma unroll
-    for (int q = 0; q < 7; ++q) w[q] = SRC_MP ? fmadd(nm0, a3A[q], s.B3[q]) : nm0 * a3A[q];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        T c = S.part[i];
-#pragma unroll
-        for (int q = 0; q < 7; ++q) c = fmadd_u(w[q], D.U[i][q], c);
-        S.part[i] = renorm(c);
+            for (int q = 0; q < 7; ++q) c = fmaf(w[q], D.U[i][q], c);
+            S.part[i] = c;
+        }
     }
 }
 
 // One multipole source into a leaf target (orders 0-1 and the correction;
 // the target has no third moment)
 // (ORDER = 2: L0 -= M0 D0 + B2.D2, L1 -= M0 D1, S_i -= B2 . D3[i, .])
-template <typename T, int ORDER = 3>
-__device__ __forceinline__ void acc_mx(T Rx, T Ry, T Rz, const Src<T> &s, Acc<T, 4> &L,
-                                       Acc<T, 3> &S)
+template <int ORDER = 3>
+__device__ __forceinline__ void acc_mx(float Rx, float Ry, float Rz, const Src<float> &s,
+                                       Acc<float, 4> &L, Acc<float, 3> &S)
 {
-    DTraceless<T> D;
-    D.template eval<ORDER == 3>(Rx, Ry, Rz);
-    T a = -s.m0 * D.D0;
+    DTraceless D;
+    D.eval<ORDER == 3>(Rx, Ry, Rz);
+    float a = -s.m0 * D.D0;
 #pragma unroll
-    for (int k = 0; k < 5; ++k) a = fmadd_u(-s.B2[k], D.D2[k], a);
+    for (int k = 0; k < 5; ++k) a = fmaf(-s.B2[k], D.D2[k], a);
     if (ORDER == 3) {
 #pragma unroll
-        for (int q = 0; q < 7; ++q) a = fmadd_u(s.B3[q], D.D3[q], a);
+        for (int q = 0; q < 7; ++q) a = fmaf(s.B3[q], D.D3[q], a);
     }
-    L.part[0] = add_u(L.part[0], renorm(a));
+    L.part[0] = L.part[0] + a;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        T b = -s.m0 * D.D1[i];
-        T c = S.part[i];
-        if (ORDER == 3) {
+        float b = -s.m0 * D.D1[i];
+        float c = S.part[i];
+        if constexpr (ORDER == 3) {
 #pragma unroll
-            for (int k = 0; k < 5; ++k) b = fmadd_u(-s.B2[k], D.d3slice(i, k), b);
+            for (int k = 0; k < 5; ++k) b = fmaf(-s.B2[k], D.d3slice(i, k), b);
 #pragma unroll
-            for (int q = 0; q < 7; ++q) c = fmadd_u(s.B3[q], D.U[i][q], c);
+            for (int q = 0; q < 7; ++q) c = fmaf(s.B3[q], D.U[i][q], c);
         } else {
 #pragma unroll
-            for (int k = 0; k < 5; ++k) c = fmadd_u(-s.B2[k], D.d3slice(i, k), c);
+            for (int k = 0; k < 5; ++k) c = fmaf(-s.B2[k], D.d3slice(i, k), c);
         }
-        L.part[1 + i] = add_u(L.part[1 + i], renorm(b));
-        S.part[i] = renorm(c);
+        L.part[1 + i] = L.part[1 + i] + b;
+        S.part[i] = c;
     }
 }
 
 // target-to-source separation in cell widths, R = (dA - d) - E, in that
-// order; float takes x and y as one pair (the offsets' x and y sit in
+// order; x and y go as one pair (the offsets' x and y sit in
 // aligned register pairs: first in their 16-byte groups)
-template <typename T>
-__device__ __forceinline__ void separation(const T dA[3], const T d[3], const float4 &E, T R[3])
+__device__ __forceinline__ void separation(const float dA[3], const float d[3], const float4 &E,
+                                           float R[3])
 {
-    if constexpr (kF32<T>) {
-        const float2 u = fsub2_rn(make_float2(dA[0], dA[1]), make_float2(d[0], d[1]));
-        const float2 r = fsub2_rn(u, make_float2(E.x, E.y));
-        R[0] = r.x;
-        R[1] = r.y;
-        R[2] = dA[2] - d[2] - E.z;
-    } else {
-        R[0] = dA[0] - d[0] - T(E.x);
-        R[1] = dA[1] - d[1] - T(E.y);
-        R[2] = dA[2] - d[2] - T(E.z);
-    }
+    const float2 u = fsub2_rn(make_float2(dA[0], dA[1]), make_float2(d[0], d[1]));
+    const float2 r = fsub2_rn(u, make_float2(E.x, E.y));
+    R[0] = r.x;
+    R[1] = r.y;
+    R[2] = dA[2] - d[2] - E.z;
 }
 
 // own packed data of a multipole target: centre-of-mass offset and
 // a3 = B3/M0 (order 3) or a2 = B2/M0 in the first five entries (order 2)
-template <typename T, int ORDER = 3>
-__device__ __forceinline__ void load_target(const KParams &P, int row, int pi, T dA[3], T aA[7])
+template <int ORDER = 3>
+__device__ __forceinline__ void load_target(const KParams &P, int row, int pi, float dA[3], float aA[7])
 {
-    Src<T> own;
-    load_source<T>(P, row, pi, own);
-    const T im0 = T(1) / own.m0;
+    Src<float> own;
+    load_source(P, row, pi, own);
+    const float im0 = 1.f / own.m0;
 #pragma unroll
     for (int a = 0; a < 3; ++a) dA[a] = own.d[a];
     if (ORDER == 3) {
@@ -776,7 +782,7 @@ __device__ __forceinline__ void load_target(const KParams &P, int row, int pi, T
     } else {
 #pragma unroll
         for (int q = 0; q < 5; ++q) aA[q] = own.B2[q] * im0;
-        aA[5] = aA[6] = T(0);
+        aA[5] = aA[6] = 0.f;
     }
 }
 
@@ -784,7 +790,7 @@ __device__ __forceinline__ double to_double(float v) { return double(v); }
 __device__ __forceinline__ double to_double(double v) { return v; }
 __device__ __forceinline__ double to_double(dfloat v) { return v.to_double(); }
 
-template <typename T, class SA>
+template <class SA>
 __device__ __forceinline__ double acc_value(const SA &S, int i)
 {
     return to_double(acc_hi(S, i)) + to_double(acc_lo(S, i));
@@ -802,8 +808,9 @@ __device__ __forceinline__ void mx_target(const KParams &P, int t)
     const int x = tg.y & 7, y = (tg.y >> 3) & 7, z = tg.y >> 6;
     const int p = (x & 1) + 2 * (y & 1) + 4 * (z & 1);
     const float4 *ent = P.stencil_f + p * P.ent_stride;   // float offsets: no conversions
-    Acc<T, 4> L;
-    Acc<T, 3> S;
+    using Low = std::conditional_t<kF32<T>, Acc<float, 4>, WideChunked<T, WideLow<T, ORDER>>>;
+    Low L;
+    Acc<float, 3> S;                               // float only
     L.zero();
     S.zero();
     int done = 0;
@@ -815,9 +822,16 @@ __device__ __forceinline__ void mx_target(const KParams &P, int t)
         const int2 pr = next;
         if (k + 1 < tg.w) next = __ldg(pairs + size_t(k + 1) * 32);
         const float4 E = __ldg(ent + pr.y);
-        Src<T> src;
-        load_source_at<T>(mp + pr.x, src);
-        acc_mx<T, ORDER>(-T(E.x) - src.d[0], -T(E.y) - src.d[1], -T(E.z) - src.d[2], src, L, S);
+        if constexpr (kF32<T>) {
+            Src<float> src;
+            load_source_at(mp + pr.x, src);
+            acc_mx<ORDER>(-E.x - src.d[0], -E.y - src.d[1], -E.z - src.d[2], src, L, S);
+        } else {
+            WideSrc<T> src;
+            load_wide<T>(mp + pr.x, src);
+            wide_add_leaf<T, ORDER>(wide_sep(T(0), src.d[0], E.x), wide_sep(T(0), src.d[1], E.y),
+                                    wide_sep(T(0), src.d[2], E.z), src, L.part);
+        }
         if (++done == kChunk) {
             L.flush();
             S.flush();
@@ -827,10 +841,10 @@ __device__ __forceinline__ void mx_target(const KParams &P, int t)
     L.flush();
     S.flush();
     const int node = tg.x, cell = tg.y;
+    if constexpr (kF32<T>) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const size_t idx = (size_t(node) * NCOMP + k) * NCELL + cell;
-        if constexpr (kF32<T>) {
+        for (int k = 0; k < 4; ++k) {
+            const size_t idx = (size_t(node) * NCOMP + k) * NCELL + cell;
             float *Lh = static_cast<float *>(P.L);
             float s, e;
             two_sum(Lh[idx], L.hi[k], s, e);
@@ -838,38 +852,51 @@ __device__ __forceinline__ void mx_target(const KParams &P, int t)
             const float s2 = s + lo;
             Lh[idx] = s2;
             P.Lc[idx] = lo - (s2 - s);
-        } else if constexpr (kDF<T>) {
-            float *Lh = static_cast<float *>(P.L);
-            const dfloat v = dfloat(Lh[idx], P.Lc[idx]) + L.part[k];
-            Lh[idx] = v.hi;
-            P.Lc[idx] = v.lo;
-        } else {
-            static_cast<double *>(P.L)[idx] += L.hi[k];
         }
-    }
 #pragma unroll
-    for (int i = 0; i < 3; ++i) P.dL1[(size_t(node) * 3 + i) * NCELL + cell] = acc_value<T>(S, i);
+        for (int i = 0; i < 3; ++i)
+            P.dL1[(size_t(node) * 3 + i) * NCELL + cell] = acc_value(S, i);
+    } else {
+        const WideLow<T, ORDER> &A = L.total();
+        const T v[4] = {-A.a0, A.a1[0], A.a1[1], A.a1[2]};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const size_t idx = (size_t(node) * NCOMP + k) * NCELL + cell;
+            if constexpr (kDF<T>) {
+                float *Lh = static_cast<float *>(P.L);
+                const dfloat w = dfloat(Lh[idx], P.Lc[idx]) + v[k];
+                Lh[idx] = w.hi;
+                P.Lc[idx] = w.lo;
+            } else {
+                static_cast<double *>(P.L)[idx] += v[k];
+            }
+        }
+        T c[3];
+        A.correction(c);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) P.dL1[(size_t(node) * 3 + i) * NCELL + cell] = to_double(c[i]);
+    }
 }
 
 // ------------------------------------------------------------ mp_kernel
 // HALVES: item k is half k & 1 (cells of z < 4 or z >= 4) of node list[k >> 1],
 // else item k is all of node list[k]
-template <typename T, int ORDER, bool HALVES>
+template <int ORDER, bool HALVES>
 // float: three CTAs per SM (at most 85 registers): the compensation pairs,
 // touched once per chunk, live in shared memory after the window
-__global__ void __launch_bounds__(kThreads, kF32<T> ? 3 : 1) mp_kernel(KParams P)
+__global__ void __launch_bounds__(kThreads, 3) mp_kernel(KParams P)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *W = reinterpret_cast<T *>(smem_raw);
-    float *Cs = reinterpret_cast<float *>(W + 8 * P.sub_stride) + threadIdx.x;   // float only
+    float *W = reinterpret_cast<float *>(smem_raw);
+    float *Cs = W + 8 * P.sub_stride + threadIdx.x;
     __shared__ int s_nbr[27], s_leaf[27], s_row[27], s_item;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int p = warp;
     const int px = p & 1, py = (p >> 1) & 1, pz = p >> 2;
     const int cx = lane & 3, cy = (lane >> 2) & 3, cz0 = lane >> 4;
     const float4 *ent = P.stencil_f + p * P.ent_stride;   // float offsets: no conversions
-    const T *mass = static_cast<const T *>(P.mass);
-    const T *mp = static_cast<const T *>(P.mp);
+    const float *mass = static_cast<const float *>(P.mass);
+    const float *mp = static_cast<const float *>(P.mp);
     for (;;) {
         const int item = pull_item(P.counter, &s_item);
         if (item >= P.n_items) break;
@@ -877,7 +904,7 @@ __global__ void __launch_bounds__(kThreads, kF32<T> ? 3 : 1) mp_kernel(KParams P
         const NodeInfo ti = P.info[node];
         // near sources contribute only if some neighbour is a leaf
         const int any_leaf = __syncthreads_or(load_slots(node, P, s_nbr, s_leaf, s_row));
-        stage_window_async<T>(W, s_nbr, s_leaf, mass, P, s_row);
+        stage_window_async<float>(W, s_nbr, s_leaf, mass, P, s_row);
         cp_async_commit();
         cp_async_wait_all();
         __syncthreads();
@@ -887,18 +914,16 @@ __global__ void __launch_bounds__(kThreads, kF32<T> ? 3 : 1) mp_kernel(KParams P
             const int cz = cz0 + 2 * half;
             const int ax = 2 * cx + px, ay = 2 * cy + py, az = 2 * cz + pz;
             const int base = cx + P.py * cy + P.pz * cz;
-            T dA[3], a3A[7];
-            load_target<T, ORDER>(P, ti.mp_row, parity_index(ax, ay, az), dA, a3A);
-            typename MpAcc<T, 16>::type L;
-            typename MpAcc<T, 3>::type S;
-            if constexpr (kF32<T>) {
-                L.col = Cs;
-                S.col = Cs + 4 * 2 * kThreads;
-            }
+            float dA[3], a3A[7];
+            load_target<ORDER>(P, ti.mp_row, parity_index(ax, ay, az), dA, a3A);
+            SmemAcc<16, 4> L;
+            SmemAcc<3> S;
+            L.col = Cs;
+            S.col = Cs + 4 * 2 * kThreads;
             L.zero();
             S.zero();
             // well-separated sources: refined (full moments) or leaf (mass).
-            // In float, a vote classifies the warp's 32 sources of one
+            // A vote classifies the warp's 32 sources of one
             // entry: all refined take the moments without a branch, all
             // leaves the mass-only form (the same operations less the zero
             // moments' terms, so the same values), a mix the general form
@@ -908,42 +933,31 @@ __global__ void __launch_bounds__(kThreads, kF32<T> ? 3 : 1) mp_kernel(KParams P
                 const int e1 = min(e0 + kChunk, P.n_far);
                 for (int e = e0; e < e1; ++e) {
                     const float4 E = __ldg(ent + e);
-                    const T wv = W[base + __float_as_int(E.w)];
+                    const float wv = W[base + __float_as_int(E.w)];
                     int idx;
-                    const bool is_mp = window_moments<T>(wv, P.mp_limit, idx);
-                    // (the double-float and double bodies are several times
-                    // larger, and extra copies of them cost more in
-                    // instruction fetch than they save: general form only)
-                    const bool all_mp = kF32<T> && __all_sync(0xffffffffu, is_mp);
-                    Src<T> src;
-                    T R[3];
+                    const bool is_mp = window_moments<float>(wv, P.mp_limit, idx);
+                    const bool all_mp = __all_sync(0xffffffffu, is_mp);
+                    Src<float> src;
+                    float R[3];
                     if (all_mp) {
-                        load_source_at<T>(mp + idx, src);
-                        separation<T>(dA, src.d, E, R);
-                        acc_mp<T, true, ORDER>(R[0], R[1], R[2], src, a3A, L, S);
-                    } else if (kF32<T> && !__any_sync(0xffffffffu, is_mp)) {
-                        if (__any_sync(0xffffffffu, window_nonzero<T>(wv))) {
+                        load_source_at(mp + idx, src);
+                        separation(dA, src.d, E, R);
+                        acc_mp<true, ORDER>(R[0], R[1], R[2], src, a3A, L, S);
+                    } else if (!__any_sync(0xffffffffu, is_mp)) {
+                        if (__any_sync(0xffffffffu, window_nonzero<float>(wv))) {
                             src.m0 = wv;
-                            acc_mp<T, false, ORDER>(dA[0] - T(E.x), dA[1] - T(E.y),
-                                                    dA[2] - T(E.z), src, a3A, L, S);
+                            acc_mp<false, ORDER>(dA[0] - E.x, dA[1] - E.y,
+                                                    dA[2] - E.z, src, a3A, L, S);
                         }
                     } else {
-                        if constexpr (kF32<T>) {
-                            if (is_mp) {
-                                load_source_at<T>(mp + idx, src);
-                            } else {
-                                src.m0 = wv;
-                                zero_moments<T>(src);
-                            }
+                        if (is_mp) {
+                            load_source_at(mp + idx, src);
                         } else {
-                            // leaf lanes read zero moments from the zero row
-                            // (no branch; the warp issues the loads anyway):
-                            // faster for the wider types, slower for float
-                            load_source_at<T>(mp + (is_mp ? idx : P.mp_limit), src);
-                            if (!is_mp) src.m0 = wv;
+                            src.m0 = wv;
+                            zero_moments(src);
                         }
-                        separation<T>(dA, src.d, E, R);
-                        acc_mp<T, true, ORDER>(R[0], R[1], R[2], src, a3A, L, S);
+                        separation(dA, src.d, E, R);
+                        acc_mp<true, ORDER>(R[0], R[1], R[2], src, a3A, L, S);
                     }
                 }
                 L.flush();
@@ -958,21 +972,21 @@ __global__ void __launch_bounds__(kThreads, kF32<T> ? 3 : 1) mp_kernel(KParams P
                 const int e1 = min(e0 + kChunk, P.n_far + P.n_near);
                 for (int e = e0; e < e1; ++e) {
                     const float4 E = __ldg(ent + e);
-                    const T wv = W[base + __float_as_int(E.w)];
-                    Src<T> src;
-                    src.m0 = window_refined<T>(wv) ? T(0) : wv;
-                    if (!__any_sync(0xffffffffu, window_nonzero<T>(src.m0))) continue;
-                    acc_mp<T, false, ORDER>(dA[0] - T(E.x), dA[1] - T(E.y), dA[2] - T(E.z), src, a3A,
-                                     L, S);
+                    const float wv = W[base + __float_as_int(E.w)];
+                    Src<float> src;
+                    src.m0 = window_refined<float>(wv) ? 0.f : wv;
+                    if (!__any_sync(0xffffffffu, window_nonzero<float>(src.m0))) continue;
+                    acc_mp<false, ORDER>(dA[0] - E.x, dA[1] - E.y, dA[2] - E.z, src, a3A, L,
+                                         S);
                 }
                 L.flush();
                 S.flush();
             }
             const int cell = ax + 8 * ay + 64 * az;
-            store_target<T>(P, node, cell, L);
+            store_target(P, node, cell, L);
 #pragma unroll
             for (int i = 0; i < 3; ++i)
-                __stcs(P.dL1 + (size_t(node) * 3 + i) * NCELL + cell, acc_value<T>(S, i));
+                __stcs(P.dL1 + (size_t(node) * 3 + i) * NCELL + cell, acc_value(S, i));
         }
         __syncthreads();
     }
@@ -981,6 +995,154 @@ __global__ void __launch_bounds__(kThreads, kF32<T> ? 3 : 1) mp_kernel(KParams P
     // from their own queue, which fills the tail that the coarse multipole
     // items leave (the monopole kernel, whose results they add to, has
     // finished before this launch)
+    if (P.n_mx > 0) {
+        for (;;) {
+            int w = 0;
+            if (lane == 0) w = atomicAdd(P.mx_counter, 1);
+            w = __shfl_sync(0xffffffffu, w, 0);
+            if (w * 32 >= P.n_mx) break;
+            if (w * 32 + lane < P.n_mx) mx_target<float, ORDER>(P, w * 32 + lane);
+        }
+    }
+}
+
+// ---------------------------------------------------------- mpw_kernel
+// The multipole kernel of the wide types (double, double-float; the
+// interaction and its sums are in fmm_wide.cuh).  Bound by the FP64 pipe
+// (double) or the FP32 pipe (double-float): one CTA per SM is enough, and
+// registers go to the 38 sums.  One loop takes far and near entries alike
+// (near ones count leaf sources only), so the large body is compiled once;
+// its second half, the moments, is skipped for entries without a refined
+// source in the warp, and entries with absent sources only altogether.
+// CTAs of four warps: three per SM in double-float (at most 168 registers),
+// whose dependent chains leave the pipe idle with two warps a scheduler; two
+// in double, which fills its pipe with those and needs the registers for the
+// chunk sums.
+//   PARTS 2, 4: an item is four of a sub-grid's eight parities (one z parity),
+//     a warp each, in both halves (z < 4, z >= 4) or one of them;
+//   PARTS 16: an item is one half of one parity, 32 cells, whose stencil
+//     entries the four warps share out (every fourth entry), the sums added
+//     through shared memory in a fixed order: for trees with too few refined
+//     nodes to fill the SMs otherwise.
+constexpr int kWideThreads = 128;
+template <typename T>
+__device__ __forceinline__ T wide_shfl_xor(T v, int mask)
+{
+    if constexpr (kDF<T>)
+        return dfloat(__shfl_xor_sync(0xffffffffu, v.hi, mask), __shfl_xor_sync(0xffffffffu, v.lo, mask));
+    else
+        return __shfl_xor_sync(0xffffffffu, v, mask);
+}
+// the sums of WideAcc as an array (order 2 leaves the last 15 at zero)
+template <int ORDER>
+constexpr int kWideSums = ORDER == 3 ? 38 : 23;
+
+template <typename T, int ORDER>
+__device__ __forceinline__ void store_wide(const KParams &P, int node, int cell, const T L[16], const T S[3])
+{
+    T zero[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) zero[k] = T(0);
+    store_target_values<T>(P, node, cell, L, zero);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+        __stcs(P.dL1 + (size_t(node) * 3 + i) * NCELL + cell, to_double(S[i]));
+}
+
+template <typename T, int ORDER, int PARTS>
+__global__ void __launch_bounds__(kWideThreads, kDF<T> ? 3 : 2) mpw_kernel(KParams P)
+{
+    static_assert(PARTS == 2 || PARTS == 4 || PARTS == 16, "items per sub-grid");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T *W = reinterpret_cast<T *>(smem_raw);
+    __shared__ int s_nbr[27], s_leaf[27], s_row[27], s_item;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cx = lane & 3, cy = (lane >> 2) & 3, cz0 = lane >> 4;
+    const T *mass = static_cast<const T *>(P.mass);
+    const T *mp = static_cast<const T *>(P.mp);
+    for (;;) {
+        const int item = pull_item(P.counter, &s_item);
+        if (item >= P.n_items) break;
+        const int node = P.list[item / PARTS];
+        const NodeInfo ti = P.info[node];
+        // near sources contribute only if some neighbour is a leaf
+        const int any_leaf = __syncthreads_or(load_slots(node, P, s_nbr, s_leaf, s_row));
+        stage_window_async<T>(W, s_nbr, s_leaf, mass, P, s_row);
+        cp_async_commit();
+        cp_async_wait_all();
+        __syncthreads();
+        const int p = PARTS == 16 ? (item >> 1) & 7 : 4 * (item / (PARTS / 2) & 1) + warp;
+        const int px = p & 1, py = (p >> 1) & 1, pz = p >> 2;
+        const float4 *ent = P.stencil_f + p * P.ent_stride;
+        const int n_ent = any_leaf ? P.n_far + P.n_near : P.n_far;
+        constexpr int step = PARTS == 16 ? kWideThreads / 32 : 1;
+        const int half0 = PARTS == 2 ? 0 : item & 1;
+        const int half1 = PARTS == 2 ? 2 : half0 + 1;
+        for (int half = half0; half < half1; ++half) {
+            const int cz = cz0 + 2 * half;
+            const int ax = 2 * cx + px, ay = 2 * cy + py, az = 2 * cz + pz;
+            const int base = cx + P.py * cy + P.pz * cz;
+            const T *own_at = mp + (size_t(ti.mp_row) * 4 * NCELL + parity_index(ax, ay, az)) * 4;
+            T dA[4];
+            load4<T>(own_at, dA);
+            WideChunked<T, WideAcc<T, ORDER>> C;
+            C.zero();
+            int done = 0;
+            for (int e = PARTS == 16 ? warp : 0; e < n_ent; e += step) {
+                const float4 E = __ldg(ent + e);
+                T wv = W[base + __float_as_int(E.w)];
+                int idx;
+                bool is_mp = window_moments<T>(wv, P.mp_limit, idx);
+                if (e >= P.n_far) {
+                    if (window_refined<T>(wv)) wv = T(0);
+                    is_mp = false;
+                }
+                if (!__any_sync(0xffffffffu, window_nonzero<T>(wv))) continue;
+                const bool any_mp = __any_sync(0xffffffffu, is_mp);
+                WideSrc<T> src;
+                T m = wv;
+                if (any_mp) {
+                    // leaf lanes read zero moments from the zero row
+                    load_wide<T>(mp + (is_mp ? idx : P.mp_limit), src);
+                    if (is_mp) m = src.m0;
+                } else {
+                    src.d[0] = src.d[1] = src.d[2] = T(0);
+                }
+                C.part.add(wide_sep(dA[0], src.d[0], E.x), wide_sep(dA[1], src.d[1], E.y),
+                           wide_sep(dA[2], src.d[2], E.z), m, src, any_mp);
+                if (++done == kChunk) {
+                    C.flush();
+                    done = 0;
+                }
+            }
+            C.flush();
+            WideAcc<T, ORDER> &A = C.total();
+            if (PARTS == 16) {
+                // the upper half of the warps hand their sums to the lower, twice
+                constexpr int NS = kWideSums<ORDER>;
+                T *sum = reinterpret_cast<T *>(&A);
+                for (int w = kWideThreads / 64; w > 0; w >>= 1) {
+                    __syncthreads();                // the window, or the last round, is done with
+                    if (warp >= w && warp < 2 * w)
+#pragma unroll
+                        for (int k = 0; k < NS; ++k) W[((warp - w) * NS + k) * 32 + lane] = sum[k];
+                    __syncthreads();
+                    if (warp < w)
+#pragma unroll
+                        for (int k = 0; k < NS; ++k) sum[k] += W[(warp * NS + k) * 32 + lane];
+                }
+            }
+            if (PARTS != 16 || warp == 0) {
+                WideSrc<T> own;
+                load_wide<T>(own_at, own);
+                T L[16], S[3];
+                A.finish(own, L, S);
+                store_wide<T, ORDER>(P, node, ax + 8 * ay + 64 * az, L, S);
+            }
+        }
+        __syncthreads();
+    }
+    // as in mp_kernel: fmm_step's monopole<-multipole targets fill the tail
     if (P.n_mx > 0) {
         for (;;) {
             int w = 0;
@@ -1008,10 +1170,10 @@ __device__ __forceinline__ void mp2_source(const KParams &P, const float *mp, fl
     // masses are not negative, so a mass's decoded offset is out of range
     const unsigned idx = unsigned(-1 - __float_as_int(wv));
     if (idx < unsigned(P.mp_limit)) {
-        load_source_at<float>(mp + idx, src);
+        load_source_at(mp + idx, src);
     } else {
         src.m0 = wv;
-        zero_moments<float>(src);
+        zero_moments(src);
     }
 }
 
@@ -1042,10 +1204,10 @@ __global__ void __launch_bounds__(kThreads, 2) mp2_kernel(KParams P)
         const int az0 = 2 * cz0 + pz, az1 = az0 + 4;
         const int base0 = cx + P.py * cy + P.pz * cz0, base1 = base0 + 2 * P.pz;
         float dA0[3], a3A0[7], dA1[3], a3A1[7];
-        load_target<float>(P, ti.mp_row, parity_index(ax, ay, az0), dA0, a3A0);
-        load_target<float>(P, ti.mp_row, parity_index(ax, ay, az1), dA1, a3A1);
-        MpAcc<float, 16>::type L0, L1;
-        MpAcc<float, 3>::type S0, S1;
+        load_target<3>(P, ti.mp_row, parity_index(ax, ay, az0), dA0, a3A0);
+        load_target<3>(P, ti.mp_row, parity_index(ax, ay, az1), dA1, a3A1);
+        SmemAcc<16, 4> L0, L1;
+        SmemAcc<3> S0, S1;
         L0.col = Cs;
         S0.col = Cs + 4 * 2 * kThreads;
         L1.col = Cs + kMpPairs * 2 * kThreads;
@@ -1066,17 +1228,17 @@ __global__ void __launch_bounds__(kThreads, 2) mp2_kernel(KParams P)
                 // the warp's 64 sources all refined: the moments without a
                 // branch (the same values as the general form)
                 if (__all_sync(0xffffffffu, i0 < unsigned(P.mp_limit) && i1 < unsigned(P.mp_limit))) {
-                    load_source_at<float>(mp + i0, s0);
-                    load_source_at<float>(mp + i1, s1);
+                    load_source_at(mp + i0, s0);
+                    load_source_at(mp + i1, s1);
                 } else {
                     mp2_source(P, mp, w0, s0);
                     mp2_source(P, mp, w1, s1);
                 }
                 float R0[3], R1[3];
-                separation<float>(dA0, s0.d, E, R0);
-                separation<float>(dA1, s1.d, E, R1);
-                acc_mp<float, true>(R0[0], R0[1], R0[2], s0, a3A0, L0, S0);
-                acc_mp<float, true>(R1[0], R1[1], R1[2], s1, a3A1, L1, S1);
+                separation(dA0, s0.d, E, R0);
+                separation(dA1, s1.d, E, R1);
+                acc_mp<true>(R0[0], R0[1], R0[2], s0, a3A0, L0, S0);
+                acc_mp<true>(R1[0], R1[1], R1[2], s1, a3A1, L1, S1);
             }
             L0.flush();
             S0.flush();
@@ -1093,8 +1255,8 @@ __global__ void __launch_bounds__(kThreads, 2) mp2_kernel(KParams P)
                 s0.m0 = unsigned(-1 - __float_as_int(w0)) < unsigned(P.mp_limit) ? 0.f : w0;
                 s1.m0 = unsigned(-1 - __float_as_int(w1)) < unsigned(P.mp_limit) ? 0.f : w1;
                 if (!__any_sync(0xffffffffu, s0.m0 != 0.f || s1.m0 != 0.f)) continue;
-                acc_mp<float, false>(dA0[0] - E.x, dA0[1] - E.y, dA0[2] - E.z, s0, a3A0, L0, S0);
-                acc_mp<float, false>(dA1[0] - E.x, dA1[1] - E.y, dA1[2] - E.z, s1, a3A1, L1, S1);
+                acc_mp<false>(dA0[0] - E.x, dA0[1] - E.y, dA0[2] - E.z, s0, a3A0, L0, S0);
+                acc_mp<false>(dA1[0] - E.x, dA1[1] - E.y, dA1[2] - E.z, s1, a3A1, L1, S1);
             }
             L0.flush();
             S0.flush();
@@ -1102,12 +1264,12 @@ __global__ void __launch_bounds__(kThreads, 2) mp2_kernel(KParams P)
             S1.flush();
         }
         const int cell0 = ax + 8 * ay + 64 * az0, cell1 = ax + 8 * ay + 64 * az1;
-        store_target<float>(P, node, cell0, L0);
-        store_target<float>(P, node, cell1, L1);
+        store_target(P, node, cell0, L0);
+        store_target(P, node, cell1, L1);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            P.dL1[(size_t(node) * 3 + i) * NCELL + cell0] = acc_value<float>(S0, i);
-            P.dL1[(size_t(node) * 3 + i) * NCELL + cell1] = acc_value<float>(S1, i);
+            P.dL1[(size_t(node) * 3 + i) * NCELL + cell0] = acc_value(S0, i);
+            P.dL1[(size_t(node) * 3 + i) * NCELL + cell1] = acc_value(S1, i);
         }
         __syncthreads();
     }
@@ -1308,23 +1470,23 @@ constexpr int kRootSlices = 8;
 constexpr int kRootThreads = 32 * kRootSlices;
 constexpr int kRootGroups = NCELL / 32;
 
-template <typename T, int ORDER>
+template <int ORDER>
 __global__ void __launch_bounds__(kRootThreads) root_kernel(KParams P)
 {
     constexpr int NV = 16 + 3;                      // L (traceless), S
-    __shared__ T sh_hi[kRootSlices][NV][32];
-    __shared__ T sh_lo[kRootSlices][kF32<T> ? NV : 1][32];   // float only
+    __shared__ float sh_hi[kRootSlices][NV][32];
+    __shared__ float sh_lo[kRootSlices][NV][32];
     const int node = P.list[blockIdx.x];
     const NodeInfo ti = P.info[node];
     const bool leaf = ti.leaf_row >= 0;
-    const T *mass = static_cast<const T *>(P.mass);
+    const float *mass = static_cast<const float *>(P.mass);
     const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
     const int cell = blockIdx.y * 32 + lane;
     const int ax = cell & 7, ay = (cell >> 3) & 7, az = cell >> 6;
-    T dA[3] = {T(0), T(0), T(0)}, a3A[7] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
-    if (!leaf) load_target<T, ORDER>(P, ti.mp_row, parity_index(ax, ay, az), dA, a3A);
-    Acc<T, 16> L;
-    Acc<T, 3> S;
+    float dA[3] = {0.f, 0.f, 0.f}, a3A[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (!leaf) load_target<ORDER>(P, ti.mp_row, parity_index(ax, ay, az), dA, a3A);
+    Acc<float, 16> L;
+    Acc<float, 3> S;
     L.zero();
     S.zero();
     int done = 0;
@@ -1334,15 +1496,15 @@ __global__ void __launch_bounds__(kRootThreads) root_kernel(KParams P)
         const bool far = ox * ox + oy * oy + oz * oz >= P.far_o2;
         if (b == cell || !(far || leaf)) continue;
         const int pi = parity_index(b & 7, (b >> 3) & 7, b >> 6);
-        Src<T> src;
+        Src<float> src;
         if (!leaf) {
-            load_source<T>(P, ti.mp_row, pi, src);
+            load_source(P, ti.mp_row, pi, src);
         } else {
             src.m0 = mass[size_t(node) * NCELL + pi];
-            zero_moments<T>(src);
+            zero_moments(src);
         }
-        acc_mp<T, true, ORDER>(dA[0] - src.d[0] - T(ox), dA[1] - src.d[1] - T(oy),
-                        dA[2] - src.d[2] - T(oz), src, a3A, L, S);
+        acc_mp<true, ORDER>(dA[0] - src.d[0] - float(ox), dA[1] - src.d[1] - float(oy),
+                        dA[2] - src.d[2] - float(oz), src, a3A, L, S);
         if (++done == kChunk) {
             L.flush();
             S.flush();
@@ -1353,38 +1515,115 @@ __global__ void __launch_bounds__(kRootThreads) root_kernel(KParams P)
     S.flush();
     for (int k = 0; k < 16; ++k) {
         sh_hi[slice][k][lane] = acc_hi(L, k);
-        if constexpr (kF32<T>) sh_lo[slice][k][lane] = acc_lo(L, k);
+        sh_lo[slice][k][lane] = acc_lo(L, k);
     }
     for (int i = 0; i < 3; ++i) {
         sh_hi[slice][16 + i][lane] = acc_hi(S, i);
-        if constexpr (kF32<T>) sh_lo[slice][16 + i][lane] = acc_lo(S, i);
+        sh_lo[slice][16 + i][lane] = acc_lo(S, i);
     }
     __syncthreads();
     if (slice != 0) return;
-    T Fh[NV], Fl[NV];
+    float Fh[NV], Fl[NV];
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
-        T hi = T(0), lo = T(0);
+        float hi = 0.f, lo = 0.f;
         for (int sl = 0; sl < kRootSlices; ++sl) {
-            if constexpr (kF32<T>) {
-                float sum, err;
-                two_sum(hi, sh_hi[sl][k][lane], sum, err);
-                hi = sum;
-                lo += err + sh_lo[sl][k][lane];
-            } else {
-                hi += sh_hi[sl][k][lane];
-            }
+            float sum, err;
+            two_sum(hi, sh_hi[sl][k][lane], sum, err);
+            hi = sum;
+            lo += err + sh_lo[sl][k][lane];
         }
         Fh[k] = hi;
         Fl[k] = lo;
     }
     if (leaf) {
-        for (int k = 0; k < 4; ++k) store_L<T>(P, node, k, cell, Fh[k], Fl[k]);
+        for (int k = 0; k < 4; ++k) store_L<float>(P, node, k, cell, Fh[k], Fl[k]);
     } else {
-        store_target_values<T>(P, node, cell, Fh, Fl);
+        store_target_values<float>(P, node, cell, Fh, Fl);
     }
     for (int i = 0; i < 3; ++i)
         P.dL1[(size_t(node) * 3 + i) * NCELL + cell] = to_double(Fh[16 + i]) + to_double(Fl[16 + i]);
+}
+
+// The root of the wide types, whose arithmetic fills an SM: four targets per
+// CTA and 128 CTAs, so that one root spreads over most SMs (16 CTAs of 32
+// targets took 741 us in FP64 and 150 us in double-float).  The 512 sources
+// of a target are shared out over 64 threads, eight each; their sums are
+// added by shuffles within a warp and in a fixed order across the warps.
+constexpr int kRootwTargets = 4;
+
+template <typename T, int ORDER>
+__global__ void __launch_bounds__(kThreads) rootw_kernel(KParams P)
+{
+    constexpr int NS = kWideSums<ORDER>, NW = kThreads / 32;
+    static_assert(sizeof(WideAcc<T, ORDER>) == 38 * sizeof(T), "sums of WideAcc");
+    __shared__ T sh[NW][NS][kRootwTargets];
+    const int node = P.list[blockIdx.x];
+    const NodeInfo ti = P.info[node];
+    const bool leaf = ti.leaf_row >= 0;
+    const T *mass = static_cast<const T *>(P.mass);
+    const T *mp = static_cast<const T *>(P.mp);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int cell = blockIdx.y * kRootwTargets + (lane & 3);
+    const int slice = warp * 8 + (lane >> 2);
+    const int ax = cell & 7, ay = (cell >> 3) & 7, az = cell >> 6;
+    const T *row = leaf ? mp : mp + size_t(ti.mp_row) * 4 * NCELL * 4;
+    const T *own_at = row + parity_index(ax, ay, az) * 4;
+    T dA[4] = {T(0), T(0), T(0), T(0)};
+    if (!leaf) load4<T>(own_at, dA);
+    WideAcc<T, ORDER> A;
+    A.zero();
+    // source x = slot + k: every slice's eight sources are one x row
+    const int by = slice & 7, bz = slice >> 3;
+    for (int bx = 0; bx < 8; ++bx) {
+        const int ox = bx - ax, oy = by - ay, oz = bz - az;
+        const int o2 = ox * ox + oy * oy + oz * oz;
+        if (o2 == 0 || !(leaf || o2 >= P.far_o2)) continue;
+        const int pi = parity_index(bx, by, bz);
+        WideSrc<T> src;
+        T m;
+        if (!leaf) {
+            load_wide<T>(row + pi * 4, src);
+            m = src.m0;
+        } else {
+            m = mass[size_t(node) * NCELL + pi];
+            src.d[0] = src.d[1] = src.d[2] = T(0);
+        }
+        A.add(wide_sep(dA[0], src.d[0], float(ox)), wide_sep(dA[1], src.d[1], float(oy)),
+              wide_sep(dA[2], src.d[2], float(oz)), m, src, !leaf);
+    }
+    A.flush();
+    T *sum = reinterpret_cast<T *>(&A);
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+#pragma unroll
+        for (int off = 4; off < 32; off <<= 1) sum[k] += wide_shfl_xor(sum[k], off);
+        if (lane < kRootwTargets) sh[warp][k][lane] = sum[k];
+    }
+    __syncthreads();
+    // (one thread per value and target adds the eight warps' sums)
+    for (int i = threadIdx.x; i < NS * kRootwTargets; i += kThreads) {
+        const int k = i / kRootwTargets, t = i % kRootwTargets;
+        T v = sh[0][k][t];
+#pragma unroll
+        for (int w = 1; w < NW; ++w) v += sh[w][k][t];
+        sh[0][k][t] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x >= kRootwTargets) return;
+#pragma unroll
+    for (int k = 0; k < NS; ++k) sum[k] = sh[0][k][threadIdx.x];
+    if (leaf) {
+        store_L<T>(P, node, 0, cell, -A.low.a0, T(0));
+        for (int i = 0; i < 3; ++i) store_L<T>(P, node, 1 + i, cell, A.low.a1[i], T(0));
+        for (int i = 0; i < 3; ++i) P.dL1[(size_t(node) * 3 + i) * NCELL + cell] = 0.0;
+        return;
+    }
+    WideSrc<T> own;
+    load_wide<T>(own_at, own);
+    T L[16], S[3];
+    A.finish(own, L, S);
+    store_wide<T, ORDER>(P, node, cell, L, S);
 }
 
 // ---------------------------------------------------------- launching
@@ -1401,11 +1640,13 @@ cudaError_t allow_smem(Kern k, size_t bytes, size_t &done)
 
 template <typename T>
 struct Kernels {
-    template <int ORDER, bool HALVES>
+    // PARTS items per sub-grid: float 1, 2; the wide types 2, 4, 16
+    template <int ORDER, int PARTS>
     static cudaError_t mp(size_t bytes)
     {
         static size_t done = 0;
-        return allow_smem(mp_kernel<T, ORDER, HALVES>, bytes, done);
+        if constexpr (kF32<T>) return allow_smem(mp_kernel<ORDER, PARTS == 2>, bytes, done);
+        else return allow_smem(mpw_kernel<T, ORDER, PARTS>, bytes, done);
     }
     static cudaError_t mp2(size_t bytes)
     {
@@ -1422,10 +1663,11 @@ struct Kernels {
 
 // persistent grid: SMs x resident CTAs (optionally capped by the tuning)
 template <typename Kern>
-int persistent_grid(Kern k, size_t smem, int64_t items, int sms, int cap_per_sm)
+int persistent_grid(Kern k, size_t smem, int64_t items, int sms, int cap_per_sm,
+                    int threads = kThreads)
 {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kThreads, smem) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem) != cudaSuccess ||
         per_sm < 1)
         per_sm = 1;
     if (cap_per_sm > 0 && cap_per_sm < per_sm) per_sm = cap_per_sm;
@@ -1459,6 +1701,24 @@ cudaError_t launch_mono(const KParams &K, size_t wbytes, int sms, int cap, cudaS
     case 7: return launch_mono_r<T, NB, 7>(K, wbytes, sms, cap, s);
     default: return cudaErrorInvalidValue;
     }
+}
+
+// the multipole launch, PARTS items per sub-grid
+template <typename T, int ORDER, int PARTS>
+cudaError_t launch_mp(KParams K, size_t bytes, int sms, int cap, cudaStream_t s)
+{
+    cudaError_t e = Kernels<T>::template mp<ORDER, PARTS>(bytes);
+    if (e != cudaSuccess) return e;
+    K.n_items *= PARTS;
+    if constexpr (kF32<T>) {
+        const int g = persistent_grid(mp_kernel<ORDER, PARTS == 2>, bytes, K.n_items, sms, cap);
+        mp_kernel<ORDER, PARTS == 2><<<g, kThreads, bytes, s>>>(K);
+    } else {
+        const int g = persistent_grid(mpw_kernel<T, ORDER, PARTS>, bytes, K.n_items, sms, cap,
+                                      kWideThreads);
+        mpw_kernel<T, ORDER, PARTS><<<g, kWideThreads, bytes, s>>>(K);
+    }
+    return cudaGetLastError();
 }
 
 template <typename T, int ORDER>
@@ -1497,9 +1757,7 @@ cudaError_t launch_all(const fmm_tree_s *t, void *L, float *Lc, double *dL1, cud
     // mp_kernel: one window (masses of leaf sources, moment offsets of
     // refined ones); float adds its compensation pairs, [7][2][threads]
     const size_t mp_bytes = wbytes + (kF32<T> ? size_t(kMpPairs) * 2 * kThreads * sizeof(float) : 0);
-    cudaError_t e = Kernels<T>::template mp<ORDER, false>(mp_bytes);
-    if (e == cudaSuccess) e = Kernels<T>::template mp<ORDER, true>(mp_bytes);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     if (parts & M2L_RESET) {
         e = cudaMemsetAsync(d.counters, 0, 4 * sizeof(int32_t), s);
         if (e != cudaSuccess) return e;
@@ -1514,7 +1772,11 @@ cudaError_t launch_all(const fmm_tree_s *t, void *L, float *Lc, double *dL1, cud
         R.list = d.lists + Pl.roots.off;
         R.n_items = int32_t(Pl.roots.count);
         timing_begin(t, FMM_K_ROOT, s);
-        root_kernel<T, ORDER><<<dim3(unsigned(Pl.roots.count), kRootGroups), kRootThreads, 0, s>>>(R);
+        if constexpr (kF32<T>)
+            root_kernel<ORDER><<<dim3(unsigned(Pl.roots.count), kRootGroups), kRootThreads, 0, s>>>(R);
+        else
+            rootw_kernel<T, ORDER><<<dim3(unsigned(Pl.roots.count), NCELL / kRootwTargets), kThreads, 0,
+                                     s>>>(R);
         timing_end(t, s);
         ++nl;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -1536,19 +1798,32 @@ cudaError_t launch_all(const fmm_tree_s *t, void *L, float *Lc, double *dL1, cud
             int g = persistent_grid(mp2_kernel, b2, Pl.work_mp.count, sms, cap);
             mp2_kernel<<<g, kThreads, b2, s>>>(K);
         } else {
-            // half sub-grids per item where whole ones would leave CTA slots
-            // idle or unbalanced (fewer nodes than twice the slots)
-            const int64_t slots =
-                persistent_grid(mp_kernel<T, ORDER, false>, mp_bytes, INT32_MAX, sms, cap);
             const int mode = t->tuning.mp_items;
-            if (mode == 2 || (mode == 0 && Pl.work_mp.count < 2 * slots)) {
-                K.n_items = int32_t(2 * Pl.work_mp.count);
-                int g = persistent_grid(mp_kernel<T, ORDER, true>, mp_bytes, K.n_items, sms, cap);
-                mp_kernel<T, ORDER, true><<<g, kThreads, mp_bytes, s>>>(K);
+            const int64_t n = Pl.work_mp.count;
+            if constexpr (kF32<T>) {
+                // half sub-grids per item where whole ones would leave CTA
+                // slots idle or unbalanced (fewer nodes than twice the slots)
+                if ((e = Kernels<T>::template mp<ORDER, 1>(mp_bytes)) != cudaSuccess) return e;
+                const int64_t slots =
+                    persistent_grid(mp_kernel<ORDER, false>, mp_bytes, INT32_MAX, sms, cap);
+                if (mode == 2 || (mode == 0 && n < 2 * slots))
+                    e = launch_mp<T, ORDER, 2>(K, mp_bytes, sms, cap, s);
+                else
+                    e = launch_mp<T, ORDER, 1>(K, mp_bytes, sms, cap, s);
             } else {
-                int g = persistent_grid(mp_kernel<T, ORDER, false>, mp_bytes, K.n_items, sms, cap);
-                mp_kernel<T, ORDER, false><<<g, kThreads, mp_bytes, s>>>(K);
+                // halves and quarters of a sub-grid (mp_items 1 and 2; by
+                // default quarters below eight nodes an SM, so that the last
+                // items to run are short), and sixteenths where even quarters would not fill the SMs once
+                // (whatever mp_items says: their sums round differently)
+                const size_t fold = size_t(kWideThreads / 64) * kWideSums<ORDER> * 32 * sizeof(T);
+                if (4 * n < sms)
+                    e = launch_mp<T, ORDER, 16>(K, std::max(wbytes, fold), sms, cap, s);
+                else if (mode == 2 || (mode == 0 && n < 8 * int64_t(sms)))
+                    e = launch_mp<T, ORDER, 4>(K, mp_bytes, sms, cap, s);
+                else
+                    e = launch_mp<T, ORDER, 2>(K, mp_bytes, sms, cap, s);
             }
+            if (e != cudaSuccess) return e;
         }
         timing_end(t, s);
         ++nl;
