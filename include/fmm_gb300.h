@@ -287,8 +287,9 @@ int fmm_forces(fmm_tree_t tree, const double *L64, const double *dL1_acc,
  * (paper_1908_03121_gb300/autotune.py); zeros select the defaults.  No
  * counterpart in the paper: its kernels had one fixed shape (Sec. 5.1). */
 typedef struct {
-    int32_t mono_subgrids;           /* sub-grids per pass of the monopole kernel:
-                                        1, 2 or 4 (float) / 1, 2 (double) */
+    int32_t mono_subgrids;           /* FMM_MIXED: sub-grids per pass of the monopole
+                                        kernel, 1, 2 or 4 (the other precisions take one
+                                        leaf node per CTA, whatever this says) */
     int32_t ctas_per_sm;             /* cap on persistent CTAs per SM (0 = occupancy) */
     int32_t dataflow;                /* 1: fmm_step runs the refined levels' shifts and
                                         every leaf's shift and forces as one persistent

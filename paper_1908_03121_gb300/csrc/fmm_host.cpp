@@ -276,20 +276,12 @@ static void build_stencils(fmm_tree_s *t)
     }
     // monopole kernel: parity 0's weights, every parity in parity 0's order
     t->coef32.assign(size_t(P.ent_stride) * 4, 0.f);
-    t->coef64.assign(size_t(P.ent_stride) * 4, 0.0);
-    t->coefdf.assign(size_t(P.ent_stride) * 8, 0.f);
     t->mono_woff.assign(size_t(8) * P.ent_stride, 0);
     for (size_t k = 0; k < lists[0].size(); ++k) {
         const StencilEntry &e = lists[0][k];
         double c[4];
         mono_coef(e.ox, e.oy, e.oz, c);
-        for (int j = 0; j < 4; ++j) {
-            t->coef64[k * 4 + j] = c[j];
-            t->coef32[k * 4 + j] = float(c[j]);
-            // double-float (hi, lo) pairs
-            t->coefdf[k * 8 + 2 * j] = float(c[j]);
-            t->coefdf[k * 8 + 2 * j + 1] = float(c[j] - double(float(c[j])));
-        }
+        for (int j = 0; j < 4; ++j) t->coef32[k * 4 + j] = float(c[j]);
         for (int p = 0; p < 8; ++p) {
             const int pp[3] = {p & 1, (p >> 1) & 1, (p >> 2) & 1};
             const int o[3] = {pp[0] ? -e.ox : e.ox, pp[1] ? -e.oy : e.oy, pp[2] ? -e.oz : e.oz};
@@ -308,6 +300,55 @@ static void build_stencils(fmm_tree_s *t)
     // (the same expression as well_separated on o2 = far_o2)
     P.far_o2 = 1;
     while (!(theta * theta * double(P.far_o2) > 1.0)) ++P.far_o2;
+}
+
+// The wide types' monopole<-monopole weights (fmm_mono_wide.cuh): near parent
+// offsets up to signs, by mask of nonzero axes, and for each the Hadamard
+// transform of the 8 x 8 weights between a block's children,
+//   K_ab = (1/64) sum_ps (-1)^(a.p + b.s) w_c(2 d + s - p),
+// stored for a = q xor b xor e_c, q over the subsets of the mask (zero for
+// the other q by symmetry).
+static void build_orbits(fmm_tree_s *t)
+{
+    const int R = int(std::floor(1.0 / t->cfg.theta));
+    t->orbits.clear();
+    t->orbit_coef.clear();
+    for (int mask = 0; mask < 8; ++mask) {
+        t->orbit_first[mask] = int32_t(t->orbits.size() / 4);
+        for (int dz = 0; dz <= R; ++dz)
+            for (int dy = 0; dy <= R; ++dy)
+                for (int dx = 0; dx <= R; ++dx) {
+                    if (((dx > 0) | (dy > 0) << 1 | (dz > 0) << 2) != mask) continue;
+                    if (well_separated(t->cfg.theta, dx, dy, dz)) continue;
+                    for (int v : {dx, dy, dz, mask}) t->orbits.push_back(v);
+                    // w[p][s][c]; a cell has no weight on itself
+                    double w[8][8][4] = {};
+                    for (int p = 0; p < 8; ++p)
+                        for (int s = 0; s < 8; ++s) {
+                            const int ox = 2 * dx + (s & 1) - (p & 1),
+                                      oy = 2 * dy + ((s >> 1) & 1) - ((p >> 1) & 1),
+                                      oz = 2 * dz + (s >> 2) - (p >> 2);
+                            if (ox || oy || oz) mono_coef(ox, oy, oz, w[p][s]);
+                        }
+                    for (int b = 0; b < 8; ++b)
+                        for (int q = 0; q < 8; ++q) {
+                            if (q & ~mask) continue;
+                            for (int c = 0; c < 4; ++c) {
+                                const int a = q ^ b ^ (c == 0 ? 0 : 1 << (c - 1));
+                                long double sum = 0.0L;
+                                for (int p = 0; p < 8; ++p)
+                                    for (int s = 0; s < 8; ++s) {
+                                        int odd = 0;
+                                        for (int m = a & p; m; m &= m - 1) odd ^= 1;
+                                        for (int m = b & s; m; m &= m - 1) odd ^= 1;
+                                        sum += odd ? -(long double)w[p][s][c] : (long double)w[p][s][c];
+                                    }
+                                t->orbit_coef.push_back(double(sum / 64.0L));
+                            }
+                        }
+                }
+    }
+    t->orbit_first[8] = int32_t(t->orbits.size() / 4);
 }
 
 // --------------------------------------------------- interaction counting
@@ -593,7 +634,7 @@ static void free_device(fmm_tree_s *t)
         t->aux = nullptr;
     }
     DeviceTables &d = t->dev;
-    void *ptrs[] = {d.info, d.children, d.nbr, d.lists, d.stencil, d.stencil_f, d.coef32, d.coef64, d.coefdf, d.mono_woff,
+    void *ptrs[] = {d.info, d.children, d.nbr, d.lists, d.stencil, d.stencil_f, d.coef32, d.mono_woff, d.orbits, d.orbit_coef,
                     d.tree_leaf_off, d.tree_leaf_rows, d.levels, d.levels_df, d.mass, d.mp, d.counters,
                     d.partials, d.chunk_sums, d.up, d.down, d.mx_targets, d.mx_pairs,
                     d.dflow_items, d.dflow_ready};
@@ -610,15 +651,25 @@ static int upload_tree(fmm_tree_s *t)
         (rc = upload(&d.nbr, t->nbr)) || (rc = upload(&d.lists, t->lists)) ||
         (rc = upload(&d.stencil, t->stencil)) || (rc = upload(&d.stencil_f, t->stencil_f)) ||
         (rc = upload(&d.coef32, t->coef32)) ||
-        (rc = upload(&d.coef64, t->coef64)) || (rc = upload(&d.coefdf, t->coefdf)) ||
         (rc = upload(&d.mono_woff, t->mono_woff)) ||
         (rc = upload(&d.tree_leaf_off, t->tree_leaf_off)) ||
         (rc = upload(&d.tree_leaf_rows, t->tree_leaf_rows)) || (rc = upload(&d.levels, t->levels)) ||
         (rc = upload(&d.levels_df, t->levels_df)) ||
         (rc = upload(reinterpret_cast<int32_t **>(&d.mx_targets), t->mx_targets)) ||
         (rc = upload(reinterpret_cast<int32_t **>(&d.mx_pairs), t->mx_pairs)) ||
-        (rc = upload(&d.dflow_items, t->dflow_items)))
+        (rc = upload(&d.dflow_items, t->dflow_items)) ||
+        (rc = upload(reinterpret_cast<int32_t **>(&d.orbits), t->orbits)))
         return rc;
+    if (t->cfg.precision == FMM_FP64) {
+        if ((rc = upload(reinterpret_cast<double **>(&d.orbit_coef), t->orbit_coef))) return rc;
+    } else if (t->cfg.precision == FMM_DFLOAT) {
+        std::vector<float> pairs;            // double-float (hi, lo)
+        for (double v : t->orbit_coef) {
+            pairs.push_back(float(v));
+            pairs.push_back(float(v - double(float(v))));
+        }
+        if ((rc = upload(reinterpret_cast<float **>(&d.orbit_coef), pairs))) return rc;
+    }
     // packed masses and moments: float (mixed), (hi, lo) float pairs (dfloat), double
     size_t es = t->cfg.precision == FMM_MIXED ? sizeof(float) : 2 * sizeof(float);
     static_assert(2 * sizeof(float) == sizeof(double), "packed element sizes");
@@ -756,6 +807,7 @@ int fmm_build_tree(const fmm_node_desc *nodes, int64_t n_nodes, const fmm_config
         }
     }
     build_stencils(t);
+    build_orbits(t);
     plan_work(t);
     plan_dataflow(t);
     // per-level geometry: h = box / (8 * 2^(l-1)) is exact up to the box edge

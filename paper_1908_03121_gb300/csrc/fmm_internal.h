@@ -75,10 +75,12 @@ struct DeviceTables {
     StencilEntry *stencil = nullptr; // [8][ent_stride]
     float *stencil_f = nullptr;      // [8][ent_stride][4] the same entries with the offset
                                      // as floats (window offset's int bits in the fourth)
+    // monopole<-monopole, mixed precision
     float *coef32 = nullptr;         // [ent_stride][4] monopole weights of parity 0
-    double *coef64 = nullptr;        // [ent_stride][4]
-    float *coefdf = nullptr;         // [ent_stride][4][hi, lo]
     int32_t *mono_woff = nullptr;    // [8][ent_stride] window offsets, parity 0's order reflected
+    // monopole<-monopole, FP64 and double-float (fmm_mono_wide.cuh)
+    int4 *orbits = nullptr;          // near parent offsets (dx, dy, dz >= 0, mask of nonzero axes)
+    void *orbit_coef = nullptr;      // [orbit][b][q][4] transformed weights: double or float pairs
     int32_t *tree_leaf_off = nullptr;   // [n_trees + 1]
     int32_t *tree_leaf_rows = nullptr;  // [n_leaf]
     double *levels = nullptr;        // [max_level + 1][LEVEL_FIELDS]
@@ -169,9 +171,10 @@ struct fmm_tree_s {
     std::vector<fmm::StencilEntry> stencil;
     std::vector<float> stencil_f;
     std::vector<float> coef32;
-    std::vector<double> coef64;
-    std::vector<float> coefdf;
     std::vector<int32_t> mono_woff;
+    std::vector<int32_t> orbits;         // [n][4]
+    std::vector<double> orbit_coef;      // [orbit][b][q][4]
+    int32_t orbit_first[9] = {0};        // the orbits of mask k: orbit_first[k] .. [k + 1]
     std::vector<int32_t> tree_leaf_off, tree_leaf_rows;
     std::vector<double> levels;
     std::vector<float> levels_df;

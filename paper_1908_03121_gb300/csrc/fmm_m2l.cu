@@ -77,7 +77,7 @@ struct KParams {
     int32_t *counter;
     const StencilEntry *stencil;
     const float4 *stencil_f;  // the same, offsets as floats, window offset's bits in w
-    const void *coef;        // monopole weights of parity 0
+    const float *coef;       // monopole weights of parity 0 (mixed)
     const int32_t *mono_woff;  // [8][ent_stride] window offsets in parity 0's order, reflected
     int n_far, n_near;       // identical for every parity
     int ent_stride;          // entries reserved per parity
@@ -505,8 +505,8 @@ constexpr int kMpPairs = 4 + 3;      // compensated float components of mp_kerne
 // Same-level results are stored with the evict-first (streaming) hint: they
 // are read once, much later, by the downward pass, and left in L2 they would
 // push out the packed source moments that the multipole kernel rereads.
-template <typename T>
-__device__ __forceinline__ void store_L(const KParams &P, int node, int k, int cell, T hi, T lo)
+template <typename T, class Params>
+__device__ __forceinline__ void store_L(const Params &P, int node, int k, int cell, T hi, T lo)
 {
     const size_t idx = (size_t(node) * NCOMP + k) * NCELL + cell;
     if constexpr (kF32<T>) {
@@ -564,6 +564,31 @@ __device__ __forceinline__ void store_target(const KParams &P, int node, int cel
     }
     store_target_values<float>(P, node, cell, hi, lo);
 }
+
+// four consecutive values from shared memory
+template <typename T>
+__device__ __forceinline__ void load4_shared(const T *p, T v[4])
+{
+    if constexpr (kDF<T>) {
+        const float4 a = reinterpret_cast<const float4 *>(p)[0];
+        const float4 b = reinterpret_cast<const float4 *>(p)[1];
+        v[0] = dfloat(a.x, a.y); v[1] = dfloat(a.z, a.w);
+        v[2] = dfloat(b.x, b.y); v[3] = dfloat(b.z, b.w);
+    } else {
+        const double2 a = reinterpret_cast<const double2 *>(p)[0];
+        const double2 b = reinterpret_cast<const double2 *>(p)[1];
+        v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+    }
+}
+
+}  // namespace
+}  // namespace fmm
+
+#include "fmm_mono_wide.cuh"
+
+namespace fmm {
+
+namespace {
 
 // packed data of one source cell (level units)
 template <typename T>
@@ -1294,72 +1319,54 @@ __global__ void __launch_bounds__(kThreads, 2) mp2_kernel(KParams P)
 // the signs of its L1 components along p's odd axes at the end (exact).  The
 // table and the window offsets sit in shared memory, loaded once per CTA;
 // every access to them is a warp-uniform broadcast.
+// (Mixed precision; the wide types' kernel is in fmm_mono_wide.cuh.)
 // Each pass takes NB sub-grids (consecutive in the cost-sorted queue), each
 // with its own halo window, staged by cp.async so that every load of the
 // window is in flight at once; every thread holds two target cells (z and
 // z+4 of one parity) per sub-grid, so each weight feeds 2 NB cells.
-template <typename T>
-__device__ __forceinline__ void load4_shared(const T *p, T v[4])
-{
-    if constexpr (kF32<T>) {
-        const float4 f = *reinterpret_cast<const float4 *>(p);
-        v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
-    } else if constexpr (kDF<T>) {
-        const float4 a = reinterpret_cast<const float4 *>(p)[0];
-        const float4 b = reinterpret_cast<const float4 *>(p)[1];
-        v[0] = dfloat(a.x, a.y); v[1] = dfloat(a.z, a.w);
-        v[2] = dfloat(b.x, b.y); v[3] = dfloat(b.z, b.w);
-    } else {
-        const double2 a = reinterpret_cast<const double2 *>(p)[0];
-        const double2 b = reinterpret_cast<const double2 *>(p)[1];
-        v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
-    }
-}
-
 // Wb = the window at this thread's first target cell; the NB windows are
 // WSTRIDE apart and the second target cell DZ1 further on (compile-time
 // offsets, folded into the shared-memory loads)
-template <typename T, int NB, int WSTRIDE, int DZ1>
-__device__ __forceinline__ void mono_entry(const T *Wb, const int *woff, const T *coef, int e,
-                                           Acc<T, 4> (&A)[NB], Acc<T, 4> (&B)[NB])
+template <int NB, int WSTRIDE, int DZ1>
+__device__ __forceinline__ void mono_entry(const float *Wb, const int *woff, const float *coef, int e,
+                                           Acc<float, 4> (&A)[NB], Acc<float, 4> (&B)[NB])
 {
-    const T *src = Wb + woff[e];
-    T c[4];
-    load4_shared<T>(coef + 4 * e, c);
+    const float *src = Wb + woff[e];
+    const float4 c4 = *reinterpret_cast<const float4 *>(coef + 4 * e);
+    const float c[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
-        const T m0 = src[b * WSTRIDE];
-        const T m1 = src[b * WSTRIDE + DZ1];
+        const float m0 = src[b * WSTRIDE];
+        const float m1 = src[b * WSTRIDE + DZ1];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            A[b].part[k] = fmadd_u(c[k], m0, A[b].part[k]);
-            B[b].part[k] = fmadd_u(c[k], m1, B[b].part[k]);
+            A[b].part[k] = fmaf(c[k], m0, A[b].part[k]);
+            B[b].part[k] = fmaf(c[k], m1, B[b].part[k]);
         }
     }
 }
 
-// dynamic shared memory of mono_kernel<T, NB, R>: NB windows, the weight table
+// dynamic shared memory of mono_kernel<NB, R>: NB windows, the weight table
 // of parity 0 and the window offsets of all parities
-template <typename T>
-size_t mono_smem_bytes(int nb, size_t window_bytes, int ent_stride)
+inline size_t mono_smem_bytes(int nb, size_t window_bytes, int ent_stride)
 {
-    return nb * window_bytes + size_t(ent_stride) * 4 * sizeof(T) + size_t(8) * ent_stride * sizeof(int);
+    return nb * window_bytes + size_t(ent_stride) * 4 * sizeof(float) + size_t(8) * ent_stride * sizeof(int);
 }
 
-template <typename T, int NB, int RR>
+template <int NB, int RR>
 __global__ void __launch_bounds__(kThreads) mono_kernel(KParams P)
 {
     using G = WinGeo<RR>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int wstride = 8 * G::SUB_STRIDE;
-    T *W = reinterpret_cast<T *>(smem_raw);
-    T *s_coef = W + NB * wstride;
+    float *W = reinterpret_cast<float *>(smem_raw);
+    float *s_coef = W + NB * wstride;
     int *s_woff = reinterpret_cast<int *>(s_coef + 4 * P.ent_stride);
     __shared__ int s_nbr[NB][27], s_leaf[NB][27], s_row[NB][27], s_item;
     const int n_ent = P.n_far + P.n_near;
     {
-        const T *gcoef = static_cast<const T *>(P.coef);          // parity 0 first
-        for (int i = threadIdx.x; i < 4 * n_ent; i += blockDim.x) s_coef[i] = ldg_t(gcoef + i);
+        const float *gcoef = P.coef;                              // parity 0's
+        for (int i = threadIdx.x; i < 4 * n_ent; i += blockDim.x) s_coef[i] = __ldg(gcoef + i);
         for (int i = threadIdx.x; i < 8 * P.ent_stride; i += blockDim.x)
             s_woff[i] = __ldg(P.mono_woff + i);
     }
@@ -1368,7 +1375,7 @@ __global__ void __launch_bounds__(kThreads) mono_kernel(KParams P)
     const int px = p & 1, py = (p >> 1) & 1, pz = p >> 2;
     const int cx = lane & 3, cy = (lane >> 2) & 3, cz = lane >> 4;
     const int *woff = s_woff + p * P.ent_stride;
-    const T *mass = static_cast<const T *>(P.mass);
+    const float *mass = static_cast<const float *>(P.mass);
     const int base0 = cx + G::PY * cy + G::PZ * cz;
     constexpr int dz1 = 2 * G::PZ;              // the second target cell, z + 4
     for (;;) {
@@ -1385,31 +1392,31 @@ __global__ void __launch_bounds__(kThreads) mono_kernel(KParams P)
         __syncthreads();
 #pragma unroll
         for (int b = 0; b < NB; ++b)
-            if (nodes[b] >= 0) stage_window_async<T, RR>(W + b * wstride, s_nbr[b], s_leaf[b], mass, P);
+            if (nodes[b] >= 0) stage_window_async<float, RR>(W + b * wstride, s_nbr[b], s_leaf[b], mass, P);
         cp_async_commit();
         cp_async_wait_all();
         __syncthreads();
-        Acc<T, 4> A[NB], B[NB];
+        Acc<float, 4> A[NB], B[NB];
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
             A[b].zero();
             B[b].zero();
         }
-        // float: 32 entries per compensated chunk (the TwoSum folds are a
-        // fifth of this kernel's instructions at 16); double-float keeps 16
-        constexpr int chunk = kF32<T> ? 2 * kChunk : kChunk;
+        // 32 entries per compensated chunk (the TwoSum folds are a
+        // fifth of this kernel's instructions at 16)
+        constexpr int chunk = 2 * kChunk;
         int e = 0;
         for (; e + chunk <= n_ent; e += chunk) {
 #pragma unroll
             for (int j = 0; j < chunk; ++j)
-                mono_entry<T, NB, wstride, dz1>(W + base0, woff, s_coef, e + j, A, B);
+                mono_entry<NB, wstride, dz1>(W + base0, woff, s_coef, e + j, A, B);
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
                 A[b].flush();
                 B[b].flush();
             }
         }
-        for (; e < n_ent; ++e) mono_entry<T, NB, wstride, dz1>(W + base0, woff, s_coef, e, A, B);
+        for (; e < n_ent; ++e) mono_entry<NB, wstride, dz1>(W + base0, woff, s_coef, e, A, B);
         const int ax = 2 * cx + px, ay = 2 * cy + py;
         const int cell0 = ax + 8 * ay + 64 * (2 * cz + pz);
         const int cell1 = cell0 + 64 * 4;
@@ -1422,10 +1429,10 @@ __global__ void __launch_bounds__(kThreads) mono_kernel(KParams P)
             for (int k = 0; k < 4; ++k) {
                 // first-order weights were parity 0's: undo the reflection
                 const bool flip = k > 0 && ((p >> (k - 1)) & 1);
-                const T ah = acc_hi(A[b], k), al = acc_lo(A[b], k);
-                const T bh = acc_hi(B[b], k), bl = acc_lo(B[b], k);
-                store_L<T>(P, nodes[b], k, cell0, flip ? -ah : ah, flip ? -al : al);
-                store_L<T>(P, nodes[b], k, cell1, flip ? -bh : bh, flip ? -bl : bl);
+                const float ah = acc_hi(A[b], k), al = acc_lo(A[b], k);
+                const float bh = acc_hi(B[b], k), bl = acc_lo(B[b], k);
+                store_L<float>(P, nodes[b], k, cell0, flip ? -ah : ah, flip ? -al : al);
+                store_L<float>(P, nodes[b], k, cell1, flip ? -bh : bh, flip ? -bl : bl);
             }
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
@@ -1657,7 +1664,12 @@ struct Kernels {
     static cudaError_t mono(size_t bytes)
     {
         static size_t done = 0;
-        return allow_smem(mono_kernel<T, NB, RR>, bytes, done);
+        return allow_smem(mono_kernel<NB, RR>, bytes, done);
+    }
+    static cudaError_t mono_wide(size_t bytes)
+    {
+        static size_t done = 0;
+        return allow_smem(mono_wide_kernel<T>, bytes, done);
     }
 };
 
@@ -1675,32 +1687,59 @@ int persistent_grid(Kern k, size_t smem, int64_t items, int sms, int cap_per_sm,
     return int(items < g ? items : g);
 }
 
-template <typename T, int NB, int RR>
+template <int NB, int RR>
 cudaError_t launch_mono_r(const KParams &K, size_t wbytes, int sms, int cap, cudaStream_t s)
 {
     // the compile-time window geometry must be the host's
     using G = WinGeo<RR>;
     if (K.reach != G::R || K.py != G::PY || K.pz != G::PZ || K.sub_stride != G::SUB_STRIDE)
         return cudaErrorInvalidValue;
-    const size_t bytes = mono_smem_bytes<T>(NB, wbytes, K.ent_stride);
-    cudaError_t e = Kernels<T>::template mono<NB, RR>(bytes);
+    const size_t bytes = mono_smem_bytes(NB, wbytes, K.ent_stride);
+    cudaError_t e = Kernels<float>::mono<NB, RR>(bytes);
     if (e != cudaSuccess) return e;
     const int64_t passes = (K.n_items + NB - 1) / NB;
-    const int g = persistent_grid(mono_kernel<T, NB, RR>, bytes, passes, sms, cap);
-    mono_kernel<T, NB, RR><<<g, kThreads, bytes, s>>>(K);
+    const int g = persistent_grid(mono_kernel<NB, RR>, bytes, passes, sms, cap);
+    mono_kernel<NB, RR><<<g, kThreads, bytes, s>>>(K);
     return cudaGetLastError();
 }
 
 // theta in (0.25, 1/sqrt(3)] gives reach 2 floor(1/theta) + 1 = 3, 5 or 7
-template <typename T, int NB>
+template <int NB>
 cudaError_t launch_mono(const KParams &K, size_t wbytes, int sms, int cap, cudaStream_t s)
 {
     switch (K.reach) {
-    case 3: return launch_mono_r<T, NB, 3>(K, wbytes, sms, cap, s);
-    case 5: return launch_mono_r<T, NB, 5>(K, wbytes, sms, cap, s);
-    case 7: return launch_mono_r<T, NB, 7>(K, wbytes, sms, cap, s);
+    case 3: return launch_mono_r<NB, 3>(K, wbytes, sms, cap, s);
+    case 5: return launch_mono_r<NB, 5>(K, wbytes, sms, cap, s);
+    case 7: return launch_mono_r<NB, 7>(K, wbytes, sms, cap, s);
     default: return cudaErrorInvalidValue;
     }
+}
+
+// the wide types' monopole kernel: one leaf node per item, one CTA per SM
+template <typename T>
+cudaError_t launch_mono_wide(const fmm_tree_s *t, const KParams &K, int sms, cudaStream_t s)
+{
+    MonoWParams P{};
+    P.info = K.info;
+    P.nbr = K.nbr;
+    P.list = K.list;
+    P.n_items = K.n_items;
+    P.counter = K.counter;
+    P.orbits = t->dev.orbits;
+    for (int k = 0; k < 9; ++k) P.first[k] = t->orbit_first[k];
+    P.coef = t->dev.orbit_coef;
+    P.n_coef = int(t->orbit_coef.size());
+    P.reach = (K.reach - 1) / 2;
+    P.mass = K.mass;
+    P.L = K.L;
+    P.Lc = K.Lc;
+    P.dL1 = K.dL1;
+    const size_t bytes = mono_wide_smem<T>(P.reach, P.n_coef);
+    cudaError_t e = Kernels<T>::mono_wide(bytes);
+    if (e != cudaSuccess) return e;
+    const int g = int(std::min<int64_t>(K.n_items, sms));
+    mono_wide_kernel<T><<<g, kMonoWThreads, bytes, s>>>(P);
+    return cudaGetLastError();
 }
 
 // the multipole launch, PARTS items per sub-grid
@@ -1732,9 +1771,7 @@ cudaError_t launch_all(const fmm_tree_s *t, void *L, float *Lc, double *dL1, cud
     P.nbr = d.nbr;
     P.stencil = d.stencil;
     P.stencil_f = reinterpret_cast<const float4 *>(d.stencil_f);
-    P.coef = kF32<T> ? static_cast<const void *>(d.coef32)
-             : kDF<T> ? static_cast<const void *>(d.coefdf)
-                      : static_cast<const void *>(d.coef64);
+    P.coef = d.coef32;
     P.n_far = Pl.n_far[0];
     P.n_near = Pl.n_near[0];
     P.ent_stride = Pl.ent_stride;
@@ -1834,16 +1871,19 @@ cudaError_t launch_all(const fmm_tree_s *t, void *L, float *Lc, double *dL1, cud
         K.list = d.lists + Pl.work_mono.off;
         K.n_items = int32_t(Pl.work_mono.count);
         K.counter = d.counters + Q_MONO;
-        int nb = t->tuning.mono_subgrids;
-        if (nb != 1 && nb != 2 && nb != 4) nb = kF32<T> ? 2 : 1;
-        if (!kF32<T> && nb == 4) nb = 2;
-        // fewer sub-grids per pass where their windows do not fit
-        const size_t smem_max = max_smem_optin_of_current_device();
-        while (nb > 1 && mono_smem_bytes<T>(nb, wbytes, Pl.ent_stride) > smem_max) nb /= 2;
         timing_begin(t, FMM_K_MONOPOLE, s);
-        e = nb == 1 ? launch_mono<T, 1>(K, wbytes, sms, cap, s)
-            : nb == 2 ? launch_mono<T, 2>(K, wbytes, sms, cap, s)
-                      : launch_mono<T, kF32<T> ? 4 : 2>(K, wbytes, sms, cap, s);
+        if constexpr (kF32<T>) {
+            int nb = t->tuning.mono_subgrids;
+            if (nb != 1 && nb != 2 && nb != 4) nb = 2;
+            // fewer sub-grids per pass where their windows do not fit
+            const size_t smem_max = max_smem_optin_of_current_device();
+            while (nb > 1 && mono_smem_bytes(nb, wbytes, Pl.ent_stride) > smem_max) nb /= 2;
+            e = nb == 1 ? launch_mono<1>(K, wbytes, sms, cap, s)
+                : nb == 2 ? launch_mono<2>(K, wbytes, sms, cap, s)
+                          : launch_mono<4>(K, wbytes, sms, cap, s);
+        } else {
+            e = launch_mono_wide<T>(t, K, sms, s);
+        }
         timing_end(t, s);
         ++nl;
         if (e != cudaSuccess) return e;
