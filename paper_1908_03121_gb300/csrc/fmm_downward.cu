@@ -13,7 +13,7 @@
 // (forming L64).  The correction is carried in FP64 in every precision.
 // forces_kernel: phi = L0, g = -(L1 + dL1), f = m g, and fixed-order FP64
 // block sums of f and x cross f (plus the |f|, |x cross f| normalisers) per
-// leaf node; reduce_chunk_kernel and reduce_final_kernel fold those per tree.
+// leaf node; reduce_kernel folds those per tree.
 #include "fmm_convert.cuh"
 #include "fmm_internal.h"
 #include "fmm_tensor.cuh"
@@ -652,35 +652,62 @@ __global__ void __launch_bounds__(kForceThreads, 12) dataflow_kernel(DflowParams
     }
 }
 
-// Per-tree sums of the per-leaf-node partials in two fixed-order stages, so
-// the FP64 adds spread over many SMs: chunks of kReduceRows leaf rows per CTA,
-// then one warp per tree over its chunks.
-__global__ void __launch_bounds__(512) reduce_chunk_kernel(const int32_t *__restrict__ off,
-                                                           const int32_t *__restrict__ rows,
-                                                           const double *__restrict__ partials,
-                                                           double *__restrict__ chunk_sums)
+// Per-tree sums of the per-leaf-node partials, in one launch and a fixed
+// order: chunks of kReduceRows leaf rows per CTA, and the tree's last CTA to
+// finish (a counter per tree, left at zero again) adds the chunks.  Both
+// stages read eight threads per row, 64 contiguous bytes, and add what one
+// component's threads hold by shuffles, then across warps through shared
+// memory.  (Two launches, with a whole row per thread and full shuffle trees of
+// FP64 adds, took 17 + 3 us whatever the tree's size; one step of 8, 64 or 512
+// leaf nodes became 12 to 15 us shorter.)
+constexpr int kReduceThreads = 256;
+
+// sum over `rows` rows of 8 values; row(i) gives row i's address; the result
+// in threads 0-7 (component = thread)
+template <class Row>
+__device__ __forceinline__ double row_sums(int rows, Row row, double (*sh)[8])
 {
-    __shared__ double sh[16][8];
-    const int tree = blockIdx.x, chunk = blockIdx.y;
-    const int lo = off[tree] + chunk * kReduceRows;
-    const int hi = min(lo + kReduceRows, off[tree + 1]);
-    double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int i = lo + threadIdx.x; i < hi; i += blockDim.x)
+    const int k = threadIdx.x & 7, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double v = 0.0;
+    for (int i = threadIdx.x >> 3; i < rows; i += kReduceThreads / 8) v += __ldcg(row(i) + k);   // past L1: other CTAs wrote the chunk sums
+    v += __shfl_xor_sync(0xffffffffu, v, 8);
+    v += __shfl_xor_sync(0xffffffffu, v, 16);
+    if (lane < 8) sh[warp][lane] = v;
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        v = sh[0][k];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] += partials[size_t(rows[i]) * 8 + k];
-    block_sum<512, double, 8>(v, sh);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 8; ++k) chunk_sums[(size_t(tree) * gridDim.y + chunk) * 8 + k] = v[k];
+        for (int w = 1; w < kReduceThreads / 32; ++w) v += sh[w][k];
+    }
+    return v;
 }
 
-__global__ void __launch_bounds__(32) reduce_final_kernel(const double *__restrict__ chunk_sums,
-                                                          int chunks, double *__restrict__ totals)
+__global__ void __launch_bounds__(kReduceThreads) reduce_kernel(const int32_t *__restrict__ off,
+                                                                const int32_t *__restrict__ rows,
+                                                                const double *__restrict__ partials,
+                                                                double *__restrict__ chunk_sums,
+                                                                int32_t *__restrict__ arrived,
+                                                                double *__restrict__ totals)
 {
-    const int tree = blockIdx.x, k = threadIdx.x;
-    if (k >= 8) return;
-    double v = 0.0;
-    for (int c = 0; c < chunks; ++c) v += chunk_sums[(size_t(tree) * chunks + c) * 8 + k];
-    totals[size_t(tree) * 8 + k] = v;
+    __shared__ double sh[kReduceThreads / 32][8];
+    __shared__ int s_last;
+    const int tree = blockIdx.x, chunk = blockIdx.y, chunks = gridDim.y;
+    const int lo = off[tree] + chunk * kReduceRows;
+    const int n = min(kReduceRows, off[tree + 1] - lo);      // may be <= 0: a smaller tree
+    const double v = row_sums(n, [&](int i) { return partials + size_t(rows[lo + i]) * 8; }, sh);
+    double *mine = chunk_sums + size_t(tree) * chunks * 8;
+    if (threadIdx.x < 8) {
+        mine[chunk * 8 + threadIdx.x] = v;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(arrived + tree, 1) == chunks - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const double t = row_sums(chunks, [&](int i) { return mine + i * 8; }, sh);
+    if (threadIdx.x < 8) totals[size_t(tree) * 8 + threadIdx.x] = t;
+    if (threadIdx.x == 0) arrived[tree] = 0;
 }
 
 }  // namespace
@@ -819,12 +846,9 @@ cudaError_t launch_forces(const fmm_tree_s *t, const double *L64, const double *
 cudaError_t launch_force_sums(const fmm_tree_s *t, double *totals, cudaStream_t s)
 {
     timing_begin(t, FMM_K_REDUCE, s);
-    const int chunks = t->plan.reduce_chunks;
-    reduce_chunk_kernel<<<dim3(unsigned(t->n_trees), unsigned(chunks)), 512, 0, s>>>(
-        t->dev.tree_leaf_off, t->dev.tree_leaf_rows, t->dev.partials, t->dev.chunk_sums);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    reduce_final_kernel<<<unsigned(t->n_trees), 32, 0, s>>>(t->dev.chunk_sums, chunks, totals);
+    reduce_kernel<<<dim3(unsigned(t->n_trees), unsigned(t->plan.reduce_chunks)), kReduceThreads, 0, s>>>(
+        t->dev.tree_leaf_off, t->dev.tree_leaf_rows, t->dev.partials, t->dev.chunk_sums,
+        t->dev.reduce_arrived, totals);
     timing_end(t, s);
     return cudaGetLastError();
 }

@@ -636,7 +636,7 @@ static void free_device(fmm_tree_s *t)
     DeviceTables &d = t->dev;
     void *ptrs[] = {d.info, d.children, d.nbr, d.lists, d.stencil, d.stencil_f, d.coef32, d.mono_woff, d.orbits, d.orbit_coef,
                     d.tree_leaf_off, d.tree_leaf_rows, d.levels, d.levels_df, d.mass, d.mp, d.counters,
-                    d.partials, d.chunk_sums, d.up, d.down, d.mx_targets, d.mx_pairs,
+                    d.partials, d.chunk_sums, d.reduce_arrived, d.up, d.down, d.mx_targets, d.mx_pairs,
                     d.dflow_items, d.dflow_ready};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -686,13 +686,16 @@ static int upload_tree(fmm_tree_s *t)
         (e = cudaMalloc(reinterpret_cast<void **>(&d.counters), 64 * sizeof(int32_t))) != cudaSuccess ||
         (e = cudaMalloc(reinterpret_cast<void **>(&d.partials), part_b)) != cudaSuccess ||
         (e = cudaMalloc(reinterpret_cast<void **>(&d.chunk_sums), chunk_b)) != cudaSuccess ||
+        (e = cudaMalloc(reinterpret_cast<void **>(&d.reduce_arrived), size_t(t->n_trees) * sizeof(int32_t))) !=
+            cudaSuccess ||
         (e = cudaMalloc(reinterpret_cast<void **>(&d.dflow_ready), size_t(t->n) * sizeof(int32_t))) !=
             cudaSuccess)
         return fail(FMM_ERR_NOMEM, std::string("workspace cudaMalloc: ") + cudaGetErrorString(e));
     d.workspace_bytes = mass_b + mp_b + part_b + chunk_b + 64 * sizeof(int32_t) +
-                        size_t(t->n) * sizeof(int32_t);
+                        size_t(t->n) * sizeof(int32_t) + size_t(t->n_trees) * sizeof(int32_t);
     // work queues and the status word start at zero
     if ((e = cudaMemset(d.counters, 0, 64 * sizeof(int32_t))) != cudaSuccess ||
+        (e = cudaMemset(d.reduce_arrived, 0, size_t(t->n_trees) * sizeof(int32_t))) != cudaSuccess ||
         (e = cudaMemset(static_cast<char *>(d.mp) + size_t(t->n_refined) * mp_row_b, 0, mp_row_b)) !=
             cudaSuccess)
         return cuda_fail(e, "cudaMemset");
@@ -902,18 +905,18 @@ int fmm_get_stats(fmm_tree_t t, fmm_stats *o)
     int down = 0;
     for (int lev = 1; lev <= t->max_level; ++lev) down += P.nodes_at[size_t(lev)].count > 0;
     o->launches_m2l = m2l;
-    o->launches_step = up + m2l + down + 3;
+    o->launches_step = up + m2l + down + 2;
     // fmm_step: P2M also packs the leaf masses, one pack launch for the
     // refined nodes; then either the refined levels' shifts per level and
     // every leaf's shift and forces in one launch, or (dataflow tuning) all
-    // of it in one persistent launch; the two force-sum launches
+    // of it in one persistent launch; the force sums
     int refined_levels = 0;
     for (int lev = 1; lev <= t->max_level; ++lev) refined_levels += P.refined_at[size_t(lev)].count > 0;
     // (the monopole<-multipole targets ride in the multipole launch)
     const int mx_alone = (P.n_mx_targets > 0) && (P.work_mp.count == 0);
     const int downward = t->tuning.dataflow ? 1 : refined_levels + (P.leaves.count > 0);
     o->launches_fused = up + (m2l - 1) - (P.n_mx_targets > 0) + mx_alone + (P.refined.count > 0) +
-                        downward + 2;
+                        downward + 1;
     if ((t->cfg.flags & FMM_FLAG_TIMING) && !t->host_only) {
         o->timing = 1;
         timing_fold(t);

@@ -31,7 +31,7 @@ constexpr int NSIDE = 8;
 constexpr int NCELL = 512;
 constexpr int NCOMP = 20;
 constexpr int NMP = 16;          // packed same-level values per refined cell
-constexpr int kReduceRows = 1024;   // leaf rows per CTA of the first force-sum stage
+constexpr int kReduceRows = 256;    // leaf rows per CTA of the force sums
 
 // pad a pitch up to the next value congruent to want (mod 32): the halo
 // window's row and plane pitches, chosen so that the 32 lanes of a warp hit
@@ -95,6 +95,7 @@ struct DeviceTables {
     int32_t *counters = nullptr;     // work-queue heads; [kStatusSlot]: FMM_STATUS_* bits
     double *partials = nullptr;      // [n_leaf][8]
     double *chunk_sums = nullptr;    // [n_trees][reduce_chunks][8]
+    int32_t *reduce_arrived = nullptr;  // [n_trees] finished CTAs of the force sums (zero between steps)
     float *up = nullptr;             // mixed, dfloat: [n_refined][20][512] double-float
                                      // (hi, lo) results of the upward pass per refined cell
     int32_t *dflow_items = nullptr;  // dataflow downward queue: refined (node, slice) items
