@@ -901,7 +901,11 @@ int fmm_get_stats(fmm_tree_t t, fmm_stats *o)
     int m2l = 1 /*pack*/ + (P.roots.count > 0) + (P.work_mp.count > 0) + (P.work_mono.count > 0) +
               (P.n_mx_targets > 0);
     int up = 1;
-    for (int lev = 1; lev < t->max_level; ++lev) up += P.refined_at[size_t(lev)].count > 0;
+    for (int lev = 1; lev < t->max_level; ++lev) {
+        ListRange lean, lanes;
+        up += t->cfg.precision == FMM_FP64 ? P.refined_at[size_t(lev)].count > 0
+                                           : m2m_split(t, lev, lean, lanes);
+    }
     int down = 0;
     for (int lev = 1; lev <= t->max_level; ++lev) down += P.nodes_at[size_t(lev)].count > 0;
     o->launches_m2l = m2l;

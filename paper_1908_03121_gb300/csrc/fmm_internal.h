@@ -203,6 +203,8 @@ cudaError_t launch_p2m(const fmm_tree_s *t, const double *rho, double *M, cudaSt
                        bool pack_leaves = false);
 cudaError_t launch_m2m_level(const fmm_tree_s *t, int level, double *M, double *com,
                              cudaStream_t s);
+// mixed and double-float: the level's nodes by kernel; returns the launches
+int m2m_split(const fmm_tree_s *t, int level, ListRange &lean, ListRange &lanes);
 // which nodes a pack launch covers
 enum { PACK_ALL = 0, PACK_LEAVES = 1, PACK_REFINED = 2 };
 cudaError_t launch_pack(const fmm_tree_s *t, const double *M, const double *com,

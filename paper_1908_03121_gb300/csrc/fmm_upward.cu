@@ -216,10 +216,9 @@ __global__ void __launch_bounds__(kSliceThreads) m2m_kernel(const NodeInfo *__re
 // (q = half a child width).  The FP64 operations left per parent cell are the
 // splits of leaf-child masses (one subtraction each) and the conversions of
 // the 17 moments and 3 coordinates written to M and com (one add each).
-// Two launch shapes: one thread per parent cell (the recurrences above, with
-// the Hadamard transform for leaf children) for levels with many nodes, and
-// eight threads per parent cell for levels with few, where one thread's long
-// dependent sequence of double-float operations would set the time.
+// Two kernels: nodes whose children are all leaves take one thread per parent
+// cell and the Hadamard transform of the recurrences above; the others take
+// four threads per parent cell.
 __device__ __forceinline__ void write_up(const NodeInfo &ni, int node, int c, int x, int y, int z,
                                          double hp, const dfloat &m0, const dfloat d[3],
                                          const dfloat M2[6], const dfloat M3[10], double *M,
@@ -249,13 +248,10 @@ __device__ __forceinline__ void write_up(const NodeInfo &ni, int node, int c, in
     for (int t = 0; t < 10; ++t) ou[(10 + t) * NCELL] = M3[t];
 }
 
-// one thread per parent cell, 8 CTAs of 64 threads per node.  LEAF_KIDS:
-// every child of the launch's nodes is a leaf (the deepest refined level,
-// the bulk of the upward pass's cells), so only the leaf-children branch is
-// compiled: far fewer registers than the general kernel, which lets the
-// launch share its SMs with the persistent monopole kernel that runs beside
-// the upward pass in fmm_step.
-template <bool LEAF_KIDS>
+// Nodes with only leaf children (the deepest refined level, the bulk of the
+// upward pass's cells): one thread per parent cell, 8 CTAs of 64 threads per
+// node, 64 registers, which lets the launch share its SMs with the persistent
+// monopole kernel that runs beside the upward pass in fmm_step.
 __global__ void __launch_bounds__(kSliceThreads) m2m_df_kernel(const NodeInfo *__restrict__ info,
                                                                const int32_t *__restrict__ children,
                                                                const int32_t *__restrict__ nodes,
@@ -271,185 +267,177 @@ __global__ void __launch_bounds__(kSliceThreads) m2m_df_kernel(const NodeInfo *_
     const int x = c & 7, y = (c >> 3) & 7, z = c >> 6;
     const int k = (x >> 2) + 2 * (y >> 2) + 4 * (z >> 2);
     const int ch = children[node * 8 + k];
-    const NodeInfo ci = info[ch];
     const double hp = levels[ni.level * LEVEL_FIELDS + LV_H];
     const dfloat q = df_from_double(0.25 * hp);           // half a child cell width
     const int c0 = 2 * (x & 3) + 16 * (y & 3) + 128 * (z & 3);   // child cell of j = 0
     dfloat m0, d[3], M2[6], M3[10];
-    if (LEAF_KIDS || ci.leaf_row >= 0) {
-        // child j sits at ref + q (e_x, e_y, e_z), e = +-1 from the bits of j
-        const size_t cbase = size_t(ch) * NCOMP * NCELL;
-        dfloat m[8];
+    // child j sits at ref + q (e_x, e_y, e_z), e = +-1 from the bits of j
+    const size_t cbase = size_t(ch) * NCOMP * NCELL;
+    dfloat m[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-            m[j] = df_from_double(M[cbase + c0 + (j & 1) + 8 * ((j >> 1) & 1) + 64 * (j >> 2)]);
-        dfloat a[8];
+    for (int j = 0; j < 8; ++j)
+        m[j] = df_from_double(M[cbase + c0 + (j & 1) + 8 * ((j >> 1) & 1) + 64 * (j >> 2)]);
+    dfloat a[8];
 #pragma unroll
-        for (int j = 0; j < 8; j += 2) { a[j] = m[j] + m[j + 1]; a[j + 1] = m[j + 1] - m[j]; }
-        dfloat b[8];
+    for (int j = 0; j < 8; j += 2) { a[j] = m[j] + m[j + 1]; a[j + 1] = m[j + 1] - m[j]; }
+    dfloat b[8];
 #pragma unroll
-        for (int j = 0; j < 8; j += 4)
+    for (int j = 0; j < 8; j += 4)
 #pragma unroll
-            for (int i = 0; i < 2; ++i) { b[j + i] = a[j + i] + a[j + i + 2]; b[j + i + 2] = a[j + i + 2] - a[j + i]; }
-        dfloat e[8];
+        for (int i = 0; i < 2; ++i) { b[j + i] = a[j + i] + a[j + i + 2]; b[j + i + 2] = a[j + i + 2] - a[j + i]; }
+    dfloat e[8];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) { e[i] = b[i] + b[i + 4]; e[i + 4] = b[i + 4] - b[i]; }
-        m0 = e[0];
-        const dfloat qm = q / m0;
-        d[0] = qm * e[1];
-        d[1] = qm * e[2];
-        d[2] = qm * e[4];
-        const dfloat q2 = q * q, q3 = q2 * q;
-        const dfloat q2m = q2 * m0;
-        const dfloat S2[6] = {q2m, q2 * e[3], q2 * e[5], q2m, q2 * e[6], q2m};
-        const dfloat q3x = q3 * e[1], q3y = q3 * e[2], q3z = q3 * e[4];
-        const dfloat S3[10] = {q3x, q3y, q3z, q3x, q3 * e[7], q3x, q3y, q3z, q3y, q3z};
-        central_from_raw(m0, d, S2, S3, M2, M3);
-    } else if constexpr (!LEAF_KIDS) {
-        const dfloat *cu = up + size_t(ci.mp_row) * 20 * NCELL;
-        dfloat mj[8], X[8][3];
-        m0 = dfloat(0.f);
-        dfloat mr[3] = {dfloat(0.f), dfloat(0.f), dfloat(0.f)};
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int cc = c0 + (j & 1) + 8 * ((j >> 1) & 1) + 64 * (j >> 2);
-            mj[j] = cu[cc];
-#pragma unroll
-            for (int t = 0; t < 3; ++t) {
-                const dfloat sq = ((j >> t) & 1) ? q : -q;
-                X[j][t] = sq + cu[(1 + t) * NCELL + cc];
-            }
-            m0 += mj[j];
-#pragma unroll
-            for (int t = 0; t < 3; ++t) mr[t] += mj[j] * X[j][t];
-        }
-#pragma unroll
-        for (int t = 0; t < 3; ++t) d[t] = mr[t] / m0;
-#pragma unroll
-        for (int t = 0; t < 6; ++t) M2[t] = dfloat(0.f);
-#pragma unroll
-        for (int t = 0; t < 10; ++t) M3[t] = dfloat(0.f);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int cc = c0 + (j & 1) + 8 * ((j >> 1) & 1) + 64 * (j >> 2);
-            const dfloat s3[3] = {X[j][0] - d[0], X[j][1] - d[1], X[j][2] - d[2]};
-            const dfloat ms[3] = {mj[j] * s3[0], mj[j] * s3[1], mj[j] * s3[2]};
-            dfloat c2[6];
-#pragma unroll
-            for (int t = 0; t < 6; ++t) c2[t] = cu[(4 + t) * NCELL + cc];
-            dfloat mss[6];
-#pragma unroll
-            for (int t = 0; t < 6; ++t) {
-                mss[t] = ms[i2_at(t, 0)] * s3[i2_at(t, 1)];
-                M2[t] += c2[t] + mss[t];
-            }
-#pragma unroll
-            for (int t = 0; t < 10; ++t) {
-                const int a = i3_at(t, 0), b = i3_at(t, 1), e = i3_at(t, 2);
-                M3[t] += cu[(10 + t) * NCELL + cc] + c2[r2_of(a, b)] * s3[e] + c2[r2_of(a, e)] * s3[b] +
-                         c2[r2_of(b, e)] * s3[a] + mss[r2_of(a, b)] * s3[e];
-            }
-        }
-    }
+    for (int i = 0; i < 4; ++i) { e[i] = b[i] + b[i + 4]; e[i + 4] = b[i + 4] - b[i]; }
+    m0 = e[0];
+    const dfloat qm = q / m0;
+    d[0] = qm * e[1];
+    d[1] = qm * e[2];
+    d[2] = qm * e[4];
+    const dfloat q2 = q * q, q3 = q2 * q;
+    const dfloat q2m = q2 * m0;
+    const dfloat S2[6] = {q2m, q2 * e[3], q2 * e[5], q2m, q2 * e[6], q2m};
+    const dfloat q3x = q3 * e[1], q3y = q3 * e[2], q3z = q3 * e[4];
+    const dfloat S3[10] = {q3x, q3y, q3z, q3x, q3 * e[7], q3x, q3y, q3z, q3y, q3z};
+    central_from_raw(m0, d, S2, S3, M2, M3);
     write_up(ni, node, c, x, y, z, hp, m0, d, M2, M3, M, com, up, lo_x, lo_y, lo_z);
 }
 
-// eight threads per parent cell, one per child cell: each forms its child's
-// raw moments about the parent cell's centre ref,
-//   m,  m X,  M2c + m X X,  M3c + (M2c X, three terms) + m X X X,
-// X = child centre of mass - ref (a leaf child's M2c, M3c vanish), the eight
-// are summed by a butterfly of shuffles (every lane ends with the same sums:
-// double-float addition is commutative), and every lane turns them into
-// central moments about X = ref + m X / m and writes its share of the outputs.
-constexpr int kCellsPerCta = 8;
-// levels with fewer refined nodes than this take eight threads per cell
-constexpr int64_t kLanesBelow = 128;
+// Every other node: four threads per parent cell, two child cells each.  The
+// mass and centre of mass first (sums over the four by a butterfly of
+// shuffles), then each thread's share of the central moments, which the four
+// add by halves (each ends with the sums of four of the sixteen components)
+// and write.  Shorter dependent chains than one thread per cell (whose eight
+// children, unrolled, were 7000 instructions), without the redundant work of
+// eight: a level of 196 nodes 110 -> 42 us, of 76 nodes 61 -> 20, of 64
+// nodes 40 -> 18, of 8 nodes 12 -> 9.
+constexpr int kLanes = 4;
+// levels of both kinds with at least this many nodes take a launch for each
+constexpr int64_t kSplitFrom = 96;
+constexpr int kCellsPerCta = kSliceThreads / kLanes;
 
 __device__ __forceinline__ dfloat shfl_xor_df(dfloat v, int mask)
 {
     return dfloat(__shfl_xor_sync(0xffffffffu, v.hi, mask), __shfl_xor_sync(0xffffffffu, v.lo, mask));
 }
 
-__global__ void __launch_bounds__(8 * kCellsPerCta) m2m_df_lanes_kernel(const NodeInfo *__restrict__ info,
-                                                                  const int32_t *__restrict__ children,
-                                                                  const int32_t *__restrict__ nodes,
-                                                                  const double *__restrict__ levels,
-                                                                  double *__restrict__ M,
-                                                                  double *__restrict__ com,
-                                                                  dfloat *__restrict__ up, double lo_x,
-                                                                  double lo_y, double lo_z)
+// the lower half of v's N values stays with the threads whose `upper` is
+// false, the upper half goes to the others; both add their partner's
+template <int N>
+__device__ __forceinline__ void add_halves(dfloat (&v)[16], bool upper, int mask)
+{
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) {
+        const dfloat keep = upper ? v[i + N / 2] : v[i], give = upper ? v[i] : v[i + N / 2];
+        v[i] = keep + shfl_xor_df(give, mask);
+    }
+}
+
+__global__ void __launch_bounds__(kSliceThreads) m2m_df_lanes_kernel(
+    const NodeInfo *__restrict__ info, const int32_t *__restrict__ children,
+    const int32_t *__restrict__ nodes, const double *__restrict__ levels, double *__restrict__ M,
+    double *__restrict__ com, dfloat *__restrict__ up, double lo_x, double lo_y, double lo_z)
 {
     constexpr int kCtasPerNode = NCELL / kCellsPerCta;
     const int node = nodes[blockIdx.x / kCtasPerNode];
     const NodeInfo ni = info[node];
-    const int c = (blockIdx.x % kCtasPerNode) * kCellsPerCta + (threadIdx.x >> 3);
-    const int j = threadIdx.x & 7;                            // child cell of this lane
+    const int c = (blockIdx.x % kCtasPerNode) * kCellsPerCta + threadIdx.x / kLanes;
+    const int lane = threadIdx.x % kLanes;                    // children 2 lane, 2 lane + 1
     const int x = c & 7, y = (c >> 3) & 7, z = c >> 6;
     const int k = (x >> 2) + 2 * (y >> 2) + 4 * (z >> 2);
     const int ch = children[node * 8 + k];
     const NodeInfo ci = info[ch];
     const double hp = levels[ni.level * LEVEL_FIELDS + LV_H];
-    const dfloat q = df_from_double(0.25 * hp);
-    const int cc = 2 * (x & 3) + 16 * (y & 3) + 128 * (z & 3) + (j & 1) + 8 * ((j >> 1) & 1) +
-                   64 * (j >> 2);
-    dfloat X[3], m, c2[6], c3[10];
+    const dfloat q = df_from_double(0.25 * hp);               // half a child cell width
+    const int cc = 2 * (x & 3) + 16 * (y & 3) + 128 * (z & 3) + 8 * (lane & 1) + 64 * (lane >> 1);
+    // child i at cc + i: offset from the parent cell's centre, moments (a
+    // leaf's vanish)
+    dfloat m[2], X[2][3], c2[2][6], c3[2][10];
 #pragma unroll
-    for (int t = 0; t < 3; ++t) X[t] = ((j >> t) & 1) ? q : -q;
+    for (int i = 0; i < 2; ++i) {
+        X[i][0] = i ? q : -q;
+        X[i][1] = (lane & 1) ? q : -q;
+        X[i][2] = (lane >> 1) ? q : -q;
+#pragma unroll
+        for (int t = 0; t < 6; ++t) c2[i][t] = dfloat(0.f);
+#pragma unroll
+        for (int t = 0; t < 10; ++t) c3[i][t] = dfloat(0.f);
+    }
     if (ci.leaf_row >= 0) {
-        m = df_from_double(M[size_t(ch) * NCOMP * NCELL + cc]);
+        const double *Mc = M + size_t(ch) * NCOMP * NCELL + cc;
 #pragma unroll
-        for (int t = 0; t < 6; ++t) c2[t] = dfloat(0.f);
-#pragma unroll
-        for (int t = 0; t < 10; ++t) c3[t] = dfloat(0.f);
+        for (int i = 0; i < 2; ++i) m[i] = df_from_double(Mc[i]);
     } else {
         const dfloat *cu = up + size_t(ci.mp_row) * 20 * NCELL + cc;
-        m = cu[0];
 #pragma unroll
-        for (int t = 0; t < 3; ++t) X[t] += cu[(1 + t) * NCELL];
+        for (int i = 0; i < 2; ++i) {
+            m[i] = cu[i];
 #pragma unroll
-        for (int t = 0; t < 6; ++t) c2[t] = cu[(4 + t) * NCELL];
+            for (int t = 0; t < 3; ++t) X[i][t] += cu[(1 + t) * NCELL + i];
 #pragma unroll
-        for (int t = 0; t < 10; ++t) c3[t] = cu[(10 + t) * NCELL];
+            for (int t = 0; t < 6; ++t) c2[i][t] = cu[(4 + t) * NCELL + i];
+#pragma unroll
+            for (int t = 0; t < 10; ++t) c3[i][t] = cu[(10 + t) * NCELL + i];
+        }
     }
-    // raw moments of this child about ref: v = (m, m X, S2, S3)
-    dfloat v[20];
-    v[0] = m;
+    // M0 and M0 d over the eight children
+    dfloat m0 = m[0] + m[1], d[3];
 #pragma unroll
-    for (int t = 0; t < 3; ++t) v[1 + t] = m * X[t];
+    for (int t = 0; t < 3; ++t) d[t] = fmadd(m[1], X[1][t], m[0] * X[0][t]);
 #pragma unroll
-    for (int t = 0; t < 6; ++t) v[4 + t] = c2[t] + v[1 + i2_at(t, 0)] * X[i2_at(t, 1)];
+    for (int off = 1; off < kLanes; off <<= 1) {
+        m0 += shfl_xor_df(m0, off);
 #pragma unroll
-    for (int t = 0; t < 10; ++t) {
-        const int a = i3_at(t, 0), b = i3_at(t, 1), e = i3_at(t, 2);
-        v[10 + t] = c3[t] + c2[r2_of(a, b)] * X[e] + c2[r2_of(a, e)] * X[b] + c2[r2_of(b, e)] * X[a] +
-                    (v[1 + a] * X[b]) * X[e];
+        for (int t = 0; t < 3; ++t) d[t] += shfl_xor_df(d[t], off);
     }
 #pragma unroll
-    for (int off = 1; off < 8; off <<= 1)
+    for (int t = 0; t < 3; ++t) d[t] = d[t] / m0;
+    // v = (M2, M3): sums of e2 = c2 + m s s and of c3 + c2 s (three terms, the
+    // first with e2) over this thread's children, s = X - d
+    dfloat v[16];
 #pragma unroll
-        for (int t = 0; t < 20; ++t) v[t] += shfl_xor_df(v[t], off);
-    const dfloat m0 = v[0];
-    dfloat d[3], M2[6], M3[10];
+    for (int t = 0; t < 16; ++t) v[t] = dfloat(0.f);
 #pragma unroll
-    for (int t = 0; t < 3; ++t) d[t] = v[1 + t] / m0;
-    central_from_raw(m0, d, v + 4, v + 10, M2, M3);
-    // lane j writes components j, j + 8, j + 16 of (M0, offset, M2, M3), and
-    // lanes 0-3 the FP64 dipole zeros, lanes 4-6 the centre of mass
-    const dfloat outv[20] = {m0,    d[0],  d[1],  d[2],  M2[0], M2[1], M2[2], M2[3], M2[4], M2[5],
-                             M3[0], M3[1], M3[2], M3[3], M3[4], M3[5], M3[6], M3[7], M3[8], M3[9]};
+    for (int i = 0; i < 2; ++i) {
+        const dfloat s3[3] = {X[i][0] - d[0], X[i][1] - d[1], X[i][2] - d[2]};
+        const dfloat ms[3] = {m[i] * s3[0], m[i] * s3[1], m[i] * s3[2]};
+        dfloat e2[6];
+#pragma unroll
+        for (int t = 0; t < 6; ++t) {
+            e2[t] = fmadd(ms[i2_at(t, 0)], s3[i2_at(t, 1)], c2[i][t]);
+            v[t] = i ? v[t] + e2[t] : e2[t];
+        }
+#pragma unroll
+        for (int t = 0; t < 10; ++t) {
+            const int a = i3_at(t, 0), b = i3_at(t, 1), e = i3_at(t, 2);
+            dfloat w = i ? add_u(v[6 + t], c3[i][t]) : c3[i][t];
+            w = fmadd_u(e2[r2_of(a, b)], s3[e], w);
+            w = fmadd_u(c2[i][r2_of(a, e)], s3[b], w);
+            v[6 + t] = renorm(fmadd_u(c2[i][r2_of(b, e)], s3[a], w));
+        }
+    }
+    add_halves<16>(v, lane >> 1, 2);
+    add_halves<8>(v, lane & 1, 1);
+    // this thread's four components of (M2, M3), and one of M0 and the offset
     double *out = M + size_t(node) * NCOMP * NCELL + c;
     dfloat *ou = up + size_t(ni.mp_row) * 20 * NCELL + c;
+    const int first = 4 + 8 * (lane >> 1) + 4 * (lane & 1);
 #pragma unroll
-    for (int comp = 0; comp < 20; ++comp) {
-        if ((comp & 7) != j) continue;
-        ou[comp * NCELL] = outv[comp];
-        if (comp == 0 || comp >= 4) out[comp * NCELL] = df_to_double(outv[comp]);
+    for (int i = 0; i < 4; ++i) {
+        out[(first + i) * NCELL] = df_to_double(v[i]);
+        ou[(first + i) * NCELL] = v[i];
     }
-    if (j >= 1 && j <= 3) out[j * NCELL] = 0.0;
-    double *cm = com + size_t(node) * 3 * NCELL + c;
-    if (j == 4) cm[0] = (lo_x + (8.0 * ni.ix + x + 0.5) * hp) + df_to_double(d[0]);
-    if (j == 5) cm[NCELL] = (lo_y + (8.0 * ni.iy + y + 0.5) * hp) + df_to_double(d[1]);
-    if (j == 6) cm[2 * NCELL] = (lo_z + (8.0 * ni.iz + z + 0.5) * hp) + df_to_double(d[2]);
+    const dfloat low = lane == 0 ? m0 : lane == 1 ? d[0] : lane == 2 ? d[1] : d[2];
+    ou[lane * NCELL] = low;
+    if (lane == 0) {
+        out[0] = df_to_double(m0);
+    } else {
+        const int a = lane - 1;
+        const int i = a == 0 ? 8 * ni.ix + x : a == 1 ? 8 * ni.iy + y : 8 * ni.iz + z;
+        const double lo = a == 0 ? lo_x : a == 1 ? lo_y : lo_z;
+        out[lane * NCELL] = 0.0;
+        com[(size_t(node) * 3 + a) * NCELL + c] =
+            fma(f2d_bits(float(i) + 0.5f), hp, lo) + df_to_double(low);
+    }
 }
 
 }  // namespace
@@ -479,32 +467,39 @@ cudaError_t launch_p2m(const fmm_tree_s *t, const double *rho, double *M, cudaSt
     return cudaGetLastError();
 }
 
+// Which nodes of a level go through which double-float kernel (and so how
+// many launches it takes).  A level that mixes both kinds takes two launches
+// only where it is large enough for the lean kernel to gain more than a
+// launch costs.
+int m2m_split(const fmm_tree_s *t, int level, ListRange &lean, ListRange &lanes)
+{
+    const ListRange &all = t->plan.refined_at[size_t(level)];
+    lean = t->plan.leafkids_at[size_t(level)];
+    lanes = t->plan.mixedkids_at[size_t(level)];
+    if (lean.count && lanes.count && all.count < kSplitFrom) {
+        lean = ListRange{};
+        lanes = all;
+    }
+    return (lean.count > 0) + (lanes.count > 0);
+}
+
 cudaError_t launch_m2m_level(const fmm_tree_s *t, int level, double *M, double *com,
                              cudaStream_t s)
 {
     const ListRange &r = t->plan.refined_at[size_t(level)];
     if (r.count == 0) return cudaSuccess;
-    if (t->cfg.precision != FMM_FP64 && r.count >= kLanesBelow) {
-        // nodes with only leaf children through the lean kernel, the others
-        // through the general one
-        const ListRange &rl = t->plan.leafkids_at[size_t(level)];
-        const ListRange &rm = t->plan.mixedkids_at[size_t(level)];
-        if (rl.count)
-            m2m_df_kernel<true><<<unsigned(rl.count * 8), kSliceThreads, 0, s>>>(
-                t->dev.info, t->dev.children, t->dev.lists + rl.off, t->dev.levels, M, com,
+    if (t->cfg.precision != FMM_FP64) {
+        ListRange lean, lanes;
+        m2m_split(t, level, lean, lanes);
+        if (lean.count)
+            m2m_df_kernel<<<unsigned(lean.count * 8), kSliceThreads, 0, s>>>(
+                t->dev.info, t->dev.children, t->dev.lists + lean.off, t->dev.levels, M, com,
                 reinterpret_cast<dfloat *>(t->dev.up), t->cfg.box_lo[0], t->cfg.box_lo[1],
                 t->cfg.box_lo[2]);
         cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess || rm.count == 0) return e;
-        m2m_df_kernel<false><<<unsigned(rm.count * 8), kSliceThreads, 0, s>>>(
-            t->dev.info, t->dev.children, t->dev.lists + rm.off, t->dev.levels, M, com,
-            reinterpret_cast<dfloat *>(t->dev.up), t->cfg.box_lo[0], t->cfg.box_lo[1],
-            t->cfg.box_lo[2]);
-        return cudaGetLastError();
-    }
-    if (t->cfg.precision != FMM_FP64) {
-        m2m_df_lanes_kernel<<<unsigned(r.count * (NCELL / kCellsPerCta)), 8 * kCellsPerCta, 0, s>>>(
-            t->dev.info, t->dev.children, t->dev.lists + r.off, t->dev.levels, M, com,
+        if (e != cudaSuccess || lanes.count == 0) return e;
+        m2m_df_lanes_kernel<<<unsigned(lanes.count * (NCELL / kCellsPerCta)), kSliceThreads, 0, s>>>(
+            t->dev.info, t->dev.children, t->dev.lists + lanes.off, t->dev.levels, M, com,
             reinterpret_cast<dfloat *>(t->dev.up), t->cfg.box_lo[0], t->cfg.box_lo[1],
             t->cfg.box_lo[2]);
         return cudaGetLastError();
