@@ -367,7 +367,8 @@ __global__ void __launch_bounds__(kSliceThreads) l2l_kernel(const NodeInfo *__re
 // integer pipe.
 constexpr int kForceThreads = 64;
 
-// block sum of NV values of type V, fixed order; result in thread 0
+// sum of NV values of type V over the block's first THREADS threads, fixed
+// order; result in thread 0
 template <int THREADS, typename V, int NV>
 __device__ __forceinline__ void block_sum(V v[NV], V (*sh)[NV])
 {
@@ -376,7 +377,7 @@ __device__ __forceinline__ void block_sum(V v[NV], V (*sh)[NV])
     for (int k = 0; k < NV; ++k)
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], off);
-    if (lane == 0)
+    if (lane == 0 && warp < THREADS / 32)
 #pragma unroll
         for (int k = 0; k < NV; ++k) sh[warp][k] = v[k];
     __syncthreads();
@@ -396,13 +397,14 @@ struct ForceColumn {
     double F[3] = {0.0, 0.0, 0.0}, T[2] = {0.0, 0.0};
     float nf = 0.f, nt = 0.f;
 
+    // column: x + 8 y
     __device__ __forceinline__ ForceColumn(const NodeInfo &ni, const double *levels,
-                                           double box_size)
+                                           double box_size, int column)
     {
         h = levels[ni.level * LEVEL_FIELDS + LV_H];
         h3 = levels[ni.level * LEVEL_FIELDS + LV_H3];
         const double half = 0.5 * box_size;
-        const int x = threadIdx.x & 7, y = threadIdx.x >> 3;
+        const int x = column & 7, y = column >> 3;
         // position from the box centre (the box corner cancels); x, y fixed per thread
         X0 = (8.0 * ni.ix + x + 0.5) * h - half;
         X1 = (8.0 * ni.iy + y + 0.5) * h - half;
@@ -413,20 +415,33 @@ struct ForceColumn {
         hf = d2f_trunc(h);
     }
 
-    // cell z of the column, of mass m: phi = L0, g = -(L1 + dL1), and its
-    // terms of the sums
-    __device__ __forceinline__ void cell(int row, int c, int z, double m, double L0,
-                                         const double L1[3], const double acc[3],
-                                         double *__restrict__ phi, double *__restrict__ g)
+    // a cell's field: phi = L0, g = -(L1 + dL1)
+    static __device__ __forceinline__ void field(int row, int c, double L0, const double L1[3],
+                                                 const double acc[3], double *__restrict__ phi,
+                                                 double *__restrict__ g, double gv[3])
     {
         phi[size_t(row) * NCELL + c] = L0;
-        double gv[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             gv[a] = -(L1[a] + acc[a]);
             g[(size_t(row) * 3 + a) * NCELL + c] = gv[a];
-            F[a] = fma(m, gv[a], F[a]);                 // f = m g
         }
+    }
+
+    // cell z of the column, of mass m: its field and its terms of the sums
+    __device__ __forceinline__ void cell(int row, int c, int z, double m, double L0,
+                                         const double L1[3], const double acc[3],
+                                         double *__restrict__ phi, double *__restrict__ g)
+    {
+        double gv[3];
+        field(row, c, L0, L1, acc, phi, g, gv);
+        add(z, m, gv);
+    }
+
+    __device__ __forceinline__ void add(int z, double m, const double gv[3])
+    {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) F[a] = fma(m, gv[a], F[a]);     // f = m g
         if (z > 0) {
             const double mz = z == 1 ? m : m * double(z);
             T[0] = fma(mz, gv[0], T[0]);
@@ -451,6 +466,7 @@ struct ForceColumn {
     // eight partial sums.  That is 63 adds per value, where a shuffle tree
     // has every lane of both warps add at each of its five levels (five
     // times the FP64 operations, on the pipe that bounds this pass).
+    // (threads past the first 64 only take part in the barriers)
     __device__ __forceinline__ void finish(int row, double *__restrict__ partials)
     {
         __shared__ double sh[6][kForceThreads];
@@ -459,8 +475,9 @@ struct ForceColumn {
         const double S0 = fma(h, T[0], Z0 * F[0]), S1 = fma(h, T[1], Z0 * F[1]);
         const double v[6] = {F[0], F[1], F[2], fma(X1, F[2], -S1), fma(-X0, F[2], S0),
                              fma(X0, F[1], -X1 * F[0])};
+        if (threadIdx.x < kForceThreads)
 #pragma unroll
-        for (int k = 0; k < 6; ++k) sh[k][threadIdx.x] = v[k];
+            for (int k = 0; k < 6; ++k) sh[k][threadIdx.x] = v[k];
         float vf[2] = {nf, nt};
         block_sum<kForceThreads, float, 2>(vf, shf);     // (its barrier publishes sh)
         if (threadIdx.x < 48) {
@@ -493,7 +510,7 @@ __global__ void __launch_bounds__(kForceThreads) forces_kernel(
     const int node = leaves[blockIdx.x];
     const NodeInfo ni = info[node];
     const int row = ni.leaf_row;
-    ForceColumn col(ni, levels, box_size);
+    ForceColumn col(ni, levels, box_size, threadIdx.x);
 #pragma unroll
     for (int z = 0; z < 8; ++z) {
         const int c = threadIdx.x + 64 * z;
@@ -528,7 +545,7 @@ __global__ void __launch_bounds__(kForceThreads, 12) leaf_finish_kernel(
     const int node = leaves[blockIdx.x];
     const NodeInfo ni = info[node];
     const int row = ni.leaf_row;
-    ForceColumn col(ni, levels, box_size);
+    ForceColumn col(ni, levels, box_size, threadIdx.x);
 #pragma unroll
     for (int z = 0; z < 8; ++z) {
         const int c = threadIdx.x + 64 * z;
@@ -541,6 +558,44 @@ __global__ void __launch_bounds__(kForceThreads, 12) leaf_finish_kernel(
         col.cell(row, c, z, M[(size_t(node) * NCOMP) * NCELL + c], out[0], out + 1, corr, phi, g);
     }
     col.finish(row, partials);
+}
+
+// The same with one thread per cell, for trees with few leaf nodes: eight cells
+// one after the other cost each thread 30 us (FP64: 52), whatever the number
+// of nodes up to a dozen per SM.  The cells' masses and fields go through
+// shared memory to the first 64 threads, which take the columns' sums in the
+// same order as above, so the results are the same bits.
+template <int MODE>
+__global__ void __launch_bounds__(NCELL, MODE == FMM_FP64 ? 1 : 2) leaf_finish_cells_kernel(
+    const NodeInfo *__restrict__ info, const int32_t *__restrict__ leaves,
+    const double *__restrict__ levels, const dfloat *__restrict__ levels_df,
+    const void *__restrict__ Lv, const float *__restrict__ Lc, const double *dL1,
+    const double *__restrict__ com, double *__restrict__ L64, double *dacc, float *down,
+    const double *__restrict__ M, double *__restrict__ phi, double *__restrict__ g,
+    double *__restrict__ partials, double lo_x, double lo_y, double lo_z, double box_size)
+{
+    __shared__ double sc[4][NCELL];
+    const int node = leaves[blockIdx.x];
+    const NodeInfo ni = info[node];
+    const int c = threadIdx.x;
+    double out[20], corr[3], gv[3];
+    const double m = M[(size_t(node) * NCOMP) * NCELL + c];
+    l2l_cell<MODE, 1>(info, ni, node, c, levels, levels_df, Lv, Lc, dL1, com, L64, dacc, down, lo_x,
+                      lo_y, lo_z, out, corr);
+    ForceColumn::field(ni.leaf_row, c, out[0], out + 1, corr, phi, g, gv);
+    sc[0][c] = m;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) sc[1 + a][c] = gv[a];
+    __syncthreads();
+    ForceColumn col(ni, levels, box_size, c & (kForceThreads - 1));
+    if (c < kForceThreads)
+#pragma unroll
+        for (int z = 0; z < 8; ++z) {
+            const int b = c + 64 * z;
+            const double gz[3] = {sc[1][b], sc[2][b], sc[3][b]};
+            col.add(z, sc[0][b], gz);
+        }
+    col.finish(ni.leaf_row, partials);
 }
 
 // ---------------------------------------------------------------- dataflow
@@ -637,7 +692,7 @@ __global__ void __launch_bounds__(kForceThreads, 12) dataflow_kernel(DflowParams
             if (threadIdx.x == 0) atomicAdd(P.ready + node, 1);
         } else {
             const int row = ni.leaf_row;
-            ForceColumn col(ni, P.levels, P.box_size);
+            ForceColumn col(ni, P.levels, P.box_size, threadIdx.x);
 #pragma unroll
             for (int z = 0; z < 8; ++z) {
                 const int c = threadIdx.x + 64 * z;
@@ -755,19 +810,25 @@ cudaError_t launch_leaf_finish(const fmm_tree_s *t, const void *L, const float *
     const dfloat *ldf = reinterpret_cast<const dfloat *>(t->dev.levels_df);
     const int32_t *nodes = t->dev.lists + r.off;
     const unsigned grid = unsigned(r.count);
+    // one thread per cell while the CTAs fit the SMs in one wave (two per SM,
+    // FP64: one), one per column of eight cells above: 64 leaf nodes 29 -> 14 us,
+    // but 512 nodes 30 -> 34; FP64, 8 nodes 52 -> 27
+    const bool cells = r.count <= (c.precision == FMM_FP64 ? 1 : 2) *
+                                      int64_t(sm_count_of_current_device());
+    auto launch = [&](auto kern, int threads) {
+        kern<<<grid, threads, 0, s>>>(t->dev.info, nodes, t->dev.levels, ldf, L, Lc, dL1, com, L64,
+                                      dacc, t->dev.down, M, phi, g, t->dev.partials, c.box_lo[0],
+                                      c.box_lo[1], c.box_lo[2], c.box_size);
+        return cudaGetLastError();
+    };
     if (c.precision == FMM_MIXED)
-        leaf_finish_kernel<FMM_MIXED><<<grid, kForceThreads, 0, s>>>(
-            t->dev.info, nodes, t->dev.levels, ldf, L, Lc, dL1, com, L64, dacc, t->dev.down, M,
-            phi, g, t->dev.partials, c.box_lo[0], c.box_lo[1], c.box_lo[2], c.box_size);
-    else if (c.precision == FMM_DFLOAT)
-        leaf_finish_kernel<FMM_DFLOAT><<<grid, kForceThreads, 0, s>>>(
-            t->dev.info, nodes, t->dev.levels, ldf, L, Lc, dL1, com, L64, dacc, t->dev.down, M,
-            phi, g, t->dev.partials, c.box_lo[0], c.box_lo[1], c.box_lo[2], c.box_size);
-    else
-        leaf_finish_kernel<FMM_FP64><<<grid, kForceThreads, 0, s>>>(
-            t->dev.info, nodes, t->dev.levels, ldf, L, Lc, dL1, com, L64, dacc, nullptr, M, phi,
-            g, t->dev.partials, c.box_lo[0], c.box_lo[1], c.box_lo[2], c.box_size);
-    return cudaGetLastError();
+        return cells ? launch(leaf_finish_cells_kernel<FMM_MIXED>, NCELL)
+                     : launch(leaf_finish_kernel<FMM_MIXED>, kForceThreads);
+    if (c.precision == FMM_DFLOAT)
+        return cells ? launch(leaf_finish_cells_kernel<FMM_DFLOAT>, NCELL)
+                     : launch(leaf_finish_kernel<FMM_DFLOAT>, kForceThreads);
+    return cells ? launch(leaf_finish_cells_kernel<FMM_FP64>, NCELL)
+                 : launch(leaf_finish_kernel<FMM_FP64>, kForceThreads);
 }
 
 cudaError_t launch_downward_dataflow(const fmm_tree_s *t, const void *L, const float *Lc,
