@@ -460,18 +460,18 @@ __device__ __forceinline__ dfloat acc_lo(const Acc<dfloat, N> &, int) { return d
 // the downward shifts, scaled by the small child offsets) are plain float
 // sums in registers.  Fewer pairs leave more of the SM's shared memory to
 // L1, where the multipole kernel rereads the sources' packed moments.
-template <int N, int NC = N>
+template <int N, int NC = N, int THREADS = kThreads>
 struct SmemAcc {
     float part[N];
-    float *col;                       // the (hi, lo) pairs of component k < NC at col[k * 2 * kThreads]
+    float *col;                       // the (hi, lo) pairs of component k < NC at col[k * 2 * THREADS]
     __device__ __forceinline__ void zero()
     {
 #pragma unroll
         for (int k = 0; k < N; ++k) part[k] = 0.f;
 #pragma unroll
         for (int k = 0; k < NC; ++k) {
-            col[k * 2 * kThreads] = 0.f;
-            col[(k * 2 + 1) * kThreads] = 0.f;
+            col[k * 2 * THREADS] = 0.f;
+            col[(k * 2 + 1) * THREADS] = 0.f;
         }
     }
     __device__ __forceinline__ void flush()
@@ -479,22 +479,22 @@ struct SmemAcc {
 #pragma unroll
         for (int k = 0; k < NC; ++k) {
             float s, e;
-            two_sum(col[k * 2 * kThreads], part[k], s, e);
-            col[k * 2 * kThreads] = s;
-            col[(k * 2 + 1) * kThreads] += e;
+            two_sum(col[k * 2 * THREADS], part[k], s, e);
+            col[k * 2 * THREADS] = s;
+            col[(k * 2 + 1) * THREADS] += e;
             part[k] = 0.f;
         }
     }
 };
-template <int N, int NC>
-__device__ __forceinline__ float acc_hi(const SmemAcc<N, NC> &a, int k)
+template <int N, int NC, int THREADS>
+__device__ __forceinline__ float acc_hi(const SmemAcc<N, NC, THREADS> &a, int k)
 {
-    return k < NC ? a.col[k * 2 * kThreads] : a.part[k];
+    return k < NC ? a.col[k * 2 * THREADS] : a.part[k];
 }
-template <int N, int NC>
-__device__ __forceinline__ float acc_lo(const SmemAcc<N, NC> &a, int k)
+template <int N, int NC, int THREADS>
+__device__ __forceinline__ float acc_lo(const SmemAcc<N, NC, THREADS> &a, int k)
 {
-    return k < NC ? a.col[(k * 2 + 1) * kThreads] : 0.f;
+    return k < NC ? a.col[(k * 2 + 1) * THREADS] : 0.f;
 }
 
 // (the multipole kernel keeps shared-memory pairs for orders 0-1 and the correction)
@@ -904,28 +904,35 @@ __device__ __forceinline__ void mx_target(const KParams &P, int t)
 }
 
 // ------------------------------------------------------------ mp_kernel
-// HALVES: item k is half k & 1 (cells of z < 4 or z >= 4) of node list[k >> 1],
-// else item k is all of node list[k]
-template <int ORDER, bool HALVES>
-// float: three CTAs per SM (at most 85 registers): the compensation pairs,
-// touched once per chunk, live in shared memory after the window
-__global__ void __launch_bounds__(kThreads, 3) mp_kernel(KParams P)
+// WARPS per CTA, PARTS items per sub-grid:
+//   8, 1: an item is a sub-grid, a warp each parity, both halves (z < 4, z >= 4);
+//   8, 2: an item is one half of a sub-grid;
+//   1, 16: an item is one half of one parity, 32 cells, and a CTA one warp.
+// Three CTAs of eight warps per SM (at most 85 registers): the compensation
+// pairs, touched once per chunk, live in shared memory after the window.
+// AHEAD: the far loop is software-pipelined by hand (below), at 112 registers
+// and two such CTAs per SM: worth it only where the items do not fill the SMs
+// anyway.
+template <int ORDER, int WARPS, int PARTS, bool AHEAD>
+__global__ void __launch_bounds__(32 * WARPS, WARPS == 1 ? 1 : AHEAD ? 2 : 3) mp_kernel(KParams P)
 {
+    static_assert((WARPS == 8 && PARTS <= 2) || (WARPS == 1 && PARTS == 16), "items per sub-grid");
+    constexpr int threads = 32 * WARPS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float *W = reinterpret_cast<float *>(smem_raw);
     float *Cs = W + 8 * P.sub_stride + threadIdx.x;
     __shared__ int s_nbr[27], s_leaf[27], s_row[27], s_item;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int p = warp;
-    const int px = p & 1, py = (p >> 1) & 1, pz = p >> 2;
     const int cx = lane & 3, cy = (lane >> 2) & 3, cz0 = lane >> 4;
-    const float4 *ent = P.stencil_f + p * P.ent_stride;   // float offsets: no conversions
     const float *mass = static_cast<const float *>(P.mass);
     const float *mp = static_cast<const float *>(P.mp);
     for (;;) {
         const int item = pull_item(P.counter, &s_item);
         if (item >= P.n_items) break;
-        const int node = P.list[HALVES ? item >> 1 : item];
+        const int node = P.list[item / PARTS];
+        const int p = WARPS == 8 ? warp : (item >> 1) & 7;
+        const int px = p & 1, py = (p >> 1) & 1, pz = p >> 2;
+        const float4 *ent = P.stencil_f + p * P.ent_stride;   // float offsets: no conversions
         const NodeInfo ti = P.info[node];
         // near sources contribute only if some neighbour is a leaf
         const int any_leaf = __syncthreads_or(load_slots(node, P, s_nbr, s_leaf, s_row));
@@ -933,60 +940,105 @@ __global__ void __launch_bounds__(kThreads, 3) mp_kernel(KParams P)
         cp_async_commit();
         cp_async_wait_all();
         __syncthreads();
-        const int half0 = HALVES ? item & 1 : 0;
-        const int half1 = HALVES ? half0 + 1 : 2;
+        const int half0 = PARTS == 1 ? 0 : item & 1;
+        const int half1 = PARTS == 1 ? 2 : half0 + 1;
         for (int half = half0; half < half1; ++half) {
             const int cz = cz0 + 2 * half;
             const int ax = 2 * cx + px, ay = 2 * cy + py, az = 2 * cz + pz;
             const int base = cx + P.py * cy + P.pz * cz;
             float dA[3], a3A[7];
             load_target<ORDER>(P, ti.mp_row, parity_index(ax, ay, az), dA, a3A);
-            SmemAcc<16, 4> L;
-            SmemAcc<3> S;
+            SmemAcc<16, 4, threads> L;
+            SmemAcc<3, 3, threads> S;
             L.col = Cs;
-            S.col = Cs + 4 * 2 * kThreads;
+            S.col = Cs + 4 * 2 * threads;
             L.zero();
             S.zero();
-            // well-separated sources: refined (full moments) or leaf (mass).
+            // Well-separated sources: refined (full moments) or leaf (mass).
             // A vote classifies the warp's 32 sources of one
             // entry: all refined take the moments without a branch, all
             // leaves the mass-only form (the same operations less the zero
             // moments' terms, so the same values), a mix the general form
             // with zero moments for the leaves, and an entry with only
             // absent sources (mass 0) is skipped.
-            for (int e0 = 0; e0 < P.n_far; e0 += kChunk) {
-                const int e1 = min(e0 + kChunk, P.n_far);
-                for (int e = e0; e < e1; ++e) {
-                    const float4 E = __ldg(ent + e);
-                    const float wv = W[base + __float_as_int(E.w)];
-                    int idx;
-                    const bool is_mp = window_moments<float>(wv, P.mp_limit, idx);
-                    const bool all_mp = __all_sync(0xffffffffu, is_mp);
-                    Src<float> src;
-                    float R[3];
-                    if (all_mp) {
-                        load_source_at(mp + idx, src);
-                        separation(dA, src.d, E, R);
-                        acc_mp<true, ORDER>(R[0], R[1], R[2], src, a3A, L, S);
-                    } else if (!__any_sync(0xffffffffu, is_mp)) {
-                        if (__any_sync(0xffffffffu, window_nonzero<float>(wv))) {
+            // AHEAD: while one entry is evaluated, the moments of the next are
+            // loaded, the window value of the one after (which says where
+            // its moments are) and the window offset of the one after that,
+            // so a warp waits for none of the three dependent loads; leaf
+            // lanes load the zero row.
+            if constexpr (AHEAD) {
+                const int last = P.n_far - 1;
+                float4 E = __ldg(ent);
+                float wv = W[base + __float_as_int(E.w)];
+                float wv1 = W[base + __float_as_int(__ldg(&ent[min(1, last)].w))];
+                int off2 = __float_as_int(__ldg(&ent[min(2, last)].w));
+                Src<float> src;
+                int idx;
+                bool is_mp = window_moments<float>(wv, P.mp_limit, idx);
+                load_source_at(mp + (is_mp ? idx : P.mp_limit), src);
+                for (int e0 = 0; e0 < P.n_far; e0 += kChunk) {
+                    const int e1 = min(e0 + kChunk, P.n_far);
+                    for (int e = e0; e < e1; ++e) {
+                        Src<float> src1;
+                        const bool is_mp1 = window_moments<float>(wv1, P.mp_limit, idx);
+                        load_source_at(mp + (is_mp1 ? idx : P.mp_limit), src1);
+                        const float wv2 = W[base + off2];
+                        off2 = __float_as_int(__ldg(&ent[min(e + 3, last)].w));
+                        const float4 E1 = __ldg(ent + min(e + 1, last));
+                        if (__any_sync(0xffffffffu, is_mp)) {
+                            if (!is_mp) src.m0 = wv;
+                            float R[3];
+                            separation(dA, src.d, E, R);
+                            acc_mp<true, ORDER>(R[0], R[1], R[2], src, a3A, L, S);
+                        } else if (__any_sync(0xffffffffu, window_nonzero<float>(wv))) {
                             src.m0 = wv;
-                            acc_mp<false, ORDER>(dA[0] - E.x, dA[1] - E.y,
-                                                    dA[2] - E.z, src, a3A, L, S);
+                            acc_mp<false, ORDER>(dA[0] - E.x, dA[1] - E.y, dA[2] - E.z, src, a3A, L,
+                                                 S);
                         }
-                    } else {
-                        if (is_mp) {
-                            load_source_at(mp + idx, src);
-                        } else {
-                            src.m0 = wv;
-                            zero_moments(src);
-                        }
-                        separation(dA, src.d, E, R);
-                        acc_mp<true, ORDER>(R[0], R[1], R[2], src, a3A, L, S);
+                        src = src1;
+                        is_mp = is_mp1;
+                        wv = wv1;
+                        wv1 = wv2;
+                        E = E1;
                     }
+                    L.flush();
+                    S.flush();
                 }
-                L.flush();
-                S.flush();
+            } else {
+                for (int e0 = 0; e0 < P.n_far; e0 += kChunk) {
+                    const int e1 = min(e0 + kChunk, P.n_far);
+                    for (int e = e0; e < e1; ++e) {
+                        const float4 E = __ldg(ent + e);
+                        const float wv = W[base + __float_as_int(E.w)];
+                        int idx;
+                        const bool is_mp = window_moments<float>(wv, P.mp_limit, idx);
+                        const bool all_mp = __all_sync(0xffffffffu, is_mp);
+                        Src<float> src;
+                        float R[3];
+                        if (all_mp) {
+                            load_source_at(mp + idx, src);
+                            separation(dA, src.d, E, R);
+                            acc_mp<true, ORDER>(R[0], R[1], R[2], src, a3A, L, S);
+                        } else if (!__any_sync(0xffffffffu, is_mp)) {
+                            if (__any_sync(0xffffffffu, window_nonzero<float>(wv))) {
+                                src.m0 = wv;
+                                acc_mp<false, ORDER>(dA[0] - E.x, dA[1] - E.y,
+                                                        dA[2] - E.z, src, a3A, L, S);
+                            }
+                        } else {
+                            if (is_mp) {
+                                load_source_at(mp + idx, src);
+                            } else {
+                                src.m0 = wv;
+                                zero_moments(src);
+                            }
+                            separation(dA, src.d, E, R);
+                            acc_mp<true, ORDER>(R[0], R[1], R[2], src, a3A, L, S);
+                        }
+                    }
+                    L.flush();
+                    S.flush();
+                }
             }
             // near sources: leaf cells only (refined ones contribute nothing
             // here: their children interact one level down); skipped when no
@@ -1647,13 +1699,18 @@ cudaError_t allow_smem(Kern k, size_t bytes, size_t &done)
 
 template <typename T>
 struct Kernels {
-    // PARTS items per sub-grid: float 1, 2; the wide types 2, 4, 16
+    // the wide types' multipole kernel, PARTS items per sub-grid
     template <int ORDER, int PARTS>
+    static cudaError_t mpw(size_t bytes)
+    {
+        static size_t done = 0;
+        return allow_smem(mpw_kernel<T, ORDER, PARTS>, bytes, done);
+    }
+    template <int ORDER, int WARPS, int PARTS, bool AHEAD>
     static cudaError_t mp(size_t bytes)
     {
         static size_t done = 0;
-        if constexpr (kF32<T>) return allow_smem(mp_kernel<ORDER, PARTS == 2>, bytes, done);
-        else return allow_smem(mpw_kernel<T, ORDER, PARTS>, bytes, done);
+        return allow_smem(mp_kernel<ORDER, WARPS, PARTS, AHEAD>, bytes, done);
     }
     static cudaError_t mp2(size_t bytes)
     {
@@ -1742,21 +1799,29 @@ cudaError_t launch_mono_wide(const fmm_tree_s *t, const KParams &K, int sms, cud
     return cudaGetLastError();
 }
 
-// the multipole launch, PARTS items per sub-grid
+// the multipole launch of the wide types, PARTS items per sub-grid
 template <typename T, int ORDER, int PARTS>
-cudaError_t launch_mp(KParams K, size_t bytes, int sms, int cap, cudaStream_t s)
+cudaError_t launch_mpw(KParams K, size_t bytes, int sms, int cap, cudaStream_t s)
 {
-    cudaError_t e = Kernels<T>::template mp<ORDER, PARTS>(bytes);
+    cudaError_t e = Kernels<T>::template mpw<ORDER, PARTS>(bytes);
     if (e != cudaSuccess) return e;
     K.n_items *= PARTS;
-    if constexpr (kF32<T>) {
-        const int g = persistent_grid(mp_kernel<ORDER, PARTS == 2>, bytes, K.n_items, sms, cap);
-        mp_kernel<ORDER, PARTS == 2><<<g, kThreads, bytes, s>>>(K);
-    } else {
-        const int g = persistent_grid(mpw_kernel<T, ORDER, PARTS>, bytes, K.n_items, sms, cap,
-                                      kWideThreads);
-        mpw_kernel<T, ORDER, PARTS><<<g, kWideThreads, bytes, s>>>(K);
-    }
+    const int g = persistent_grid(mpw_kernel<T, ORDER, PARTS>, bytes, K.n_items, sms, cap, kWideThreads);
+    mpw_kernel<T, ORDER, PARTS><<<g, kWideThreads, bytes, s>>>(K);
+    return cudaGetLastError();
+}
+
+// and of the mixed precision: WARPS per CTA; window plus compensation pairs
+template <int ORDER, int WARPS, int PARTS, bool AHEAD>
+cudaError_t launch_mp(KParams K, size_t wbytes, int sms, int cap, cudaStream_t s)
+{
+    const size_t bytes = wbytes + size_t(kMpPairs) * 2 * 32 * WARPS * sizeof(float);
+    cudaError_t e = Kernels<float>::mp<ORDER, WARPS, PARTS, AHEAD>(bytes);
+    if (e != cudaSuccess) return e;
+    K.n_items *= PARTS;
+    const int g = persistent_grid(mp_kernel<ORDER, WARPS, PARTS, AHEAD>, bytes, K.n_items, sms, cap,
+                                  32 * WARPS);
+    mp_kernel<ORDER, WARPS, PARTS, AHEAD><<<g, 32 * WARPS, bytes, s>>>(K);
     return cudaGetLastError();
 }
 
@@ -1791,9 +1856,6 @@ cudaError_t launch_all(const fmm_tree_s *t, void *L, float *Lc, double *dL1, cud
     P.mono_woff = d.mono_woff;
     const int cap = t->tuning.ctas_per_sm;
     const size_t wbytes = size_t(8) * Pl.sub_stride * sizeof(T);
-    // mp_kernel: one window (masses of leaf sources, moment offsets of
-    // refined ones); float adds its compensation pairs, [7][2][threads]
-    const size_t mp_bytes = wbytes + (kF32<T> ? size_t(kMpPairs) * 2 * kThreads * sizeof(float) : 0);
     cudaError_t e;
     if (parts & M2L_RESET) {
         e = cudaMemsetAsync(d.counters, 0, 4 * sizeof(int32_t), s);
@@ -1838,15 +1900,19 @@ cudaError_t launch_all(const fmm_tree_s *t, void *L, float *Lc, double *dL1, cud
             const int mode = t->tuning.mp_items;
             const int64_t n = Pl.work_mp.count;
             if constexpr (kF32<T>) {
-                // half sub-grids per item where whole ones would leave CTA
-                // slots idle or unbalanced (fewer nodes than twice the slots)
-                if ((e = Kernels<T>::template mp<ORDER, 1>(mp_bytes)) != cudaSuccess) return e;
-                const int64_t slots =
-                    persistent_grid(mp_kernel<ORDER, false>, mp_bytes, INT32_MAX, sms, cap);
-                if (mode == 2 || (mode == 0 && n < 2 * slots))
-                    e = launch_mp<T, ORDER, 2>(K, mp_bytes, sms, cap, s);
+                // Few sub-grids: one warp per CTA up to two warps an SM, then
+                // halves with the loads ahead up to two such CTAs an SM.
+                // Else half sub-grids per item where whole ones would leave
+                // CTA slots idle or unbalanced (fewer nodes than twice the
+                // slots).  Same bits throughout.
+                if (mode == 0 && 16 * n <= 2 * int64_t(sms))
+                    e = launch_mp<ORDER, 1, 16, true>(K, wbytes, sms, cap, s);
+                else if (mode == 0 && 2 * n <= 2 * int64_t(sms))
+                    e = launch_mp<ORDER, 8, 2, true>(K, wbytes, sms, cap, s);
+                else if (mode == 2 || (mode == 0 && n < 2 * int64_t(cap > 0 && cap < 3 ? cap : 3) * sms))
+                    e = launch_mp<ORDER, 8, 2, false>(K, wbytes, sms, cap, s);
                 else
-                    e = launch_mp<T, ORDER, 1>(K, mp_bytes, sms, cap, s);
+                    e = launch_mp<ORDER, 8, 1, false>(K, wbytes, sms, cap, s);
             } else {
                 // halves and quarters of a sub-grid (mp_items 1 and 2; by
                 // default quarters below eight nodes an SM, so that the last
@@ -1854,11 +1920,11 @@ cudaError_t launch_all(const fmm_tree_s *t, void *L, float *Lc, double *dL1, cud
                 // (whatever mp_items says: their sums round differently)
                 const size_t fold = size_t(kWideThreads / 64) * kWideSums<ORDER> * 32 * sizeof(T);
                 if (4 * n < sms)
-                    e = launch_mp<T, ORDER, 16>(K, std::max(wbytes, fold), sms, cap, s);
+                    e = launch_mpw<T, ORDER, 16>(K, std::max(wbytes, fold), sms, cap, s);
                 else if (mode == 2 || (mode == 0 && n < 8 * int64_t(sms)))
-                    e = launch_mp<T, ORDER, 4>(K, mp_bytes, sms, cap, s);
+                    e = launch_mpw<T, ORDER, 4>(K, wbytes, sms, cap, s);
                 else
-                    e = launch_mp<T, ORDER, 2>(K, mp_bytes, sms, cap, s);
+                    e = launch_mpw<T, ORDER, 2>(K, wbytes, sms, cap, s);
             }
             if (e != cudaSuccess) return e;
         }
