@@ -14,6 +14,7 @@
 // forces_kernel: phi = L0, g = -(L1 + dL1), f = m g, and fixed-order FP64
 // block sums of f and x cross f (plus the |f|, |x cross f| normalisers) per
 // leaf node; reduce_kernel folds those per tree.
+#include "fmm_chain.cuh"
 #include "fmm_convert.cuh"
 #include "fmm_internal.h"
 #include "fmm_tensor.cuh"
@@ -348,6 +349,7 @@ __global__ void __launch_bounds__(kSliceThreads) l2l_kernel(const NodeInfo *__re
     const int node = nodes[blockIdx.x >> 3];
     const NodeInfo ni = info[node];
     const int c = (blockIdx.x & 7) * kSliceThreads + threadIdx.x;
+    chain_begin();
     double out[20], corr[3];
     if (ni.leaf_row >= 0)
         l2l_cell<MODE, 1>(info, ni, node, c, levels, levels_df, Lv, Lc, dL1, com, L64, dacc, down,
@@ -511,6 +513,7 @@ __global__ void __launch_bounds__(kForceThreads) forces_kernel(
     const NodeInfo ni = info[node];
     const int row = ni.leaf_row;
     ForceColumn col(ni, levels, box_size, threadIdx.x);
+    chain_begin();
 #pragma unroll
     for (int z = 0; z < 8; ++z) {
         const int c = threadIdx.x + 64 * z;
@@ -546,6 +549,7 @@ __global__ void __launch_bounds__(kForceThreads, 12) leaf_finish_kernel(
     const NodeInfo ni = info[node];
     const int row = ni.leaf_row;
     ForceColumn col(ni, levels, box_size, threadIdx.x);
+    chain_begin();
 #pragma unroll
     for (int z = 0; z < 8; ++z) {
         const int c = threadIdx.x + 64 * z;
@@ -578,6 +582,7 @@ __global__ void __launch_bounds__(NCELL, MODE == FMM_FP64 ? 1 : 2) leaf_finish_c
     const int node = leaves[blockIdx.x];
     const NodeInfo ni = info[node];
     const int c = threadIdx.x;
+    chain_begin();
     double out[20], corr[3], gv[3];
     const double m = M[(size_t(node) * NCOMP) * NCELL + c];
     l2l_cell<MODE, 1>(info, ni, node, c, levels, levels_df, Lv, Lc, dL1, com, L64, dacc, down, lo_x,
@@ -749,6 +754,7 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_kernel(const int32_t *_
     const int tree = blockIdx.x, chunk = blockIdx.y, chunks = gridDim.y;
     const int lo = off[tree] + chunk * kReduceRows;
     const int n = min(kReduceRows, off[tree + 1] - lo);      // may be <= 0: a smaller tree
+    chain_begin();
     const double v = row_sums(n, [&](int i) { return partials + size_t(rows[lo + i]) * 8; }, sh);
     double *mine = chunk_sums + size_t(tree) * chunks * 8;
     if (threadIdx.x < 8) {
@@ -785,19 +791,13 @@ cudaError_t launch_l2l_nodes(const fmm_tree_s *t, const ListRange &r, const void
     const unsigned grid = unsigned(r.count * 8);
     const int32_t *nodes = t->dev.lists + r.off;
     const dfloat *ldf = reinterpret_cast<const dfloat *>(t->dev.levels_df);
-    if (c.precision == FMM_MIXED)
-        l2l_kernel<FMM_MIXED><<<grid, kSliceThreads, 0, s>>>(t->dev.info, nodes, t->dev.levels, ldf, L,
-                                                            Lc, dL1, com, L64, dacc, t->dev.down,
-                                                            c.box_lo[0], c.box_lo[1], c.box_lo[2]);
-    else if (c.precision == FMM_DFLOAT)
-        l2l_kernel<FMM_DFLOAT><<<grid, kSliceThreads, 0, s>>>(t->dev.info, nodes, t->dev.levels, ldf, L,
-                                                             Lc, dL1, com, L64, dacc, t->dev.down,
-                                                             c.box_lo[0], c.box_lo[1], c.box_lo[2]);
-    else
-        l2l_kernel<FMM_FP64><<<grid, kSliceThreads, 0, s>>>(t->dev.info, nodes, t->dev.levels, ldf, L,
-                                                           Lc, dL1, com, L64, dacc, nullptr,
-                                                           c.box_lo[0], c.box_lo[1], c.box_lo[2]);
-    return cudaGetLastError();
+    auto launch = [&](auto kern) {
+        return launch_chained(kern, grid, kSliceThreads, s, t->dev.info, nodes, t->dev.levels, ldf, L, Lc,
+                              dL1, com, L64, dacc, t->dev.down, c.box_lo[0], c.box_lo[1], c.box_lo[2]);
+    };
+    if (c.precision == FMM_MIXED) return launch(l2l_kernel<FMM_MIXED>);
+    if (c.precision == FMM_DFLOAT) return launch(l2l_kernel<FMM_DFLOAT>);
+    return launch(l2l_kernel<FMM_FP64>);
 }
 
 cudaError_t launch_leaf_finish(const fmm_tree_s *t, const void *L, const float *Lc,
@@ -816,10 +816,9 @@ cudaError_t launch_leaf_finish(const fmm_tree_s *t, const void *L, const float *
     const bool cells = r.count <= (c.precision == FMM_FP64 ? 1 : 2) *
                                       int64_t(sm_count_of_current_device());
     auto launch = [&](auto kern, int threads) {
-        kern<<<grid, threads, 0, s>>>(t->dev.info, nodes, t->dev.levels, ldf, L, Lc, dL1, com, L64,
-                                      dacc, t->dev.down, M, phi, g, t->dev.partials, c.box_lo[0],
-                                      c.box_lo[1], c.box_lo[2], c.box_size);
-        return cudaGetLastError();
+        return launch_chained(kern, grid, threads, s, t->dev.info, nodes, t->dev.levels, ldf, L, Lc, dL1,
+                              com, L64, dacc, t->dev.down, M, phi, g, t->dev.partials, c.box_lo[0],
+                              c.box_lo[1], c.box_lo[2], c.box_size);
     };
     if (c.precision == FMM_MIXED)
         return cells ? launch(leaf_finish_cells_kernel<FMM_MIXED>, NCELL)
@@ -894,11 +893,10 @@ cudaError_t launch_forces(const fmm_tree_s *t, const double *L64, const double *
     const ListRange &r = t->plan.leaves;
     if (r.count > 0) {
         timing_begin(t, FMM_K_FORCES, s);
-        forces_kernel<<<unsigned(r.count), kForceThreads, 0, s>>>(
-            t->dev.info, t->dev.lists + r.off, t->dev.levels, L64, dacc, rho, phi, g,
-            t->dev.partials, t->cfg.box_size);
+        cudaError_t e = launch_chained(forces_kernel, unsigned(r.count), kForceThreads, s, t->dev.info,
+                                       t->dev.lists + r.off, t->dev.levels, L64, dacc, rho, phi, g,
+                                       t->dev.partials, t->cfg.box_size);
         timing_end(t, s);
-        cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     return launch_force_sums(t, totals, s);
@@ -907,11 +905,12 @@ cudaError_t launch_forces(const fmm_tree_s *t, const double *L64, const double *
 cudaError_t launch_force_sums(const fmm_tree_s *t, double *totals, cudaStream_t s)
 {
     timing_begin(t, FMM_K_REDUCE, s);
-    reduce_kernel<<<dim3(unsigned(t->n_trees), unsigned(t->plan.reduce_chunks)), kReduceThreads, 0, s>>>(
+    const cudaError_t e = launch_chained(
+        reduce_kernel, dim3(unsigned(t->n_trees), unsigned(t->plan.reduce_chunks)), kReduceThreads, s,
         t->dev.tree_leaf_off, t->dev.tree_leaf_rows, t->dev.partials, t->dev.chunk_sums,
         t->dev.reduce_arrived, totals);
     timing_end(t, s);
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace fmm

@@ -1051,17 +1051,16 @@ int fmm_step(fmm_tree_t t, const double *rho, double *M, double *com, void *L, f
     int nl = 0;
 #define FMM_STEP_TRY(call, what) \
     if ((e = (call)) != cudaSuccess) return cuda_fail(e, what)
-    // main: reset the work queues, P2M, fork
-    FMM_STEP_TRY(launch_m2l(t, L, L_comp, dL1, s, &nl, M2L_RESET), "queue reset");
+    // main: P2M (which resets the work queues), fork
     FMM_STEP_TRY(launch_p2m(t, rho, M, s, true), "p2m launch");
     FMM_STEP_TRY(cudaEventRecord(ev[0], s), "cudaEventRecord");
-    // Events: 0 P2M done, 1 refined sources packed, 2 refined shifts done,
-    // 3 second stream done, 4 roots done, 5 monopole kernel done.
+    // Events: 0 P2M done, 1 refined sources packed, 2 roots done, 3 monopole
+    // kernel done.
     // aux: leaf masses, monopole<-monopole
     // (P2M has stored the leaf masses in their packed form)
     FMM_STEP_TRY(cudaStreamWaitEvent(a, ev[0], 0), "cudaStreamWaitEvent");
     FMM_STEP_TRY(launch_m2l(t, L, L_comp, dL1, a, &nl, M2L_MONO), "m2l launch");
-    FMM_STEP_TRY(cudaEventRecord(ev[5], a), "cudaEventRecord");
+    FMM_STEP_TRY(cudaEventRecord(ev[3], a), "cudaEventRecord");
     // main: M2M, refined sources, multipole targets
     for (int lev = t->max_level - 1; lev >= 1; --lev)
         if (P.refined_at[size_t(lev)].count)
@@ -1076,14 +1075,14 @@ int fmm_step(fmm_tree_t t, const double *rho, double *M, double *com, void *L, f
     // leave SMs idle; as a launch of its own it held its SMs for its whole
     // run and delayed whichever of the multipole kernel and the shifts
     // came second.
-    FMM_STEP_TRY(cudaStreamWaitEvent(s, ev[5], 0), "cudaStreamWaitEvent");
+    FMM_STEP_TRY(cudaStreamWaitEvent(s, ev[3], 0), "cudaStreamWaitEvent");
     FMM_STEP_TRY(launch_m2l(t, L, L_comp, dL1, s, &nl, M2L_MP | M2L_MPX), "m2l launch");
     // aux: the roots (16 CTAs per root) beside the multipole launch rather
     // than before it on the main stream, where the GPU idled around them
     FMM_STEP_TRY(cudaStreamWaitEvent(a, ev[1], 0), "cudaStreamWaitEvent");
     FMM_STEP_TRY(launch_m2l(t, L, L_comp, dL1, a, &nl, M2L_ROOT), "m2l launch");
-    FMM_STEP_TRY(cudaEventRecord(ev[4], a), "cudaEventRecord");
-    FMM_STEP_TRY(cudaStreamWaitEvent(s, ev[4], 0), "cudaStreamWaitEvent");
+    FMM_STEP_TRY(cudaEventRecord(ev[2], a), "cudaEventRecord");
+    FMM_STEP_TRY(cudaStreamWaitEvent(s, ev[2], 0), "cudaStreamWaitEvent");
     if (t->tuning.dataflow) {
         // main: the refined shifts and the leaf pass in one persistent
         // launch, each item started by its parent's readiness counter; the
@@ -1097,15 +1096,11 @@ int fmm_step(fmm_tree_t t, const double *rho, double *M, double *com, void *L, f
     for (int lev = 1; lev <= t->max_level; ++lev)
         FMM_STEP_TRY(launch_l2l_nodes(t, P.refined_at[size_t(lev)], L, L_comp, dL1, com, L64,
                                       dL1_acc, s), "l2l launch");
-    FMM_STEP_TRY(cudaEventRecord(ev[2], s), "cudaEventRecord");
-    // aux: every leaf's shift and forces in one pass (the shifted expansion
-    // feeds the forces from registers), the sums; join
-    FMM_STEP_TRY(cudaStreamWaitEvent(a, ev[2], 0), "cudaStreamWaitEvent");
-    FMM_STEP_TRY(launch_leaf_finish(t, L, L_comp, dL1, com, L64, dL1_acc, M, phi, g, a),
+    // every leaf's shift and forces in one pass (the shifted expansion feeds
+    // the forces from registers), the sums
+    FMM_STEP_TRY(launch_leaf_finish(t, L, L_comp, dL1, com, L64, dL1_acc, M, phi, g, s),
                  "leaf launch");
-    FMM_STEP_TRY(launch_force_sums(t, totals, a), "reduce launch");
-    FMM_STEP_TRY(cudaEventRecord(ev[3], a), "cudaEventRecord");
-    FMM_STEP_TRY(cudaStreamWaitEvent(s, ev[3], 0), "cudaStreamWaitEvent");
+    FMM_STEP_TRY(launch_force_sums(t, totals, s), "reduce launch");
 #undef FMM_STEP_TRY
     return FMM_OK;
 }

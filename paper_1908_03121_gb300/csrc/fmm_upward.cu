@@ -11,6 +11,7 @@
 // shifted to the centre of mass afterwards.
 #include <type_traits>
 
+#include "fmm_chain.cuh"
 #include "fmm_convert.cuh"
 #include "fmm_internal.h"
 #include "fmm_tensor.cuh"
@@ -40,7 +41,8 @@ __device__ __forceinline__ T packed_mass(double m)
 // the status word: the centres of mass divide by masses.  With a packed-mass
 // array (T not void), the kernel also stores the masses in the same-level
 // pass's parity-split order and element type, which the pack kernel would
-// otherwise do for the leaves in a launch of its own.
+// otherwise do for the leaves in a launch of its own, and zeroes the work
+// queues' heads (queues) for the kernels after it.
 template <typename T>
 __global__ void __launch_bounds__(NCELL / 2) p2m_kernel(const NodeInfo *__restrict__ info,
                                                         const int32_t *__restrict__ leaves,
@@ -48,8 +50,11 @@ __global__ void __launch_bounds__(NCELL / 2) p2m_kernel(const NodeInfo *__restri
                                                         const double *__restrict__ rho,
                                                         double *__restrict__ M,
                                                         int32_t *__restrict__ status,
-                                                        T *__restrict__ mass)
+                                                        T *__restrict__ mass,
+                                                        int32_t *__restrict__ queues)
 {
+    chain_begin();
+    if (queues && blockIdx.x == 0 && threadIdx.x < 4) queues[threadIdx.x] = 0;
     const int node = leaves[blockIdx.x];
     const NodeInfo ni = info[node];
     const double h3 = levels[ni.level * LEVEL_FIELDS + LV_H3];
@@ -116,6 +121,7 @@ __global__ void __launch_bounds__(kSliceThreads) m2m_kernel(const NodeInfo *__re
     const int k = (x >> 2) + 2 * (y >> 2) + 4 * (z >> 2);
     const int ch = children[node * 8 + k];
     const bool child_leaf = info[ch].leaf_row >= 0;
+    chain_begin();
     const double hp = levels[ni.level * LEVEL_FIELDS + LV_H];
     const double q = 0.25 * hp;                 // half a child cell width
     const double ref[3] = {lo_x + (8.0 * ni.ix + x + 0.5) * hp, lo_y + (8.0 * ni.iy + y + 0.5) * hp,
@@ -269,6 +275,7 @@ __global__ void __launch_bounds__(kSliceThreads) m2m_df_kernel(const NodeInfo *_
     const int ch = children[node * 8 + k];
     const double hp = levels[ni.level * LEVEL_FIELDS + LV_H];
     const dfloat q = df_from_double(0.25 * hp);           // half a child cell width
+    chain_begin();
     const int c0 = 2 * (x & 3) + 16 * (y & 3) + 128 * (z & 3);   // child cell of j = 0
     dfloat m0, d[3], M2[6], M3[10];
     // child j sits at ref + q (e_x, e_y, e_z), e = +-1 from the bits of j
@@ -348,6 +355,7 @@ __global__ void __launch_bounds__(kSliceThreads) m2m_df_lanes_kernel(
     const NodeInfo ci = info[ch];
     const double hp = levels[ni.level * LEVEL_FIELDS + LV_H];
     const dfloat q = df_from_double(0.25 * hp);               // half a child cell width
+    chain_begin();
     const int cc = 2 * (x & 3) + 16 * (y & 3) + 128 * (z & 3) + 8 * (lane & 1) + 64 * (lane >> 1);
     // child i at cc + i: offset from the parent cell's centre, moments (a
     // leaf's vanish)
@@ -454,16 +462,16 @@ cudaError_t launch_p2m(const fmm_tree_s *t, const double *rho, double *M, cudaSt
     int32_t *status = t->dev.counters + kStatusSlot;
     if (!pack_leaves)
         p2m_kernel<void><<<grid, NCELL / 2, 0, s>>>(t->dev.info, leaves, t->dev.levels, rho, M,
-                                                   status, nullptr);
+                                                   status, nullptr, nullptr);
     else if (t->cfg.precision == FMM_MIXED)
         p2m_kernel<float><<<grid, NCELL / 2, 0, s>>>(t->dev.info, leaves, t->dev.levels, rho, M,
-                                                    status, static_cast<float *>(t->dev.mass));
+                                                    status, static_cast<float *>(t->dev.mass), t->dev.counters);
     else if (t->cfg.precision == FMM_DFLOAT)
         p2m_kernel<dfloat><<<grid, NCELL / 2, 0, s>>>(t->dev.info, leaves, t->dev.levels, rho, M,
-                                                     status, static_cast<dfloat *>(t->dev.mass));
+                                                     status, static_cast<dfloat *>(t->dev.mass), t->dev.counters);
     else
         p2m_kernel<double><<<grid, NCELL / 2, 0, s>>>(t->dev.info, leaves, t->dev.levels, rho, M,
-                                                     status, static_cast<double *>(t->dev.mass));
+                                                     status, static_cast<double *>(t->dev.mass), t->dev.counters);
     return cudaGetLastError();
 }
 
@@ -491,24 +499,20 @@ cudaError_t launch_m2m_level(const fmm_tree_s *t, int level, double *M, double *
     if (t->cfg.precision != FMM_FP64) {
         ListRange lean, lanes;
         m2m_split(t, level, lean, lanes);
-        if (lean.count)
-            m2m_df_kernel<<<unsigned(lean.count * 8), kSliceThreads, 0, s>>>(
-                t->dev.info, t->dev.children, t->dev.lists + lean.off, t->dev.levels, M, com,
-                reinterpret_cast<dfloat *>(t->dev.up), t->cfg.box_lo[0], t->cfg.box_lo[1],
-                t->cfg.box_lo[2]);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess || lanes.count == 0) return e;
-        m2m_df_lanes_kernel<<<unsigned(lanes.count * (NCELL / kCellsPerCta)), kSliceThreads, 0, s>>>(
-            t->dev.info, t->dev.children, t->dev.lists + lanes.off, t->dev.levels, M, com,
-            reinterpret_cast<dfloat *>(t->dev.up), t->cfg.box_lo[0], t->cfg.box_lo[1],
-            t->cfg.box_lo[2]);
-        return cudaGetLastError();
+        auto run = [&](auto kern, const ListRange &l, int ctas_per_node) {
+            return launch_chained(kern, unsigned(l.count * ctas_per_node), kSliceThreads, s, t->dev.info,
+                                  t->dev.children, t->dev.lists + l.off, t->dev.levels, M, com,
+                                  reinterpret_cast<dfloat *>(t->dev.up), t->cfg.box_lo[0],
+                                  t->cfg.box_lo[1], t->cfg.box_lo[2]);
+        };
+        cudaError_t e = cudaSuccess;
+        if (lean.count) e = run(m2m_df_kernel, lean, 8);
+        if (e == cudaSuccess && lanes.count) e = run(m2m_df_lanes_kernel, lanes, NCELL / kCellsPerCta);
+        return e;
     }
-    m2m_kernel<<<unsigned(r.count * 8), kSliceThreads, 0, s>>>(t->dev.info, t->dev.children,
-                                                               t->dev.lists + r.off,
-                                                 t->dev.levels, M, com, t->cfg.box_lo[0],
-                                                 t->cfg.box_lo[1], t->cfg.box_lo[2]);
-    return cudaGetLastError();
+    return launch_chained(m2m_kernel, unsigned(r.count * 8), kSliceThreads, s, t->dev.info, t->dev.children,
+                          t->dev.lists + r.off, t->dev.levels, M, com, t->cfg.box_lo[0],
+                          t->cfg.box_lo[1], t->cfg.box_lo[2]);
 }
 
 }  // namespace fmm
