@@ -1,6 +1,7 @@
 // Downward pass (Sec. 4.3, third step) and leaf forces.
 //
-// l2l_kernel, one launch per level from the root down: each cell converts its
+// l2l_kernel, one launch per level of refined nodes from the root down, and
+// l2l_leaf_kernel for the leaf nodes: each cell converts its
 // own same-level result from level units to physical units, adds its parent's
 // final expansion re-centred at its own centre of mass,
 //   L^(n) += sum_{k=0}^{3-n} (1/k!) L_parent^(n+k) . d^k,  d = X - X_parent,
@@ -351,12 +352,28 @@ __global__ void __launch_bounds__(kSliceThreads) l2l_kernel(const NodeInfo *__re
     const int c = (blockIdx.x & 7) * kSliceThreads + threadIdx.x;
     chain_begin();
     double out[20], corr[3];
-    if (ni.leaf_row >= 0)
-        l2l_cell<MODE, 1>(info, ni, node, c, levels, levels_df, Lv, Lc, dL1, com, L64, dacc, down,
-                          lo_x, lo_y, lo_z, out, corr);
-    else
-        l2l_cell<MODE, 3>(info, ni, node, c, levels, levels_df, Lv, Lc, dL1, com, L64, dacc, down,
-                          lo_x, lo_y, lo_z, out, corr);
+    l2l_cell<MODE, 3>(info, ni, node, c, levels, levels_df, Lv, Lc, dL1, com, L64, dacc, down, lo_x, lo_y,
+                      lo_z, out, corr);
+}
+
+// the same for leaf nodes (all of them in one launch): half a node per CTA
+constexpr int kLeafThreads = NCELL / 2;
+
+template <int MODE>
+__global__ void __launch_bounds__(kLeafThreads) l2l_leaf_kernel(
+    const NodeInfo *__restrict__ info, const int32_t *__restrict__ nodes,
+    const double *__restrict__ levels, const dfloat *__restrict__ levels_df,
+    const void *__restrict__ Lv, const float *__restrict__ Lc, const double *dL1,
+    const double *__restrict__ com, double *__restrict__ L64, double *dacc, float *__restrict__ down,
+    double lo_x, double lo_y, double lo_z)
+{
+    const int node = nodes[blockIdx.x >> 1];
+    const NodeInfo ni = info[node];
+    const int c = (blockIdx.x & 1) * kLeafThreads + threadIdx.x;
+    chain_begin();
+    double out[20], corr[3];
+    l2l_cell<MODE, 1>(info, ni, node, c, levels, levels_df, Lv, Lc, dL1, com, L64, dacc, down, lo_x, lo_y,
+                      lo_z, out, corr);
 }
 
 // 64 threads per leaf node, one (x, y) column of 8 cells each.
@@ -773,31 +790,39 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_kernel(const int32_t *_
 
 }  // namespace
 
+// node lists whose parents are done
+template <class Kern>
+static cudaError_t launch_l2l(Kern kern, unsigned grid, int threads, const fmm_tree_s *t,
+                              const ListRange &r, const void *L, const float *Lc, const double *dL1,
+                              const double *com, double *L64, double *dacc, cudaStream_t s)
+{
+    const auto &c = t->cfg;
+    return launch_chained(kern, grid, threads, s, t->dev.info, t->dev.lists + r.off, t->dev.levels,
+                          reinterpret_cast<const dfloat *>(t->dev.levels_df), L, Lc, dL1, com, L64, dacc,
+                          t->dev.down, c.box_lo[0], c.box_lo[1], c.box_lo[2]);
+}
+
 cudaError_t launch_l2l_level(const fmm_tree_s *t, int level, const void *L, const float *Lc,
                              const double *dL1, const double *com, double *L64, double *dacc,
                              cudaStream_t s)
 {
-    return launch_l2l_nodes(t, t->plan.nodes_at[size_t(level)], L, Lc, dL1, com, L64, dacc, s);
+    const ListRange &r = t->plan.refined_at[size_t(level)];
+    if (r.count == 0) return cudaSuccess;
+    auto kern = t->cfg.precision == FMM_MIXED    ? l2l_kernel<FMM_MIXED>
+                : t->cfg.precision == FMM_DFLOAT ? l2l_kernel<FMM_DFLOAT>
+                                                 : l2l_kernel<FMM_FP64>;
+    return launch_l2l(kern, unsigned(r.count * 8), kSliceThreads, t, r, L, Lc, dL1, com, L64, dacc, s);
 }
 
-// any list of nodes whose parents are done (one level, the refined nodes of
-// one level, or every leaf once every refined node is done)
-cudaError_t launch_l2l_nodes(const fmm_tree_s *t, const ListRange &r, const void *L,
-                             const float *Lc, const double *dL1, const double *com, double *L64,
-                             double *dacc, cudaStream_t s)
+cudaError_t launch_l2l_leaves(const fmm_tree_s *t, const void *L, const float *Lc, const double *dL1,
+                              const double *com, double *L64, double *dacc, cudaStream_t s)
 {
+    const ListRange &r = t->plan.leaves;
     if (r.count == 0) return cudaSuccess;
-    const auto &c = t->cfg;
-    const unsigned grid = unsigned(r.count * 8);
-    const int32_t *nodes = t->dev.lists + r.off;
-    const dfloat *ldf = reinterpret_cast<const dfloat *>(t->dev.levels_df);
-    auto launch = [&](auto kern) {
-        return launch_chained(kern, grid, kSliceThreads, s, t->dev.info, nodes, t->dev.levels, ldf, L, Lc,
-                              dL1, com, L64, dacc, t->dev.down, c.box_lo[0], c.box_lo[1], c.box_lo[2]);
-    };
-    if (c.precision == FMM_MIXED) return launch(l2l_kernel<FMM_MIXED>);
-    if (c.precision == FMM_DFLOAT) return launch(l2l_kernel<FMM_DFLOAT>);
-    return launch(l2l_kernel<FMM_FP64>);
+    auto kern = t->cfg.precision == FMM_MIXED    ? l2l_leaf_kernel<FMM_MIXED>
+                : t->cfg.precision == FMM_DFLOAT ? l2l_leaf_kernel<FMM_DFLOAT>
+                                                 : l2l_leaf_kernel<FMM_FP64>;
+    return launch_l2l(kern, unsigned(r.count * 2), kLeafThreads, t, r, L, Lc, dL1, com, L64, dacc, s);
 }
 
 cudaError_t launch_leaf_finish(const fmm_tree_s *t, const void *L, const float *Lc,

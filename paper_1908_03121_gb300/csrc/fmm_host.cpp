@@ -586,13 +586,11 @@ static void plan_work(fmm_tree_s *t)
     P.refined_at.assign(size_t(t->max_level) + 2, {});
     P.leafkids_at.assign(size_t(t->max_level) + 2, {});
     P.mixedkids_at.assign(size_t(t->max_level) + 2, {});
-    P.nodes_at.assign(size_t(t->max_level) + 2, {});
     for (int lev = 1; lev <= t->max_level; ++lev) {
-        std::vector<int32_t> ref, all, leafkids, mixedkids;
+        std::vector<int32_t> ref, leafkids, mixedkids;
         for (int64_t i = 0; i < n; ++i) {
             const NodeInfo &x = t->info[size_t(i)];
             if (x.level != lev) continue;
-            all.push_back(int32_t(i));
             if (x.leaf_row >= 0) continue;
             ref.push_back(int32_t(i));
             bool kids_leaves = true;
@@ -604,7 +602,6 @@ static void plan_work(fmm_tree_s *t)
         P.refined_at[size_t(lev)] = push_range(ref);
         P.leafkids_at[size_t(lev)] = push_range(leafkids);
         P.mixedkids_at[size_t(lev)] = push_range(mixedkids);
-        P.nodes_at[size_t(lev)] = push_range(all);
     }
 }
 
@@ -898,29 +895,29 @@ int fmm_get_stats(fmm_tree_t t, fmm_stats *o)
     o->work_items[3] = P.roots.count;
     for (int k = 0; k < 4; ++k) o->kernel_interactions[k] = P.kernel_interactions[k];
     o->reach = P.reach;
-    int m2l = 1 /*pack*/ + (P.roots.count > 0) + (P.work_mp.count > 0) + (P.work_mono.count > 0) +
-              (P.n_mx_targets > 0);
+    // (the monopole<-multipole targets ride in the multipole launch, except
+    // where kernels are timed one by one)
+    const int mx_alone =
+        P.n_mx_targets > 0 && (P.work_mp.count == 0 || (t->cfg.flags & FMM_FLAG_TIMING));
+    const int m2l = 1 /*pack*/ + (P.roots.count > 0) + (P.work_mp.count > 0) + (P.work_mono.count > 0) +
+                    mx_alone;
     int up = 1;
     for (int lev = 1; lev < t->max_level; ++lev) {
         ListRange lean, lanes;
         up += t->cfg.precision == FMM_FP64 ? P.refined_at[size_t(lev)].count > 0
                                            : m2m_split(t, lev, lean, lanes);
     }
-    int down = 0;
-    for (int lev = 1; lev <= t->max_level; ++lev) down += P.nodes_at[size_t(lev)].count > 0;
+    int refined_levels = 0;
+    for (int lev = 1; lev <= t->max_level; ++lev) refined_levels += P.refined_at[size_t(lev)].count > 0;
+    const int down = refined_levels + (P.leaves.count > 0);
     o->launches_m2l = m2l;
     o->launches_step = up + m2l + down + 2;
     // fmm_step: P2M also packs the leaf masses, one pack launch for the
     // refined nodes; then either the refined levels' shifts per level and
     // every leaf's shift and forces in one launch, or (dataflow tuning) all
     // of it in one persistent launch; the force sums
-    int refined_levels = 0;
-    for (int lev = 1; lev <= t->max_level; ++lev) refined_levels += P.refined_at[size_t(lev)].count > 0;
-    // (the monopole<-multipole targets ride in the multipole launch)
-    const int mx_alone = (P.n_mx_targets > 0) && (P.work_mp.count == 0);
-    const int downward = t->tuning.dataflow ? 1 : refined_levels + (P.leaves.count > 0);
-    o->launches_fused = up + (m2l - 1) - (P.n_mx_targets > 0) + mx_alone + (P.refined.count > 0) +
-                        downward + 1;
+    const int downward = t->tuning.dataflow ? 1 : down;
+    o->launches_fused = up + (m2l - 1) + (P.refined.count > 0) + downward + 1;
     if ((t->cfg.flags & FMM_FLAG_TIMING) && !t->host_only) {
         o->timing = 1;
         timing_fold(t);
@@ -975,14 +972,30 @@ int fmm_m2l(fmm_tree_t t, const double *M, const double *com, void *L, float *L_
     if (t->cfg.precision != FMM_FP64 && !L_comp)
         return fail(FMM_ERR_INVALID_ARG, "L_comp is required in FMM_MIXED and FMM_DFLOAT");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    timing_begin(t, FMM_K_PACK, s);
-    cudaError_t e = launch_pack(t, M, com, s);
-    timing_end(t, s);
-    if (e != cudaSuccess) return cuda_fail(e, "pack launch");
     int nl = 0;
-    e = launch_m2l(t, L, L_comp, dL1, s, &nl);
-    if (e != cudaSuccess) return cuda_fail(e, "m2l launch");
-    return FMM_OK;
+    if (t->cfg.flags & FMM_FLAG_TIMING) {
+        // per-kernel events: one kernel after the other
+        timing_begin(t, FMM_K_PACK, s);
+        cudaError_t e = launch_pack(t, M, com, s);
+        timing_end(t, s);
+        if (e != cudaSuccess) return cuda_fail(e, "pack launch");
+        e = launch_m2l(t, L, L_comp, dL1, s, &nl);
+        return e == cudaSuccess ? FMM_OK : cuda_fail(e, "m2l launch");
+    }
+    // The roots' few CTAs beside the monopole kernel, and the
+    // monopole<-multipole targets in the tail of the multipole launch
+    // (level-6 binary: 989 -> 817 us against the five kernels in sequence)
+    cudaStream_t a = t->aux;
+    cudaError_t e = launch_pack(t, M, com, s);
+    if (e == cudaSuccess) e = launch_m2l(t, L, L_comp, dL1, s, &nl, M2L_RESET);
+    if (e == cudaSuccess) e = cudaEventRecord(t->step_ev[0], s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(a, t->step_ev[0], 0);
+    if (e == cudaSuccess) e = launch_m2l(t, L, L_comp, dL1, a, &nl, M2L_ROOT);
+    if (e == cudaSuccess) e = cudaEventRecord(t->step_ev[1], a);
+    if (e == cudaSuccess) e = launch_m2l(t, L, L_comp, dL1, s, &nl, M2L_MONO);
+    if (e == cudaSuccess) e = launch_m2l(t, L, L_comp, dL1, s, &nl, M2L_MP | M2L_MPX);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, t->step_ev[1], 0);
+    return e == cudaSuccess ? FMM_OK : cuda_fail(e, "m2l launch");
 }
 
 int fmm_downward(fmm_tree_t t, const void *L, const float *L_comp, const double *dL1,
@@ -994,10 +1007,13 @@ int fmm_downward(fmm_tree_t t, const void *L, const float *L_comp, const double 
     if (t->cfg.precision != FMM_FP64 && !L_comp)
         return fail(FMM_ERR_INVALID_ARG, "L_comp is required in FMM_MIXED and FMM_DFLOAT");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    for (int lev = 1; lev <= t->max_level; ++lev) {
-        if (t->plan.nodes_at[size_t(lev)].count == 0) continue;
+    // the refined nodes level by level, then every leaf node at once
+    for (int lev = 1; lev <= t->max_level + 1; ++lev) {
+        const bool leaves = lev > t->max_level;
+        if ((leaves ? t->plan.leaves : t->plan.refined_at[size_t(lev)]).count == 0) continue;
         timing_begin(t, FMM_K_L2L, s);
-        cudaError_t e = launch_l2l_level(t, lev, L, L_comp, dL1, com, L64, dL1_acc, s);
+        cudaError_t e = leaves ? launch_l2l_leaves(t, L, L_comp, dL1, com, L64, dL1_acc, s)
+                               : launch_l2l_level(t, lev, L, L_comp, dL1, com, L64, dL1_acc, s);
         timing_end(t, s);
         if (e != cudaSuccess) return cuda_fail(e, "l2l launch");
     }
@@ -1094,8 +1110,7 @@ int fmm_step(fmm_tree_t t, const double *rho, double *M, double *com, void *L, f
     }
     // main: shifts of the refined nodes, root level first
     for (int lev = 1; lev <= t->max_level; ++lev)
-        FMM_STEP_TRY(launch_l2l_nodes(t, P.refined_at[size_t(lev)], L, L_comp, dL1, com, L64,
-                                      dL1_acc, s), "l2l launch");
+        FMM_STEP_TRY(launch_l2l_level(t, lev, L, L_comp, dL1, com, L64, dL1_acc, s), "l2l launch");
     // every leaf's shift and forces in one pass (the shifted expansion feeds
     // the forces from registers), the sums
     FMM_STEP_TRY(launch_leaf_finish(t, L, L_comp, dL1, com, L64, dL1_acc, M, phi, g, s),

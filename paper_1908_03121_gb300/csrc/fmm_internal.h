@@ -136,10 +136,9 @@ struct Plan {
     int64_t stencil_union = 0;
     // node lists
     ListRange leaves;                // all leaf nodes (P2M, forces)
-    std::vector<ListRange> refined_at;   // [level] refined nodes (M2M)
+    std::vector<ListRange> refined_at;   // [level] refined nodes (M2M, L2L)
     std::vector<ListRange> leafkids_at;  // [level] refined nodes whose 8 children are leaves
     std::vector<ListRange> mixedkids_at; // [level] the other refined nodes
-    std::vector<ListRange> nodes_at;     // [level] all nodes (L2L)
     ListRange work_mp, work_mono, work_mx, roots;
     ListRange refined;                    // every refined node (roots included)
     int64_t n_mx_targets = 0;             // leaf cells with refined sources
@@ -216,12 +215,14 @@ enum { M2L_RESET = 1, M2L_ROOT = 2, M2L_MP = 4, M2L_MONO = 8, M2L_MX = 16, M2L_A
        M2L_MPX = 32 };
 cudaError_t launch_m2l(const fmm_tree_s *t, void *L, float *Lc, double *dL1,
                        cudaStream_t s, int *n_launches, int parts = M2L_ALL);
+// one level's refined nodes (their parents done); every leaf node (every
+// refined node done)
 cudaError_t launch_l2l_level(const fmm_tree_s *t, int level, const void *L,
                              const float *Lc, const double *dL1, const double *com,
                              double *L64, double *dacc, cudaStream_t s);
-cudaError_t launch_l2l_nodes(const fmm_tree_s *t, const ListRange &r, const void *L,
-                             const float *Lc, const double *dL1, const double *com,
-                             double *L64, double *dacc, cudaStream_t s);
+cudaError_t launch_l2l_leaves(const fmm_tree_s *t, const void *L, const float *Lc,
+                              const double *dL1, const double *com, double *L64, double *dacc,
+                              cudaStream_t s);
 cudaError_t launch_leaf_finish(const fmm_tree_s *t, const void *L, const float *Lc,
                                const double *dL1, const double *com, double *L64, double *dacc,
                                const double *M, double *phi, double *g, cudaStream_t s);
