@@ -630,6 +630,10 @@ static void free_device(fmm_tree_s *t)
         cudaStreamDestroy(t->aux);
         t->aux = nullptr;
     }
+    if (t->scf_host) {
+        cudaFreeHost(t->scf_host);
+        t->scf_host = nullptr;
+    }
     DeviceTables &d = t->dev;
     void *ptrs[] = {d.info, d.children, d.nbr, d.lists, d.stencil, d.stencil_f, d.coef32, d.mono_woff, d.orbits, d.orbit_coef,
                     d.tree_leaf_off, d.tree_leaf_rows, d.levels, d.levels_df, d.mass, d.mp, d.counters,

@@ -11,12 +11,15 @@
 //   Omega^2, C_1, C_2 from H = 0 at surface points A, B (star 1) and C
 //   (star 2),  rho' = max(rho_floor, rho_max,i (H / H_max,i)^n) where H > 0.
 // The per-cell work (centre of mass, H and its per-star maximum, the new
-// density) runs in three kernels over the leaf nodes; the host reads back
-// per-node partial sums and the potential at the three surface cells, and
-// forms the few scalars of the iteration in FP64.
+// density) runs in three kernels over the leaf nodes; the last CTA of the first
+// two to finish combines the nodes' values in a fixed order and writes them
+// into page-locked host memory (with the potential at the three surface
+// cells), from which the host forms the few scalars of the iteration in FP64.
+// (An update of 512 leaf nodes, with its solve: 355 -> 293 us against copies of every
+// node's partial sums through pageable memory and full shuffle trees of FP64
+// adds per node.)
 #include <cmath>
 #include <string>
-#include <vector>
 
 #include "fmm_internal.h"
 
@@ -39,39 +42,81 @@ __device__ __forceinline__ void cell_centre(const NodeInfo &ni, const double *le
     x[2] = g.lo[2] + (8.0 * ni.iz + (c >> 6) + 0.5) * h;
 }
 
-// fixed-order block sum / max of NV values over kScfThreads threads; result
-// in thread 0
+// fixed-order sum or maximum of every component k of the 256 threads' v[k]; the
+// results in threads 0 .. NV - 1.  Sixteen threads per component combine
+// sixteen values each, then one the sixteen: 31 dependent FP64 operations,
+// where a shuffle tree has all eight warps at work on each of its levels.
 template <int NV, bool MAX>
-__device__ __forceinline__ void block_reduce(double v[NV])
+__device__ __forceinline__ double block_combine(const double v[NV])
 {
-    __shared__ double sh[kScfThreads / 32][NV];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ double sh[NV][kScfThreads + kScfThreads / 16];
+    __shared__ double part[NV][16];
+    auto both = [](double a, double b) { return MAX ? fmax(a, b) : a + b; };
 #pragma unroll
-    for (int k = 0; k < NV; ++k)
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const double o = __shfl_down_sync(0xffffffffu, v[k], off);
-            v[k] = MAX ? fmax(v[k], o) : v[k] + o;
-        }
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < NV; ++k) sh[warp][k] = v[k];
+    for (int k = 0; k < NV; ++k) sh[k][threadIdx.x + threadIdx.x / 16] = v[k];
     __syncthreads();
-    if (threadIdx.x == 0)
-        for (int k = 0; k < NV; ++k) {
-            double s = sh[0][k];
-            for (int w = 1; w < kScfThreads / 32; ++w) s = MAX ? fmax(s, sh[w][k]) : s + sh[w][k];
-            v[k] = s;
-        }
+    if (threadIdx.x < 16 * NV) {
+        const int k = threadIdx.x >> 4, q = threadIdx.x & 15;
+        double t = sh[k][17 * q];
+#pragma unroll
+        for (int i = 1; i < 16; ++i) t = both(t, sh[k][17 * q + i]);
+        part[k][q] = t;
+    }
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x < NV) {
+        t = part[threadIdx.x][0];
+#pragma unroll
+        for (int q = 1; q < 16; ++q) t = both(t, part[threadIdx.x][q]);
+    }
+    return t;
 }
 
-// per leaf node: sum m, sum m x, sum m y, sum m z (m = rho h^3) into
-// partials[row][0..3]
+// the node's value of component k (threads 0 .. NV - 1) into its row; in the
+// last CTA of the launch, true, with the rows' combined values in threads
+// 0 .. NV - 1 of `all`
+template <int NV, bool MAX>
+__device__ __forceinline__ bool combine_nodes(double mine, int row, double *partials, int32_t *arrived,
+                                              double &all)
+{
+    __shared__ int s_last;
+    if (threadIdx.x < NV) {
+        partials[size_t(row) * 8 + threadIdx.x] = mine;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(arrived, 1) == int(gridDim.x) - 1;
+    __syncthreads();
+    if (!s_last) return false;
+    __threadfence();
+    double v[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = MAX ? -1e300 : 0.0;
+    for (int i = threadIdx.x; i < int(gridDim.x); i += kScfThreads)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            const double o = __ldcg(partials + size_t(i) * 8 + k);      // past L1: other CTAs' rows
+            v[k] = MAX ? fmax(v[k], o) : v[k] + o;
+        }
+    all = block_combine<NV, MAX>(v);
+    if (threadIdx.x == 0) *arrived = 0;
+    return true;
+}
+
+// the potential's address at up to three surface cells
+struct ScfPoints {
+    const double *phi[3];
+};
+
+// sum m, sum m x, sum m y, sum m z (m = rho h^3) over the leaf nodes into
+// host[0..3], the potentials at the points into host[4..6]
 __global__ void __launch_bounds__(kScfThreads) scf_com_kernel(const NodeInfo *__restrict__ info,
                                                                const int32_t *__restrict__ leaves,
                                                                const double *__restrict__ levels,
                                                                const double *__restrict__ rho,
-                                                               double *__restrict__ partials, ScfGeo g)
+                                                               double *__restrict__ partials,
+                                                               int32_t *__restrict__ arrived, ScfGeo g,
+                                                               ScfPoints points, double *host)
 {
     const NodeInfo ni = info[leaves[blockIdx.x]];
     const double h3 = levels[ni.level * LEVEL_FIELDS + LV_H3];
@@ -84,9 +129,14 @@ __global__ void __launch_bounds__(kScfThreads) scf_com_kernel(const NodeInfo *__
 #pragma unroll
         for (int a = 0; a < 3; ++a) v[1 + a] = fma(m, x[a], v[1 + a]);
     }
-    block_reduce<4, false>(v);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 4; ++k) partials[size_t(ni.leaf_row) * 8 + k] = v[k];
+    const double mine = block_combine<4, false>(v);
+    double all;
+    if (!combine_nodes<4, false>(mine, ni.leaf_row, partials, arrived, all)) return;
+    if (threadIdx.x < 4) host[threadIdx.x] = all;
+    else if (threadIdx.x < 7) {
+        const double *at = points.phi[threadIdx.x - 4];
+        host[threadIdx.x] = at ? *at : 0.0;
+    }
 }
 
 struct ScfStars {
@@ -112,13 +162,14 @@ __device__ __forceinline__ double enthalpy(const double x[3], double phi, int st
     return s.C[star] - phi + 0.5 * s.omega2 * fma(wx, wx, wy * wy);
 }
 
-// per leaf node: the largest H of each star's cells into partials[row][4..5]
+// the largest H of each star's cells into host[0..1]
 __global__ void __launch_bounds__(kScfThreads) scf_hmax_kernel(const NodeInfo *__restrict__ info,
                                                                 const int32_t *__restrict__ leaves,
                                                                 const double *__restrict__ levels,
                                                                 const double *__restrict__ phi,
-                                                                double *__restrict__ partials, ScfGeo g,
-                                                                ScfStars s)
+                                                                double *__restrict__ partials,
+                                                                int32_t *__restrict__ arrived, ScfGeo g,
+                                                                ScfStars s, double *host)
 {
     const NodeInfo ni = info[leaves[blockIdx.x]];
     double v[2] = {-1e300, -1e300};
@@ -131,11 +182,20 @@ __global__ void __launch_bounds__(kScfThreads) scf_hmax_kernel(const NodeInfo *_
             v[star] = fmax(v[star], H);
         }
     }
-    block_reduce<2, true>(v);
-    if (threadIdx.x == 0) {
-        partials[size_t(ni.leaf_row) * 8 + 4] = v[0];
-        partials[size_t(ni.leaf_row) * 8 + 5] = v[1];
-    }
+    const double mine = block_combine<2, true>(v);
+    double all;
+    if (!combine_nodes<2, true>(mine, ni.leaf_row, partials, arrived, all)) return;
+    if (threadIdx.x < 2) host[threadIdx.x] = all;
+}
+
+// u^n, u > 0; half: 2 n where that is a whole number up to 16 (the usual
+// indices: products and a square root, a tenth of pow's FP64 operations)
+__device__ __forceinline__ double power(double u, double n, int half)
+{
+    if (half == 0) return pow(u, n);
+    double r = (half & 1) ? sqrt(u) : 1.0;
+    for (int k = half >> 1; k > 0; --k) r *= u;
+    return r;
 }
 
 // the new density: max(floor, rho_max,i (H / H_max,i)^n) inside star i where
@@ -144,8 +204,8 @@ __global__ void __launch_bounds__(kScfThreads) scf_hmax_kernel(const NodeInfo *_
 __global__ void __launch_bounds__(kScfThreads) scf_density_kernel(
     const NodeInfo *__restrict__ info, const int32_t *__restrict__ leaves,
     const double *__restrict__ levels, const double *__restrict__ phi, double *__restrict__ rho_out,
-    ScfGeo g, ScfStars s, double n, double rho_max0, double rho_max1, double ih0, double ih1,
-    double floor_value)
+    ScfGeo g, ScfStars s, double n, int half, double rho_max0, double rho_max1, double ih0,
+    double ih1, double floor_value)
 {
     const NodeInfo ni = info[leaves[blockIdx.x]];
     for (int c = threadIdx.x; c < NCELL; c += kScfThreads) {
@@ -157,7 +217,7 @@ __global__ void __launch_bounds__(kScfThreads) scf_density_kernel(
         if (star >= 0) {
             const double H = enthalpy(x, phi[idx], star, s);
             if (H > 0.0)
-                r = fmax(floor_value, (star ? rho_max1 : rho_max0) * pow(H * (star ? ih1 : ih0), n));
+                r = fmax(floor_value, (star ? rho_max1 : rho_max0) * power(H * (star ? ih1 : ih0), n, half));
         }
         rho_out[idx] = r;
     }
@@ -173,27 +233,32 @@ int scf_fail(int code, const std::string &msg)
 // if none)
 bool find_cell(const fmm_tree_s *t, const double p[3], int64_t &row, int &cell, double centre[3])
 {
+    // the point in units of the domain, and from the root down the child that
+    // holds it
     const double *lo = t->cfg.box_lo;
-    for (const NodeInfo &ni : t->info) {
-        if (ni.leaf_row < 0) continue;
-        const double n = std::ldexp(1.0, ni.level - 1);
-        double q[3];
-        const int32_t ij[3] = {ni.ix, ni.iy, ni.iz};
-        bool in = true;
-        for (int a = 0; a < 3; ++a) {
-            q[a] = (p[a] - lo[a]) / t->cfg.box_size * n - ij[a];
-            in = in && q[a] >= 0.0 && q[a] < 1.0;
-        }
-        if (!in) continue;
-        row = ni.leaf_row;
-        int k[3];
-        for (int a = 0; a < 3; ++a) k[a] = int(std::floor(q[a] * 8.0));
-        cell = k[0] + 8 * k[1] + 64 * k[2];
-        const double h = t->cfg.box_size / (8.0 * n);
-        for (int a = 0; a < 3; ++a) centre[a] = lo[a] + (8.0 * ij[a] + k[a] + 0.5) * h;
-        return true;
+    double f[3];
+    for (int a = 0; a < 3; ++a) {
+        f[a] = (p[a] - lo[a]) / t->cfg.box_size;
+        if (!(f[a] >= 0.0 && f[a] < 1.0)) return false;
     }
-    return false;
+    int64_t node = t->lists[size_t(t->plan.roots.off)];
+    for (double n = 2.0; t->info[size_t(node)].leaf_row < 0; n *= 2.0) {
+        int k = 0;
+        for (int a = 0; a < 3; ++a) k |= (int64_t(std::floor(f[a] * n)) & 1) << a;
+        node = t->children[size_t(node) * 8 + k];
+    }
+    const NodeInfo &ni = t->info[size_t(node)];
+    const double n = std::ldexp(1.0, ni.level - 1);
+    const int32_t ij[3] = {ni.ix, ni.iy, ni.iz};
+    const double h = t->cfg.box_size / (8.0 * n);
+    int k[3];
+    for (int a = 0; a < 3; ++a) {
+        k[a] = int(std::floor((f[a] * n - ij[a]) * 8.0));
+        centre[a] = lo[a] + (8.0 * ij[a] + k[a] + 0.5) * h;
+    }
+    row = ni.leaf_row;
+    cell = k[0] + 8 * k[1] + 64 * k[2];
+    return true;
 }
 
 }  // namespace
@@ -215,7 +280,7 @@ extern "C" int fmm_scf_update(fmm_tree_t t, const fmm_scf_params *p, const doubl
     const int64_t nl = t->n_leaf;
     // the surface conditions hold at the centres of the cells containing the
     // points, where the potential is known
-    int64_t row[3] = {0, 0, 0};
+    int64_t row[3] = {-1, -1, -1};
     int cell[3] = {0, 0, 0};
     double ctr[3][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
     const double *pts[3] = {p->point_a, p->point_b, p->point_c};
@@ -229,26 +294,25 @@ extern "C" int fmm_scf_update(fmm_tree_t t, const fmm_scf_params *p, const doubl
     const int32_t *leaves = t->dev.lists + t->plan.leaves.off;
     const ScfGeo g{{t->cfg.box_lo[0], t->cfg.box_lo[1], t->cfg.box_lo[2]}, t->cfg.box_size};
     // 1. centre of mass; the potential at the surface cells
+    cudaError_t e = cudaSuccess;
+    if (!t->scf_host) {
+        e = cudaMallocHost(reinterpret_cast<void **>(&t->scf_host), 8 * sizeof(double));
+        if (e != cudaSuccess) {
+            t->scf_host = nullptr;
+            return scf_fail(FMM_ERR_NOMEM, cudaGetErrorString(e));
+        }
+    }
+    ScfPoints points{};
+    for (int k = 0; k < 3; ++k)
+        if (row[k] >= 0) points.phi[k] = phi + row[k] * NCELL + cell[k];
     scf_com_kernel<<<unsigned(nl), kScfThreads, 0, s>>>(t->dev.info, leaves, t->dev.levels, rho,
-                                                         t->dev.partials, g);
-    cudaError_t e = cudaGetLastError();
-    std::vector<double> part(size_t(nl) * 8);
-    double phis[3] = {0.0, 0.0, 0.0};
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(part.data(), t->dev.partials, part.size() * sizeof(double),
-                            cudaMemcpyDeviceToHost, s);
-    for (int k = 0; k < 3 && e == cudaSuccess; ++k)
-        e = cudaMemcpyAsync(&phis[k], phi + row[k] * NCELL + cell[k], sizeof(double),
-                            cudaMemcpyDeviceToHost, s);
+                                                         t->dev.partials, t->dev.reduce_arrived, g,
+                                                         points, t->scf_host);
+    e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return scf_fail(FMM_ERR_CUDA, cudaGetErrorString(e));
-    double msum = 0.0, mx = 0.0, my = 0.0, mz = 0.0;
-    for (int64_t r = 0; r < nl; ++r) {        // fixed order
-        msum += part[size_t(r) * 8];
-        mx += part[size_t(r) * 8 + 1];
-        my += part[size_t(r) * 8 + 2];
-        mz += part[size_t(r) * 8 + 3];
-    }
+    const double msum = t->scf_host[0], mx = t->scf_host[1], my = t->scf_host[2], mz = t->scf_host[3];
+    const double phis[3] = {t->scf_host[4], t->scf_host[5], t->scf_host[6]};
     if (!(msum > 0.0)) return scf_fail(FMM_ERR_INVALID_ARG, "the density has no positive mass");
     ScfStars st{};
     st.com[0] = mx / msum;
@@ -274,22 +338,19 @@ extern "C" int fmm_scf_update(fmm_tree_t t, const fmm_scf_params *p, const doubl
     }
     // 3. each star's largest enthalpy
     scf_hmax_kernel<<<unsigned(nl), kScfThreads, 0, s>>>(t->dev.info, leaves, t->dev.levels, phi,
-                                                          t->dev.partials, g, st);
+                                                          t->dev.partials, t->dev.reduce_arrived, g, st,
+                                                          t->scf_host);
     e = cudaGetLastError();
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(part.data(), t->dev.partials, part.size() * sizeof(double),
-                            cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return scf_fail(FMM_ERR_CUDA, cudaGetErrorString(e));
-    double hmax[2] = {-1e300, -1e300};
-    for (int64_t r = 0; r < nl; ++r)
-        for (int i = 0; i < 2; ++i) hmax[i] = std::fmax(hmax[i], part[size_t(r) * 8 + 4 + i]);
+    const double hmax[2] = {t->scf_host[0], t->scf_host[1]};
     for (int i = 0; i < 2; ++i)
         if (st.live[i] && !(hmax[i] > 0.0))
             return scf_fail(FMM_ERR_INVALID_ARG, "a star has no cell with positive enthalpy");
     // 4. the new density
+    const int half = 2.0 * p->n <= 16.0 && 2.0 * p->n == std::floor(2.0 * p->n) ? int(2.0 * p->n) : 0;
     scf_density_kernel<<<unsigned(nl), kScfThreads, 0, s>>>(
-        t->dev.info, leaves, t->dev.levels, phi, rho_out, g, st, p->n, p->rho_max[0],
+        t->dev.info, leaves, t->dev.levels, phi, rho_out, g, st, p->n, half, p->rho_max[0],
         p->rho_max[1], 1.0 / hmax[0], st.live[1] ? 1.0 / hmax[1] : 0.0, p->rho_floor);
     e = cudaGetLastError();
     if (e != cudaSuccess) return scf_fail(FMM_ERR_CUDA, cudaGetErrorString(e));
