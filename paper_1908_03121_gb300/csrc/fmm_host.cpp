@@ -1095,14 +1095,23 @@ int fmm_step(fmm_tree_t t, const double *rho, double *M, double *com, void *L, f
     // leave SMs idle; as a launch of its own it held its SMs for its whole
     // run and delayed whichever of the multipole kernel and the shifts
     // came second.
-    FMM_STEP_TRY(cudaStreamWaitEvent(s, ev[3], 0), "cudaStreamWaitEvent");
-    FMM_STEP_TRY(launch_m2l(t, L, L_comp, dL1, s, &nl, M2L_MP | M2L_MPX), "m2l launch");
-    // aux: the roots (16 CTAs per root) beside the multipole launch rather
-    // than before it on the main stream, where the GPU idled around them
-    FMM_STEP_TRY(cudaStreamWaitEvent(a, ev[1], 0), "cudaStreamWaitEvent");
-    FMM_STEP_TRY(launch_m2l(t, L, L_comp, dL1, a, &nl, M2L_ROOT), "m2l launch");
-    FMM_STEP_TRY(cudaEventRecord(ev[2], a), "cudaEventRecord");
-    FMM_STEP_TRY(cudaStreamWaitEvent(s, ev[2], 0), "cudaStreamWaitEvent");
+    if (P.work_mp.count > 0) {
+        FMM_STEP_TRY(cudaStreamWaitEvent(s, ev[3], 0), "cudaStreamWaitEvent");
+        FMM_STEP_TRY(launch_m2l(t, L, L_comp, dL1, s, &nl, M2L_MP | M2L_MPX), "m2l launch");
+    }
+    // the roots (16 CTAs per root) on aux, beside the multipole launch rather
+    // than before it on the main stream, where the GPU idled around them;
+    // without one they need not wait for the monopole kernel on aux
+    const bool roots_aux = P.work_mp.count > 0;
+    if (roots_aux) FMM_STEP_TRY(cudaStreamWaitEvent(a, ev[1], 0), "cudaStreamWaitEvent");
+    FMM_STEP_TRY(launch_m2l(t, L, L_comp, dL1, roots_aux ? a : s, &nl, M2L_ROOT), "m2l launch");
+    if (roots_aux) {
+        FMM_STEP_TRY(cudaEventRecord(ev[2], a), "cudaEventRecord");
+        FMM_STEP_TRY(cudaStreamWaitEvent(s, ev[2], 0), "cudaStreamWaitEvent");
+    } else {
+        FMM_STEP_TRY(cudaStreamWaitEvent(s, ev[3], 0), "cudaStreamWaitEvent");
+        FMM_STEP_TRY(launch_m2l(t, L, L_comp, dL1, s, &nl, M2L_MPX), "m2l launch");
+    }
     if (t->tuning.dataflow) {
         // main: the refined shifts and the leaf pass in one persistent
         // launch, each item started by its parent's readiness counter; the

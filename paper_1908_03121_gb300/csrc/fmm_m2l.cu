@@ -1723,10 +1723,11 @@ struct Kernels {
         static size_t done = 0;
         return allow_smem(mono_kernel<NB, RR>, bytes, done);
     }
+    template <int PLANES>
     static cudaError_t mono_wide(size_t bytes)
     {
         static size_t done = 0;
-        return allow_smem(mono_wide_kernel<T>, bytes, done);
+        return allow_smem(mono_wide_kernel<T, PLANES>, bytes, done);
     }
 };
 
@@ -1772,7 +1773,7 @@ cudaError_t launch_mono(const KParams &K, size_t wbytes, int sms, int cap, cudaS
     }
 }
 
-// the wide types' monopole kernel: one leaf node per item, one CTA per SM
+// the wide types' monopole kernel
 template <typename T>
 cudaError_t launch_mono_wide(const fmm_tree_s *t, const KParams &K, int sms, cudaStream_t s)
 {
@@ -1791,11 +1792,18 @@ cudaError_t launch_mono_wide(const fmm_tree_s *t, const KParams &K, int sms, cud
     P.L = K.L;
     P.Lc = K.Lc;
     P.dL1 = K.dL1;
-    const size_t bytes = mono_wide_smem<T>(P.reach, P.n_coef);
-    cudaError_t e = Kernels<T>::mono_wide(bytes);
+    // a CTA per node, or per plane of one while those do not fill the SMs
+    const bool planes = K.n_items <= sms;
+    const size_t bytes = mono_wide_smem<T>(P.reach, planes ? 1 : 4, P.n_coef);
+    cudaError_t e = planes ? Kernels<T>::template mono_wide<1>(bytes) : Kernels<T>::template mono_wide<4>(bytes);
     if (e != cudaSuccess) return e;
-    const int g = int(std::min<int64_t>(K.n_items, sms));
-    mono_wide_kernel<T><<<g, kMonoWThreads, bytes, s>>>(P);
+    if (planes) {
+        P.n_items = 4 * K.n_items;
+        const int g = persistent_grid(mono_wide_kernel<T, 1>, bytes, P.n_items, sms, 0, 128);
+        mono_wide_kernel<T, 1><<<g, 128, bytes, s>>>(P);
+    } else {
+        mono_wide_kernel<T, 4><<<std::min(P.n_items, sms), 512, bytes, s>>>(P);
+    }
     return cudaGetLastError();
 }
 

@@ -25,7 +25,10 @@
 // A thread has one target block and one b (the same for a whole warp, so the
 // weights are broadcasts); its 32 sums A[q][c] belong to a = q xor b xor e_c and
 // meet those of the other b at the end, through shared memory, in a fixed
-// order.  One CTA of 16 warps takes one leaf node.
+// order.  A CTA takes PLANES of the four planes of blocks of a leaf node: all
+// four with 16 warps, one CTA per SM, or one with four warps where there are
+// few leaf nodes.  Same bits.  (A 9-sub-grid step in FP64, its root beside this
+// kernel: 172 -> 148 us.)
 #pragma once
 
 #include "fmm_internal.h"
@@ -35,8 +38,6 @@ namespace fmm {
 
 namespace {
 
-// one CTA per SM, 128 registers a thread
-constexpr int kMonoWThreads = 512;
 
 struct MonoWParams {
     const NodeInfo *info;
@@ -55,20 +56,20 @@ struct MonoWParams {
     double *dL1;
 };
 
-// window of (4 + 2 R)^3 blocks; the row pitch 12 puts the 16 (x, y) lanes of a
-// half warp on distinct banks for 8-byte elements
+// window of (4 + 2 R)^2 (planes + 2 R) blocks; the row pitch 12 puts the 16
+// (x, y) lanes of a half warp on distinct banks for 8-byte elements
 constexpr int kMonoWPitch = 12;
-__host__ __device__ constexpr int mono_wide_window(int reach)
+__host__ __device__ constexpr int mono_wide_window(int reach, int planes)
 {
-    return kMonoWPitch * (4 + 2 * reach) * (4 + 2 * reach);
+    return kMonoWPitch * (4 + 2 * reach) * (planes + 2 * reach);
 }
 
 // shared memory: the window (later the sums' exchange buffer, two components
-// of 8 x 64 threads x 8 values) and the weights
+// of 8 values of every thread) and the weights
 template <typename T>
-size_t mono_wide_smem(int reach, int n_coef)
+size_t mono_wide_smem(int reach, int planes, int n_coef)
 {
-    const size_t window = size_t(8) * mono_wide_window(reach), fold = size_t(2) * 8 * 512;
+    const size_t window = size_t(8) * mono_wide_window(reach, planes), fold = size_t(2) * 8 * 128 * planes;
     return ((window > fold ? window : fold) + size_t(n_coef)) * sizeof(T);
 }
 
@@ -123,26 +124,27 @@ __device__ __forceinline__ void mono_wide_orbits(const MonoWParams &P, const T *
         for (int k = 0; k < 4; ++k) A[q][k] = renorm(A[q][k]);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kMonoWThreads, 1) mono_wide_kernel(MonoWParams P)
+template <typename T, int PLANES>
+__global__ void __launch_bounds__(128 * PLANES, PLANES == 4 ? 1 : 4) mono_wide_kernel(MonoWParams P)
 {
+    constexpr int blocks = 16 * PLANES;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_nbr[27], s_item;
-    const int R = P.reach, E = 4 + 2 * R, pz = kMonoWPitch * E;
-    const int plane = pz * E;                            // blocks of one b
-    const int fold = 2 * 8 * 512;
+    const int R = P.reach, E = 4 + 2 * R, EZ = PLANES + 2 * R, pz = kMonoWPitch * E;
+    const int plane = pz * EZ;                           // blocks of one b
+    const int fold = 2 * 8 * 8 * blocks;
     T *W = reinterpret_cast<T *>(smem_raw);
     T *s_coef = W + (8 * plane > fold ? 8 * plane : fold);
     const T *mass = static_cast<const T *>(P.mass);
     for (int i = threadIdx.x; i < P.n_coef; i += blockDim.x)
         s_coef[i] = ldg_t(static_cast<const T *>(P.coef) + i);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int b = warp >> 1, block = (warp & 1) * 32 + lane;   // target block x + 4 y + 16 z
+    const int b = threadIdx.x / blocks, block = threadIdx.x % blocks;   // target block x + 4 y + 16 z
     const int tx = block & 3, ty = (block >> 2) & 3, tz = block >> 4;
     for (;;) {
         const int item = pull_item(P.counter, &s_item);
         if (item >= P.n_items) break;
-        const int node = P.list[item];
+        const int node = P.list[item / (4 / PLANES)];
+        const int z0 = item % (4 / PLANES) * PLANES;           // the CTA's first plane
         // leaf neighbours (-1: absent or refined)
         if (threadIdx.x < 27) {
             const int nb = P.nbr[node * 27 + threadIdx.x];
@@ -151,9 +153,9 @@ __global__ void __launch_bounds__(kMonoWThreads, 1) mono_wide_kernel(MonoWParams
         __syncthreads();
         // the window's masses, child s of block u to plane s (the packed mass
         // array has a node's child-s cells contiguous)
-        for (int i = threadIdx.x; i < E * E * E; i += blockDim.x) {
+        for (int i = threadIdx.x; i < E * E * EZ; i += blockDim.x) {
             const int ux = i % E, uy = (i / E) % E, uz = i / (E * E);
-            const int bx = ux - R + 4, by = uy - R + 4, bz = uz - R + 4;      // >= 1
+            const int bx = ux - R + 4, by = uy - R + 4, bz = uz - R + z0 + 4; // >= 1
             const int nb = s_nbr[(bx >> 2) + 3 * (by >> 2) + 9 * (bz >> 2)];
             const int src = (bx & 3) + 4 * (by & 3) + 16 * (bz & 3);
             const T *from = nb >= 0 ? mass + size_t(nb) * NCELL + src : mass;
@@ -164,7 +166,7 @@ __global__ void __launch_bounds__(kMonoWThreads, 1) mono_wide_kernel(MonoWParams
         cp_async_commit();
         cp_async_wait_all();
         // (each thread transforms the blocks that it staged itself)
-        for (int i = threadIdx.x; i < E * E * E; i += blockDim.x) {
+        for (int i = threadIdx.x; i < E * E * EZ; i += blockDim.x) {
             T *at = W + i % E + kMonoWPitch * ((i / E) % E) + pz * (i / (E * E));
             T m[8];
 #pragma unroll
@@ -205,18 +207,18 @@ __global__ void __launch_bounds__(kMonoWThreads, 1) mono_wide_kernel(MonoWParams
 #pragma unroll
             for (int k = 0; k < 2; ++k)
 #pragma unroll
-                for (int q = 0; q < 8; ++q) W[((k * 8 + b) * 8 + q) * 64 + block] = A[q][2 * half + k];
+                for (int q = 0; q < 8; ++q) W[((k * 8 + b) * 8 + q) * blocks + block] = A[q][2 * half + k];
             __syncthreads();
-            if (threadIdx.x < 128) {
-                const int k = threadIdx.x >> 6, t = threadIdx.x & 63;
+            if (threadIdx.x < 2 * blocks) {
+                const int k = threadIdx.x / blocks, t = threadIdx.x % blocks;
                 const int c = 2 * half + k;
                 const int ec = c == 0 ? 0 : 1 << (c - 1);
                 T o[8];
 #pragma unroll
                 for (int a = 0; a < 8; ++a) {
-                    T v = W[(k * 64 + (a ^ ec)) * 64 + t];
+                    T v = W[(k * 64 + (a ^ ec)) * blocks + t];
 #pragma unroll
-                    for (int s = 1; s < 8; ++s) v += W[((k * 8 + s) * 8 + (a ^ s ^ ec)) * 64 + t];
+                    for (int s = 1; s < 8; ++s) v += W[((k * 8 + s) * 8 + (a ^ s ^ ec)) * blocks + t];
                     o[a] = v;
                 }
 #pragma unroll
@@ -228,14 +230,14 @@ __global__ void __launch_bounds__(kMonoWThreads, 1) mono_wide_kernel(MonoWParams
                         o[a] = u + v;
                         o[a | ax] = u - v;
                     }
-                const int cell = 2 * (t & 3) + 16 * ((t >> 2) & 3) + 128 * (t >> 4);
+                const int cell = 2 * (t & 3) + 16 * ((t >> 2) & 3) + 128 * (z0 + (t >> 4));
 #pragma unroll
                 for (int p = 0; p < 8; ++p)
                     store_L<T>(P, node, c, cell + (p & 1) + 8 * ((p >> 1) & 1) + 64 * (p >> 2), o[p], T(0));
             }
         }
 #pragma unroll
-        for (int i = 0; i < 3; ++i) __stcs(P.dL1 + (size_t(node) * 3 + i) * NCELL + threadIdx.x, 0.0);
+        for (int i = 0; i < 3; ++i) __stcs(P.dL1 + (size_t(node) * 3 + i) * NCELL + 128 * z0 + threadIdx.x, 0.0);
         __syncthreads();
     }
 }
