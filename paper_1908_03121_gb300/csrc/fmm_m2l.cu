@@ -669,76 +669,86 @@ __device__ __forceinline__ void zero_moments(Src<float> &s)
 // n = 1, m = 2 term with the target's share added (D3 is odd):
 //   S_i -= sum_k (B2_B + M0_B a2_A)_k D3[i, k],  a2_A = B2_A / M0_A
 // (aA holds a2_A in its first five entries then).
-template <bool SRC_MP, int ORDER = 3, class LA, class SA>
+// WHAT: 1 only the Taylor coefficients, 2 only the correction, 3 both.
+template <bool SRC_MP, int ORDER = 3, int WHAT = 3, class LA, class SA>
 __device__ __forceinline__ void acc_mp(float Rx, float Ry, float Rz, const Src<float> &s,
                                        const float aA[7], LA &L, SA &S)
 {
     DTraceless D;
     D.eval<ORDER == 3>(Rx, Ry, Rz);
     const float nm0 = -s.m0;
-    float a = fmaf(nm0, D.D0, L.part[0]);
-    if (SRC_MP) {
+    if constexpr (WHAT & 1) {
+        float a = fmaf(nm0, D.D0, L.part[0]);
+        if (SRC_MP) {
 #pragma unroll
-        for (int k = 0; k < 5; ++k) a = fmaf(-s.B2[k], D.D2[k], a);
-        if (ORDER == 3) {
+            for (int k = 0; k < 5; ++k) a = fmaf(-s.B2[k], D.D2[k], a);
+            if (ORDER == 3) {
 #pragma unroll
-            for (int q = 0; q < 7; ++q) a = fmaf(s.B3[q], D.D3[q], a);
+                for (int q = 0; q < 7; ++q) a = fmaf(s.B3[q], D.D3[q], a);
+            }
         }
-    }
-    L.part[0] = a;
+        L.part[0] = a;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        float b = fmaf(nm0, D.D1[i], L.part[1 + i]);
-        if (SRC_MP && ORDER == 3) {
+        for (int i = 0; i < 3; ++i) {
+            float b = fmaf(nm0, D.D1[i], L.part[1 + i]);
+            if (SRC_MP && ORDER == 3) {
 #pragma unroll
-            for (int k = 0; k < 5; ++k) b = fmaf(-s.B2[k], D.d3slice(i, k), b);
+                for (int k = 0; k < 5; ++k) b = fmaf(-s.B2[k], D.d3slice(i, k), b);
+            }
+            L.part[1 + i] = b;
         }
-        L.part[1 + i] = b;
     }
     if constexpr (ORDER == 2) {
+        if constexpr (WHAT & 1)
 #pragma unroll
-        for (int k = 0; k < 5; ++k) L.part[4 + k] = fmaf(nm0, D.D2[k], L.part[4 + k]);
-        float wn[5];
+            for (int k = 0; k < 5; ++k) L.part[4 + k] = fmaf(nm0, D.D2[k], L.part[4 + k]);
+        if constexpr (WHAT & 2) {
+            float wn[5];
 #pragma unroll
-        for (int k = 0; k < 5; ++k) wn[k] = SRC_MP ? fmaf(nm0, aA[k], -s.B2[k]) : nm0 * aA[k];
+            for (int k = 0; k < 5; ++k) wn[k] = SRC_MP ? fmaf(nm0, aA[k], -s.B2[k]) : nm0 * aA[k];
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            float c = S.part[i];
+            for (int i = 0; i < 3; ++i) {
+                float c = S.part[i];
 #pragma unroll
-            for (int k = 0; k < 5; ++k) c = fmaf(wn[k], D.d3slice(i, k), c);
-            S.part[i] = c;
+                for (int k = 0; k < 5; ++k) c = fmaf(wn[k], D.d3slice(i, k), c);
+                S.part[i] = c;
+            }
         }
     } else {
-        // orders 2-3 (12 components): the pairs in which the derivative
-        // tensors come out of DTraceless (xx yy | xz yz of D2, xxx yyy
-        // | xxz yyz of D3) on the paired FP32 pipe (fma.rn.f32x2: each half
-        // rounds as fmaf does), the other four scalar
-        constexpr int pair_a[4] = {4, 7, 9, 11}, pair_b[4] = {5, 8, 14, 15};
-        const float dv[16] = {0.f, 0.f, 0.f, 0.f, D.D2[0], D.D2[1], D.D2[2], D.D2[3],
-                              D.D2[4], D.D3[0], D.D3[1], D.D3[2], D.D3[3], D.D3[4],
-                              D.D3[5], D.D3[6]};
-        const float2 nm2 = make_float2(nm0, nm0);
+        if constexpr (WHAT & 1) {
+            // orders 2-3 (12 components): the pairs in which the derivative
+            // tensors come out of DTraceless (xx yy | xz yz of D2, xxx yyy
+            // | xxz yyz of D3) on the paired FP32 pipe (fma.rn.f32x2: each half
+            // rounds as fmaf does), the other four scalar
+            constexpr int pair_a[4] = {4, 7, 9, 11}, pair_b[4] = {5, 8, 14, 15};
+            const float dv[16] = {0.f, 0.f, 0.f, 0.f, D.D2[0], D.D2[1], D.D2[2], D.D2[3],
+                                  D.D2[4], D.D3[0], D.D3[1], D.D3[2], D.D3[3], D.D3[4],
+                                  D.D3[5], D.D3[6]};
+            const float2 nm2 = make_float2(nm0, nm0);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int a = pair_a[j], b = pair_b[j];
-            const float2 r = __ffma2_rn(nm2, make_float2(dv[a], dv[b]),
-                                        make_float2(L.part[a], L.part[b]));
-            L.part[a] = r.x;
-            L.part[b] = r.y;
+            for (int j = 0; j < 4; ++j) {
+                const int a = pair_a[j], b = pair_b[j];
+                const float2 r = __ffma2_rn(nm2, make_float2(dv[a], dv[b]),
+                                            make_float2(L.part[a], L.part[b]));
+                L.part[a] = r.x;
+                L.part[b] = r.y;
+            }
+            L.part[6] = fmaf(nm0, dv[6], L.part[6]);
+            L.part[10] = fmaf(nm0, dv[10], L.part[10]);
+            L.part[12] = fmaf(nm0, dv[12], L.part[12]);
+            L.part[13] = fmaf(nm0, dv[13], L.part[13]);
         }
-        L.part[6] = fmaf(nm0, dv[6], L.part[6]);
-        L.part[10] = fmaf(nm0, dv[10], L.part[10]);
-        L.part[12] = fmaf(nm0, dv[12], L.part[12]);
-        L.part[13] = fmaf(nm0, dv[13], L.part[13]);
-        float w[7];
+        if constexpr (WHAT & 2) {
+            float w[7];
 #pragma unroll
-        for (int q = 0; q < 7; ++q) w[q] = SRC_MP ? fmaf(nm0, aA[q], s.B3[q]) : nm0 * aA[q];
+            for (int q = 0; q < 7; ++q) w[q] = SRC_MP ? fmaf(nm0, aA[q], s.B3[q]) : nm0 * aA[q];
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            float c = S.part[i];
+            for (int i = 0; i < 3; ++i) {
+                float c = S.part[i];
 #pragma unroll
-            for (int q = 0; q < 7; ++q) c = fmaf(w[q], D.U[i][q], c);
-            S.part[i] = c;
+                for (int q = 0; q < 7; ++q) c = fmaf(w[q], D.U[i][q], c);
+                S.part[i] = c;
+            }
         }
     }
 }
@@ -904,20 +914,106 @@ __device__ __forceinline__ void mx_target(const KParams &P, int t)
 }
 
 // ------------------------------------------------------------ mp_kernel
-// WARPS per CTA, PARTS items per sub-grid:
-//   8, 1: an item is a sub-grid, a warp each parity, both halves (z < 4, z >= 4);
-//   8, 2: an item is one half of a sub-grid;
-//   1, 16: an item is one half of one parity, 32 cells, and a CTA one warp.
+// The far loop of a warp's 32 targets, software-pipelined by hand: while one
+// entry is evaluated, the moments of the next are loaded, the window value of
+// the one after (which says where its moments are) and the window offset of
+// the one after that, so a warp waits for none of the three dependent loads;
+// leaf lanes load the zero row.
+template <int ORDER, int WHAT, int THREADS>
+__device__ __forceinline__ void mp_far_ahead(const KParams &P, const float *W, const float *mp,
+                                             const float4 *ent, int base, const float dA[3],
+                                             const float a3A[7], SmemAcc<16, 4, THREADS> &L,
+                                             SmemAcc<3, 3, THREADS> &S)
+{
+    const int last = P.n_far - 1;
+    float4 E = __ldg(ent);
+    float wv = W[base + __float_as_int(E.w)];
+    float wv1 = W[base + __float_as_int(__ldg(&ent[min(1, last)].w))];
+    int off2 = __float_as_int(__ldg(&ent[min(2, last)].w));
+    Src<float> src;
+    int idx;
+    bool is_mp = window_moments<float>(wv, P.mp_limit, idx);
+    load_source_at(mp + (is_mp ? idx : P.mp_limit), src);
+    for (int e0 = 0; e0 < P.n_far; e0 += kChunk) {
+        const int e1 = min(e0 + kChunk, P.n_far);
+        for (int e = e0; e < e1; ++e) {
+            Src<float> src1;
+            const bool is_mp1 = window_moments<float>(wv1, P.mp_limit, idx);
+            load_source_at(mp + (is_mp1 ? idx : P.mp_limit), src1);
+            const float wv2 = W[base + off2];
+            off2 = __float_as_int(__ldg(&ent[min(e + 3, last)].w));
+            const float4 E1 = __ldg(ent + min(e + 1, last));
+            if (__any_sync(0xffffffffu, is_mp)) {
+                if (!is_mp) src.m0 = wv;
+                float R[3];
+                separation(dA, src.d, E, R);
+                acc_mp<true, ORDER, WHAT>(R[0], R[1], R[2], src, a3A, L, S);
+            } else if (__any_sync(0xffffffffu, window_nonzero<float>(wv))) {
+                src.m0 = wv;
+                acc_mp<false, ORDER, WHAT>(dA[0] - E.x, dA[1] - E.y, dA[2] - E.z, src, a3A, L, S);
+            }
+            src = src1;
+            is_mp = is_mp1;
+            wv = wv1;
+            wv1 = wv2;
+            E = E1;
+        }
+        if (WHAT & 1) L.flush();
+        if (WHAT & 2) S.flush();
+    }
+}
+
+// Near sources: leaf cells only (refined ones contribute nothing here: their
+// children interact one level down); entries are skipped when none of the
+// warp's 32 sources is a leaf with mass (skipping exact zeros changes no sum).
+template <int ORDER, int WHAT, int THREADS>
+__device__ __forceinline__ void mp_near(const KParams &P, const float *W, const float4 *ent, int base,
+                                        const float dA[3], const float a3A[7],
+                                        SmemAcc<16, 4, THREADS> &L, SmemAcc<3, 3, THREADS> &S)
+{
+    for (int e0 = P.n_far; e0 < P.n_far + P.n_near; e0 += kChunk) {
+        const int e1 = min(e0 + kChunk, P.n_far + P.n_near);
+        for (int e = e0; e < e1; ++e) {
+            const float4 E = __ldg(ent + e);
+            const float wv = W[base + __float_as_int(E.w)];
+            Src<float> src;
+            src.m0 = window_refined<float>(wv) ? 0.f : wv;
+            if (!__any_sync(0xffffffffu, window_nonzero<float>(src.m0))) continue;
+            acc_mp<false, ORDER, WHAT>(dA[0] - E.x, dA[1] - E.y, dA[2] - E.z, src, a3A, L, S);
+        }
+        if (WHAT & 1) L.flush();
+        if (WHAT & 2) S.flush();
+    }
+}
+
+// fmm_step also hands the multipole launch the monopole<-multipole targets:
+// once the multipole queue is empty, each warp pulls 32 of them at a time
+// from their own queue, which fills the tail that the coarse multipole
+// items leave (the monopole kernel, whose results they add to, has
+// finished before this launch)
+template <int ORDER>
+__device__ __forceinline__ void mx_tail(const KParams &P)
+{
+    const int lane = threadIdx.x & 31;
+    while (P.n_mx > 0) {
+        int w = 0;
+        if (lane == 0) w = atomicAdd(P.mx_counter, 1);
+        w = __shfl_sync(0xffffffffu, w, 0);
+        if (w * 32 >= P.n_mx) break;
+        if (w * 32 + lane < P.n_mx) mx_target<float, ORDER>(P, w * 32 + lane);
+    }
+}
+
+// PARTS 1: an item is a sub-grid, a warp each parity, both halves (z < 4, z >=
+// 4); 2: one half of a sub-grid.
 // Three CTAs of eight warps per SM (at most 85 registers): the compensation
 // pairs, touched once per chunk, live in shared memory after the window.
-// AHEAD: the far loop is software-pipelined by hand (below), at 112 registers
-// and two such CTAs per SM: worth it only where the items do not fill the SMs
-// anyway.
-template <int ORDER, int WARPS, int PARTS, bool AHEAD>
-__global__ void __launch_bounds__(32 * WARPS, WARPS == 1 ? 1 : AHEAD ? 2 : 3) mp_kernel(KParams P)
+// AHEAD (mp_far_ahead) takes 112 registers and two such CTAs per SM: worth it
+// only where the items do not fill the SMs anyway.
+template <int ORDER, int PARTS, bool AHEAD>
+__global__ void __launch_bounds__(kThreads, AHEAD ? 2 : 3) mp_kernel(KParams P)
 {
-    static_assert((WARPS == 8 && PARTS <= 2) || (WARPS == 1 && PARTS == 16), "items per sub-grid");
-    constexpr int threads = 32 * WARPS;
+    constexpr int threads = kThreads;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float *W = reinterpret_cast<float *>(smem_raw);
     float *Cs = W + 8 * P.sub_stride + threadIdx.x;
@@ -930,7 +1026,7 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS == 1 ? 1 : AHEAD ? 2 : 3) mp
         const int item = pull_item(P.counter, &s_item);
         if (item >= P.n_items) break;
         const int node = P.list[item / PARTS];
-        const int p = WARPS == 8 ? warp : (item >> 1) & 7;
+        const int p = warp;
         const int px = p & 1, py = (p >> 1) & 1, pz = p >> 2;
         const float4 *ent = P.stencil_f + p * P.ent_stride;   // float offsets: no conversions
         const NodeInfo ti = P.info[node];
@@ -961,49 +1057,8 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS == 1 ? 1 : AHEAD ? 2 : 3) mp
             // moments' terms, so the same values), a mix the general form
             // with zero moments for the leaves, and an entry with only
             // absent sources (mass 0) is skipped.
-            // AHEAD: while one entry is evaluated, the moments of the next are
-            // loaded, the window value of the one after (which says where
-            // its moments are) and the window offset of the one after that,
-            // so a warp waits for none of the three dependent loads; leaf
-            // lanes load the zero row.
             if constexpr (AHEAD) {
-                const int last = P.n_far - 1;
-                float4 E = __ldg(ent);
-                float wv = W[base + __float_as_int(E.w)];
-                float wv1 = W[base + __float_as_int(__ldg(&ent[min(1, last)].w))];
-                int off2 = __float_as_int(__ldg(&ent[min(2, last)].w));
-                Src<float> src;
-                int idx;
-                bool is_mp = window_moments<float>(wv, P.mp_limit, idx);
-                load_source_at(mp + (is_mp ? idx : P.mp_limit), src);
-                for (int e0 = 0; e0 < P.n_far; e0 += kChunk) {
-                    const int e1 = min(e0 + kChunk, P.n_far);
-                    for (int e = e0; e < e1; ++e) {
-                        Src<float> src1;
-                        const bool is_mp1 = window_moments<float>(wv1, P.mp_limit, idx);
-                        load_source_at(mp + (is_mp1 ? idx : P.mp_limit), src1);
-                        const float wv2 = W[base + off2];
-                        off2 = __float_as_int(__ldg(&ent[min(e + 3, last)].w));
-                        const float4 E1 = __ldg(ent + min(e + 1, last));
-                        if (__any_sync(0xffffffffu, is_mp)) {
-                            if (!is_mp) src.m0 = wv;
-                            float R[3];
-                            separation(dA, src.d, E, R);
-                            acc_mp<true, ORDER>(R[0], R[1], R[2], src, a3A, L, S);
-                        } else if (__any_sync(0xffffffffu, window_nonzero<float>(wv))) {
-                            src.m0 = wv;
-                            acc_mp<false, ORDER>(dA[0] - E.x, dA[1] - E.y, dA[2] - E.z, src, a3A, L,
-                                                 S);
-                        }
-                        src = src1;
-                        is_mp = is_mp1;
-                        wv = wv1;
-                        wv1 = wv2;
-                        E = E1;
-                    }
-                    L.flush();
-                    S.flush();
-                }
+                mp_far_ahead<ORDER, 3>(P, W, mp, ent, base, dA, a3A, L, S);
             } else {
                 for (int e0 = 0; e0 < P.n_far; e0 += kChunk) {
                     const int e1 = min(e0 + kChunk, P.n_far);
@@ -1040,25 +1095,8 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS == 1 ? 1 : AHEAD ? 2 : 3) mp
                     S.flush();
                 }
             }
-            // near sources: leaf cells only (refined ones contribute nothing
-            // here: their children interact one level down); skipped when no
-            // neighbour is a leaf, and entry by entry when none of the
-            // warp's 32 sources is a leaf with mass (skipping exact zeros
-            // changes no sum)
-            for (int e0 = P.n_far; any_leaf && e0 < P.n_far + P.n_near; e0 += kChunk) {
-                const int e1 = min(e0 + kChunk, P.n_far + P.n_near);
-                for (int e = e0; e < e1; ++e) {
-                    const float4 E = __ldg(ent + e);
-                    const float wv = W[base + __float_as_int(E.w)];
-                    Src<float> src;
-                    src.m0 = window_refined<float>(wv) ? 0.f : wv;
-                    if (!__any_sync(0xffffffffu, window_nonzero<float>(src.m0))) continue;
-                    acc_mp<false, ORDER>(dA[0] - E.x, dA[1] - E.y, dA[2] - E.z, src, a3A, L,
-                                         S);
-                }
-                L.flush();
-                S.flush();
-            }
+            // skipped when no neighbour is a leaf
+            if (any_leaf) mp_near<ORDER, 3>(P, W, ent, base, dA, a3A, L, S);
             const int cell = ax + 8 * ay + 64 * az;
             store_target(P, node, cell, L);
 #pragma unroll
@@ -1067,20 +1105,66 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS == 1 ? 1 : AHEAD ? 2 : 3) mp
         }
         __syncthreads();
     }
-    // fmm_step also hands this launch the monopole<-multipole targets: once
-    // the multipole queue is empty, each warp pulls 32 of them at a time
-    // from their own queue, which fills the tail that the coarse multipole
-    // items leave (the monopole kernel, whose results they add to, has
-    // finished before this launch)
-    if (P.n_mx > 0) {
-        for (;;) {
-            int w = 0;
-            if (lane == 0) w = atomicAdd(P.mx_counter, 1);
-            w = __shfl_sync(0xffffffffu, w, 0);
-            if (w * 32 >= P.n_mx) break;
-            if (w * 32 + lane < P.n_mx) mx_target<float, ORDER>(P, w * 32 + lane);
+    mx_tail<ORDER>(P);
+}
+
+// Trees with few refined sub-grids, whose time is that of one warp's walk
+// through the stencil: two warps share 32 targets (one parity of one half of a
+// sub-grid), one forming their Taylor coefficients and one their correction,
+// which have no operation in common but the separation's powers.  The walk goes
+// from 158 instructions per entry to 100: nine sub-grids (a three-level tree's
+// step) 149 -> 137 us, against one warp for both.  Same sums in the same order.
+// A CTA is one such pair, an item a sixteenth of a sub-grid.
+constexpr int kSplitParts = 16, kSplitThreads = 64;
+template <int ORDER>
+__global__ void __launch_bounds__(kSplitThreads, 2) mp_split_kernel(KParams P)
+{
+    constexpr int threads = kSplitThreads;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float *W = reinterpret_cast<float *>(smem_raw);
+    float *Cs = W + 8 * P.sub_stride + threadIdx.x;
+    __shared__ int s_nbr[27], s_leaf[27], s_row[27], s_item;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cx = lane & 3, cy = (lane >> 2) & 3;
+    const float *mass = static_cast<const float *>(P.mass);
+    const float *mp = static_cast<const float *>(P.mp);
+    for (;;) {
+        const int item = pull_item(P.counter, &s_item);
+        if (item >= P.n_items) break;
+        const int node = P.list[item / kSplitParts];
+        const int p = (item >> 1) & 7;
+        const float4 *ent = P.stencil_f + p * P.ent_stride;
+        const NodeInfo ti = P.info[node];
+        const int any_leaf = __syncthreads_or(load_slots(node, P, s_nbr, s_leaf, s_row));
+        stage_window_async<float>(W, s_nbr, s_leaf, mass, P, s_row);
+        cp_async_commit();
+        cp_async_wait_all();
+        __syncthreads();
+        const int cz = (lane >> 4) + 2 * (item & 1);
+        const int ax = 2 * cx + (p & 1), ay = 2 * cy + ((p >> 1) & 1), az = 2 * cz + (p >> 2);
+        const int base = cx + P.py * cy + P.pz * cz, cell = ax + 8 * ay + 64 * az;
+        float dA[3], a3A[7];
+        load_target<ORDER>(P, ti.mp_row, parity_index(ax, ay, az), dA, a3A);
+        SmemAcc<16, 4, threads> L;
+        SmemAcc<3, 3, threads> S;
+        L.col = Cs;
+        S.col = Cs + 4 * 2 * threads;
+        L.zero();
+        S.zero();
+        if (warp == 0) {
+            mp_far_ahead<ORDER, 1>(P, W, mp, ent, base, dA, a3A, L, S);
+            if (any_leaf) mp_near<ORDER, 1>(P, W, ent, base, dA, a3A, L, S);
+            store_target(P, node, cell, L);
+        } else {
+            mp_far_ahead<ORDER, 2>(P, W, mp, ent, base, dA, a3A, L, S);
+            if (any_leaf) mp_near<ORDER, 2>(P, W, ent, base, dA, a3A, L, S);
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+                __stcs(P.dL1 + (size_t(node) * 3 + i) * NCELL + cell, acc_value(S, i));
         }
+        __syncthreads();
     }
+    mx_tail<ORDER>(P);
 }
 
 // ---------------------------------------------------------- mpw_kernel
@@ -1350,15 +1434,7 @@ __global__ void __launch_bounds__(kThreads, 2) mp2_kernel(KParams P)
         }
         __syncthreads();
     }
-    if (P.n_mx > 0) {
-        for (;;) {
-            int w = 0;
-            if (lane == 0) w = atomicAdd(P.mx_counter, 1);
-            w = __shfl_sync(0xffffffffu, w, 0);
-            if (w * 32 >= P.n_mx) break;
-            if (w * 32 + lane < P.n_mx) mx_target<float>(P, w * 32 + lane);
-        }
-    }
+    mx_tail<3>(P);
 }
 
 // ---------------------------------------------------------- mono_kernel
@@ -1706,11 +1782,17 @@ struct Kernels {
         static size_t done = 0;
         return allow_smem(mpw_kernel<T, ORDER, PARTS>, bytes, done);
     }
-    template <int ORDER, int WARPS, int PARTS, bool AHEAD>
+    template <int ORDER, int PARTS, bool AHEAD>
     static cudaError_t mp(size_t bytes)
     {
         static size_t done = 0;
-        return allow_smem(mp_kernel<ORDER, WARPS, PARTS, AHEAD>, bytes, done);
+        return allow_smem(mp_kernel<ORDER, PARTS, AHEAD>, bytes, done);
+    }
+    template <int ORDER>
+    static cudaError_t mp_split(size_t bytes)
+    {
+        static size_t done = 0;
+        return allow_smem(mp_split_kernel<ORDER>, bytes, done);
     }
     static cudaError_t mp2(size_t bytes)
     {
@@ -1819,17 +1901,27 @@ cudaError_t launch_mpw(KParams K, size_t bytes, int sms, int cap, cudaStream_t s
     return cudaGetLastError();
 }
 
-// and of the mixed precision: WARPS per CTA; window plus compensation pairs
-template <int ORDER, int WARPS, int PARTS, bool AHEAD>
+// and of the mixed precision; window plus compensation pairs
+template <int ORDER, int PARTS, bool AHEAD>
 cudaError_t launch_mp(KParams K, size_t wbytes, int sms, int cap, cudaStream_t s)
 {
-    const size_t bytes = wbytes + size_t(kMpPairs) * 2 * 32 * WARPS * sizeof(float);
-    cudaError_t e = Kernels<float>::mp<ORDER, WARPS, PARTS, AHEAD>(bytes);
+    const size_t bytes = wbytes + size_t(kMpPairs) * 2 * kThreads * sizeof(float);
+    cudaError_t e = Kernels<float>::mp<ORDER, PARTS, AHEAD>(bytes);
     if (e != cudaSuccess) return e;
     K.n_items *= PARTS;
-    const int g = persistent_grid(mp_kernel<ORDER, WARPS, PARTS, AHEAD>, bytes, K.n_items, sms, cap,
-                                  32 * WARPS);
-    mp_kernel<ORDER, WARPS, PARTS, AHEAD><<<g, 32 * WARPS, bytes, s>>>(K);
+    const int g = persistent_grid(mp_kernel<ORDER, PARTS, AHEAD>, bytes, K.n_items, sms, cap);
+    mp_kernel<ORDER, PARTS, AHEAD><<<g, kThreads, bytes, s>>>(K);
+    return cudaGetLastError();
+}
+template <int ORDER>
+cudaError_t launch_mp_split(KParams K, size_t wbytes, int sms, int cap, cudaStream_t s)
+{
+    const size_t bytes = wbytes + size_t(kMpPairs) * 2 * kSplitThreads * sizeof(float);
+    cudaError_t e = Kernels<float>::mp_split<ORDER>(bytes);
+    if (e != cudaSuccess) return e;
+    K.n_items *= kSplitParts;
+    const int g = persistent_grid(mp_split_kernel<ORDER>, bytes, K.n_items, sms, cap, kSplitThreads);
+    mp_split_kernel<ORDER><<<g, kSplitThreads, bytes, s>>>(K);
     return cudaGetLastError();
 }
 
@@ -1908,19 +2000,20 @@ cudaError_t launch_all(const fmm_tree_s *t, void *L, float *Lc, double *dL1, cud
             const int mode = t->tuning.mp_items;
             const int64_t n = Pl.work_mp.count;
             if constexpr (kF32<T>) {
-                // Few sub-grids: one warp per CTA up to two warps an SM, then
-                // halves with the loads ahead up to two such CTAs an SM.
-                // Else half sub-grids per item where whole ones would leave
-                // CTA slots idle or unbalanced (fewer nodes than twice the
-                // slots).  Same bits throughout.
+                // Few sub-grids: pairs of warps up to two pairs an SM, halves
+                // with the loads ahead up to two such CTAs (73 sub-grids in
+                // quarters of four pairs each: 10 us slower).  Else half
+                // sub-grids per item where whole ones would leave CTA slots
+                // idle or unbalanced (fewer nodes than twice the slots).
+                // Same bits throughout.
                 if (mode == 0 && 16 * n <= 2 * int64_t(sms))
-                    e = launch_mp<ORDER, 1, 16, true>(K, wbytes, sms, cap, s);
+                    e = launch_mp_split<ORDER>(K, wbytes, sms, cap, s);
                 else if (mode == 0 && 2 * n <= 2 * int64_t(sms))
-                    e = launch_mp<ORDER, 8, 2, true>(K, wbytes, sms, cap, s);
+                    e = launch_mp<ORDER, 2, true>(K, wbytes, sms, cap, s);
                 else if (mode == 2 || (mode == 0 && n < 2 * int64_t(cap > 0 && cap < 3 ? cap : 3) * sms))
-                    e = launch_mp<ORDER, 8, 2, false>(K, wbytes, sms, cap, s);
+                    e = launch_mp<ORDER, 2, false>(K, wbytes, sms, cap, s);
                 else
-                    e = launch_mp<ORDER, 8, 1, false>(K, wbytes, sms, cap, s);
+                    e = launch_mp<ORDER, 1, false>(K, wbytes, sms, cap, s);
             } else {
                 // halves and quarters of a sub-grid (mp_items 1 and 2; by
                 // default quarters below eight nodes an SM, so that the last

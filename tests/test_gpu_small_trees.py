@@ -1,5 +1,5 @@
-"""The mixed precision's launch shapes for trees that do not fill the SMs (one
-warp per CTA, halves with the loads ahead, one thread per leaf cell) against
+"""The mixed precision's launch shapes for trees that do not fill the SMs (pairs
+of warps, halves with the loads ahead, one thread per leaf cell) against
 the shapes of large trees, bit for bit, and against the oracle."""
 
 import numpy as np
@@ -26,7 +26,7 @@ def _corner(max_level):
     return adaptive_tree(want, max_level)
 
 
-# refined sub-grids below the root: 8 and 16 (one warp per CTA), 72 (halves
+# refined sub-grids below the root: 8 and 16 (pairs of warps), 72 (halves
 # with the loads ahead); leaf sub-grids: 64 and 120 (a thread per cell), 512
 @pytest.mark.parametrize("tree,theta,order", [("uniform3", 0.5, 3), ("corner4", 0.5, 3),
                                               ("corner4", 0.35, 2), ("corner4", 0.28, 3),
