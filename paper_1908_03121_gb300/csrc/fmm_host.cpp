@@ -262,7 +262,7 @@ static void build_stencils(fmm_tree_s *t)
         if (P.n_far[p] != P.n_far[0] || P.n_near[p] != P.n_near[0]) std::abort();
     int stride = 0;
     for (int p = 0; p < 8; ++p) stride = std::max(stride, int(lists[p].size()));
-    P.ent_stride = (stride + 3) & ~3;
+    P.ent_stride = (stride + 7) & ~7;          // (rows of 16-bit offsets start on 16 bytes)
     t->stencil.assign(size_t(8) * P.ent_stride, StencilEntry{0, 0, 0, 0});
     for (int p = 0; p < 8; ++p)
         for (size_t k = 0; k < lists[p].size(); ++k) t->stencil[size_t(p) * P.ent_stride + k] = lists[p][k];
@@ -277,6 +277,7 @@ static void build_stencils(fmm_tree_s *t)
     // monopole kernel: parity 0's weights, every parity in parity 0's order
     t->coef32.assign(size_t(P.ent_stride) * 4, 0.f);
     t->mono_woff.assign(size_t(8) * P.ent_stride, 0);
+    t->mono_woff16.assign(size_t(8) * P.ent_stride, 0);
     for (size_t k = 0; k < lists[0].size(); ++k) {
         const StencilEntry &e = lists[0][k];
         double c[4];
@@ -290,7 +291,9 @@ static void build_stencils(fmm_tree_s *t)
             if (!in_stencil(pp, o) ||
                 well_separated(theta, o[0], o[1], o[2]) != (int(k) < P.n_far[0]))
                 std::abort();
-            t->mono_woff[size_t(p) * P.ent_stride + k] = entry(pp, o[0], o[1], o[2]).woff;
+            const size_t at = size_t(p) * P.ent_stride + k;
+            t->mono_woff[at] = entry(pp, o[0], o[1], o[2]).woff;
+            t->mono_woff16[at] = uint16_t(sizeof(float) * t->mono_woff[at]);   // 8 * 1584 cells at most
         }
     }
     P.stencil_union = 0;
@@ -635,7 +638,8 @@ static void free_device(fmm_tree_s *t)
         t->scf_host = nullptr;
     }
     DeviceTables &d = t->dev;
-    void *ptrs[] = {d.info, d.children, d.nbr, d.lists, d.stencil, d.stencil_f, d.coef32, d.mono_woff, d.orbits, d.orbit_coef,
+    void *ptrs[] = {d.info, d.children, d.nbr, d.lists, d.stencil, d.stencil_f, d.coef32, d.mono_woff,
+                    d.mono_woff16, d.orbits, d.orbit_coef,
                     d.tree_leaf_off, d.tree_leaf_rows, d.levels, d.levels_df, d.mass, d.mp, d.counters,
                     d.partials, d.chunk_sums, d.reduce_arrived, d.up, d.down, d.mx_targets, d.mx_pairs,
                     d.dflow_items, d.dflow_ready};
@@ -652,7 +656,7 @@ static int upload_tree(fmm_tree_s *t)
         (rc = upload(&d.nbr, t->nbr)) || (rc = upload(&d.lists, t->lists)) ||
         (rc = upload(&d.stencil, t->stencil)) || (rc = upload(&d.stencil_f, t->stencil_f)) ||
         (rc = upload(&d.coef32, t->coef32)) ||
-        (rc = upload(&d.mono_woff, t->mono_woff)) ||
+        (rc = upload(&d.mono_woff, t->mono_woff)) || (rc = upload(&d.mono_woff16, t->mono_woff16)) ||
         (rc = upload(&d.tree_leaf_off, t->tree_leaf_off)) ||
         (rc = upload(&d.tree_leaf_rows, t->tree_leaf_rows)) || (rc = upload(&d.levels, t->levels)) ||
         (rc = upload(&d.levels_df, t->levels_df)) ||

@@ -78,6 +78,7 @@ struct DeviceTables {
     // monopole<-monopole, mixed precision
     float *coef32 = nullptr;         // [ent_stride][4] monopole weights of parity 0
     int32_t *mono_woff = nullptr;    // [8][ent_stride] window offsets, parity 0's order reflected
+    uint16_t *mono_woff16 = nullptr; // the same, in bytes
     // monopole<-monopole, FP64 and double-float (fmm_mono_wide.cuh)
     int4 *orbits = nullptr;          // near parent offsets (dx, dy, dz >= 0, mask of nonzero axes)
     void *orbit_coef = nullptr;      // [orbit][b][q][4] transformed weights: double or float pairs
@@ -172,6 +173,7 @@ struct fmm_tree_s {
     std::vector<float> stencil_f;
     std::vector<float> coef32;
     std::vector<int32_t> mono_woff;
+    std::vector<uint16_t> mono_woff16;
     std::vector<int32_t> orbits;         // [n][4]
     std::vector<double> orbit_coef;      // [orbit][b][q][4]
     int32_t orbit_first[9] = {0};        // the orbits of mask k: orbit_first[k] .. [k + 1]

@@ -79,6 +79,7 @@ struct KParams {
     const float4 *stencil_f;  // the same, offsets as floats, window offset's bits in w
     const float *coef;       // monopole weights of parity 0 (mixed)
     const int32_t *mono_woff;  // [8][ent_stride] window offsets in parity 0's order, reflected
+    const uint16_t *mono_woff16;  // the same, in bytes
     int n_far, n_near;       // identical for every parity
     int ent_stride;          // entries reserved per parity
     const int4 *mx_targets;  // monopole<-multipole targets (node, cell, warp's pair base, count)
@@ -1452,14 +1453,13 @@ __global__ void __launch_bounds__(kThreads, 2) mp2_kernel(KParams P)
 // with its own halo window, staged by cp.async so that every load of the
 // window is in flight at once; every thread holds two target cells (z and
 // z+4 of one parity) per sub-grid, so each weight feeds 2 NB cells.
-// Wb = the window at this thread's first target cell; the NB windows are
-// WSTRIDE apart and the second target cell DZ1 further on (compile-time
+// src = the entry's source of this thread's first target cell; the NB windows
+// are WSTRIDE apart and the second target cell DZ1 further on (compile-time
 // offsets, folded into the shared-memory loads)
 template <int NB, int WSTRIDE, int DZ1>
-__device__ __forceinline__ void mono_entry(const float *Wb, const int *woff, const float *coef, int e,
+__device__ __forceinline__ void mono_entry(const float *src, const float *coef, int e,
                                            Acc<float, 4> (&A)[NB], Acc<float, 4> (&B)[NB])
 {
-    const float *src = Wb + woff[e];
     const float4 c4 = *reinterpret_cast<const float4 *>(coef + 4 * e);
     const float c[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
@@ -1474,14 +1474,24 @@ __device__ __forceinline__ void mono_entry(const float *Wb, const int *woff, con
     }
 }
 
-// dynamic shared memory of mono_kernel<NB, R>: NB windows, the weight table
-// of parity 0 and the window offsets of all parities
-inline size_t mono_smem_bytes(int nb, size_t window_bytes, int ent_stride)
+__device__ __forceinline__ const float *byte_offset(const float *p, unsigned bytes)
 {
-    return nb * window_bytes + size_t(ent_stride) * 4 * sizeof(float) + size_t(8) * ent_stride * sizeof(int);
+    return reinterpret_cast<const float *>(reinterpret_cast<const char *>(p) + bytes);
 }
 
-template <int NB, int RR>
+// dynamic shared memory of mono_kernel<NB, R>: NB windows, the weight table
+// of parity 0 and the window offsets of all parities
+inline size_t mono_smem_bytes(int nb, size_t window_bytes, int ent_stride, bool packed)
+{
+    return nb * window_bytes + size_t(ent_stride) * 4 * sizeof(float) +
+           size_t(8) * ent_stride * (packed ? sizeof(uint16_t) : sizeof(int));
+}
+
+// PACKED: the window offsets stay 16-bit in shared memory and are read eight
+// to a load.  Shared-memory wavefronts bound the loop: five per entry and warp
+// instead of six.  The unpacking costs a little latency per chunk, so only
+// trees with many passes per CTA use it (launch_mono_r).
+template <int NB, int RR, bool PACKED>
 __global__ void __launch_bounds__(kThreads) mono_kernel(KParams P)
 {
     using G = WinGeo<RR>;
@@ -1489,20 +1499,27 @@ __global__ void __launch_bounds__(kThreads) mono_kernel(KParams P)
     constexpr int wstride = 8 * G::SUB_STRIDE;
     float *W = reinterpret_cast<float *>(smem_raw);
     float *s_coef = W + NB * wstride;
-    int *s_woff = reinterpret_cast<int *>(s_coef + 4 * P.ent_stride);
+    using Off = std::conditional_t<PACKED, uint16_t, int>;
+    Off *s_woff = reinterpret_cast<Off *>(s_coef + 4 * P.ent_stride);
     __shared__ int s_nbr[NB][27], s_leaf[NB][27], s_row[NB][27], s_item;
     const int n_ent = P.n_far + P.n_near;
     {
         const float *gcoef = P.coef;                              // parity 0's
         for (int i = threadIdx.x; i < 4 * n_ent; i += blockDim.x) s_coef[i] = __ldg(gcoef + i);
-        for (int i = threadIdx.x; i < 8 * P.ent_stride; i += blockDim.x)
-            s_woff[i] = __ldg(P.mono_woff + i);
+        if constexpr (PACKED) {                        // eight offsets each
+            for (int i = threadIdx.x; i < P.ent_stride; i += blockDim.x)
+                reinterpret_cast<uint4 *>(s_woff)[i] =
+                    __ldg(reinterpret_cast<const uint4 *>(P.mono_woff16) + i);
+        } else {
+            for (int i = threadIdx.x; i < 8 * P.ent_stride; i += blockDim.x)
+                s_woff[i] = __ldg(P.mono_woff + i);
+        }
     }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int p = warp;
     const int px = p & 1, py = (p >> 1) & 1, pz = p >> 2;
     const int cx = lane & 3, cy = (lane >> 2) & 3, cz = lane >> 4;
-    const int *woff = s_woff + p * P.ent_stride;
+    const Off *woff = s_woff + p * P.ent_stride;
     const float *mass = static_cast<const float *>(P.mass);
     const int base0 = cx + G::PY * cy + G::PZ * cz;
     constexpr int dz1 = 2 * G::PZ;              // the second target cell, z + 4
@@ -1535,16 +1552,31 @@ __global__ void __launch_bounds__(kThreads) mono_kernel(KParams P)
         constexpr int chunk = 2 * kChunk;
         int e = 0;
         for (; e + chunk <= n_ent; e += chunk) {
+            if constexpr (PACKED) {
 #pragma unroll
-            for (int j = 0; j < chunk; ++j)
-                mono_entry<NB, wstride, dz1>(W + base0, woff, s_coef, e + j, A, B);
+                for (int j = 0; j < chunk; j += 8) {
+                    const uint4 o = *reinterpret_cast<const uint4 *>(woff + e + j);
+                    const unsigned w[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const unsigned off = i % 2 ? w[i / 2] >> 16 : w[i / 2] & 0xffffu;
+                        mono_entry<NB, wstride, dz1>(byte_offset(W + base0, off), s_coef, e + j + i, A, B);
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < chunk; ++j)
+                    mono_entry<NB, wstride, dz1>(W + base0 + woff[e + j], s_coef, e + j, A, B);
+            }
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
                 A[b].flush();
                 B[b].flush();
             }
         }
-        for (; e < n_ent; ++e) mono_entry<NB, wstride, dz1>(W + base0, woff, s_coef, e, A, B);
+        for (; e < n_ent; ++e)
+            mono_entry<NB, wstride, dz1>(PACKED ? byte_offset(W + base0, woff[e]) : W + base0 + woff[e],
+                                         s_coef, e, A, B);
         const int ax = 2 * cx + px, ay = 2 * cy + py;
         const int cell0 = ax + 8 * ay + 64 * (2 * cz + pz);
         const int cell1 = cell0 + 64 * 4;
@@ -1799,11 +1831,11 @@ struct Kernels {
         static size_t done = 0;
         return allow_smem(mp2_kernel, bytes, done);
     }
-    template <int NB, int RR>
+    template <int NB, int RR, bool PACKED>
     static cudaError_t mono(size_t bytes)
     {
         static size_t done = 0;
-        return allow_smem(mono_kernel<NB, RR>, bytes, done);
+        return allow_smem(mono_kernel<NB, RR, PACKED>, bytes, done);
     }
     template <int PLANES>
     static cudaError_t mono_wide(size_t bytes)
@@ -1827,6 +1859,25 @@ int persistent_grid(Kern k, size_t smem, int64_t items, int sms, int cap_per_sm,
     return int(items < g ? items : g);
 }
 
+template <int NB, int RR, bool PACKED>
+cudaError_t launch_mono_p(const KParams &K, size_t wbytes, int sms, int cap, cudaStream_t s)
+{
+    const size_t bytes = mono_smem_bytes(NB, wbytes, K.ent_stride, PACKED);
+    cudaError_t e = Kernels<float>::mono<NB, RR, PACKED>(bytes);
+    if (e != cudaSuccess) return e;
+    const int64_t passes = (K.n_items + NB - 1) / NB;
+    int g = persistent_grid(mono_kernel<NB, RR, PACKED>, bytes, passes, sms, cap);
+    if (PACKED) g = std::min(g, 5 * sms / 2);
+    mono_kernel<NB, RR, PACKED><<<g, kThreads, bytes, s>>>(K);
+    return cudaGetLastError();
+}
+
+// Packed offsets for pairs of sub-grids and at least eight passes an SM: with
+// 15 passes (4572 leaf sub-grids) the same-level pass takes 818 -> 801 us and
+// a theta = 0.35 step 2238 -> 2177 us, with five (1457) a step 399 -> 408 us.
+// The smaller table lets a third CTA onto an SM at theta = 0.5, but only half
+// of the SMs get one (level-7 tree's step 2439 -> 2413 us): beside three CTAs
+// on each SM the upward pass finds no room (2461 us).
 template <int NB, int RR>
 cudaError_t launch_mono_r(const KParams &K, size_t wbytes, int sms, int cap, cudaStream_t s)
 {
@@ -1834,13 +1885,9 @@ cudaError_t launch_mono_r(const KParams &K, size_t wbytes, int sms, int cap, cud
     using G = WinGeo<RR>;
     if (K.reach != G::R || K.py != G::PY || K.pz != G::PZ || K.sub_stride != G::SUB_STRIDE)
         return cudaErrorInvalidValue;
-    const size_t bytes = mono_smem_bytes(NB, wbytes, K.ent_stride);
-    cudaError_t e = Kernels<float>::mono<NB, RR>(bytes);
-    if (e != cudaSuccess) return e;
-    const int64_t passes = (K.n_items + NB - 1) / NB;
-    const int g = persistent_grid(mono_kernel<NB, RR>, bytes, passes, sms, cap);
-    mono_kernel<NB, RR><<<g, kThreads, bytes, s>>>(K);
-    return cudaGetLastError();
+    if constexpr (NB == 2)
+        if (K.n_items >= 8 * int64_t(sms) * NB) return launch_mono_p<NB, RR, true>(K, wbytes, sms, cap, s);
+    return launch_mono_p<NB, RR, false>(K, wbytes, sms, cap, s);
 }
 
 // theta in (0.25, 1/sqrt(3)] gives reach 2 floor(1/theta) + 1 = 3, 5 or 7
@@ -1954,6 +2001,7 @@ cudaError_t launch_all(const fmm_tree_s *t, void *L, float *Lc, double *dL1, cud
     P.mx_targets = d.mx_targets;
     P.mx_pairs = d.mx_pairs;
     P.mono_woff = d.mono_woff;
+    P.mono_woff16 = d.mono_woff16;
     const int cap = t->tuning.ctas_per_sm;
     const size_t wbytes = size_t(8) * Pl.sub_stride * sizeof(T);
     cudaError_t e;
@@ -2044,7 +2092,7 @@ cudaError_t launch_all(const fmm_tree_s *t, void *L, float *Lc, double *dL1, cud
             if (nb != 1 && nb != 2 && nb != 4) nb = 2;
             // fewer sub-grids per pass where their windows do not fit
             const size_t smem_max = max_smem_optin_of_current_device();
-            while (nb > 1 && mono_smem_bytes(nb, wbytes, Pl.ent_stride) > smem_max) nb /= 2;
+            while (nb > 1 && mono_smem_bytes(nb, wbytes, Pl.ent_stride, false) > smem_max) nb /= 2;
             e = nb == 1 ? launch_mono<1>(K, wbytes, sms, cap, s)
                 : nb == 2 ? launch_mono<2>(K, wbytes, sms, cap, s)
                           : launch_mono<4>(K, wbytes, sms, cap, s);
