@@ -238,6 +238,9 @@ int fmm_upward(fmm_tree_t tree, const double *rho, double *M, double *com,
  * double, contracts in float with two-sum compensated accumulation, and
  * finishes the correction in double; FMM_DFLOAT evaluates every step (offsets,
  * derivative tensors, contraction, sums) in double-float.
+ * The roots run beside the other kernels on the tree's second stream, which
+ * forks from and joins back into `stream` through events (not with
+ * FMM_FLAG_TIMING), so the call can be captured as part of a graph.
  * Errors: FMM_ERR_INVALID_ARG (NULL tree or buffer, L_comp NULL in FMM_MIXED
  * or FMM_DFLOAT, a FMM_FLAG_HOST_ONLY tree), FMM_ERR_CUDA (a launch failed).
  */
@@ -311,7 +314,9 @@ typedef struct {
                                         items to balance a tree with few refined
                                         nodes, the halo staged twice); 0 = 2 when the
                                         tree has fewer refined nodes than twice the
-                                        kernel's resident CTAs, else 1.  FMM_FP64 and
+                                        kernel's resident CTAs (and shapes of their own
+                                        where even halves would not fill the SMs),
+                                        else 1.  FMM_FP64 and
                                         FMM_DFLOAT take half of that: 1 a half, 2 a
                                         quarter, 0 = 2 below eight refined nodes per SM.
                                         Same results. */

@@ -5,10 +5,10 @@ so co-resident kernels share SMs as they will in the real step) on the
 caller's tree for every candidate of
 ``fmm_tuning`` (sub-grids per pass of the monopole kernel, persistent CTAs per
 SM, the dataflow downward pass or the level-by-level one, one or two multipole
-target cells per thread in flight, whole or half sub-grids per multipole work
-item), each captured as a CUDA graph and replayed, with CUDA events on the
-current stream; keeps the fastest and leaves it set on the tree.  Each
-candidate is replayed ``reps`` times after one warm-up; the four fastest are
+target cells per thread in flight, the multipole work items the library picks
+by the tree's size, whole or half sub-grids), each captured as a CUDA graph and
+replayed, with CUDA events on the current stream; keeps the fastest and leaves
+it set on the tree.  Each candidate is replayed ``reps`` times after one warm-up; the four fastest are
 then timed again, round-robin, with about 100 ms of steps each, and the
 median decides.  Results are cached per tree size and precision for the
 process.
@@ -24,7 +24,7 @@ MONO_SUBGRIDS = (1, 2, 4)
 CTAS_PER_SM = (0, 1, 2)
 DATAFLOW = (0, 1)
 PAIR_TARGETS = (0, 1)
-MP_ITEMS = (1, 2)
+MP_ITEMS = (0, 1, 2)      # 0: by the tree's size
 _CACHE = {}
 
 

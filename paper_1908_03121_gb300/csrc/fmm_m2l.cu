@@ -12,12 +12,16 @@
 // multipole<-monopole:
 //   mp_kernel    refined targets: multipole<-multipole (well-separated
 //                sources) and multipole<-monopole (all candidate leaf
-//                sources) -- the "455 flop" kernel of Sec. 4.3;
+//                sources) -- the "455 flop" kernel of Sec. 4.3; in the mixed
+//                precision also mp_split_kernel (trees with few sub-grids)
+//                and mp2_kernel (two targets per thread, a tuning), in the
+//                wide element types mpw_kernel (fmm_wide.cuh's algebra);
 //   mono_kernel  leaf targets, leaf sources: monopole<-monopole, a 1-in,
-//                4-out convolution whose per-offset weights are tabulated;
+//                4-out convolution whose per-offset weights are tabulated
+//                (wide types: mono_wide_kernel in fmm_mono_wide.cuh);
 //   mx_kernel    leaf targets next to refined nodes: monopole<-multipole;
 //   root_kernel  the single node of level 1 of each tree (all pairs are
-//                candidates there).
+//                candidates there); wide types: rootw_kernel.
 // Design (GB300-first, unlike the paper's 8x64-thread launches per node fed
 // from 128 streams): persistent CTAs pull whole sub-grids from cost-sorted
 // work queues; a warp holds 32 targets of one child parity so the stencil
@@ -32,10 +36,12 @@
 // (packed as offsets from the cell centre, in cell widths), the contraction
 // runs in float with per-chunk sums folded into (hi, lo) pairs by TwoSum, and
 // the correction's compensated sum is stored and carried down in double.
-// Conserving precision: the same kernels instantiated on dfloat (pairs of
-// floats, fmm_dfloat.cuh) evaluate offsets, derivative tensors, contraction
-// and sums in double-float, so each pair's contributions to A and to B cancel
-// in momentum and angular momentum to about 1e-13, as in FP64.
+// Wide element types (double, and dfloat: pairs of floats, fmm_dfloat.cuh, the
+// conserving precision): both are bound by their arithmetic pipe, so their
+// kernels are written for the fewest operations (fmm_wide.cuh); dfloat
+// evaluates offsets, contraction and sums in double-float, so each pair's
+// contributions to A and to B cancel in momentum and angular momentum to about
+// 1e-13, as in FP64.
 #include <algorithm>
 #include <cstdio>
 #include <type_traits>
@@ -761,7 +767,7 @@ template <int ORDER = 3>
 __device__ __forceinline__ void acc_mx(float Rx, float Ry, float Rz, const Src<float> &s,
                                        Acc<float, 4> &L, Acc<float, 3> &S)
 {
-    DTraceless D;
+    DTraceless D{};
     D.eval<ORDER == 3>(Rx, Ry, Rz);
     float a = -s.m0 * D.D0;
 #pragma unroll

@@ -38,7 +38,6 @@ namespace fmm {
 
 namespace {
 
-
 struct MonoWParams {
     const NodeInfo *info;
     const int32_t *nbr;
