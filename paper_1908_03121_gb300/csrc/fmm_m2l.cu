@@ -254,6 +254,16 @@ __device__ __forceinline__ void cp_async_elem(T *dst, const T *src, bool valid)
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+// all but the newest N groups
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+// 16 bytes, zeros if not valid
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool valid)
+{
+    const unsigned d = unsigned(__cvta_generic_to_shared(dst));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(valid ? 16 : 0)
+                 : "memory");
+}
 
 // With s_row given (the multipole-target kernel), a refined source's cell
 // holds instead the offset of its packed moments (row and parity index),
@@ -621,17 +631,22 @@ __device__ __forceinline__ void load4(const T *p, T v[4])
     }
 }
 
-__device__ __forceinline__ void load_source_at(const float *base, Src<float> &s)
+__device__ __forceinline__ void unpack_source(const float (&v)[16], Src<float> &s)
 {
-    float v[16];
-#pragma unroll
-    for (int g = 0; g < 4; ++g) load4<float>(base + size_t(g) * NCELL * 4, v + 4 * g);
     s.d[0] = v[0]; s.d[1] = v[1]; s.d[2] = v[2];
     s.m0 = v[3];
 #pragma unroll
     for (int k = 0; k < 5; ++k) s.B2[k] = v[4 + k];
 #pragma unroll
     for (int q = 0; q < 7; ++q) s.B3[q] = v[9 + q];
+}
+
+__device__ __forceinline__ void load_source_at(const float *base, Src<float> &s)
+{
+    float v[16];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) load4<float>(base + size_t(g) * NCELL * 4, v + 4 * g);
+    unpack_source(v, s);
 }
 
 // the same for the wide types; base also names the zero row of leaf sources
@@ -926,7 +941,7 @@ __device__ __forceinline__ void mx_target(const KParams &P, int t)
 // the one after (which says where its moments are) and the window offset of
 // the one after that, so a warp waits for none of the three dependent loads;
 // leaf lanes load the zero row.
-template <int ORDER, int WHAT, int THREADS>
+template <int ORDER, int THREADS>
 __device__ __forceinline__ void mp_far_ahead(const KParams &P, const float *W, const float *mp,
                                              const float4 *ent, int base, const float dA[3],
                                              const float a3A[7], SmemAcc<16, 4, THREADS> &L,
@@ -954,10 +969,10 @@ __device__ __forceinline__ void mp_far_ahead(const KParams &P, const float *W, c
                 if (!is_mp) src.m0 = wv;
                 float R[3];
                 separation(dA, src.d, E, R);
-                acc_mp<true, ORDER, WHAT>(R[0], R[1], R[2], src, a3A, L, S);
+                acc_mp<true, ORDER>(R[0], R[1], R[2], src, a3A, L, S);
             } else if (__any_sync(0xffffffffu, window_nonzero<float>(wv))) {
                 src.m0 = wv;
-                acc_mp<false, ORDER, WHAT>(dA[0] - E.x, dA[1] - E.y, dA[2] - E.z, src, a3A, L, S);
+                acc_mp<false, ORDER>(dA[0] - E.x, dA[1] - E.y, dA[2] - E.z, src, a3A, L, S);
             }
             src = src1;
             is_mp = is_mp1;
@@ -965,9 +980,85 @@ __device__ __forceinline__ void mp_far_ahead(const KParams &P, const float *W, c
             wv1 = wv2;
             E = E1;
         }
+        L.flush();
+        S.flush();
+    }
+}
+
+// The far loop where so few warps share an SM that neither the moment loads nor
+// the arithmetic's latency is hidden by other warps: the moments of the next
+// DEPTH - 2 entries are in flight to a ring in shared memory (cp.async, zeros for
+// leaf lanes; each lane copies and reads its own 64 bytes per entry, so no
+// barrier is needed), and two entries are evaluated side by side, their terms
+// added in order (an absent source's terms are exact zeros).
+// ring: DEPTH entries of four 16-byte groups, 32 lanes apart, from this lane's
+template <int ORDER, int WHAT, int DEPTH, int THREADS>
+__device__ __forceinline__ void mp_far_staged(const KParams &P, const float *W, const float *mp,
+                                              const float4 *ent, int base, const float dA[3],
+                                              const float a3A[7], float4 *ring,
+                                              SmemAcc<16, 4, THREADS> &L, SmemAcc<3, 3, THREADS> &S)
+{
+    static_assert(DEPTH % 2 == 0 && DEPTH >= 4 && kChunk % 2 == 0, "pairs");
+    const int last = P.n_far - 1;
+    // window value of entry i (0, an absent source, past the last)
+    auto value = [&](int i, float w) { return i <= last ? W[base + __float_as_int(w)] : 0.f; };
+    auto issue = [&](int i, float w) {
+        int idx;
+        const bool is_mp = window_moments<float>(value(i, w), P.mp_limit, idx);
+        const float *src = mp + (is_mp ? idx : P.mp_limit);
+        float4 *slot = ring + (i % DEPTH) * 128;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) cp_async16(slot + 32 * g, src + size_t(g) * NCELL * 4, is_mp);
+    };
+    for (int i = 0; i < DEPTH - 2; i += 2) {
+        issue(i, __ldg(&ent[min(i, last)].w));
+        issue(i + 1, __ldg(&ent[min(i + 1, last)].w));
+        cp_async_commit();
+    }
+    float4 E[2] = {__ldg(ent), __ldg(ent + min(1, last))};
+    float off[2] = {__ldg(&ent[min(DEPTH - 2, last)].w), __ldg(&ent[min(DEPTH - 1, last)].w)};
+    for (int e0 = 0; e0 < P.n_far; e0 += kChunk) {
+        const int e1 = min(e0 + kChunk, P.n_far);
+        for (int e = e0; e < e1; e += 2) {
+            cp_async_wait<DEPTH / 2 - 2>();
+            Src<float> src[2];
+            float R[2][3];
+            bool some = false;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const float wv = value(e + k, E[k].w);
+                int idx;
+                const bool is_mp = window_moments<float>(wv, P.mp_limit, idx);
+                const float4 *slot = ring + ((e + k) % DEPTH) * 128;
+                float v[16];
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    const float4 q = slot[32 * g];
+                    v[4 * g] = q.x; v[4 * g + 1] = q.y; v[4 * g + 2] = q.z; v[4 * g + 3] = q.w;
+                }
+                unpack_source(v, src[k]);
+                if (!is_mp) src[k].m0 = wv;
+                some = some || is_mp || window_nonzero<float>(wv);
+                separation(dA, src[k].d, E[k], R[k]);
+            }
+            // (into the slots of the pair before, whose values have been used)
+            issue(e + DEPTH - 2, off[0]);
+            issue(e + DEPTH - 1, off[1]);
+            cp_async_commit();
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                off[k] = __ldg(&ent[min(e + DEPTH + k, last)].w);
+                E[k] = __ldg(ent + min(e + 2 + k, last));
+            }
+            if (!__any_sync(0xffffffffu, some)) continue;
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                acc_mp<true, ORDER, WHAT>(R[k][0], R[k][1], R[k][2], src[k], a3A, L, S);
+        }
         if (WHAT & 1) L.flush();
         if (WHAT & 2) S.flush();
     }
+    cp_async_wait_all();
 }
 
 // Near sources: leaf cells only (refined ones contribute nothing here: their
@@ -1012,15 +1103,17 @@ __device__ __forceinline__ void mx_tail(const KParams &P)
 }
 
 // PARTS 1: an item is a sub-grid, a warp each parity, both halves (z < 4, z >=
-// 4); 2: one half of a sub-grid.
+// 4); 2: one half of a sub-grid; 4, WARPS 4: one half of four parities.
 // Three CTAs of eight warps per SM (at most 85 registers): the compensation
 // pairs, touched once per chunk, live in shared memory after the window.
-// AHEAD (mp_far_ahead) takes 112 registers and two such CTAs per SM: worth it
-// only where the items do not fill the SMs anyway.
-template <int ORDER, int PARTS, bool AHEAD>
-__global__ void __launch_bounds__(kThreads, AHEAD ? 2 : 3) mp_kernel(KParams P)
+// AHEAD (mp_far_ahead) takes 112 registers and two such CTAs per SM, WARPS 4
+// mp_far_staged: worth it only where the items do not fill the SMs anyway.
+constexpr int kMpDepth = 4;      // entries of the ring of WARPS 4
+template <int ORDER, int PARTS, bool AHEAD, int WARPS = 8>
+__global__ void __launch_bounds__(32 * WARPS, AHEAD || WARPS == 4 ? 2 : 3) mp_kernel(KParams P)
 {
-    constexpr int threads = kThreads;
+    static_assert(WARPS == 8 ? PARTS <= 2 : WARPS == 4 && PARTS == 4, "items per sub-grid");
+    constexpr int threads = 32 * WARPS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float *W = reinterpret_cast<float *>(smem_raw);
     float *Cs = W + 8 * P.sub_stride + threadIdx.x;
@@ -1033,7 +1126,7 @@ __global__ void __launch_bounds__(kThreads, AHEAD ? 2 : 3) mp_kernel(KParams P)
         const int item = pull_item(P.counter, &s_item);
         if (item >= P.n_items) break;
         const int node = P.list[item / PARTS];
-        const int p = warp;
+        const int p = WARPS == 8 ? warp : 4 * ((item >> 1) & 1) + warp;
         const int px = p & 1, py = (p >> 1) & 1, pz = p >> 2;
         const float4 *ent = P.stencil_f + p * P.ent_stride;   // float offsets: no conversions
         const NodeInfo ti = P.info[node];
@@ -1064,8 +1157,12 @@ __global__ void __launch_bounds__(kThreads, AHEAD ? 2 : 3) mp_kernel(KParams P)
             // moments' terms, so the same values), a mix the general form
             // with zero moments for the leaves, and an entry with only
             // absent sources (mass 0) is skipped.
-            if constexpr (AHEAD) {
-                mp_far_ahead<ORDER, 3>(P, W, mp, ent, base, dA, a3A, L, S);
+            if constexpr (WARPS == 4) {
+                float4 *ring = reinterpret_cast<float4 *>(W + 8 * P.sub_stride + 2 * kMpPairs * threads) +
+                               warp * kMpDepth * 128 + lane;
+                mp_far_staged<ORDER, 3, kMpDepth>(P, W, mp, ent, base, dA, a3A, ring, L, S);
+            } else if constexpr (AHEAD) {
+                mp_far_ahead<ORDER>(P, W, mp, ent, base, dA, a3A, L, S);
             } else {
                 for (int e0 = 0; e0 < P.n_far; e0 += kChunk) {
                     const int e1 = min(e0 + kChunk, P.n_far);
@@ -1119,10 +1216,11 @@ __global__ void __launch_bounds__(kThreads, AHEAD ? 2 : 3) mp_kernel(KParams P)
 // through the stencil: two warps share 32 targets (one parity of one half of a
 // sub-grid), one forming their Taylor coefficients and one their correction,
 // which have no operation in common but the separation's powers.  The walk goes
-// from 158 instructions per entry to 100: nine sub-grids (a three-level tree's
-// step) 149 -> 137 us, against one warp for both.  Same sums in the same order.
+// from 158 instructions per entry to 100: eight sub-grids below the root (a
+// three-level tree's step) 149 -> 137 us, against one warp for both, and
+// 137 -> 115 us with mp_far_staged.  Same sums in the same order.
 // A CTA is one such pair, an item a sixteenth of a sub-grid.
-constexpr int kSplitParts = 16, kSplitThreads = 64;
+constexpr int kSplitParts = 16, kSplitThreads = 64, kSplitDepth = 8;
 template <int ORDER>
 __global__ void __launch_bounds__(kSplitThreads, 2) mp_split_kernel(KParams P)
 {
@@ -1132,6 +1230,8 @@ __global__ void __launch_bounds__(kSplitThreads, 2) mp_split_kernel(KParams P)
     float *Cs = W + 8 * P.sub_stride + threadIdx.x;
     __shared__ int s_nbr[27], s_leaf[27], s_row[27], s_item;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float4 *ring = reinterpret_cast<float4 *>(W + 8 * P.sub_stride + 2 * kMpPairs * threads) +
+                   warp * kSplitDepth * 128 + lane;
     const int cx = lane & 3, cy = (lane >> 2) & 3;
     const float *mass = static_cast<const float *>(P.mass);
     const float *mp = static_cast<const float *>(P.mp);
@@ -1159,11 +1259,11 @@ __global__ void __launch_bounds__(kSplitThreads, 2) mp_split_kernel(KParams P)
         L.zero();
         S.zero();
         if (warp == 0) {
-            mp_far_ahead<ORDER, 1>(P, W, mp, ent, base, dA, a3A, L, S);
+            mp_far_staged<ORDER, 1, kSplitDepth>(P, W, mp, ent, base, dA, a3A, ring, L, S);
             if (any_leaf) mp_near<ORDER, 1>(P, W, ent, base, dA, a3A, L, S);
             store_target(P, node, cell, L);
         } else {
-            mp_far_ahead<ORDER, 2>(P, W, mp, ent, base, dA, a3A, L, S);
+            mp_far_staged<ORDER, 2, kSplitDepth>(P, W, mp, ent, base, dA, a3A, ring, L, S);
             if (any_leaf) mp_near<ORDER, 2>(P, W, ent, base, dA, a3A, L, S);
 #pragma unroll
             for (int i = 0; i < 3; ++i)
@@ -1820,11 +1920,11 @@ struct Kernels {
         static size_t done = 0;
         return allow_smem(mpw_kernel<T, ORDER, PARTS>, bytes, done);
     }
-    template <int ORDER, int PARTS, bool AHEAD>
+    template <int ORDER, int PARTS, bool AHEAD, int WARPS>
     static cudaError_t mp(size_t bytes)
     {
         static size_t done = 0;
-        return allow_smem(mp_kernel<ORDER, PARTS, AHEAD>, bytes, done);
+        return allow_smem(mp_kernel<ORDER, PARTS, AHEAD, WARPS>, bytes, done);
     }
     template <int ORDER>
     static cudaError_t mp_split(size_t bytes)
@@ -1954,22 +2054,25 @@ cudaError_t launch_mpw(KParams K, size_t bytes, int sms, int cap, cudaStream_t s
     return cudaGetLastError();
 }
 
-// and of the mixed precision; window plus compensation pairs
-template <int ORDER, int PARTS, bool AHEAD>
+// and of the mixed precision; window, compensation pairs and ring
+template <int ORDER, int PARTS, bool AHEAD, int WARPS = 8>
 cudaError_t launch_mp(KParams K, size_t wbytes, int sms, int cap, cudaStream_t s)
 {
-    const size_t bytes = wbytes + size_t(kMpPairs) * 2 * kThreads * sizeof(float);
-    cudaError_t e = Kernels<float>::mp<ORDER, PARTS, AHEAD>(bytes);
+    constexpr int threads = 32 * WARPS;
+    const size_t bytes = wbytes + size_t(kMpPairs) * 2 * threads * sizeof(float) +
+                         size_t(threads) * (WARPS == 4 ? kMpDepth : 0) * 64;
+    cudaError_t e = Kernels<float>::mp<ORDER, PARTS, AHEAD, WARPS>(bytes);
     if (e != cudaSuccess) return e;
     K.n_items *= PARTS;
-    const int g = persistent_grid(mp_kernel<ORDER, PARTS, AHEAD>, bytes, K.n_items, sms, cap);
-    mp_kernel<ORDER, PARTS, AHEAD><<<g, kThreads, bytes, s>>>(K);
+    const int g = persistent_grid(mp_kernel<ORDER, PARTS, AHEAD, WARPS>, bytes, K.n_items, sms, cap, threads);
+    mp_kernel<ORDER, PARTS, AHEAD, WARPS><<<g, threads, bytes, s>>>(K);
     return cudaGetLastError();
 }
 template <int ORDER>
 cudaError_t launch_mp_split(KParams K, size_t wbytes, int sms, int cap, cudaStream_t s)
 {
-    const size_t bytes = wbytes + size_t(kMpPairs) * 2 * kSplitThreads * sizeof(float);
+    const size_t bytes = wbytes + size_t(kMpPairs) * 2 * kSplitThreads * sizeof(float) +
+                         size_t(kSplitThreads) * kSplitDepth * 64;
     cudaError_t e = Kernels<float>::mp_split<ORDER>(bytes);
     if (e != cudaSuccess) return e;
     K.n_items *= kSplitParts;
@@ -2054,14 +2157,19 @@ cudaError_t launch_all(const fmm_tree_s *t, void *L, float *Lc, double *dL1, cud
             const int mode = t->tuning.mp_items;
             const int64_t n = Pl.work_mp.count;
             if constexpr (kF32<T>) {
-                // Few sub-grids: pairs of warps up to two pairs an SM, halves
-                // with the loads ahead up to two such CTAs (73 sub-grids in
-                // quarters of four pairs each: 10 us slower).  Else half
-                // sub-grids per item where whole ones would leave CTA slots
-                // idle or unbalanced (fewer nodes than twice the slots).
-                // Same bits throughout.
-                if (mode == 0 && 16 * n <= 2 * int64_t(sms))
+                // Few sub-grids, whose time is that of one warp's walk: pairs of
+                // warps up to three pairs an SM, quarters of a sub-grid up to
+                // two four-warp CTAs an SM, halves with the loads ahead up to
+                // two such CTAs.  Steps of binaries, us, halves with the
+                // loads ahead / this: 21 sub-grids 184 / 160, 41 204 / 177,
+                // 72 272 / 257; above 76 quarters take two rounds (113:
+                // 323 / 347).  Else half sub-grids per item where
+                // whole ones would leave CTA slots idle or unbalanced (fewer
+                // nodes than twice the slots).  Same bits throughout.
+                if (mode == 0 && 16 * n <= 3 * int64_t(sms))
                     e = launch_mp_split<ORDER>(K, wbytes, sms, cap, s);
+                else if (mode == 0 && 4 * n <= 2 * int64_t(sms))
+                    e = launch_mp<ORDER, 4, false, 4>(K, wbytes, sms, cap, s);
                 else if (mode == 0 && 2 * n <= 2 * int64_t(sms))
                     e = launch_mp<ORDER, 2, true>(K, wbytes, sms, cap, s);
                 else if (mode == 2 || (mode == 0 && n < 2 * int64_t(cap > 0 && cap < 3 ? cap : 3) * sms))

@@ -1,5 +1,5 @@
 """The mixed precision's launch shapes for trees that do not fill the SMs (pairs
-of warps, halves with the loads ahead, one thread per leaf cell) against
+of warps, quarters, halves with the loads ahead, one thread per leaf cell) against
 the shapes of large trees, bit for bit, and against the oracle."""
 
 import numpy as np
@@ -17,23 +17,27 @@ pytestmark = pytest.mark.gpu
 FORCE_TOL = 1e-6                 # the mixed precision's bar
 
 
-def _corner(max_level):
+def _corner(max_level, radius=0.1):
     c = np.array([0.2, 0.25, 0.3])
 
     def want(lo, hi):
         d = np.clip(c, lo, hi) - c
-        return float(d @ d) < 0.1 ** 2
+        return float(d @ d) < radius ** 2
     return adaptive_tree(want, max_level)
 
 
-# refined sub-grids below the root: 8 and 16 (pairs of warps), 72 (halves
-# with the loads ahead); leaf sub-grids: 64 and 120 (a thread per cell), 512
+# refined sub-grids below the root: 8 and 16 (pairs of warps), 44 and 72
+# (quarters, four warps), 80 (halves with the loads ahead); leaf sub-grids: 64,
+# 120 (a thread per cell), 316, 512 and 568
 @pytest.mark.parametrize("tree,theta,order", [("uniform3", 0.5, 3), ("corner4", 0.5, 3),
                                               ("corner4", 0.35, 2), ("corner4", 0.28, 3),
-                                              ("corner4", 0.57, 3), ("uniform4", 0.5, 3)])
+                                              ("corner4", 0.57, 3), ("uniform4", 0.5, 3),
+                                              ("corner5", 0.5, 2), ("corner5", 0.28, 3),
+                                              ("corner5", 0.57, 3), ("wide5", 0.5, 3)])
 def test_launch_shapes_agree(tree, theta, order):
     desc = {"uniform3": lambda: uniform_tree(3), "uniform4": lambda: uniform_tree(4),
-            "corner4": lambda: _corner(4)}[tree]()
+            "corner4": lambda: _corner(4), "corner5": lambda: _corner(5, 0.13),
+            "wide5": lambda: _corner(5, 0.2)}[tree]()
     rng = np.random.default_rng(3)
     rho = gaussian_blobs(leaf_cell_centres(desc), rng.uniform(0.2, 0.5, (2, 3)), 0.06, 1.0).reshape(-1, 512)
     c = dict(desc=desc, theta=theta, G=1.0, box_lo=(0.0, 0.0, 0.0), box_size=1.0, order=order)
