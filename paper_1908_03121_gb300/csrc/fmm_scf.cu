@@ -15,31 +15,35 @@
 // two to finish combines the nodes' values in a fixed order and writes them
 // into page-locked host memory (with the potential at the three surface
 // cells), from which the host forms the few scalars of the iteration in FP64.
-// (An update of 512 leaf nodes, with its solve: 355 -> 293 us against copies of every
-// node's partial sums through pageable memory and full shuffle trees of FP64
-// adds per node.)
+// An update of 512 leaf nodes, with its solve: 355 -> 293 us against copies of
+// every node's partial sums through pageable memory and full shuffle trees of
+// FP64 adds per node.  FP64 operations bound the three kernels, so nodes that
+// neither star reaches are sorted out in float, a thread's two cells share what
+// x and y set, and the mass sums are taken in cell indices: 273 -> 257 us.
 #include <cmath>
 #include <string>
 
+#include "fmm_convert.cuh"
 #include "fmm_internal.h"
 
 namespace fmm {
 namespace {
 
-constexpr int kScfThreads = 256;       // 2 cells per thread
+constexpr int kScfThreads = 256;       // 2 cells per thread, four planes apart
+static_assert(NCELL == 2 * kScfThreads, "two cells per thread");
 
 struct ScfGeo {
     double lo[3];
     double size;
 };
 
-__device__ __forceinline__ void cell_centre(const NodeInfo &ni, const double *levels, const ScfGeo &g,
-                                            int c, double x[3])
+// a small whole number as a double, on the integer pipe
+__device__ __forceinline__ double whole(int i) { return f2d_bits(float(i)); }
+
+// centre of a cell along one axis: node index i, cell index k
+__device__ __forceinline__ double centre_of(double lo, int i, int k, double h)
 {
-    const double h = levels[ni.level * LEVEL_FIELDS + LV_H];
-    x[0] = g.lo[0] + (8.0 * ni.ix + (c & 7) + 0.5) * h;
-    x[1] = g.lo[1] + (8.0 * ni.iy + ((c >> 3) & 7) + 0.5) * h;
-    x[2] = g.lo[2] + (8.0 * ni.iz + (c >> 6) + 0.5) * h;
+    return lo + (8.0 * i + whole(k) + 0.5) * h;
 }
 
 // fixed-order sum or maximum of every component k of the 256 threads' v[k]; the
@@ -118,18 +122,26 @@ __global__ void __launch_bounds__(kScfThreads) scf_com_kernel(const NodeInfo *__
                                                                int32_t *__restrict__ arrived, ScfGeo g,
                                                                ScfPoints points, double *host)
 {
+    // density sums in cell indices; the node's scale and corner at the end
     const NodeInfo ni = info[leaves[blockIdx.x]];
-    const double h3 = levels[ni.level * LEVEL_FIELDS + LV_H3];
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int c = threadIdx.x; c < NCELL; c += kScfThreads) {
-        double x[3];
-        cell_centre(ni, levels, g, c, x);
-        const double m = rho[size_t(ni.leaf_row) * NCELL + c] * h3;
-        v[0] += m;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) v[1 + a] = fma(m, x[a], v[1 + a]);
+    const double *r = rho + size_t(ni.leaf_row) * NCELL + threadIdx.x;
+    const double r0 = r[0], r1 = r[kScfThreads], both = r0 + r1;
+    const int c = threadIdx.x;
+    const double v[4] = {both, both * whole(c & 7), both * whole((c >> 3) & 7),
+                         fma(r0, whole(c >> 6), r1 * whole((c >> 6) + 4))};
+    double mine = block_combine<4, false>(v);
+    if (threadIdx.x < 32) {
+        const double sum = __shfl_sync(0xffffffffu, mine, 0);
+        const double h = levels[ni.level * LEVEL_FIELDS + LV_H], h3 = levels[ni.level * LEVEL_FIELDS + LV_H3];
+        if (threadIdx.x > 0 && threadIdx.x < 4) {
+            const int a = threadIdx.x;
+            const double corner = a == 1   ? centre_of(g.lo[0], ni.ix, 0, h)
+                                  : a == 2 ? centre_of(g.lo[1], ni.iy, 0, h)
+                                           : centre_of(g.lo[2], ni.iz, 0, h);
+            mine = fma(corner, sum, h * mine);
+        }
+        mine *= h3;
     }
-    const double mine = block_combine<4, false>(v);
     double all;
     if (!combine_nodes<4, false>(mine, ni.leaf_row, partials, arrived, all)) return;
     if (threadIdx.x < 4) host[threadIdx.x] = all;
@@ -143,24 +155,62 @@ struct ScfStars {
     double omega2, C[2], com[2], x_split;
     double centre[2][3], r2lim[2];
     int live[2];                         // star i exists (rho_max > 0)
+    float box_centre[2][3], box_reach[2];  // in box widths; the reach rounded up
 };
 
-// the star a cell belongs to (0, 1) or -1, and its enthalpy
-__device__ __forceinline__ int star_of(const double x[3], const ScfStars &s)
+// whether any cell of the node can lie within a star's reach: the distance from
+// the star's centre to the box of the node's cell centres, in float, against
+// the reach with a margin far above float's rounding.  Most nodes lie in
+// neither star and take none of the FP64 operations per cell, which bound both
+// kernels
+__device__ __forceinline__ bool near_star(const NodeInfo &ni, const ScfStars &s)
 {
-    const int i = x[0] < s.x_split ? 0 : 1;
-    if (!s.live[i]) return -1;
-    double d2 = 0.0;
+    const int at[3] = {ni.ix, ni.iy, ni.iz};
+    const float w = exp2f(float(1 - ni.level));
+    bool near = false;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) d2 = fma(x[a] - s.centre[i][a], x[a] - s.centre[i][a], d2);
-    return d2 < s.r2lim[i] ? i : -1;
+    for (int i = 0; i < 2; ++i) {
+        float d2 = 0.f;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const float lo = (float(at[a]) + 0.0625f) * w, hi = (float(at[a]) + 0.9375f) * w;
+            const float d = fmaxf(fmaxf(lo - s.box_centre[i][a], s.box_centre[i][a] - hi), 0.f);
+            d2 = fmaf(d, d, d2);
+        }
+        near = near || (s.live[i] && !(d2 > s.box_reach[i] * s.box_reach[i]));
+    }
+    return near;
 }
 
-__device__ __forceinline__ double enthalpy(const double x[3], double phi, int star, const ScfStars &s)
-{
-    const double wx = x[0] - s.com[0], wy = x[1] - s.com[1];
-    return s.C[star] - phi + 0.5 * s.omega2 * fma(wx, wx, wy * wy);
-}
+// a thread's two cells (x, y alike): the star they may belong to, 0 or 1, or -1,
+// and the parts of the distance and the enthalpy that x and y set
+struct ScfColumn {
+    int star;
+    double d2, rot, h;
+    __device__ __forceinline__ ScfColumn(const NodeInfo &ni, double h_, const ScfGeo &g, const ScfStars &s)
+        : h(h_)
+    {
+        const int c = threadIdx.x;
+        const double x = centre_of(g.lo[0], ni.ix, c & 7, h), y = centre_of(g.lo[1], ni.iy, (c >> 3) & 7, h);
+        star = x < s.x_split ? 0 : 1;
+        const double dx = x - s.centre[star][0], dy = y - s.centre[star][1];
+        d2 = fma(dy, dy, fma(dx, dx, 0.0));
+        if (!s.live[star]) star = -1;
+        const double wx = x - s.com[0], wy = y - s.com[1];
+        rot = 0.5 * s.omega2 * fma(wx, wx, wy * wy);
+    }
+    // whether cell threadIdx.x + 256 j is inside the star
+    __device__ __forceinline__ bool inside(const NodeInfo &ni, const ScfGeo &g, const ScfStars &s, int j) const
+    {
+        if (star < 0) return false;
+        const double dz = centre_of(g.lo[2], ni.iz, (int(threadIdx.x) >> 6) + 4 * j, h) - s.centre[star][2];
+        return fma(dz, dz, d2) < s.r2lim[star];
+    }
+    __device__ __forceinline__ double enthalpy(double phi, const ScfStars &s) const
+    {
+        return s.C[star] - phi + rot;
+    }
+};
 
 // the largest H of each star's cells into host[0..1]
 __global__ void __launch_bounds__(kScfThreads) scf_hmax_kernel(const NodeInfo *__restrict__ info,
@@ -172,17 +222,17 @@ __global__ void __launch_bounds__(kScfThreads) scf_hmax_kernel(const NodeInfo *_
                                                                 ScfStars s, double *host)
 {
     const NodeInfo ni = info[leaves[blockIdx.x]];
-    double v[2] = {-1e300, -1e300};
-    for (int c = threadIdx.x; c < NCELL; c += kScfThreads) {
-        double x[3];
-        cell_centre(ni, levels, g, c, x);
-        const int star = star_of(x, s);
-        if (star >= 0) {
-            const double H = enthalpy(x, phi[size_t(ni.leaf_row) * NCELL + c], star, s);
-            v[star] = fmax(v[star], H);
-        }
+    double mine = -1e300;
+    if (near_star(ni, s)) {              // (the same for the whole CTA)
+        const ScfColumn col(ni, levels[ni.level * LEVEL_FIELDS + LV_H], g, s);
+        const double *at = phi + size_t(ni.leaf_row) * NCELL + threadIdx.x;
+        double m = -1e300;
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+            if (col.inside(ni, g, s, j)) m = fmax(m, col.enthalpy(at[j * kScfThreads], s));
+        const double v[2] = {col.star == 0 ? m : -1e300, col.star == 1 ? m : -1e300};
+        mine = block_combine<2, true>(v);
     }
-    const double mine = block_combine<2, true>(v);
     double all;
     if (!combine_nodes<2, true>(mine, ni.leaf_row, partials, arrived, all)) return;
     if (threadIdx.x < 2) host[threadIdx.x] = all;
@@ -208,19 +258,21 @@ __global__ void __launch_bounds__(kScfThreads) scf_density_kernel(
     double ih1, double floor_value)
 {
     const NodeInfo ni = info[leaves[blockIdx.x]];
-    for (int c = threadIdx.x; c < NCELL; c += kScfThreads) {
-        double x[3];
-        cell_centre(ni, levels, g, c, x);
-        const size_t idx = size_t(ni.leaf_row) * NCELL + c;
-        const int star = star_of(x, s);
-        double r = floor_value;
-        if (star >= 0) {
-            const double H = enthalpy(x, phi[idx], star, s);
-            if (H > 0.0)
-                r = fmax(floor_value, (star ? rho_max1 : rho_max0) * power(H * (star ? ih1 : ih0), n, half));
-        }
-        rho_out[idx] = r;
+    const size_t at = size_t(ni.leaf_row) * NCELL + threadIdx.x;
+    double r[2] = {floor_value, floor_value};
+    if (near_star(ni, s)) {
+        const ScfColumn col(ni, levels[ni.level * LEVEL_FIELDS + LV_H], g, s);
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+            if (col.inside(ni, g, s, j)) {
+                const double H = col.enthalpy(phi[at + j * kScfThreads], s);
+                if (H > 0.0)
+                    r[j] = fmax(floor_value, (col.star ? rho_max1 : rho_max0) *
+                                                 power(H * (col.star ? ih1 : ih0), n, half));
+            }
     }
+    rho_out[at] = r[0];
+    rho_out[at + kScfThreads] = r[1];
 }
 
 int scf_fail(int code, const std::string &msg)
@@ -335,6 +387,13 @@ extern "C" int fmm_scf_update(fmm_tree_t t, const fmm_scf_params *p, const doubl
         for (int a = 0; a < 3; ++a) st.centre[i][a] = p->centre[i][a];
         st.r2lim[i] = p->r_lim[i] * p->r_lim[i];
         st.live[i] = p->rho_max[i] > 0.0;
+        double far = 1.0;
+        for (int a = 0; a < 3; ++a) {
+            const double c = (p->centre[i][a] - g.lo[a]) / g.size;
+            st.box_centre[i][a] = float(c);
+            far += std::abs(c);
+        }
+        st.box_reach[i] = float(p->r_lim[i] / g.size + 1e-5 * far);
     }
     // 3. each star's largest enthalpy
     scf_hmax_kernel<<<unsigned(nl), kScfThreads, 0, s>>>(t->dev.info, leaves, t->dev.levels, phi,
