@@ -581,13 +581,16 @@ __global__ void __launch_bounds__(kForceThreads, 12) leaf_finish_kernel(
     col.finish(row, partials);
 }
 
-// The same with one thread per cell, for trees with few leaf nodes: eight cells
-// one after the other cost each thread 30 us (FP64: 52), whatever the number
-// of nodes up to a dozen per SM.  The cells' masses and fields go through
-// shared memory to the first 64 threads, which take the columns' sums in the
-// same order as above, so the results are the same bits.
-template <int MODE>
-__global__ void __launch_bounds__(NCELL, MODE == FMM_FP64 ? 1 : 2) leaf_finish_cells_kernel(
+// The same with fewer cells per thread, for trees with few leaf nodes: eight
+// cells one after the other cost each thread 30 us (FP64: 52), whatever the
+// number of nodes up to a dozen per SM.  One cell per thread up to two nodes an
+// SM, four up to six (launch_leaf_finish).
+// The cells' masses and fields go through shared memory to the first 64
+// threads, which take the columns' sums in the same order as above, so the
+// results are the same bits.
+template <int MODE, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == NCELL ? (MODE == FMM_FP64 ? 1 : 2)
+                                           : MODE == FMM_MIXED ? 6 : 4) leaf_finish_cells_kernel(
     const NodeInfo *__restrict__ info, const int32_t *__restrict__ leaves,
     const double *__restrict__ levels, const dfloat *__restrict__ levels_df,
     const void *__restrict__ Lv, const float *__restrict__ Lc, const double *dL1,
@@ -598,22 +601,25 @@ __global__ void __launch_bounds__(NCELL, MODE == FMM_FP64 ? 1 : 2) leaf_finish_c
     __shared__ double sc[4][NCELL];
     const int node = leaves[blockIdx.x];
     const NodeInfo ni = info[node];
-    const int c = threadIdx.x;
     chain_begin();
-    double out[20], corr[3], gv[3];
-    const double m = M[(size_t(node) * NCOMP) * NCELL + c];
-    l2l_cell<MODE, 1>(info, ni, node, c, levels, levels_df, Lv, Lc, dL1, com, L64, dacc, down, lo_x,
-                      lo_y, lo_z, out, corr);
-    ForceColumn::field(ni.leaf_row, c, out[0], out + 1, corr, phi, g, gv);
-    sc[0][c] = m;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) sc[1 + a][c] = gv[a];
+    for (int k = 0; k < NCELL / THREADS; ++k) {
+        const int c = threadIdx.x + THREADS * k;
+        double out[20], corr[3], gv[3];
+        const double m = M[(size_t(node) * NCOMP) * NCELL + c];
+        l2l_cell<MODE, 1>(info, ni, node, c, levels, levels_df, Lv, Lc, dL1, com, L64, dacc, down, lo_x,
+                          lo_y, lo_z, out, corr);
+        ForceColumn::field(ni.leaf_row, c, out[0], out + 1, corr, phi, g, gv);
+        sc[0][c] = m;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) sc[1 + a][c] = gv[a];
+    }
     __syncthreads();
-    ForceColumn col(ni, levels, box_size, c & (kForceThreads - 1));
-    if (c < kForceThreads)
+    ForceColumn col(ni, levels, box_size, threadIdx.x & (kForceThreads - 1));
+    if (threadIdx.x < kForceThreads)
 #pragma unroll
         for (int z = 0; z < 8; ++z) {
-            const int b = c + 64 * z;
+            const int b = threadIdx.x + 64 * z;
             const double gz[3] = {sc[1][b], sc[2][b], sc[3][b]};
             col.add(z, sc[0][b], gz);
         }
@@ -835,24 +841,30 @@ cudaError_t launch_leaf_finish(const fmm_tree_s *t, const void *L, const float *
     const dfloat *ldf = reinterpret_cast<const dfloat *>(t->dev.levels_df);
     const int32_t *nodes = t->dev.lists + r.off;
     const unsigned grid = unsigned(r.count);
-    // one thread per cell while the CTAs fit the SMs in one wave (two per SM,
-    // FP64: one), one per column of eight cells above: 64 leaf nodes 29 -> 14 us,
-    // but 512 nodes 30 -> 34; FP64, 8 nodes 52 -> 27
-    const bool cells = r.count <= (c.precision == FMM_FP64 ? 1 : 2) *
-                                      int64_t(sm_count_of_current_device());
+    // one cell per thread while the CTAs fit the SMs in one wave (two per SM,
+    // FP64: one), four up to six nodes an SM, else eight: 64 leaf nodes
+    // 29 -> 14 us with one, but 512 nodes 30 -> 34; FP64, 8 nodes 52 -> 27.
+    // With four, steps of 512 nodes: mixed 185 -> 169 us, double-float
+    // 778 -> 730; 288 nodes in FP64 2481 -> 2342.  Beyond, eight in the mixed
+    // precision (11768 nodes: 2413 us, 2451 with four) and in FP64 (equal), four
+    // in double-float, which has no spills there (4572 nodes: 4695 -> 4590)
     auto launch = [&](auto kern, int threads) {
         return launch_chained(kern, grid, threads, s, t->dev.info, nodes, t->dev.levels, ldf, L, Lc, dL1,
                               com, L64, dacc, t->dev.down, M, phi, g, t->dev.partials, c.box_lo[0],
                               c.box_lo[1], c.box_lo[2], c.box_size);
     };
+    const int64_t sms = sm_count_of_current_device();
+    const bool one = r.count <= (c.precision == FMM_FP64 ? 1 : 2) * sms, four = r.count <= 6 * sms;
     if (c.precision == FMM_MIXED)
-        return cells ? launch(leaf_finish_cells_kernel<FMM_MIXED>, NCELL)
-                     : launch(leaf_finish_kernel<FMM_MIXED>, kForceThreads);
+        return one    ? launch(leaf_finish_cells_kernel<FMM_MIXED, NCELL>, NCELL)
+               : four ? launch(leaf_finish_cells_kernel<FMM_MIXED, 128>, 128)
+                      : launch(leaf_finish_kernel<FMM_MIXED>, kForceThreads);
     if (c.precision == FMM_DFLOAT)
-        return cells ? launch(leaf_finish_cells_kernel<FMM_DFLOAT>, NCELL)
-                     : launch(leaf_finish_kernel<FMM_DFLOAT>, kForceThreads);
-    return cells ? launch(leaf_finish_cells_kernel<FMM_FP64>, NCELL)
-                 : launch(leaf_finish_kernel<FMM_FP64>, kForceThreads);
+        return one ? launch(leaf_finish_cells_kernel<FMM_DFLOAT, NCELL>, NCELL)
+                   : launch(leaf_finish_cells_kernel<FMM_DFLOAT, 128>, 128);
+    return one    ? launch(leaf_finish_cells_kernel<FMM_FP64, NCELL>, NCELL)
+           : four ? launch(leaf_finish_cells_kernel<FMM_FP64, 128>, 128)
+                  : launch(leaf_finish_kernel<FMM_FP64>, kForceThreads);
 }
 
 cudaError_t launch_downward_dataflow(const fmm_tree_s *t, const void *L, const float *Lc,

@@ -59,3 +59,22 @@ def test_launch_shapes_agree(tree, theta, order):
             assert np.array_equal(a, b)
     assert np.abs(out[0][3] - ref["g"]).max() <= FORCE_TOL * np.abs(ref["g"]).max()
     s.close()
+
+
+# leaf sub-grids: 120, 260 (one cell per thread; FP64 four), 316, 568 (four)
+@pytest.mark.parametrize("precision", ["mixed", "dfloat", "fp64"])
+@pytest.mark.parametrize("radius,level", [(0.1, 4), (0.1, 5), (0.13, 5), (0.2, 5)])
+def test_leaf_pass_shapes_agree(precision, radius, level):
+    desc = _corner(level, radius)
+    rng = np.random.default_rng(4)
+    rho = gaussian_blobs(leaf_cell_centres(desc), rng.uniform(0.2, 0.5, (2, 3)), 0.06, 1.0).reshape(-1, 512)
+    s = F.Solver(desc, 0.5, precision=precision)
+    s.rho.copy_(torch.from_numpy(rho).cuda())
+    out = []
+    for run in (s.step, s.step_passes):      # the fused pass, and shifts and forces apart
+        run()
+        torch.cuda.synchronize()
+        out.append([t.cpu().numpy().copy() for t in (s.phi, s.g, s.dacc, s.totals)])
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+    s.close()
