@@ -276,8 +276,8 @@ static void build_stencils(fmm_tree_s *t)
     }
     // monopole kernel: parity 0's weights, every parity in parity 0's order
     t->coef32.assign(size_t(P.ent_stride) * 4, 0.f);
-    t->mono_woff.assign(size_t(8) * P.ent_stride, 0);
-    t->mono_woff16.assign(size_t(8) * P.ent_stride, 0);
+    t->mono_woff.assign(size_t(8) * P.ent_stride + size_t(4) * P.ent_stride, 0);
+    std::vector<uint16_t> woff16(size_t(8) * P.ent_stride, 0);
     for (size_t k = 0; k < lists[0].size(); ++k) {
         const StencilEntry &e = lists[0][k];
         double c[4];
@@ -293,9 +293,10 @@ static void build_stencils(fmm_tree_s *t)
                 std::abort();
             const size_t at = size_t(p) * P.ent_stride + k;
             t->mono_woff[at] = entry(pp, o[0], o[1], o[2]).woff;
-            t->mono_woff16[at] = uint16_t(sizeof(float) * t->mono_woff[at]);   // 8 * 1584 cells at most
+            woff16[at] = uint16_t(sizeof(float) * t->mono_woff[at]);   // 8 * 1584 cells at most
         }
     }
+    std::memcpy(&t->mono_woff[size_t(8) * P.ent_stride], woff16.data(), woff16.size() * sizeof(uint16_t));
     P.stencil_union = 0;
     for (char c : in_union) P.stencil_union += c;
     // the opening test on an integer squared offset n, as a threshold: the
@@ -333,20 +334,26 @@ static void build_orbits(fmm_tree_s *t)
                                       oz = 2 * dz + (s >> 2) - (p >> 2);
                             if (ox || oy || oz) mono_coef(ox, oy, oz, w[p][s]);
                         }
+                    // both transforms by butterflies over the six bits of
+                    // (p, s), in long double
+                    long double K[64][4];
+                    for (int i = 0; i < 64; ++i)
+                        for (int c = 0; c < 4; ++c) K[i][c] = w[i >> 3][i & 7][c];
+                    for (int bit = 1; bit < 64; bit <<= 1)
+                        for (int i = 0; i < 64; ++i) {
+                            if (i & bit) continue;
+                            for (int c = 0; c < 4; ++c) {
+                                const long double u = K[i][c], v = K[i | bit][c];
+                                K[i][c] = u + v;
+                                K[i | bit][c] = u - v;
+                            }
+                        }
                     for (int b = 0; b < 8; ++b)
                         for (int q = 0; q < 8; ++q) {
                             if (q & ~mask) continue;
                             for (int c = 0; c < 4; ++c) {
                                 const int a = q ^ b ^ (c == 0 ? 0 : 1 << (c - 1));
-                                long double sum = 0.0L;
-                                for (int p = 0; p < 8; ++p)
-                                    for (int s = 0; s < 8; ++s) {
-                                        int odd = 0;
-                                        for (int m = a & p; m; m &= m - 1) odd ^= 1;
-                                        for (int m = b & s; m; m &= m - 1) odd ^= 1;
-                                        sum += odd ? -(long double)w[p][s][c] : (long double)w[p][s][c];
-                                    }
-                                t->orbit_coef.push_back(double(sum / 64.0L));
+                                t->orbit_coef.push_back(double(K[8 * a + b][c] / 64.0L));
                             }
                         }
                 }
@@ -639,9 +646,9 @@ static void free_device(fmm_tree_s *t)
     }
     DeviceTables &d = t->dev;
     void *ptrs[] = {d.info, d.children, d.nbr, d.lists, d.stencil, d.stencil_f, d.coef32, d.mono_woff,
-                    d.mono_woff16, d.orbits, d.orbit_coef,
+                    d.orbits, d.orbit_coef,
                     d.tree_leaf_off, d.tree_leaf_rows, d.levels, d.levels_df, d.mass, d.mp, d.counters,
-                    d.partials, d.chunk_sums, d.reduce_arrived, d.up, d.down, d.mx_targets, d.mx_pairs,
+                    d.partials, d.chunk_sums, d.up, d.down, d.mx_targets, d.mx_pairs,
                     d.dflow_items, d.dflow_ready};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -655,8 +662,6 @@ static int upload_tree(fmm_tree_s *t)
     if ((rc = upload(&d.info, t->info)) || (rc = upload(&d.children, t->children)) ||
         (rc = upload(&d.nbr, t->nbr)) || (rc = upload(&d.lists, t->lists)) ||
         (rc = upload(&d.stencil, t->stencil)) || (rc = upload(&d.stencil_f, t->stencil_f)) ||
-        (rc = upload(&d.coef32, t->coef32)) ||
-        (rc = upload(&d.mono_woff, t->mono_woff)) || (rc = upload(&d.mono_woff16, t->mono_woff16)) ||
         (rc = upload(&d.tree_leaf_off, t->tree_leaf_off)) ||
         (rc = upload(&d.tree_leaf_rows, t->tree_leaf_rows)) || (rc = upload(&d.levels, t->levels)) ||
         (rc = upload(&d.levels_df, t->levels_df)) ||
@@ -665,9 +670,12 @@ static int upload_tree(fmm_tree_s *t)
         (rc = upload(&d.dflow_items, t->dflow_items)) ||
         (rc = upload(reinterpret_cast<int32_t **>(&d.orbits), t->orbits)))
         return rc;
-    if (t->cfg.precision == FMM_FP64) {
+    if (t->cfg.precision == FMM_MIXED) {
+        if ((rc = upload(&d.coef32, t->coef32)) || (rc = upload(&d.mono_woff, t->mono_woff))) return rc;
+        d.mono_woff16 = reinterpret_cast<const uint16_t *>(d.mono_woff + size_t(8) * t->plan.ent_stride);
+    } else if (t->cfg.precision == FMM_FP64) {
         if ((rc = upload(reinterpret_cast<double **>(&d.orbit_coef), t->orbit_coef))) return rc;
-    } else if (t->cfg.precision == FMM_DFLOAT) {
+    } else {
         std::vector<float> pairs;            // double-float (hi, lo)
         for (double v : t->orbit_coef) {
             pairs.push_back(float(v));
@@ -685,22 +693,20 @@ static int upload_tree(fmm_tree_s *t)
     size_t mp_b = size_t(t->n_refined + 1) * mp_row_b;
     size_t part_b = size_t(std::max<int64_t>(t->n_leaf, 1)) * 8 * sizeof(double);
     size_t chunk_b = size_t(t->n_trees) * t->plan.reduce_chunks * 8 * sizeof(double);
+    size_t counters_b = size_t(64 + t->n_trees) * sizeof(int32_t);
     cudaError_t e;
     if ((e = cudaMalloc(&d.mass, mass_b)) != cudaSuccess ||
         (e = cudaMalloc(&d.mp, mp_b)) != cudaSuccess ||
-        (e = cudaMalloc(reinterpret_cast<void **>(&d.counters), 64 * sizeof(int32_t))) != cudaSuccess ||
+        (e = cudaMalloc(reinterpret_cast<void **>(&d.counters), counters_b)) != cudaSuccess ||
         (e = cudaMalloc(reinterpret_cast<void **>(&d.partials), part_b)) != cudaSuccess ||
         (e = cudaMalloc(reinterpret_cast<void **>(&d.chunk_sums), chunk_b)) != cudaSuccess ||
-        (e = cudaMalloc(reinterpret_cast<void **>(&d.reduce_arrived), size_t(t->n_trees) * sizeof(int32_t))) !=
-            cudaSuccess ||
         (e = cudaMalloc(reinterpret_cast<void **>(&d.dflow_ready), size_t(t->n) * sizeof(int32_t))) !=
             cudaSuccess)
         return fail(FMM_ERR_NOMEM, std::string("workspace cudaMalloc: ") + cudaGetErrorString(e));
-    d.workspace_bytes = mass_b + mp_b + part_b + chunk_b + 64 * sizeof(int32_t) +
-                        size_t(t->n) * sizeof(int32_t) + size_t(t->n_trees) * sizeof(int32_t);
+    d.reduce_arrived = d.counters + 64;
+    d.workspace_bytes = mass_b + mp_b + part_b + chunk_b + counters_b + size_t(t->n) * sizeof(int32_t);
     // work queues and the status word start at zero
-    if ((e = cudaMemset(d.counters, 0, 64 * sizeof(int32_t))) != cudaSuccess ||
-        (e = cudaMemset(d.reduce_arrived, 0, size_t(t->n_trees) * sizeof(int32_t))) != cudaSuccess ||
+    if ((e = cudaMemset(d.counters, 0, counters_b)) != cudaSuccess ||
         (e = cudaMemset(static_cast<char *>(d.mp) + size_t(t->n_refined) * mp_row_b, 0, mp_row_b)) !=
             cudaSuccess)
         return cuda_fail(e, "cudaMemset");
@@ -815,7 +821,7 @@ int fmm_build_tree(const fmm_node_desc *nodes, int64_t n_nodes, const fmm_config
         }
     }
     build_stencils(t);
-    build_orbits(t);
+    if (t->cfg.precision != FMM_MIXED) build_orbits(t);
     plan_work(t);
     plan_dataflow(t);
     // per-level geometry: h = box / (8 * 2^(l-1)) is exact up to the box edge

@@ -78,7 +78,7 @@ struct DeviceTables {
     // monopole<-monopole, mixed precision
     float *coef32 = nullptr;         // [ent_stride][4] monopole weights of parity 0
     int32_t *mono_woff = nullptr;    // [8][ent_stride] window offsets, parity 0's order reflected
-    uint16_t *mono_woff16 = nullptr; // the same, in bytes
+    const uint16_t *mono_woff16 = nullptr;  // the same, in bytes (behind them)
     // monopole<-monopole, FP64 and double-float (fmm_mono_wide.cuh)
     int4 *orbits = nullptr;          // near parent offsets (dx, dy, dz >= 0, mask of nonzero axes)
     void *orbit_coef = nullptr;      // [orbit][b][q][4] transformed weights: double or float pairs
@@ -96,7 +96,7 @@ struct DeviceTables {
     int32_t *counters = nullptr;     // work-queue heads; [kStatusSlot]: FMM_STATUS_* bits
     double *partials = nullptr;      // [n_leaf][8]
     double *chunk_sums = nullptr;    // [n_trees][reduce_chunks][8]
-    int32_t *reduce_arrived = nullptr;  // [n_trees] finished CTAs of the force sums (zero between steps)
+    int32_t *reduce_arrived = nullptr;  // (in counters) [n_trees] finished CTAs of the force sums (zero between steps)
     float *up = nullptr;             // mixed, dfloat: [n_refined][20][512] double-float
                                      // (hi, lo) results of the upward pass per refined cell
     int32_t *dflow_items = nullptr;  // dataflow downward queue: refined (node, slice) items
@@ -172,8 +172,7 @@ struct fmm_tree_s {
     std::vector<fmm::StencilEntry> stencil;
     std::vector<float> stencil_f;
     std::vector<float> coef32;
-    std::vector<int32_t> mono_woff;
-    std::vector<uint16_t> mono_woff16;
+    std::vector<int32_t> mono_woff;      // and behind them the same in bytes, 16-bit
     std::vector<int32_t> orbits;         // [n][4]
     std::vector<double> orbit_coef;      // [orbit][b][q][4]
     int32_t orbit_first[9] = {0};        // the orbits of mask k: orbit_first[k] .. [k + 1]
