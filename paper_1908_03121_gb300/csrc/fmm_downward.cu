@@ -101,8 +101,8 @@ __device__ __forceinline__ double whole(int i) { return f2d_bits(float(i)); }
 template <int NMAX>
 __device__ __forceinline__ void l2l_cell_fp64(const NodeInfo &ni, int node, int c,
                                               const double *__restrict__ lv,
-                                              const void *__restrict__ Lv, const double *dL1,
-                                              const double *__restrict__ com,
+                                              const void *Lv, const double *dL1,
+                                              const double *com,
                                               double *__restrict__ L64, double *dacc, double lo_x,
                                               double lo_y, double lo_z, double (&out)[20],
                                               double (&corr)[3])
@@ -163,9 +163,8 @@ __device__ __forceinline__ void l2l_cell_mixed(const NodeInfo &ni, int node, int
                                                const NodeInfo *__restrict__ info,
                                                const double *__restrict__ lv,
                                                const dfloat *__restrict__ lvdf,
-                                               const float *__restrict__ Lhi,
-                                               const float *__restrict__ Llo, const double *dL1,
-                                               const double *__restrict__ com,
+                                               const float *Lhi, const float *Llo,
+                                               const double *dL1, const double *com,
                                                double *__restrict__ L64, double *dacc,
                                                dfloat *__restrict__ down, double lo_x,
                                                double lo_y, double lo_z, double (&out)[20],
@@ -264,9 +263,8 @@ __device__ __forceinline__ void l2l_cell_df(const NodeInfo &ni, int node, int c,
                                             const NodeInfo *__restrict__ info,
                                             const double *__restrict__ lv,
                                             const dfloat *__restrict__ lvdf,
-                                            const float *__restrict__ Lhi,
-                                            const float *__restrict__ Llo, const double *dL1,
-                                            const double *__restrict__ com,
+                                            const float *Lhi, const float *Llo,
+                                            const double *dL1, const double *com,
                                             double *__restrict__ L64, double *dacc,
                                             dfloat *__restrict__ down, double lo_x, double lo_y,
                                             double lo_z, double (&out)[20], double (&corr)[3])
@@ -342,8 +340,8 @@ template <int MODE, int NMAX>
 __device__ __forceinline__ void l2l_cell(const NodeInfo *__restrict__ info, const NodeInfo &ni,
                                          int node, int c, const double *__restrict__ levels,
                                          const dfloat *__restrict__ levels_df,
-                                         const void *__restrict__ Lv, const float *__restrict__ Lc,
-                                         const double *dL1, const double *__restrict__ com,
+                                         const void *Lv, const float *Lc,
+                                         const double *dL1, const double *com,
                                          double *__restrict__ L64, double *dacc, float *down,
                                          double lo_x, double lo_y, double lo_z, double (&out)[20],
                                          double (&corr)[3])
@@ -371,12 +369,10 @@ __global__ void __launch_bounds__(kSliceThreads) l2l_kernel(const NodeInfo *__re
                                                             const int32_t *__restrict__ nodes,
                                                             const double *__restrict__ levels,
                                                             const dfloat *__restrict__ levels_df,
-                                                            const void *__restrict__ Lv,
-                                                            const float *__restrict__ Lc,
+                                                            const void *Lv, const float *Lc,
                                                             const double *dL1,  // may alias dacc
-                                                            const double *__restrict__ com,
-                                                            double *__restrict__ L64, double *dacc,
-                                                            float *__restrict__ down, double lo_x,
+                                                            const double *com, double *L64,
+                                                            double *dacc, float *down, double lo_x,
                                                             double lo_y, double lo_z)
 {
     const int node = nodes[blockIdx.x >> 3];
@@ -395,9 +391,8 @@ template <int MODE>
 __global__ void __launch_bounds__(kLeafThreads) l2l_leaf_kernel(
     const NodeInfo *__restrict__ info, const int32_t *__restrict__ nodes,
     const double *__restrict__ levels, const dfloat *__restrict__ levels_df,
-    const void *__restrict__ Lv, const float *__restrict__ Lc, const double *dL1,
-    const double *__restrict__ com, double *__restrict__ L64, double *dacc, float *__restrict__ down,
-    double lo_x, double lo_y, double lo_z)
+    const void *Lv, const float *Lc, const double *dL1, const double *com, double *L64, double *dacc,
+    float *down, double lo_x, double lo_y, double lo_z)
 {
     const int node = nodes[blockIdx.x >> 1];
     const NodeInfo ni = info[node];
@@ -552,17 +547,11 @@ struct ForceColumn {
     }
 };
 
-__global__ void __launch_bounds__(kForceThreads) forces_kernel(
-    const NodeInfo *__restrict__ info, const int32_t *__restrict__ leaves,
-    const double *__restrict__ levels, const double *__restrict__ L64,
-    const double *__restrict__ dacc, const double *__restrict__ rho, double *__restrict__ phi,
-    double *__restrict__ g, double *__restrict__ partials, double box_size)
+// a leaf node's forces: eight cells per thread (after chain_begin())
+__device__ __forceinline__ void forces_columns(ForceColumn &col, int node, int row, const double *L64,
+                                               const double *dacc, const double *rho,
+                                               double *__restrict__ phi, double *__restrict__ g)
 {
-    const int node = leaves[blockIdx.x];
-    const NodeInfo ni = info[node];
-    const int row = ni.leaf_row;
-    ForceColumn col(ni, levels, box_size, threadIdx.x);
-    chain_begin();
 #pragma unroll
     for (int z = 0; z < 8; ++z) {
         const int c = threadIdx.x + 64 * z;
@@ -575,7 +564,19 @@ __global__ void __launch_bounds__(kForceThreads) forces_kernel(
         col.cell(row, c, z, rho[size_t(row) * NCELL + c] * col.h3, L64[(size_t(node) * NCOMP) * NCELL + c],
                  L1, acc, phi, g);
     }
-    col.finish(row, partials);
+}
+
+__global__ void __launch_bounds__(kForceThreads) forces_kernel(
+    const NodeInfo *__restrict__ info, const int32_t *__restrict__ leaves,
+    const double *__restrict__ levels, const double *L64, const double *dacc, const double *rho,
+    double *phi, double *g, double *partials, double box_size)
+{
+    const int node = leaves[blockIdx.x];
+    const NodeInfo ni = info[node];
+    ForceColumn col(ni, levels, box_size, threadIdx.x);
+    chain_begin();
+    forces_columns(col, node, ni.leaf_row, L64, dacc, rho, phi, g);
+    col.finish(ni.leaf_row, partials);
 }
 
 // fmm_step's last pass over the leaves: each leaf cell's shift (as
@@ -586,19 +587,13 @@ __global__ void __launch_bounds__(kForceThreads) forces_kernel(
 // and the extra warps keep more FP64 operations in flight than the 96
 // registers it would otherwise take
 template <int MODE>
-__global__ void __launch_bounds__(kForceThreads, 12) leaf_finish_kernel(
-    const NodeInfo *__restrict__ info, const int32_t *__restrict__ leaves,
-    const double *__restrict__ levels, const dfloat *__restrict__ levels_df,
-    const void *__restrict__ Lv, const float *__restrict__ Lc, const double *dL1,
-    const double *__restrict__ com, double *__restrict__ L64, double *dacc, float *down,
-    const double *__restrict__ M, double *__restrict__ phi, double *__restrict__ g,
-    double *__restrict__ partials, double lo_x, double lo_y, double lo_z, double box_size)
+__device__ __forceinline__ void leaf_finish_columns(
+    ForceColumn &col, const NodeInfo *__restrict__ info, const NodeInfo &ni, int node,
+    const double *__restrict__ levels, const dfloat *__restrict__ levels_df, const void *Lv,
+    const float *Lc, const double *dL1, const double *com, double *__restrict__ L64, double *dacc,
+    float *down, const double *M, double *__restrict__ phi, double *__restrict__ g, double lo_x,
+    double lo_y, double lo_z)
 {
-    const int node = leaves[blockIdx.x];
-    const NodeInfo ni = info[node];
-    const int row = ni.leaf_row;
-    ForceColumn col(ni, levels, box_size, threadIdx.x);
-    chain_begin();
 #pragma unroll
     for (int z = 0; z < 8; ++z) {
         const int c = threadIdx.x + 64 * z;
@@ -608,9 +603,25 @@ __global__ void __launch_bounds__(kForceThreads, 12) leaf_finish_kernel(
         // the cell mass as P2M left it in M (rho h^3, the same product): the
         // step reads the density in P2M only, so it may sit in pinned host
         // memory
-        col.cell(row, c, z, M[(size_t(node) * NCOMP) * NCELL + c], out[0], out + 1, corr, phi, g);
+        col.cell(ni.leaf_row, c, z, M[(size_t(node) * NCOMP) * NCELL + c], out[0], out + 1, corr, phi, g);
     }
-    col.finish(row, partials);
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kForceThreads, 12) leaf_finish_kernel(
+    const NodeInfo *__restrict__ info, const int32_t *__restrict__ leaves,
+    const double *__restrict__ levels, const dfloat *__restrict__ levels_df, const void *Lv,
+    const float *Lc, const double *dL1, const double *com, double *L64, double *dacc, float *down,
+    const double *M, double *phi, double *g, double *partials, double lo_x, double lo_y, double lo_z,
+    double box_size)
+{
+    const int node = leaves[blockIdx.x];
+    const NodeInfo ni = info[node];
+    ForceColumn col(ni, levels, box_size, threadIdx.x);
+    chain_begin();
+    leaf_finish_columns<MODE>(col, info, ni, node, levels, levels_df, Lv, Lc, dL1, com, L64, dacc, down,
+                              M, phi, g, lo_x, lo_y, lo_z);
+    col.finish(ni.leaf_row, partials);
 }
 
 // The same with fewer cells per thread, for trees with few leaf nodes: eight
@@ -621,19 +632,13 @@ __global__ void __launch_bounds__(kForceThreads, 12) leaf_finish_kernel(
 // threads, which take the columns' sums in the same order as above, so the
 // results are the same bits.
 template <int MODE, int THREADS>
-__global__ void __launch_bounds__(THREADS, THREADS == NCELL ? (MODE == FMM_FP64 ? 1 : 2)
-                                           : MODE == FMM_MIXED ? 6 : 4) leaf_finish_cells_kernel(
-    const NodeInfo *__restrict__ info, const int32_t *__restrict__ leaves,
-    const double *__restrict__ levels, const dfloat *__restrict__ levels_df,
-    const void *__restrict__ Lv, const float *__restrict__ Lc, const double *dL1,
-    const double *__restrict__ com, double *__restrict__ L64, double *dacc, float *down,
-    const double *__restrict__ M, double *__restrict__ phi, double *__restrict__ g,
-    double *__restrict__ partials, double lo_x, double lo_y, double lo_z, double box_size)
+__device__ __forceinline__ void leaf_finish_cells(
+    double (*sc)[NCELL], const NodeInfo *__restrict__ info, const NodeInfo &ni, int node,
+    const double *__restrict__ levels, const dfloat *__restrict__ levels_df, const void *Lv,
+    const float *Lc, const double *dL1, const double *com, double *__restrict__ L64, double *dacc,
+    float *down, const double *M, double *__restrict__ phi, double *__restrict__ g, double lo_x,
+    double lo_y, double lo_z)
 {
-    __shared__ double sc[4][NCELL];
-    const int node = leaves[blockIdx.x];
-    const NodeInfo ni = info[node];
-    chain_begin();
 #pragma unroll
     for (int k = 0; k < NCELL / THREADS; ++k) {
         const int c = threadIdx.x + THREADS * k;
@@ -646,6 +651,23 @@ __global__ void __launch_bounds__(THREADS, THREADS == NCELL ? (MODE == FMM_FP64 
 #pragma unroll
         for (int a = 0; a < 3; ++a) sc[1 + a][c] = gv[a];
     }
+}
+
+template <int MODE, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == NCELL ? (MODE == FMM_FP64 ? 1 : 2)
+                                           : MODE == FMM_MIXED ? 6 : 4) leaf_finish_cells_kernel(
+    const NodeInfo *__restrict__ info, const int32_t *__restrict__ leaves,
+    const double *__restrict__ levels, const dfloat *__restrict__ levels_df, const void *Lv,
+    const float *Lc, const double *dL1, const double *com, double *L64, double *dacc, float *down,
+    const double *M, double *phi, double *g, double *partials, double lo_x, double lo_y, double lo_z,
+    double box_size)
+{
+    __shared__ double sc[4][NCELL];
+    const int node = leaves[blockIdx.x];
+    const NodeInfo ni = info[node];
+    chain_begin();
+    leaf_finish_cells<MODE, THREADS>(sc, info, ni, node, levels, levels_df, Lv, Lc, dL1, com, L64, dacc,
+                                     down, M, phi, g, lo_x, lo_y, lo_z);
     __syncthreads();
     ForceColumn col(ni, levels, box_size, threadIdx.x & (kForceThreads - 1));
     if (threadIdx.x < kForceThreads)
@@ -784,7 +806,7 @@ __device__ __forceinline__ double row_sums(int rows, Row row, double (*sh)[8])
 {
     const int k = threadIdx.x & 7, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double v = 0.0;
-    for (int i = threadIdx.x >> 3; i < rows; i += kReduceThreads / 8) v += __ldcg(row(i) + k);   // past L1: other CTAs wrote the chunk sums
+    for (int i = threadIdx.x >> 3; i < rows; i += kReduceThreads / 8) v += load_cg(row(i) + k);
     v += __shfl_xor_sync(0xffffffffu, v, 8);
     v += __shfl_xor_sync(0xffffffffu, v, 16);
     if (lane < 8) sh[warp][lane] = v;
@@ -799,10 +821,9 @@ __device__ __forceinline__ double row_sums(int rows, Row row, double (*sh)[8])
 
 __global__ void __launch_bounds__(kReduceThreads) reduce_kernel(const int32_t *__restrict__ off,
                                                                 const int32_t *__restrict__ rows,
-                                                                const double *__restrict__ partials,
-                                                                double *__restrict__ chunk_sums,
-                                                                int32_t *__restrict__ arrived,
-                                                                double *__restrict__ totals)
+                                                                const double *partials,
+                                                                double *chunk_sums, int32_t *arrived,
+                                                                double *totals)
 {
     __shared__ double sh[kReduceThreads / 32][8];
     __shared__ int s_last;

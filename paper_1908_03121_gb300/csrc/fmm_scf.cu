@@ -23,6 +23,7 @@
 #include <cmath>
 #include <string>
 
+#include "fmm_chain.cuh"
 #include "fmm_convert.cuh"
 #include "fmm_internal.h"
 
@@ -99,7 +100,7 @@ __device__ __forceinline__ bool combine_nodes(double mine, int row, double *part
     for (int i = threadIdx.x; i < int(gridDim.x); i += kScfThreads)
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
-            const double o = __ldcg(partials + size_t(i) * 8 + k);      // past L1: other CTAs' rows
+            const double o = load_cg(partials + size_t(i) * 8 + k);     // other CTAs' rows
             v[k] = MAX ? fmax(v[k], o) : v[k] + o;
         }
     all = block_combine<NV, MAX>(v);

@@ -47,11 +47,8 @@ template <typename T>
 __global__ void __launch_bounds__(NCELL / 2) p2m_kernel(const NodeInfo *__restrict__ info,
                                                         const int32_t *__restrict__ leaves,
                                                         const double *__restrict__ levels,
-                                                        const double *__restrict__ rho,
-                                                        double *__restrict__ M,
-                                                        int32_t *__restrict__ status,
-                                                        T *__restrict__ mass,
-                                                        int32_t *__restrict__ queues)
+                                                        const double *rho, double *M,
+                                                        int32_t *status, T *mass, int32_t *queues)
 {
     chain_begin();
     if (queues && blockIdx.x == 0 && threadIdx.x < 4) queues[threadIdx.x] = 0;
@@ -110,8 +107,7 @@ __global__ void __launch_bounds__(kSliceThreads) m2m_kernel(const NodeInfo *__re
                                                             const int32_t *__restrict__ children,
                                                             const int32_t *__restrict__ nodes,
                                                             const double *__restrict__ levels,
-                                                            double *__restrict__ M,
-                                                            double *__restrict__ com, double lo_x,
+                                                            double *M, double *com, double lo_x,
                                                             double lo_y, double lo_z)
 {
     const int node = nodes[blockIdx.x >> 3];
@@ -262,10 +258,8 @@ __global__ void __launch_bounds__(kSliceThreads) m2m_df_kernel(const NodeInfo *_
                                                                const int32_t *__restrict__ children,
                                                                const int32_t *__restrict__ nodes,
                                                                const double *__restrict__ levels,
-                                                               double *__restrict__ M,
-                                                               double *__restrict__ com,
-                                                               dfloat *__restrict__ up, double lo_x,
-                                                               double lo_y, double lo_z)
+                                                               double *M, double *com, dfloat *up,
+                                                               double lo_x, double lo_y, double lo_z)
 {
     const int node = nodes[blockIdx.x >> 3];
     const NodeInfo ni = info[node];
@@ -341,8 +335,8 @@ __device__ __forceinline__ void add_halves(dfloat (&v)[16], bool upper, int mask
 
 __global__ void __launch_bounds__(kSliceThreads) m2m_df_lanes_kernel(
     const NodeInfo *__restrict__ info, const int32_t *__restrict__ children,
-    const int32_t *__restrict__ nodes, const double *__restrict__ levels, double *__restrict__ M,
-    double *__restrict__ com, dfloat *__restrict__ up, double lo_x, double lo_y, double lo_z)
+    const int32_t *__restrict__ nodes, const double *__restrict__ levels, double *M, double *com,
+    dfloat *up, double lo_x, double lo_y, double lo_z)
 {
     constexpr int kCtasPerNode = NCELL / kCellsPerCta;
     const int node = nodes[blockIdx.x / kCtasPerNode];
