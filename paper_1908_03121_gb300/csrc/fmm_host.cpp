@@ -307,17 +307,20 @@ static void build_stencils(fmm_tree_s *t)
 }
 
 // The wide types' monopole<-monopole weights (fmm_mono_wide.cuh): near parent
-// offsets up to signs, by mask of nonzero axes, and for each the Hadamard
+// offsets up to signs (not 0: a block's own cells are summed directly), by mask
+// of nonzero axes, and for each the Hadamard
 // transform of the 8 x 8 weights between a block's children,
 //   K_ab = (1/64) sum_ps (-1)^(a.p + b.s) w_c(2 d + s - p),
 // stored for a = q xor b xor e_c, q over the subsets of the mask (zero for
-// the other q by symmetry).
+// the other q by symmetry).  Behind them the weights within a block: c = 0 and
+// an axis c for cells apart in one, two and three axes (and a zero).
 static void build_orbits(fmm_tree_s *t)
 {
     const int R = int(std::floor(1.0 / t->cfg.theta));
     t->orbits.clear();
     t->orbit_coef.clear();
-    for (int mask = 0; mask < 8; ++mask) {
+    t->orbit_first[0] = 0;
+    for (int mask = 1; mask < 8; ++mask) {
         t->orbit_first[mask] = int32_t(t->orbits.size() / 4);
         for (int dz = 0; dz <= R; ++dz)
             for (int dy = 0; dy <= R; ++dy)
@@ -325,14 +328,14 @@ static void build_orbits(fmm_tree_s *t)
                     if (((dx > 0) | (dy > 0) << 1 | (dz > 0) << 2) != mask) continue;
                     if (well_separated(t->cfg.theta, dx, dy, dz)) continue;
                     for (int v : {dx, dy, dz, mask}) t->orbits.push_back(v);
-                    // w[p][s][c]; a cell has no weight on itself
+                    // w[p][s][c]
                     double w[8][8][4] = {};
                     for (int p = 0; p < 8; ++p)
                         for (int s = 0; s < 8; ++s) {
                             const int ox = 2 * dx + (s & 1) - (p & 1),
                                       oy = 2 * dy + ((s >> 1) & 1) - ((p >> 1) & 1),
                                       oz = 2 * dz + (s >> 2) - (p >> 2);
-                            if (ox || oy || oz) mono_coef(ox, oy, oz, w[p][s]);
+                            mono_coef(ox, oy, oz, w[p][s]);
                         }
                     // both transforms by butterflies over the six bits of
                     // (p, s), in long double
@@ -359,6 +362,10 @@ static void build_orbits(fmm_tree_s *t)
                 }
     }
     t->orbit_first[8] = int32_t(t->orbits.size() / 4);
+    double near[3][4];
+    for (int k = 0; k < 3; ++k) mono_coef(1, k > 0, k > 1, near[k]);
+    for (int c = 0; c < 2; ++c)
+        for (int k = 0; k < 4; ++k) t->orbit_coef.push_back(k < 3 ? near[k][c] : 0.0);
 }
 
 // --------------------------------------------------- interaction counting

@@ -81,7 +81,8 @@ struct DeviceTables {
     const uint16_t *mono_woff16 = nullptr;  // the same, in bytes (behind them)
     // monopole<-monopole, FP64 and double-float (fmm_mono_wide.cuh)
     int4 *orbits = nullptr;          // near parent offsets (dx, dy, dz >= 0, mask of nonzero axes)
-    void *orbit_coef = nullptr;      // [orbit][b][q][4] transformed weights: double or float pairs
+    void *orbit_coef = nullptr;      // [orbit][b][q][4] transformed weights, [2][4] within a block: double or
+                                     // float pairs
     int32_t *tree_leaf_off = nullptr;   // [n_trees + 1]
     int32_t *tree_leaf_rows = nullptr;  // [n_leaf]
     double *levels = nullptr;        // [max_level + 1][LEVEL_FIELDS]
@@ -174,7 +175,7 @@ struct fmm_tree_s {
     std::vector<float> coef32;
     std::vector<int32_t> mono_woff;      // and behind them the same in bytes, 16-bit
     std::vector<int32_t> orbits;         // [n][4]
-    std::vector<double> orbit_coef;      // [orbit][b][q][4]
+    std::vector<double> orbit_coef;      // [orbit][b][q][4], and [2][4] within a block
     int32_t orbit_first[9] = {0};        // the orbits of mask k: orbit_first[k] .. [k + 1]
     std::vector<int32_t> tree_leaf_off, tree_leaf_rows;
     std::vector<double> levels;

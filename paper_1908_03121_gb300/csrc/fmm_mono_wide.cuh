@@ -18,10 +18,18 @@
 //       S_b^q(C) = sum_signs (product of the signs of q's axes) m^_b(C + d),
 //     and O_a += K_ab(|d|) S_b^q: one product per (b, q, c), where the direct
 //     form has one per (p, s, c) and sign.
-// theta = 0.5: 1056 products, 480 additions, 192 + 320 for the transforms per
-// block of eight cells, against 8416 products (direct form).  A level-6 binary
+//   - only the own block (d = 0) is summed directly, cell by cell: in the
+//     transformed basis a cell's own mass would enter its sums and cancel to
+//     rounding of that mass alone, far above the field of a thin surrounding (a
+//     dense cell in a floor of 1e-10: 9e-9 of g in FP64).  A heavier cell of
+//     another block attracts the target by as much as its roundings scale with.
+// theta = 0.5: 1024 products, 480 additions, 192 + 320 for the transforms and 152
+// products in the own block per block of eight cells, against 8416 products
+// (direct form).  A level-6 binary
 // (4572 leaf nodes), whole step: FP64 24.1 -> 20.9 ms (this kernel 4.4 -> 1.2),
-// double-float 5.43 -> 4.79 ms; 8 leaf nodes in FP64, step 318 -> 207 us.
+// double-float 5.43 -> 4.79 ms; 8 leaf nodes in FP64, step 318 -> 207 us.  (The
+// own block's products cost 0.13 and 0.07 ms of a level-6 step, 2 us of 8 leaf
+// nodes'.)
 // A thread has one target block and one b (the same for a whole warp, so the
 // weights are broadcasts); its 32 sums A[q][c] belong to a = q xor b xor e_c and
 // meet those of the other b at the end, through shared memory, in a fixed
@@ -46,7 +54,7 @@ struct MonoWParams {
     int32_t *counter;
     const int4 *orbits;          // [n] (dx, dy, dz >= 0, mask of nonzero axes), by mask
     int first[9];                // orbits of mask k: first[k] .. first[k + 1]
-    const void *coef;            // [orbit][b][q in mask][c]
+    const void *coef;            // [orbit][b][q in mask][c]; the last eight: [2][4] within a block
     int n_coef;                  // values
     int reach;                   // in blocks
     const void *mass;
@@ -123,6 +131,29 @@ __device__ __forceinline__ void mono_wide_orbits(const MonoWParams &P, const T *
         for (int k = 0; k < 4; ++k) A[q][k] = renorm(A[q][k]);
 }
 
+// the own block's terms of one component: ec = 0 for L0, else the axis's bit (a
+// first-order weight is nonzero between cells apart in that axis only, and its
+// sign is the target's side of it)
+template <typename T>
+__device__ __forceinline__ void mono_wide_own(const T m[8], const T *near, int ec, T (&o)[8])
+{
+    T v[8];
+#pragma unroll
+    for (int p = 0; p < 8; ++p) v[p] = T(0);
+#pragma unroll
+    for (int x = 1; x < 8; ++x) {
+        if (ec != 0 && !(x & ec)) continue;
+        const T w = near[(ec ? 4 : 0) + (x & 1) + ((x >> 1) & 1) + (x >> 2) - 1];
+#pragma unroll
+        for (int p = 0; p < 8; ++p) v[p] = fmadd_u(w, m[p ^ x], v[p]);
+    }
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+        const T a = renorm(v[p]);
+        o[p] += (p & ec) ? -a : a;
+    }
+}
+
 template <typename T, int PLANES>
 __global__ void __launch_bounds__(128 * PLANES, PLANES == 4 ? 1 : 4) mono_wide_kernel(MonoWParams P)
 {
@@ -190,7 +221,6 @@ __global__ void __launch_bounds__(128 * PLANES, PLANES == 4 ? 1 : 4) mono_wide_k
             for (int k = 0; k < 4; ++k) A[q][k] = T(0);
         const T *own = W + b * plane + (tx + R) + kMonoWPitch * (ty + R) + pz * (tz + R);
         const T *coef = s_coef;
-        mono_wide_orbits<T, 0>(P, own, pz, b, coef, A);
         mono_wide_orbits<T, 1>(P, own, pz, b, coef, A);
         mono_wide_orbits<T, 2>(P, own, pz, b, coef, A);
         mono_wide_orbits<T, 3>(P, own, pz, b, coef, A);
@@ -229,6 +259,11 @@ __global__ void __launch_bounds__(128 * PLANES, PLANES == 4 ? 1 : 4) mono_wide_k
                         o[a] = u + v;
                         o[a | ax] = u - v;
                     }
+                T m[8];
+                const T *at = mass + size_t(node) * NCELL + (t & 3) + 4 * ((t >> 2) & 3) + 16 * (z0 + (t >> 4));
+#pragma unroll
+                for (int s = 0; s < 8; ++s) m[s] = ldg_t(at + 64 * s);
+                mono_wide_own<T>(m, s_coef + P.n_coef - 8, ec, o);
                 const int cell = 2 * (t & 3) + 16 * ((t >> 2) & 3) + 128 * (z0 + (t >> 4));
 #pragma unroll
                 for (int p = 0; p < 8; ++p)
