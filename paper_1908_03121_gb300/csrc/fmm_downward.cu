@@ -384,19 +384,20 @@ __global__ void __launch_bounds__(kSliceThreads) l2l_kernel(const NodeInfo *__re
                       lo_z, out, corr);
 }
 
-// the same for leaf nodes (all of them in one launch): half a node per CTA
-constexpr int kLeafThreads = NCELL / 2;
-
+// the same for leaf nodes, all of them in one launch: the same small CTAs, which
+// share a few hundred nodes out evenly over the SMs (with two CTAs of 256
+// threads a node the shifts and forces of 176 to 316 leaf nodes in double-float
+// took as long as level by level; 4572 nodes 371 us against 325)
 template <int MODE>
-__global__ void __launch_bounds__(kLeafThreads) l2l_leaf_kernel(
+__global__ void __launch_bounds__(kSliceThreads) l2l_leaf_kernel(
     const NodeInfo *__restrict__ info, const int32_t *__restrict__ nodes,
     const double *__restrict__ levels, const dfloat *__restrict__ levels_df,
     const void *Lv, const float *Lc, const double *dL1, const double *com, double *L64, double *dacc,
     float *down, double lo_x, double lo_y, double lo_z)
 {
-    const int node = nodes[blockIdx.x >> 1];
+    const int node = nodes[blockIdx.x >> 3];
     const NodeInfo ni = info[node];
-    const int c = (blockIdx.x & 1) * kLeafThreads + threadIdx.x;
+    const int c = (blockIdx.x & 7) * kSliceThreads + threadIdx.x;
     chain_begin();
     double out[20], corr[3];
     l2l_cell<MODE, 1>(info, ni, node, c, levels, levels_df, Lv, Lc, dL1, com, L64, dacc, down, lo_x, lo_y,
@@ -579,6 +580,61 @@ __global__ void __launch_bounds__(kForceThreads) forces_kernel(
     col.finish(ni.leaf_row, partials);
 }
 
+// the sums of a node's columns from its cells' masses and fields in shared
+// memory, in the order of the columns above (after a barrier)
+__device__ __forceinline__ void finish_cells(const double (*sc)[NCELL], const NodeInfo &ni,
+                                             const double *levels, double box_size, double *partials)
+{
+    ForceColumn col(ni, levels, box_size, threadIdx.x & (kForceThreads - 1));
+    if (threadIdx.x < kForceThreads)
+#pragma unroll
+        for (int z = 0; z < 8; ++z) {
+            const int b = threadIdx.x + 64 * z;
+            const double gz[3] = {sc[1][b], sc[2][b], sc[3][b]};
+            col.add(z, sc[0][b], gz);
+        }
+    col.finish(ni.leaf_row, partials);
+}
+
+// The same with fewer cells per thread, whose chains leave the memory idle on
+// trees with few leaf nodes (launch_forces); same bits
+template <int THREADS>
+__device__ __forceinline__ void forces_cells(double (*sc)[NCELL], int node, int row, double h3,
+                                             const double *L64, const double *dacc, const double *rho,
+                                             double *__restrict__ phi, double *__restrict__ g)
+{
+#pragma unroll
+    for (int k = 0; k < NCELL / THREADS; ++k) {
+        const int c = threadIdx.x + THREADS * k;
+        double L1[3], acc[3], gv[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            L1[a] = L64[(size_t(node) * NCOMP + 1 + a) * NCELL + c];
+            acc[a] = dacc[(size_t(node) * 3 + a) * NCELL + c];
+        }
+        sc[0][c] = rho[size_t(row) * NCELL + c] * h3;
+        ForceColumn::field(row, c, L64[(size_t(node) * NCOMP) * NCELL + c], L1, acc, phi, g, gv);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) sc[1 + a][c] = gv[a];
+    }
+}
+
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) forces_cells_kernel(
+    const NodeInfo *__restrict__ info, const int32_t *__restrict__ leaves,
+    const double *__restrict__ levels, const double *L64, const double *dacc, const double *rho,
+    double *phi, double *g, double *partials, double box_size)
+{
+    __shared__ double sc[4][NCELL];
+    const int node = leaves[blockIdx.x];
+    const NodeInfo ni = info[node];
+    const double h3 = levels[ni.level * LEVEL_FIELDS + LV_H3];
+    chain_begin();
+    forces_cells<THREADS>(sc, node, ni.leaf_row, h3, L64, dacc, rho, phi, g);
+    __syncthreads();
+    finish_cells(sc, ni, levels, box_size, partials);
+}
+
 // fmm_step's last pass over the leaves: each leaf cell's shift (as
 // l2l_kernel) and its forces (as forces_kernel) in one kernel, the shifted
 // expansion going straight from registers into the force terms; the same
@@ -669,15 +725,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == NCELL ? (MODE == FMM_FP64 
     leaf_finish_cells<MODE, THREADS>(sc, info, ni, node, levels, levels_df, Lv, Lc, dL1, com, L64, dacc,
                                      down, M, phi, g, lo_x, lo_y, lo_z);
     __syncthreads();
-    ForceColumn col(ni, levels, box_size, threadIdx.x & (kForceThreads - 1));
-    if (threadIdx.x < kForceThreads)
-#pragma unroll
-        for (int z = 0; z < 8; ++z) {
-            const int b = threadIdx.x + 64 * z;
-            const double gz[3] = {sc[1][b], sc[2][b], sc[3][b]};
-            col.add(z, sc[0][b], gz);
-        }
-    col.finish(ni.leaf_row, partials);
+    finish_cells(sc, ni, levels, box_size, partials);
 }
 
 // ---------------------------------------------------------------- dataflow
@@ -881,7 +929,7 @@ cudaError_t launch_l2l_leaves(const fmm_tree_s *t, const void *L, const float *L
     auto kern = t->cfg.precision == FMM_MIXED    ? l2l_leaf_kernel<FMM_MIXED>
                 : t->cfg.precision == FMM_DFLOAT ? l2l_leaf_kernel<FMM_DFLOAT>
                                                  : l2l_leaf_kernel<FMM_FP64>;
-    return launch_l2l(kern, unsigned(r.count * 2), kLeafThreads, t, r, L, Lc, dL1, com, L64, dacc, s);
+    return launch_l2l(kern, unsigned(r.count * 8), kSliceThreads, t, r, L, Lc, dL1, com, L64, dacc, s);
 }
 
 cudaError_t launch_leaf_finish(const fmm_tree_s *t, const void *L, const float *Lc,
@@ -982,10 +1030,22 @@ cudaError_t launch_forces(const fmm_tree_s *t, const double *L64, const double *
 {
     const ListRange &r = t->plan.leaves;
     if (r.count > 0) {
+        auto launch = [&](auto kern, int threads) {
+            return launch_chained(kern, unsigned(r.count), threads, s, t->dev.info, t->dev.lists + r.off,
+                                  t->dev.levels, L64, dacc, rho, phi, g, t->dev.partials, t->cfg.box_size);
+        };
+        // one cell per thread up to six leaf nodes an SM, four up to twelve, else
+        // eight.  fmm_downward and fmm_forces with one / four / eight, us: 64
+        // nodes 28 / 42 / 53, 512 nodes 47 / 56 / 67, 848 (5.6 an SM) 69 / 71 /
+        // 82, 932 75 / 73 / 84, 1520 (10 an SM) 108 / 95 / 105, 1968 132 / 117 /
+        // 117, 4572 265 / 223 / 217 (mixed; FP64 and double-float cross at the
+        // same sizes)
+        const int64_t sms = sm_count_of_current_device();
+        const bool one = r.count <= 6 * sms, four = r.count <= 12 * sms;
         timing_begin(t, FMM_K_FORCES, s);
-        cudaError_t e = launch_chained(forces_kernel, unsigned(r.count), kForceThreads, s, t->dev.info,
-                                       t->dev.lists + r.off, t->dev.levels, L64, dacc, rho, phi, g,
-                                       t->dev.partials, t->cfg.box_size);
+        const cudaError_t e = one    ? launch(forces_cells_kernel<NCELL>, NCELL)
+                              : four ? launch(forces_cells_kernel<128>, 128)
+                                     : launch(forces_kernel, kForceThreads);
         timing_end(t, s);
         if (e != cudaSuccess) return e;
     }
