@@ -984,6 +984,14 @@ int fmm_upward(fmm_tree_t t, const double *rho, double *M, double *com, fmm_stre
     return FMM_OK;
 }
 
+// stream s waits for what the second stream has been given, also after an
+// error on the way: its kernels may still write the caller's buffers
+static cudaError_t join_aux(fmm_tree_t t, cudaEvent_t ev, cudaStream_t s)
+{
+    const cudaError_t e = cudaEventRecord(ev, t->aux);
+    return e == cudaSuccess ? cudaStreamWaitEvent(s, ev, 0) : e;
+}
+
 int fmm_m2l(fmm_tree_t t, const double *M, const double *com, void *L, float *L_comp,
             double *dL1, fmm_stream_t stream)
 {
@@ -1011,11 +1019,12 @@ int fmm_m2l(fmm_tree_t t, const double *M, const double *com, void *L, float *L_
     if (e == cudaSuccess) e = launch_m2l(t, L, L_comp, dL1, s, &nl, M2L_RESET);
     if (e == cudaSuccess) e = cudaEventRecord(t->step_ev[0], s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(a, t->step_ev[0], 0);
-    if (e == cudaSuccess) e = launch_m2l(t, L, L_comp, dL1, a, &nl, M2L_ROOT);
-    if (e == cudaSuccess) e = cudaEventRecord(t->step_ev[1], a);
+    if (e != cudaSuccess) return cuda_fail(e, "m2l launch");
+    e = launch_m2l(t, L, L_comp, dL1, a, &nl, M2L_ROOT);
     if (e == cudaSuccess) e = launch_m2l(t, L, L_comp, dL1, s, &nl, M2L_MONO);
     if (e == cudaSuccess) e = launch_m2l(t, L, L_comp, dL1, s, &nl, M2L_MP | M2L_MPX);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, t->step_ev[1], 0);
+    const cudaError_t joined = join_aux(t, t->step_ev[1], s);
+    if (e == cudaSuccess) e = joined;
     return e == cudaSuccess ? FMM_OK : cuda_fail(e, "m2l launch");
 }
 
@@ -1086,8 +1095,12 @@ int fmm_step(fmm_tree_t t, const double *rho, double *M, double *com, void *L, f
     const Plan &P = t->plan;
     cudaError_t e;
     int nl = 0;
-#define FMM_STEP_TRY(call, what) \
-    if ((e = (call)) != cudaSuccess) return cuda_fail(e, what)
+    bool forked = false;
+#define FMM_STEP_TRY(call, what)                                                  \
+    if ((e = (call)) != cudaSuccess) {                                            \
+        if (forked) (void)join_aux(t, ev[2], s);                                  \
+        return cuda_fail(e, what);                                                \
+    }
     // main: P2M (which resets the work queues), fork
     FMM_STEP_TRY(launch_p2m(t, rho, M, s, true), "p2m launch");
     FMM_STEP_TRY(cudaEventRecord(ev[0], s), "cudaEventRecord");
@@ -1096,6 +1109,7 @@ int fmm_step(fmm_tree_t t, const double *rho, double *M, double *com, void *L, f
     // aux: leaf masses, monopole<-monopole
     // (P2M has stored the leaf masses in their packed form)
     FMM_STEP_TRY(cudaStreamWaitEvent(a, ev[0], 0), "cudaStreamWaitEvent");
+    forked = true;
     FMM_STEP_TRY(launch_m2l(t, L, L_comp, dL1, a, &nl, M2L_MONO), "m2l launch");
     FMM_STEP_TRY(cudaEventRecord(ev[3], a), "cudaEventRecord");
     // main: M2M, refined sources, multipole targets
