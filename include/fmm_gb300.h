@@ -31,9 +31,13 @@
  * Memory and streams
  *   - The caller owns every data buffer (device memory, raw pointers).  The
  *     library owns only what fmm_build_tree allocates (tree tables on the
- *     device and a fixed workspace), released by fmm_destroy_tree.
- *   - fmm_upward / fmm_m2l / fmm_downward / fmm_forces only enqueue work on
- *     the given stream (a cudaStream_t; NULL = legacy default stream).  They
+ *     device, a fixed workspace, a stream and its events, and for a single
+ *     tree 64 bytes of page-locked host memory), released by fmm_destroy_tree.
+ *   - fmm_upward / fmm_m2l / fmm_downward / fmm_forces / fmm_step only enqueue
+ *     work, ordered by the given stream (a cudaStream_t; NULL = legacy default
+ *     stream): fmm_m2l and fmm_step run part of it on the tree's own stream
+ *     (of default priority), which forks from and joins back into the given
+ *     one through events, also when they return an error.  They
  *     do not allocate, free or synchronise.  A tree's workspace is shared by
  *     its calls, so calls on one tree must not overlap in time (serialise
  *     them on one stream).
@@ -498,8 +502,8 @@ typedef struct {
  *   rho_out: device double [n_leaf][512], receives
  *            max(rho_floor, rho_max,i (H / H_max,i)^n) where H > 0 in star i,
  *            else rho_floor (may be rho itself).
- * The centre of mass is summed per leaf node on the device and over the
- * nodes on the host in a fixed order; the surface conditions hold at the
+ * The centre of mass is summed on the device, per leaf node and then over the
+ * nodes in a fixed order; the surface conditions hold at the
  * centres of the leaf cells containing A, B, C (w measured there); then
  *   Omega^2 = 2 (Phi_A - Phi_B) / (w_A^2 - w_B^2)   (0 unless rotate),
  *   C_1 = Phi_A - Omega^2 w_A^2 / 2,  C_2 = Phi_C - Omega^2 w_C^2 / 2.

@@ -710,6 +710,9 @@ static int upload_tree(fmm_tree_s *t)
         (e = cudaMalloc(reinterpret_cast<void **>(&d.dflow_ready), size_t(t->n) * sizeof(int32_t))) !=
             cudaSuccess)
         return fail(FMM_ERR_NOMEM, std::string("workspace cudaMalloc: ") + cudaGetErrorString(e));
+    if (t->n_trees == 1 &&
+        (e = cudaMallocHost(reinterpret_cast<void **>(&t->scf_host), 8 * sizeof(double))) != cudaSuccess)
+        return fail(FMM_ERR_NOMEM, std::string("workspace cudaMallocHost: ") + cudaGetErrorString(e));
     d.reduce_arrived = d.counters + 64;
     d.workspace_bytes = mass_b + mp_b + part_b + chunk_b + counters_b + size_t(t->n) * sizeof(int32_t);
     // work queues and the status word start at zero

@@ -190,7 +190,7 @@ struct fmm_tree_s {
     int device = -1;
     fmm::DeviceTables dev;
     mutable fmm::TimerState timer;
-    double *scf_host = nullptr;          // fmm_scf_update's scalars, page-locked, from its first call
+    double *scf_host = nullptr;          // fmm_scf_update's scalars, page-locked (single trees)
     // fmm_step's second stream and its fork/join events (device trees only)
     cudaStream_t aux = nullptr;
     cudaEvent_t step_ev[4] = {nullptr, nullptr, nullptr, nullptr};

@@ -347,21 +347,13 @@ extern "C" int fmm_scf_update(fmm_tree_t t, const fmm_scf_params *p, const doubl
     const int32_t *leaves = t->dev.lists + t->plan.leaves.off;
     const ScfGeo g{{t->cfg.box_lo[0], t->cfg.box_lo[1], t->cfg.box_lo[2]}, t->cfg.box_size};
     // 1. centre of mass; the potential at the surface cells
-    cudaError_t e = cudaSuccess;
-    if (!t->scf_host) {
-        e = cudaMallocHost(reinterpret_cast<void **>(&t->scf_host), 8 * sizeof(double));
-        if (e != cudaSuccess) {
-            t->scf_host = nullptr;
-            return scf_fail(FMM_ERR_NOMEM, cudaGetErrorString(e));
-        }
-    }
     ScfPoints points{};
     for (int k = 0; k < 3; ++k)
         if (row[k] >= 0) points.phi[k] = phi + row[k] * NCELL + cell[k];
     scf_com_kernel<<<unsigned(nl), kScfThreads, 0, s>>>(t->dev.info, leaves, t->dev.levels, rho,
                                                          t->dev.partials, t->dev.reduce_arrived, g,
                                                          points, t->scf_host);
-    e = cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return scf_fail(FMM_ERR_CUDA, cudaGetErrorString(e));
     const double msum = t->scf_host[0], mx = t->scf_host[1], my = t->scf_host[2], mz = t->scf_host[3];
