@@ -491,7 +491,8 @@ typedef struct {
     double com[3];                   /* centre of mass of the input density */
     double H_max[2];                 /* each star's largest enthalpy (K_i = H_max,i /
                                         ((n + 1) rho_max,i^(1/n))) */
-    double phi_points[3];            /* potential at the cells of A, B, C */
+    double phi_points[3];            /* potential at the cells of A, B, C (a point that
+                                        the model does not use: of the first leaf cell) */
     double mass;                     /* total mass of the input density */
 } fmm_scf_result;
 

@@ -108,7 +108,7 @@ __device__ __forceinline__ bool combine_nodes(double mine, int row, double *part
     return true;
 }
 
-// the potential's address at up to three surface cells
+// the potential's address at the three surface cells
 struct ScfPoints {
     const double *phi[3];
 };
@@ -146,10 +146,7 @@ __global__ void __launch_bounds__(kScfThreads) scf_com_kernel(const NodeInfo *__
     double all;
     if (!combine_nodes<4, false>(mine, ni.leaf_row, partials, arrived, all)) return;
     if (threadIdx.x < 4) host[threadIdx.x] = all;
-    else if (threadIdx.x < 7) {
-        const double *at = points.phi[threadIdx.x - 4];
-        host[threadIdx.x] = at ? *at : 0.0;
-    }
+    else if (threadIdx.x < 7) host[threadIdx.x] = *points.phi[threadIdx.x - 4];
 }
 
 struct ScfStars {
@@ -333,7 +330,7 @@ extern "C" int fmm_scf_update(fmm_tree_t t, const fmm_scf_params *p, const doubl
     const int64_t nl = t->n_leaf;
     // the surface conditions hold at the centres of the cells containing the
     // points, where the potential is known
-    int64_t row[3] = {-1, -1, -1};
+    int64_t row[3] = {0, 0, 0};       // (a point that is not used: the first leaf cell)
     int cell[3] = {0, 0, 0};
     double ctr[3][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
     const double *pts[3] = {p->point_a, p->point_b, p->point_c};
@@ -348,8 +345,7 @@ extern "C" int fmm_scf_update(fmm_tree_t t, const fmm_scf_params *p, const doubl
     const ScfGeo g{{t->cfg.box_lo[0], t->cfg.box_lo[1], t->cfg.box_lo[2]}, t->cfg.box_size};
     // 1. centre of mass; the potential at the surface cells
     ScfPoints points{};
-    for (int k = 0; k < 3; ++k)
-        if (row[k] >= 0) points.phi[k] = phi + row[k] * NCELL + cell[k];
+    for (int k = 0; k < 3; ++k) points.phi[k] = phi + row[k] * NCELL + cell[k];
     scf_com_kernel<<<unsigned(nl), kScfThreads, 0, s>>>(t->dev.info, leaves, t->dev.levels, rho,
                                                          t->dev.partials, t->dev.reduce_arrived, g,
                                                          points, t->scf_host);
