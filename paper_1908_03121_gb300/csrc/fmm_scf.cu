@@ -237,13 +237,24 @@ __global__ void __launch_bounds__(kScfThreads) scf_hmax_kernel(const NodeInfo *_
 }
 
 // u^n, u > 0; half: 2 n where that is a whole number up to 16 (the usual
-// indices: products and a square root, a tenth of pow's FP64 operations)
+// indices: products and a square root, a fifth of pow's FP64 operations).  What
+// each rounding leaves out is carried along, so that the result is as near as
+// pow's (0.6 units in the last place at n = 8, 2.5 without)
 __device__ __forceinline__ double power(double u, double n, int half)
 {
     if (half == 0) return pow(u, n);
-    double r = (half & 1) ? sqrt(u) : 1.0;
-    for (int k = half >> 1; k > 0; --k) r *= u;
-    return r;
+    double r = 1.0, e = 0.0;             // the power so far is r + e
+    if (half & 1) {
+        r = sqrt(u);
+        const float rf = d2f_trunc(r);   // (e to a float's bits)
+        if (rf > 0.f) e = fma(-r, r, u) * f2d_bits(0.5f / rf);
+    }
+    for (int k = half >> 1; k > 0; --k) {
+        const double p = r * u;
+        e = fma(e, u, fma(r, u, -p));
+        r = p;
+    }
+    return r + e;
 }
 
 // the new density: max(floor, rho_max,i (H / H_max,i)^n) inside star i where
