@@ -1278,7 +1278,7 @@ __global__ void __launch_bounds__(kSplitThreads, 2) mp_split_kernel(KParams P)
 // The multipole kernel of the wide types (double, double-float; the
 // interaction and its sums are in fmm_wide.cuh).  Bound by the FP64 pipe
 // (double) or the FP32 pipe (double-float): one CTA per SM is enough, and
-// registers go to the 38 sums.  One loop takes far and near entries alike
+// registers go to the 34 sums.  One loop takes far and near entries alike
 // (near ones count leaf sources only), so the large body is compiled once;
 // its second half, the moments, is skipped for entries without a refined
 // source in the warp, and entries with absent sources only altogether.
@@ -1301,9 +1301,9 @@ __device__ __forceinline__ T wide_shfl_xor(T v, int mask)
     else
         return __shfl_xor_sync(0xffffffffu, v, mask);
 }
-// the sums of WideAcc as an array (order 2 leaves the last 15 at zero)
+// the sums of WideAcc as an array
 template <int ORDER>
-constexpr int kWideSums = ORDER == 3 ? 38 : 23;
+constexpr int kWideSums = ORDER == 3 ? 34 : 22;
 
 template <typename T, int ORDER>
 __device__ __forceinline__ void store_wide(const KParams &P, int node, int cell, const T L[16], const T S[3])
@@ -1829,7 +1829,7 @@ template <typename T, int ORDER>
 __global__ void __launch_bounds__(kThreads) rootw_kernel(KParams P)
 {
     constexpr int NS = kWideSums<ORDER>, NW = kThreads / 32;
-    static_assert(sizeof(WideAcc<T, ORDER>) == 38 * sizeof(T), "sums of WideAcc");
+    static_assert(sizeof(WideAcc<T, ORDER>) == NS * sizeof(T), "sums of WideAcc");
     __shared__ T sh[NW][NS][kRootwTargets];
     const int node = P.list[blockIdx.x];
     const NodeInfo ti = P.info[node];

@@ -14,20 +14,23 @@
 //       dL1 += 7 e9 s3 R - 3 e7 b                       (the source's share);
 //   - what depends on the source's mass alone (orders 2 and 3 of the Taylor
 //     coefficients, and the target's share of the correction,
-//     -sum m D4 : M3_A / (6 M0_A)) is summed as plain moments
-//     sum m e_k R R.. of the separations: the delta terms of D2..D4 and the
-//     contraction with the target's own third moment are linear in those
-//     sums, so they are formed once per target cell (finish()) instead of
-//     once per source.
-// 69 operations for a leaf source and 124 for a refined one (fused
+//     -sum m D4 : M3_A / (6 M0_A)) is summed as moments m e_k R R.. of the
+//     separations: those of L2 and L3 made traceless term by term, the others
+//     plain, since the delta terms of D4 and the contraction with the target's
+//     own third moment are linear in the sums and so are formed once per target
+//     cell (finish()) instead of once per source.
+// 72 operations for a leaf source and 127 for a refined one (fused
 // multiply-add = 1), where evaluating the derivative tensors and contracting
 // them takes about 145 and 173 (with the divide and square root of
 // 1 / sqrt).  A level-6 binary (5225 sub-grids, theta 0.5), whole step: FP64
-// 31.4 -> 24.1 ms (multipole kernel 26.1 -> 18.8, its FP64 pipe 91 % busy
-// before and after), double-float 6.65 -> 5.43 ms; a 9-sub-grid FP64 step 968
-// -> 318 us (the root over 128 CTAs).  Errors against 64 bits unchanged: g
-// 4.6e-16 (FP64), 1.2e-14 -> 1.3e-14 and phi 8.1e-15 -> 6.8e-15
-// (double-float).
+// 31.4 -> 24.4 ms (multipole kernel 26.1 -> 19.1, its FP64 pipe 91 % busy
+// before and after), double-float 6.65 -> 5.48 ms; a 9-sub-grid FP64 step 968
+// -> 318 us (the root over 128 CTAs).  Errors against 64 bits, level-5 binary,
+// tensors / this: double-float g 1.2e-14 / 9e-15, phi 8.0e-15 / 4.4e-15, L2
+// 2.0e-14 / 9e-15, L3 3.1e-14 / 1.3e-14; FP64 g 4.6e-16 / 4.6e-16, L3 1.1e-15 /
+// 1.0e-15.  (L2 and L3 as plain moments, whose traces do not cancel, and sums
+// normalised every 16 entries only: 3 % faster in double-float, 1.5 % in FP64,
+// with L3 at 4.7e-14 and 1.2e-15.)
 #pragma once
 
 #include "fmm_convert.cuh"
@@ -47,6 +50,13 @@ __device__ __forceinline__ double scaled(float c, double v) { return __dmul_rn(d
 __device__ __forceinline__ dfloat scaled(float c, dfloat v) { return c * v; }
 __device__ __forceinline__ double twice(double v) { return v + v; }
 __device__ __forceinline__ dfloat twice(dfloat v) { return dfloat(v.hi + v.hi, v.lo + v.lo); }
+// n a + b, n a small whole number
+__device__ __forceinline__ double multiple(float n, double a, double b) { return fma(double(n), a, b); }
+__device__ __forceinline__ dfloat multiple(float n, dfloat a, dfloat b)
+{
+    const float p = n * a.hi, e = fmaf(n, a.lo, fmaf(n, a.hi, -p));
+    return renorm(add_u(dfloat(p, e), b));
+}
 
 // 1/sqrt(v): the hardware's float estimate y0 of a float of v, refined by the
 // binomial series of (1 - e)^(-1/2), e = 1 - v y0^2 (|e| < 2^-21): with the
@@ -91,13 +101,17 @@ struct WideSrc {
 template <typename T>
 struct WideGeo {
     T R[3], e1, e3, e5, e7, e9;
-    T xx, yy, zz, xy2, xz2, yz2;     // the mixed products doubled
+    T xx, yy, xy2, xz2, yz2;         // the mixed products doubled
+    T r2, u, v;                      // xx - zz, yy - zz
     template <int ORDER>
     __device__ __forceinline__ void eval(T x, T y, T z)
     {
         R[0] = x; R[1] = y; R[2] = z;
-        xx = renorm(product(x, x)); yy = renorm(product(y, y)); zz = renorm(product(z, z));
-        const T r2 = wide_r2(x, y, xx, yy, zz);
+        xx = renorm(product(x, x)); yy = renorm(product(y, y));
+        const T zz = renorm(product(z, z));
+        r2 = wide_r2(x, y, xx, yy, zz);
+        u = xx - zz;
+        v = yy - zz;
         e1 = rsqrt_wide(r2);
         const T i2 = e1 * e1;
         e3 = e1 * i2;
@@ -118,11 +132,11 @@ __device__ __forceinline__ void wide_t2R(const T t2[5], const T R[3], T q[3])
     q[2] = renorm(fmadd_u(-(t2[0] + t2[1]), R[2], fmadd_u(t2[4], R[1], mul_u(t2[3], R[0]))));
 }
 
-// b = t3 : R R for the traceless t3 (zz eliminated: u = xx - zz, v = yy - zz)
+// b = t3 : R R for the traceless t3 (zz eliminated)
 template <typename T>
 __device__ __forceinline__ void wide_t3RR(const T t3[7], const WideGeo<T> &g, T b[3])
 {
-    const T u = g.xx - g.zz, v = g.yy - g.zz;
+    const T u = g.u, v = g.v;
     const T nxzz = t3[0] + t3[3], nyzz = t3[1] + t3[5];       // -xzz, -yzz
     b[0] = renorm(fmadd_u(t3[4], g.yz2, fmadd_u(t3[2], g.xz2, fmadd_u(t3[1], g.xy2, fmadd_u(t3[3], v, mul_u(t3[0], u))))));
     b[1] = renorm(fmadd_u(t3[6], g.yz2, fmadd_u(t3[4], g.xz2, fmadd_u(t3[3], g.xy2, fmadd_u(t3[5], v, mul_u(t3[1], u))))));
@@ -190,13 +204,13 @@ struct WideLow {
             }
             t0 = renorm(t0);
         }
-        a0 = add_u(a0, t0);
+        a0 = renorm(add_u(a0, t0));
         if (ORDER == 3 && mp) {
 #pragma unroll
-            for (int i = 0; i < 3; ++i) a1[i] = add_u(a1[i], renorm(fmadd_u(f, g.R[i], t1[i])));
+            for (int i = 0; i < 3; ++i) a1[i] = renorm(add_u(a1[i], renorm(fmadd_u(f, g.R[i], t1[i]))));
         } else {
 #pragma unroll
-            for (int i = 0; i < 3; ++i) a1[i] = fmadd_u(f, g.R[i], a1[i]);
+            for (int i = 0; i < 3; ++i) a1[i] = renorm(fmadd_u(f, g.R[i], a1[i]));
         }
     }
     __device__ __forceinline__ void correction(T S[3]) const
@@ -207,71 +221,65 @@ struct WideLow {
 };
 
 // Sums of a refined target: WideLow's and the mass-weighted moments of the
-// separations (products of two different axes doubled, as in WideGeo).
+// separations (products of two different axes doubled, as in WideGeo).  The
+// terms of L2 and L3 are made traceless one by one: as plain moments, their
+// traces (sums of one sign) carried more rounding than the results have.
 template <typename T, int ORDER>
 struct WideAcc {
     WideLow<T, ORDER> low;
-    T tr, c2[5];             // sum m e3;  m e5 (xx yy xy xz yz)
-    T v[3], c3[7];           // m e5 (x y z);  m e7 (xxx xxy xxz xyy xyz yyy yyz)
-    T e5, c7[5], c4[9];      // order 3: sum m e5;  m e7 (xx yy xy xz yz);
-                             // m e9 (xxxx xxxy xxxz xxyy xxyz xyyy xyyz yyyy yyyz)
+    T c2[5];                 // sum m e5 (2 xx - yy - zz, 2 yy - xx - zz, xy xz yz)
+    T c3[7];                 // order 3: m e7 (x (5 xx - 3 r2), y (5 xx - r2), z (5 xx - r2),
+                             // x (5 yy - r2), xyz, y (5 yy - 3 r2), z (5 yy - r2));
+                             // order 2: m e7 (xxx xxy xxz xyy xyz yyy yyz)
+    T more[ORDER == 3 ? 15 : 3];
+    // order 3: sum m e5;  m e7 (xx yy xy xz yz);  m e9 (xxxx xxxy xxxz xxyy xxyz
+    // xyyy xyyz yyyy yyyz);  order 2: m e5 (x y z)
+    static constexpr int kE5 = 0, kC7 = 1, kC4 = 6, kV = 0;
     __device__ __forceinline__ void zero()
     {
         low.zero();
-        tr = e5 = T(0);
 #pragma unroll
-        for (int k = 0; k < 5; ++k) c2[k] = c7[k] = T(0);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) v[k] = T(0);
+        for (int k = 0; k < 5; ++k) c2[k] = T(0);
 #pragma unroll
         for (int k = 0; k < 7; ++k) c3[k] = T(0);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) c4[k] = T(0);
+        for (int k = 0; k < (ORDER == 3 ? 15 : 3); ++k) more[k] = T(0);
     }
     // double-float: restore the canonical form (the sums take unnormalised
     // terms); called every 16 stencil entries
     __device__ __forceinline__ void flush()
     {
         low.flush();
-        tr = renorm(tr);
-        e5 = renorm(e5);
 #pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            c2[k] = renorm(c2[k]);
-            c7[k] = renorm(c7[k]);
-        }
-#pragma unroll
-        for (int k = 0; k < 3; ++k) v[k] = renorm(v[k]);
+        for (int k = 0; k < 5; ++k) c2[k] = renorm(c2[k]);
 #pragma unroll
         for (int k = 0; k < 7; ++k) c3[k] = renorm(c3[k]);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) c4[k] = renorm(c4[k]);
+        for (int k = 0; k < (ORDER == 3 ? 15 : 3); ++k) more[k] = renorm(more[k]);
     }
     __device__ __forceinline__ void add(T x, T y, T z, T m, const WideSrc<T> &src, bool mp)
     {
         WideGeo<T> g;
         g.template eval<ORDER>(x, y, z);
         const T me3 = product(m, g.e3), me5 = product(m, g.e5), me7 = mul_u(m, g.e7);
-        tr = add_u(tr, me3);
-        const T two[5] = {g.xx, g.yy, g.xy2, g.xz2, g.yz2};
+        const T two[5] = {multiple(2.f, g.u, -g.v), multiple(2.f, g.v, -g.u), g.xy2, g.xz2, g.yz2};
 #pragma unroll
-        for (int k = 0; k < 5; ++k) c2[k] = fmadd_u(me5, two[k], c2[k]);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) v[k] = fmadd_u(me5, g.R[k], v[k]);
+        for (int k = 0; k < 5; ++k) c2[k] = renorm(fmadd_u(me5, two[k], c2[k]));
         const T gx = mul_u(me7, x), gy = mul_u(me7, y);
-        c3[0] = fmadd_u(gx, g.xx, c3[0]);
-        c3[1] = fmadd_u(gy, g.xx, c3[1]);
-        c3[2] = fmadd_u(gx, g.xz2, c3[2]);
-        c3[3] = fmadd_u(gx, g.yy, c3[3]);
-        c3[4] = fmadd_u(gx, g.yz2, c3[4]);
-        c3[5] = fmadd_u(gy, g.yy, c3[5]);
-        c3[6] = fmadd_u(gy, g.yz2, c3[6]);
         if constexpr (ORDER == 3) {
-            e5 = add_u(e5, me5);
+            const T gz = mul_u(me7, z);
+            const T a = multiple(5.f, g.xx, -g.r2), b = multiple(5.f, g.yy, -g.r2);
+            const T t[7] = {multiple(-2.f, g.r2, a), a, a, b, g.yz2, multiple(-2.f, g.r2, b), b};
+            const T f[7] = {gx, gy, gz, gx, gx, gy, gz};
 #pragma unroll
-            for (int k = 0; k < 5; ++k) c7[k] = fmadd_u(me7, two[k], c7[k]);
+            for (int k = 0; k < 7; ++k) c3[k] = renorm(fmadd_u(f[k], t[k], c3[k]));
+            more[kE5] = add_u(more[kE5], me5);
+            const T w[5] = {g.xx, g.yy, g.xy2, g.xz2, g.yz2};
+#pragma unroll
+            for (int k = 0; k < 5; ++k) more[kC7 + k] = fmadd_u(me7, w[k], more[kC7 + k]);
             const T me9 = mul_u(m, g.e9);
             const T hx = mul_u(me9, g.xx), hy = mul_u(me9, g.yy);
+            T *c4 = more + kC4;
             c4[0] = fmadd_u(hx, g.xx, c4[0]);
             c4[1] = fmadd_u(hx, g.xy2, c4[1]);
             c4[2] = fmadd_u(hx, g.xz2, c4[2]);
@@ -281,6 +289,12 @@ struct WideAcc {
             c4[6] = fmadd_u(hy, g.xz2, c4[6]);
             c4[7] = fmadd_u(hy, g.yy, c4[7]);
             c4[8] = fmadd_u(hy, g.yz2, c4[8]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) more[kV + k] = fmadd_u(me5, g.R[k], more[kV + k]);
+            const T f[7] = {gx, gy, gx, gx, gx, gy, gy}, t[7] = {g.xx, g.xx, g.xz2, g.yy, g.yz2, g.yy, g.yz2};
+#pragma unroll
+            for (int k = 0; k < 7; ++k) c3[k] = fmadd_u(f[k], t[k], c3[k]);
         }
         low.add(g, me3, m, src, mp);
     }
@@ -294,19 +308,15 @@ struct WideAcc {
         L[0] = -low.a0;
 #pragma unroll
         for (int i = 0; i < 3; ++i) L[1 + i] = low.a1[i];
-        L[4] = tr - scaled(3.f, c2[0]);
-        L[5] = tr - scaled(3.f, c2[1]);
+        L[4] = -c2[0];
+        L[5] = -c2[1];
 #pragma unroll
         for (int k = 2; k < 5; ++k) L[4 + k] = scaled(-1.5f, c2[k]);
         low.correction(S);
         if constexpr (ORDER == 3) {
-            L[9] = scaled(15.f, c3[0]) - scaled(9.f, v[0]);
-            L[10] = scaled(15.f, c3[1]) - scaled(3.f, v[1]);
-            L[11] = scaled(7.5f, c3[2]) - scaled(3.f, v[2]);
-            L[12] = scaled(15.f, c3[3]) - scaled(3.f, v[0]);
-            L[13] = scaled(7.5f, c3[4]);
-            L[14] = scaled(15.f, c3[5]) - scaled(9.f, v[1]);
-            L[15] = scaled(7.5f, c3[6]) - scaled(3.f, v[2]);
+#pragma unroll
+            for (int k = 0; k < 7; ++k) L[9 + k] = scaled(k == 4 ? 7.5f : 3.f, c3[k]);
+            const T e5 = more[kE5], *c7 = more + kC7, *c4 = more + kC4;
             // S_i -= 7 C4_ijkl a_jkl - 3 C7_kl a_ikl, a = t3 / M0 of the target;
             // the zz components of the sums follow from r^2 e_k = e_(k-2)
             T a[7];
@@ -343,6 +353,7 @@ struct WideAcc {
 #pragma unroll
             for (int k = 0; k < 5; ++k) a[k] = own.t2[k] / own.m0;
             const T azz = -(a[0] + a[1]);
+            const T *v = more + kV;
             const T xxx = c3[0], xxy = c3[1], xyy = c3[3], yyy = c3[5];
             const T xxz = scaled(0.5f, c3[2]), xyz = scaled(0.5f, c3[4]), yyz = scaled(0.5f, c3[6]);
             const T C3[10] = {xxx, xxy, xxz, xyy, xyz, v[0] - xxx - xyy, yyy, yyz, v[1] - xxy - yyy,
