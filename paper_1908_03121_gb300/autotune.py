@@ -23,7 +23,6 @@ from . import fmm as B
 MONO_SUBGRIDS = (1, 2, 4)
 CTAS_PER_SM = (0, 1, 2)
 DATAFLOW = (0, 1)
-PAIR_TARGETS = (0, 1)
 MP_ITEMS = (0, 1, 2)      # 0: by the tree's size
 _CACHE = {}
 
@@ -32,6 +31,25 @@ def _key(solver):
     s = solver.tree.sizes
     return (s["n_nodes"], s["n_leaf"], s["n_refined"], s["precision"],
             int(solver.tree.stats["stencil_union"]), getattr(solver, "order", 3))
+
+
+def candidates(precision, order, n_multipole, sms):
+    """The tunings to time: every launch shape once.  ``n_multipole``: refined
+    sub-grids below the roots (the multipole launch's), ``sms``: the GPU's SMs.
+    What a precision's kernels do not read stays at its default."""
+    mixed = precision == B.FMM_MIXED
+    if precision == B.FMM_FP64:
+        items = (0,)         # long steps: automatic
+    elif mixed:
+        # by size has shapes of its own up to one sub-grid an SM, above it is one of the others
+        items = MP_ITEMS if n_multipole <= sms else MP_ITEMS[1:]
+    else:
+        # sixteenths, whatever is asked for, where quarters do not fill the SMs
+        items = MP_ITEMS[1:] if 4 * n_multipole >= sms else (0,)
+    shapes = [(0, it) for it in items] + ([(1, 0)] if mixed and order == 3 else [])
+    return [dict(mono_subgrids=nb, ctas_per_sm=cap, dataflow=df, mp_pair_targets=pt, mp_items=it)
+            for nb, cap, df, (pt, it) in itertools.product(MONO_SUBGRIDS if mixed else (0,), CTAS_PER_SM,
+                                                           DATAFLOW, shapes)]
 
 
 def tune(solver, reps=5, verbose=False, flush=None, graph=True):
@@ -46,14 +64,6 @@ def tune(solver, reps=5, verbose=False, flush=None, graph=True):
     if key in _CACHE:
         B.fmm_set_tuning(solver.tree, **_CACHE[key][0])
         return _CACHE[key]
-    mixed = solver.mixed
-    # the FP64 kernels' steps are long: their multipole items stay automatic
-    items = MP_ITEMS if solver.tree.sizes["precision"] != B.FMM_FP64 else (0,)
-    candidates = [dict(mono_subgrids=nb, ctas_per_sm=cap, dataflow=df, mp_pair_targets=pt,
-                       mp_items=it)
-                  for nb, cap, df, pt, it in itertools.product(MONO_SUBGRIDS, CTAS_PER_SM,
-                                                               DATAFLOW, PAIR_TARGETS, items)
-                  if (mixed or (nb != 4 and pt == 0)) and not (pt and it == 2)]
     stream = torch.cuda.current_stream()
 
     def runner(cand):
@@ -79,7 +89,9 @@ def tune(solver, reps=5, verbose=False, flush=None, graph=True):
         return a.elapsed_time(b)
 
     results = []
-    for cand in candidates:
+    sms = torch.cuda.get_device_properties(stream.device).multi_processor_count
+    for cand in candidates(solver.tree.sizes["precision"], getattr(solver, "order", 3),
+                           solver.tree.stats["work_items"][0], sms):
         g, run = runner(cand)
         times = [timed(run) for _ in range(reps)]
         del g

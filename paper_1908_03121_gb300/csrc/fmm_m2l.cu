@@ -2010,7 +2010,7 @@ cudaError_t launch_mono(const KParams &K, size_t wbytes, int sms, int cap, cudaS
 
 // the wide types' monopole kernel
 template <typename T>
-cudaError_t launch_mono_wide(const fmm_tree_s *t, const KParams &K, int sms, cudaStream_t s)
+cudaError_t launch_mono_wide(const fmm_tree_s *t, const KParams &K, int sms, int cap, cudaStream_t s)
 {
     MonoWParams P{};
     P.info = K.info;
@@ -2034,7 +2034,7 @@ cudaError_t launch_mono_wide(const fmm_tree_s *t, const KParams &K, int sms, cud
     if (e != cudaSuccess) return e;
     if (planes) {
         P.n_items = 4 * K.n_items;
-        const int g = persistent_grid(mono_wide_kernel<T, 1>, bytes, P.n_items, sms, 0, 128);
+        const int g = persistent_grid(mono_wide_kernel<T, 1>, bytes, P.n_items, sms, cap, 128);
         mono_wide_kernel<T, 1><<<g, 128, bytes, s>>>(P);
     } else {
         mono_wide_kernel<T, 4><<<std::min(P.n_items, sms), 512, bytes, s>>>(P);
@@ -2211,7 +2211,7 @@ cudaError_t launch_all(const fmm_tree_s *t, void *L, float *Lc, double *dL1, cud
                 : nb == 2 ? launch_mono<2>(K, wbytes, sms, cap, s)
                           : launch_mono<4>(K, wbytes, sms, cap, s);
         } else {
-            e = launch_mono_wide<T>(t, K, sms, s);
+            e = launch_mono_wide<T>(t, K, sms, cap, s);
         }
         timing_end(t, s);
         ++nl;
