@@ -147,7 +147,8 @@ typedef struct {
     int64_t stencil_far;             /* well-separated offsets per parity */
     int64_t stencil_near;            /* near offsets per parity */
     int64_t stencil_union;           /* distinct offsets over the 8 parities */
-    double flops_per_interaction[4]; /* operation count of one interaction */
+    double flops_per_interaction[4]; /* operations of one interaction as the precision's
+                                        kernels evaluate it (FMM_DFLOAT: in double-float) */
     int64_t work_items[4];           /* nodes handled by each same-level kernel:
                                         multipole, monopole, monopole<-multipole, root */
     int64_t kernel_interactions[4];  /* interactions evaluated by each of those kernels */

@@ -414,11 +414,32 @@ static void slot_tables(const fmm_tree_s *t, std::vector<int64_t> &tab)
 static const double kFlops[4] = {240.0, 176.0, 8.0, 199.0};
 static const double kFlops2[4] = {125.0, 107.0, 8.0, 102.0};
 // The FP64 and double-float kernels sum moments of the separations instead
-// (fmm_wide.cuh): multipole<-monopole 29 + 33 fused (95), multipole<-multipole
-// three more for the offset and 85 for the moments (183), monopole<-multipole
-// 113; order 2: 62, 103 and 65.
-static const double kFlopsWide[4] = {183.0, 95.0, 8.0, 113.0};
-static const double kFlopsWide2[4] = {103.0, 62.0, 8.0, 65.0};
+// (fmm_wide.cuh), operations and fused multiply-adds (two each): separation 6
+// (from a leaf source, or of a leaf target, 3); powers and products of its
+// components 17 + 5 fused; a refined target's sums 10 + 32; a leaf source's
+// orders 0-1 2 + 3, a refined source's 34 + 23 moments, orders 0-1 and
+// correction (91); at order 2 16 + 5, 5 + 17 and 20 + 13 (46).  The
+// monopole<-monopole count follows from the transforms (wide_mono_flops).
+static const double kFlopsWide[4] = {198.0, 112.0, 0.0, 122.0};
+static const double kFlopsWide2[4] = {117.0, 76.0, 0.0, 76.0};
+
+// Operations per cell pair of the wide monopole<-monopole kernel
+// (fmm_mono_wide.cuh) on a block of 2 x 2 x 2 target cells, per pair of a
+// complete stencil: the weights' products, the sums over signs, the transforms
+// of the window's blocks (a node's window has (4 + 2 R)^3 for its 64) and of the
+// four components, and the own block.
+static double wide_mono_flops(const fmm_tree_s *t)
+{
+    double ops = 2.0 * double(t->orbit_coef.size() - 8);
+    for (size_t i = 0; i < t->orbits.size(); i += 4) {
+        const int mask = t->orbits[i + 3], axes = (mask & 1) + ((mask >> 1) & 1) + (mask >> 2);
+        ops += 8.0 * axes * (1 << axes);
+    }
+    const double edge = 4.0 + (t->plan.reach - 1);
+    ops += 24.0 * edge * edge * edge / 64.0 + 4.0 * (8 * 7 + 24);
+    ops += 2.0 * (8 * 7 + 3 * 8 * 4) + 4.0 * 8;
+    return ops / (8.0 * (t->plan.n_far[0] + t->plan.n_near[0]));
+}
 
 // Monopole<-multipole work as pair lists: for every cell of a leaf node next
 // to a refined node, the stencil entries whose source cell is refined, each
@@ -910,6 +931,7 @@ int fmm_get_stats(fmm_tree_t t, fmm_stats *o)
         o->interactions[k] = P.interactions[k];
         o->flops_per_interaction[k] = flops[k];
     }
+    if (t->cfg.precision != FMM_MIXED) o->flops_per_interaction[2] = wide_mono_flops(t);
     o->stencil_far = P.n_far[0];
     o->stencil_near = P.n_near[0];
     o->stencil_union = P.stencil_union;
