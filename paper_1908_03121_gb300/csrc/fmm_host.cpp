@@ -274,6 +274,14 @@ static void build_stencils(fmm_tree_s *t)
         t->stencil_f[4 * i + 2] = float(e.oz);
         std::memcpy(&t->stencil_f[4 * i + 3], &e.woff, sizeof(float));
     }
+    P.stencil_union = 0;
+    for (char c : in_union) P.stencil_union += c;
+    // the opening test on an integer squared offset n, as a threshold: the
+    // smallest n that is well separated (kernels compare integers only)
+    // (the same expression as well_separated on o2 = far_o2)
+    P.far_o2 = 1;
+    while (!(theta * theta * double(P.far_o2) > 1.0)) ++P.far_o2;
+    if (t->cfg.precision != FMM_MIXED) return;         // (build_orbits)
     // monopole kernel: parity 0's weights, every parity in parity 0's order
     t->coef32.assign(size_t(P.ent_stride) * 4, 0.f);
     t->mono_woff.assign(size_t(8) * P.ent_stride + size_t(4) * P.ent_stride, 0);
@@ -297,13 +305,6 @@ static void build_stencils(fmm_tree_s *t)
         }
     }
     std::memcpy(&t->mono_woff[size_t(8) * P.ent_stride], woff16.data(), woff16.size() * sizeof(uint16_t));
-    P.stencil_union = 0;
-    for (char c : in_union) P.stencil_union += c;
-    // the opening test on an integer squared offset n, as a threshold: the
-    // smallest n that is well separated (kernels compare integers only)
-    // (the same expression as well_separated on o2 = far_o2)
-    P.far_o2 = 1;
-    while (!(theta * theta * double(P.far_o2) > 1.0)) ++P.far_o2;
 }
 
 // The wide types' monopole<-monopole weights (fmm_mono_wide.cuh): near parent
@@ -314,6 +315,18 @@ static void build_stencils(fmm_tree_s *t)
 // stored for a = q xor b xor e_c, q over the subsets of the mask (zero for
 // the other q by symmetry).  Behind them the weights within a block: c = 0 and
 // an axis c for cells apart in one, two and three axes (and a zero).
+// a sum of doubles as hi + lo, |lo| <= ulp(hi) / 2
+struct Pair {
+    double hi, lo;
+};
+static Pair sum(Pair a, Pair b)
+{
+    const double s = a.hi + b.hi, v = s - a.hi;
+    const double lo = ((a.hi - (s - v)) + (b.hi - v)) + (a.lo + b.lo);
+    const double hi = s + lo;
+    return {hi, lo - (hi - s)};
+}
+
 static void build_orbits(fmm_tree_s *t)
 {
     const int R = int(std::floor(1.0 / t->cfg.theta));
@@ -338,17 +351,18 @@ static void build_orbits(fmm_tree_s *t)
                             mono_coef(ox, oy, oz, w[p][s]);
                         }
                     // both transforms by butterflies over the six bits of
-                    // (p, s), in long double
-                    long double K[64][4];
+                    // (p, s), in pairs of doubles (the same on every host;
+                    // long double is 64 bits on one and software on another)
+                    Pair K[64][4];
                     for (int i = 0; i < 64; ++i)
-                        for (int c = 0; c < 4; ++c) K[i][c] = w[i >> 3][i & 7][c];
+                        for (int c = 0; c < 4; ++c) K[i][c] = {w[i >> 3][i & 7][c], 0.0};
                     for (int bit = 1; bit < 64; bit <<= 1)
                         for (int i = 0; i < 64; ++i) {
                             if (i & bit) continue;
                             for (int c = 0; c < 4; ++c) {
-                                const long double u = K[i][c], v = K[i | bit][c];
-                                K[i][c] = u + v;
-                                K[i | bit][c] = u - v;
+                                const Pair u = K[i][c], v = K[i | bit][c];
+                                K[i][c] = sum(u, v);
+                                K[i | bit][c] = sum(u, {-v.hi, -v.lo});
                             }
                         }
                     for (int b = 0; b < 8; ++b)
@@ -356,7 +370,7 @@ static void build_orbits(fmm_tree_s *t)
                             if (q & ~mask) continue;
                             for (int c = 0; c < 4; ++c) {
                                 const int a = q ^ b ^ (c == 0 ? 0 : 1 << (c - 1));
-                                t->orbit_coef.push_back(double(K[8 * a + b][c] / 64.0L));
+                                t->orbit_coef.push_back(K[8 * a + b][c].hi / 64.0);
                             }
                         }
                 }

@@ -2,7 +2,8 @@
 // launches, which keeps count of what each stream has been given and of what it
 // waits for.  For every launch of fmm_m2l and fmm_step in turn, that launch
 // fails; whatever was enqueued by then, on either stream, must be ordered
-// before what the caller enqueues on the stream next.
+// before what the caller enqueues on the stream next.  With an argument: prints
+// the monopole weights of the FP64 kernels at that opening angle.
 #include <cstdio>
 #include <cstdlib>
 #include <map>
@@ -73,7 +74,7 @@ cudaError_t launch_force_sums(const fmm_tree_s *, double *, cudaStream_t s) { re
 }  // namespace fmm
 
 // a root, its 8 children, and with levels = 3 theirs
-static fmm_tree_t build(int levels)
+static fmm_tree_t build(int levels, double theta = 0.5, int precision = FMM_MIXED)
 {
     std::vector<fmm_node_desc> d;
     std::vector<int> first;
@@ -94,10 +95,10 @@ static fmm_tree_t build(int levels)
     for (size_t i = 1; i < d.size(); ++i)
         d[size_t(d[i].parent)].child[(d[i].ix & 1) + 2 * (d[i].iy & 1) + 4 * (d[i].iz & 1)] = int(i);
     fmm_config c{};
-    c.theta = 0.5;
+    c.theta = theta;
     c.G = 1.0;
     c.box_size = 1.0;
-    c.precision = FMM_MIXED;
+    c.precision = precision;
     c.max_level = 20;
     fmm_tree_t t = nullptr;
     if (fmm_build_tree(d.data(), int64_t(d.size()), &c, &t) != FMM_OK) {
@@ -107,8 +108,17 @@ static fmm_tree_t build(int levels)
     return t;
 }
 
-int main()
+int main(int argc, char **argv)
 {
+    if (argc > 1) {
+        // the FP64 monopole weights' table at an opening angle
+        fmm_tree_t t = build(2, std::atof(argv[1]), FMM_FP64);
+        std::printf("%zu\n", t->orbits.size() / 4);
+        for (int32_t v : t->orbits) std::printf("%d\n", v);
+        for (double v : t->orbit_coef) std::printf("%a\n", v);
+        fmm_destroy_tree(t);
+        return 0;
+    }
     int bad = 0, tried = 0;
     alignas(16) static double buf[2];
     float f;
