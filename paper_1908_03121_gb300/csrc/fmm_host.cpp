@@ -687,7 +687,7 @@ static void free_device(fmm_tree_s *t)
         t->scf_host = nullptr;
     }
     DeviceTables &d = t->dev;
-    void *ptrs[] = {d.info, d.children, d.nbr, d.lists, d.stencil, d.stencil_f, d.coef32, d.mono_woff,
+    void *ptrs[] = {d.info, d.children, d.nbr, d.lists, d.stencil_f, d.coef32, d.mono_woff,
                     d.orbits, d.orbit_coef,
                     d.tree_leaf_off, d.tree_leaf_rows, d.levels, d.levels_df, d.mass, d.mp, d.counters,
                     d.partials, d.chunk_sums, d.up, d.down, d.mx_targets, d.mx_pairs,
@@ -703,7 +703,7 @@ static int upload_tree(fmm_tree_s *t)
     int rc;
     if ((rc = upload(&d.info, t->info)) || (rc = upload(&d.children, t->children)) ||
         (rc = upload(&d.nbr, t->nbr)) || (rc = upload(&d.lists, t->lists)) ||
-        (rc = upload(&d.stencil, t->stencil)) || (rc = upload(&d.stencil_f, t->stencil_f)) ||
+        (rc = upload(&d.stencil_f, t->stencil_f)) ||
         (rc = upload(&d.tree_leaf_off, t->tree_leaf_off)) ||
         (rc = upload(&d.tree_leaf_rows, t->tree_leaf_rows)) || (rc = upload(&d.levels, t->levels)) ||
         (rc = upload(&d.levels_df, t->levels_df)) ||

@@ -72,8 +72,7 @@ struct DeviceTables {
     int32_t *children = nullptr;     // [n][8]
     int32_t *nbr = nullptr;          // [n][27], slot (dx+1)+3(dy+1)+9(dz+1)
     int32_t *lists = nullptr;        // all node-index lists, see Plan offsets
-    StencilEntry *stencil = nullptr; // [8][ent_stride]
-    float *stencil_f = nullptr;      // [8][ent_stride][4] the same entries with the offset
+    float *stencil_f = nullptr;      // [8][ent_stride][4] the stencil's entries, the offset
                                      // as floats (window offset's int bits in the fourth)
     // monopole<-monopole, mixed precision
     float *coef32 = nullptr;         // [ent_stride][4] monopole weights of parity 0

@@ -81,8 +81,7 @@ struct KParams {
     const int32_t *list;
     int32_t n_items;
     int32_t *counter;
-    const StencilEntry *stencil;
-    const float4 *stencil_f;  // the same, offsets as floats, window offset's bits in w
+    const float4 *stencil_f;  // stencil entries: offsets as floats, window offset's bits in w
     const float *coef;       // monopole weights of parity 0 (mixed)
     const int32_t *mono_woff;  // [8][ent_stride] window offsets in parity 0's order, reflected
     const uint16_t *mono_woff16;  // the same, in bytes
@@ -283,22 +282,6 @@ __device__ __forceinline__ T window_index(int idx)
     }
 }
 
-// the moment offset encoded in a window cell, or -1 for a mass
-template <typename T>
-__device__ __forceinline__ int window_decode(T v)
-{
-    if constexpr (kF32<T>) {
-        const int b = __float_as_int(v);
-        return b < 0 ? -1 - b : -1;
-    } else if constexpr (kDF<T>) {
-        const int b = __float_as_int(v.hi);
-        return b < 0 ? -1 - b : -1;
-    } else {
-        const long long b = __double_as_longlong(v);
-        return b < 0 ? int(-1ll - b) : -1;
-    }
-}
-
 // whether a window value is a refined source's moment offset below limit,
 // and that offset: -1 - bits is the offset for a refined source and
 // negative (a large unsigned value) for a mass, whose bits are not
@@ -413,62 +396,35 @@ __device__ __forceinline__ bool window_nonzero(T v)
 }
 
 // Compensated accumulator: float partial sums per chunk, folded into a
-// (hi, lo) pair by TwoSum; in double precision a plain sum.
-template <typename T, int N>
+// (hi, lo) pair by TwoSum.
+template <int N>
 struct Acc {
-    T part[N];
-    T hi[N];
-    T lo[N];
+    float part[N];
+    float hi[N];
+    float lo[N];
     __device__ __forceinline__ void zero()
     {
 #pragma unroll
-        for (int k = 0; k < N; ++k) part[k] = hi[k] = lo[k] = T(0);
+        for (int k = 0; k < N; ++k) part[k] = hi[k] = lo[k] = 0.f;
     }
     __device__ __forceinline__ void flush()
     {
 #pragma unroll
         for (int k = 0; k < N; ++k) {
-            if constexpr (kF32<T>) {
-                float s, e;
-                two_sum(hi[k], part[k], s, e);
-                hi[k] = s;
-                lo[k] += e;
-            } else {
-                hi[k] += part[k];
-            }
-            part[k] = T(0);
+            float s, e;
+            two_sum(hi[k], part[k], s, e);
+            hi[k] = s;
+            lo[k] += e;
+            part[k] = 0.f;
         }
     }
 };
 
-// double-float: every term already lands in a double-float running sum,
-// so there is nothing to fold
-template <int N>
-struct Acc<dfloat, N> {
-    dfloat part[N];
-    __device__ __forceinline__ void zero()
-    {
-#pragma unroll
-        for (int k = 0; k < N; ++k) part[k] = dfloat(0.f);
-    }
-    // the running sums take unnormalised terms (fmadd_u, add_u): restore
-    // the canonical (hi, lo) form every chunk
-    __device__ __forceinline__ void flush()
-    {
-#pragma unroll
-        for (int k = 0; k < N; ++k) part[k] = renorm(part[k]);
-    }
-};
-
 // the (hi, lo) value of accumulator k
-template <typename T, int N>
-__device__ __forceinline__ T acc_hi(const Acc<T, N> &a, int k) { return a.hi[k]; }
 template <int N>
-__device__ __forceinline__ dfloat acc_hi(const Acc<dfloat, N> &a, int k) { return a.part[k]; }
-template <typename T, int N>
-__device__ __forceinline__ T acc_lo(const Acc<T, N> &a, int k) { return a.lo[k]; }
+__device__ __forceinline__ float acc_hi(const Acc<N> &a, int k) { return a.hi[k]; }
 template <int N>
-__device__ __forceinline__ dfloat acc_lo(const Acc<dfloat, N> &, int) { return dfloat(0.f); }
+__device__ __forceinline__ float acc_lo(const Acc<N> &a, int k) { return a.lo[k]; }
 
 // Float accumulator whose (hi, lo) pairs live in shared memory, in this
 // thread's column of a [components][2][threads] array: only the chunk sums
@@ -780,7 +736,7 @@ __device__ __forceinline__ void acc_mp(float Rx, float Ry, float Rz, const Src<f
 // (ORDER = 2: L0 -= M0 D0 + B2.D2, L1 -= M0 D1, S_i -= B2 . D3[i, .])
 template <int ORDER = 3>
 __device__ __forceinline__ void acc_mx(float Rx, float Ry, float Rz, const Src<float> &s,
-                                       Acc<float, 4> &L, Acc<float, 3> &S)
+                                       Acc<4> &L, Acc<3> &S)
 {
     DTraceless D{};
     D.eval<ORDER == 3>(Rx, Ry, Rz);
@@ -865,9 +821,9 @@ __device__ __forceinline__ void mx_target(const KParams &P, int t)
     const int x = tg.y & 7, y = (tg.y >> 3) & 7, z = tg.y >> 6;
     const int p = (x & 1) + 2 * (y & 1) + 4 * (z & 1);
     const float4 *ent = P.stencil_f + p * P.ent_stride;   // float offsets: no conversions
-    using Low = std::conditional_t<kF32<T>, Acc<float, 4>, WideChunked<T, WideLow<T, ORDER>>>;
+    using Low = std::conditional_t<kF32<T>, Acc<4>, WideChunked<T, WideLow<T, ORDER>>>;
     Low L;
-    Acc<float, 3> S;                               // float only
+    Acc<3> S;                               // float only
     L.zero();
     S.zero();
     int done = 0;
@@ -1564,7 +1520,7 @@ __global__ void __launch_bounds__(kThreads, 2) mp2_kernel(KParams P)
 // offsets, folded into the shared-memory loads)
 template <int NB, int WSTRIDE, int DZ1>
 __device__ __forceinline__ void mono_entry(const float *src, const float *coef, int e,
-                                           Acc<float, 4> (&A)[NB], Acc<float, 4> (&B)[NB])
+                                           Acc<4> (&A)[NB], Acc<4> (&B)[NB])
 {
     const float4 c4 = *reinterpret_cast<const float4 *>(coef + 4 * e);
     const float c[4] = {c4.x, c4.y, c4.z, c4.w};
@@ -1647,7 +1603,7 @@ __global__ void __launch_bounds__(kThreads) mono_kernel(KParams P)
         cp_async_commit();
         cp_async_wait_all();
         __syncthreads();
-        Acc<float, 4> A[NB], B[NB];
+        Acc<4> A[NB], B[NB];
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
             A[b].zero();
@@ -1758,8 +1714,8 @@ __global__ void __launch_bounds__(kRootThreads) root_kernel(KParams P)
     const int ax = cell & 7, ay = (cell >> 3) & 7, az = cell >> 6;
     float dA[3] = {0.f, 0.f, 0.f}, a3A[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (!leaf) load_target<ORDER>(P, ti.mp_row, parity_index(ax, ay, az), dA, a3A);
-    Acc<float, 16> L;
-    Acc<float, 3> S;
+    Acc<16> L;
+    Acc<3> S;
     L.zero();
     S.zero();
     int done = 0;
@@ -2090,7 +2046,6 @@ cudaError_t launch_all(const fmm_tree_s *t, void *L, float *Lc, double *dL1, cud
     KParams P{};
     P.info = d.info;
     P.nbr = d.nbr;
-    P.stencil = d.stencil;
     P.stencil_f = reinterpret_cast<const float4 *>(d.stencil_f);
     P.coef = d.coef32;
     P.n_far = Pl.n_far[0];
