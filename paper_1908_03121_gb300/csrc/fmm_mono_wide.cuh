@@ -28,8 +28,8 @@
 // (direct form).  A level-6 binary
 // (4572 leaf nodes), whole step: FP64 24.1 -> 20.9 ms (this kernel 4.4 -> 1.2),
 // double-float 5.43 -> 4.79 ms; 8 leaf nodes in FP64, step 318 -> 207 us.  (The
-// own block's products cost 0.13 and 0.07 ms of a level-6 step, 2 us of 8 leaf
-// nodes'.)
+// own block's products, spread over all threads, cost 0.11 and 0.04 ms of a level-6
+// step, 1 us of 8 leaf nodes'; by the 128 threads of the exchange 0.13, 0.07 and 2.)
 // A thread has one target block and one b (the same for a whole warp, so the
 // weights are broadcasts); its 32 sums A[q][c] belong to a = q xor b xor e_c and
 // meet those of the other b at the end, through shared memory, in a fixed
@@ -71,12 +71,12 @@ __host__ __device__ constexpr int mono_wide_window(int reach, int planes)
     return kMonoWPitch * (4 + 2 * reach) * (planes + 2 * reach);
 }
 
-// shared memory: the window (later the sums' exchange buffer, two components
-// of 8 values of every thread) and the weights
+// shared memory: the window (later the exchange buffer, two components of 8 sums
+// and one own-block value of every thread) and the weights
 template <typename T>
 size_t mono_wide_smem(int reach, int planes, int n_coef)
 {
-    const size_t window = size_t(8) * mono_wide_window(reach, planes), fold = size_t(2) * 8 * 128 * planes;
+    const size_t window = size_t(8) * mono_wide_window(reach, planes), fold = size_t(2) * 9 * 128 * planes;
     return ((window > fold ? window : fold) + size_t(n_coef)) * sizeof(T);
 }
 
@@ -131,27 +131,20 @@ __device__ __forceinline__ void mono_wide_orbits(const MonoWParams &P, const T *
         for (int k = 0; k < 4; ++k) A[q][k] = renorm(A[q][k]);
 }
 
-// the own block's terms of one component: ec = 0 for L0, else the axis's bit (a
-// first-order weight is nonzero between cells apart in that axis only, and its
-// sign is the target's side of it)
-template <typename T>
-__device__ __forceinline__ void mono_wide_own(const T m[8], const T *near, int ec, T (&o)[8])
+// the own block's terms of one component for target child p, from the masses
+// m[x] of its children p xor x: EC = 0 for L0, else the axis's bit (a first-order
+// weight is nonzero between cells apart in that axis only, and its sign is the
+// target's side of it)
+template <typename T, int EC>
+__device__ __forceinline__ T mono_wide_own(const T m[8], const T *near, int p)
 {
-    T v[8];
+    T v = T(0);
 #pragma unroll
-    for (int p = 0; p < 8; ++p) v[p] = T(0);
-#pragma unroll
-    for (int x = 1; x < 8; ++x) {
-        if (ec != 0 && !(x & ec)) continue;
-        const T w = near[(ec ? 4 : 0) + (x & 1) + ((x >> 1) & 1) + (x >> 2) - 1];
-#pragma unroll
-        for (int p = 0; p < 8; ++p) v[p] = fmadd_u(w, m[p ^ x], v[p]);
-    }
-#pragma unroll
-    for (int p = 0; p < 8; ++p) {
-        const T a = renorm(v[p]);
-        o[p] += (p & ec) ? -a : a;
-    }
+    for (int x = 1; x < 8; ++x)
+        if (EC == 0 || (x & EC))
+            v = fmadd_u(near[(EC ? 4 : 0) + (x & 1) + ((x >> 1) & 1) + (x >> 2) - 1], m[x], v);
+    v = renorm(v);
+    return (p & EC) ? -v : v;
 }
 
 template <typename T, int PLANES>
@@ -162,7 +155,7 @@ __global__ void __launch_bounds__(128 * PLANES, PLANES == 4 ? 1 : 4) mono_wide_k
     __shared__ int s_nbr[27], s_item;
     const int R = P.reach, E = 4 + 2 * R, EZ = PLANES + 2 * R, pz = kMonoWPitch * E;
     const int plane = pz * EZ;                           // blocks of one b
-    const int fold = 2 * 8 * 8 * blocks;
+    const int sums = 2 * 8 * 8 * blocks, fold = sums + 2 * 8 * blocks;
     T *W = reinterpret_cast<T *>(smem_raw);
     T *s_coef = W + (8 * plane > fold ? 8 * plane : fold);
     const T *mass = static_cast<const T *>(P.mass);
@@ -232,7 +225,15 @@ __global__ void __launch_bounds__(128 * PLANES, PLANES == 4 ? 1 : 4) mono_wide_k
         // components 0-1, then 2-3, one thread per (component, target block)
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
+            // the own block's terms for child b of this thread's block
+            T m[8];
+            const T *at = mass + size_t(node) * NCELL + tx + 4 * ty + 16 * (z0 + tz);
+#pragma unroll
+            for (int x = 1; x < 8; ++x) m[x] = ldg_t(at + 64 * (b ^ x));
+            const T *near = s_coef + P.n_coef - 8;
             __syncthreads();                           // the window (the first half) is done with
+            W[sums + b * blocks + block] = half ? mono_wide_own<T, 2>(m, near, b) : mono_wide_own<T, 0>(m, near, b);
+            W[sums + (8 + b) * blocks + block] = half ? mono_wide_own<T, 4>(m, near, b) : mono_wide_own<T, 1>(m, near, b);
 #pragma unroll
             for (int k = 0; k < 2; ++k)
 #pragma unroll
@@ -259,11 +260,8 @@ __global__ void __launch_bounds__(128 * PLANES, PLANES == 4 ? 1 : 4) mono_wide_k
                         o[a] = u + v;
                         o[a | ax] = u - v;
                     }
-                T m[8];
-                const T *at = mass + size_t(node) * NCELL + (t & 3) + 4 * ((t >> 2) & 3) + 16 * (z0 + (t >> 4));
 #pragma unroll
-                for (int s = 0; s < 8; ++s) m[s] = ldg_t(at + 64 * s);
-                mono_wide_own<T>(m, s_coef + P.n_coef - 8, ec, o);
+                for (int p = 0; p < 8; ++p) o[p] += W[sums + (8 * k + p) * blocks + t];
                 const int cell = 2 * (t & 3) + 16 * ((t >> 2) & 3) + 128 * (z0 + (t >> 4));
 #pragma unroll
                 for (int p = 0; p < 8; ++p)
