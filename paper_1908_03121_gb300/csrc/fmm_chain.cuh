@@ -8,14 +8,16 @@
 // still reads: it waits until the kernel before has completed with all its
 // stores visible, then lets the next one start its own prologue.  A kernel that
 // calls it before its predecessor's completion has waited for that one too, so
-// the order holds along the whole chain.  What earlier kernels write changes
-// while such a kernel is resident, so its parameters carry no __restrict__ but
-// for the tables: the compiler could move accesses through it before the wait,
-// and with const use the non-coherent load path (tests/test_chained_kernels.py).
-// Functions called after chain_begin() may promise it again for what they store.  Upward pass of a level-6 binary 107 ->
-// 93 us, downward pass and forces 257 -> 236 us, step of 73 sub-grids 157 -> 148
-// us (of which the queue reset in P2M instead of a memset, and the leaf pass on
-// the main stream instead of behind two event waits, are part).
+// the order holds along the whole chain.
+// What earlier kernels write changes while such a kernel is resident, so its
+// parameters carry no __restrict__ but for the tables: the compiler could move
+// accesses through it before the wait, and with const use the non-coherent load
+// path (tests/test_chained_kernels.py).  Functions called after chain_begin()
+// may promise it again for what they store.
+// Upward pass of a level-6 binary 107 -> 93 us, downward pass and forces 257 ->
+// 236 us, step of 73 sub-grids 157 -> 148 us (of which the queue reset in P2M
+// instead of a memset, and the leaf pass on the main stream instead of behind two
+// event waits, are part).
 #pragma once
 
 #include <cuda_runtime.h>

@@ -238,8 +238,8 @@ __global__ void __launch_bounds__(kScfThreads) scf_hmax_kernel(const NodeInfo *_
 
 // u^n, u > 0; half: 2 n where that is a whole number up to 16 (the usual
 // indices: products and a square root, a fifth of pow's FP64 operations).  What
-// each rounding leaves out is carried along, so that the result is as near as
-// pow's (0.6 units in the last place at n = 8, 2.5 without)
+// each rounding leaves out is carried along, so that the result is within one
+// unit in the last place, as pow's is (2.6 without, at n = 7.5)
 __device__ __forceinline__ double power(double u, double n, int half)
 {
     if (half == 0) return pow(u, n);
